@@ -94,8 +94,8 @@ typedef struct gs_camera {
  * row by row its ellipse).  Both give the same images and derivatives; 1 gives
  * fewer pairs.
  * batch: records a tile's block stages in shared memory per step of its list in
- * the blends (gs_raster_fwd, gs_raster_bwd, gs_hvp_diag): 0 for one per thread,
- * else a multiple of 32 from 32 to 512.  It changes speed, not results. */
+ * the forward blend (gs_raster_fwd): 0 for one per thread, else a multiple of 32
+ * from 32 to 512.  It changes speed, not results. */
 typedef struct gs_frame {
   int32_t n_views, width, height, tile_w, tile_h, footprint_bins, batch;
 } gs_frame;

@@ -7,21 +7,20 @@
 //                  in the same sweep, the Gauss-Newton products J^T diag(w) J z_k
 //   gs_hvp_diag    the Gauss-Newton products alone
 //
-// One CTA renders one tile of one view with two pixels per thread; each warp
-// owns an 8 x 8 pixel block.  The tile's splat records are staged through
-// shared memory in batches (one record per pixel of the tile), each record moved
-// by a 48-byte TMA bulk copy (cp.async.bulk, no multicast) completing on an
+// Forward: one CTA renders one tile of one view with two pixels per thread;
+// each warp owns an 8 x 8 pixel block.  The tile's splat records are staged
+// through shared memory in batches (one record per pixel of the tile), each
+// record moved by a TMA bulk copy (cp.async.bulk, no multicast) completing on an
 // mbarrier, double-buffered so that the next batch lands while the current one
 // is blended.  Per batch every splat gets a mask of the warp blocks its
 // alpha >= 1/255 footprint can reach, and each warp walks only its own visible
-// splats (one ballot per 32).  In the reverse pass the warps release the two
-// buffers one by one instead of meeting at block barriers, and the last warp
-// out refills a buffer.  The reverse pass walks the list back to front,
-// recovers T_i = T_{i+1} / (1 - a_i) from the final transmittance (nothing per
-// pair is stored), sums each splat's 9 x streams partial derivatives over the
-// warp's 64 pixels with a reduction that ends in quads, and adds them with float4
-// atomics.  The projection's reverse pass (2-D cotangents -> 11 + 3K parameter
-// rows) runs one thread per Gaussian and sums over the views.
+// splats (one ballot per 32).  Reverse: one warp per CTA and 8 x 8 block.  It
+// walks the list back to front, recovers T_i = T_{i+1} / (1 - a_i) from the final
+// transmittance (nothing per pair is stored), merges each splat's 9 x streams
+// partial derivatives over the block's 64 pixels, four splats at a time, and
+// adds them with float4 reductions.  The projection's reverse pass (2-D
+// cotangents -> 11 + 3K parameter rows) runs one thread per Gaussian and sums
+// over the views.
 #include "common.cuh"
 
 namespace gs {
@@ -39,6 +38,27 @@ static_assert(sizeof(Rec) == 48, "record size");
 __device__ __forceinline__ float splat_power(const Rec& r, float dx, float dy) {
   const float q = __fmaf_rn(r.b.x, __fmul_rn(dy, dy), __fmul_rn(r.a.z, __fmul_rn(dx, dx)));
   return __fmaf_rn(-0.5f, q, -__fmul_rn(r.a.w, __fmul_rn(dx, dy)));
+}
+
+__device__ __forceinline__ float ex2_approx(float x) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+// The splat at a thread's two pixels, which share their column: dx and the
+// negated centres -py of the pair give dy, then power and exp(power) per pixel.
+// Each lane rounds exactly as splat_power does.
+__device__ __forceinline__ void splat_gauss2(const Rec& r, float pxc, f32x2 npy, float& dx, f32x2& dy,
+                                             float (&power)[2], f32x2& G) {
+  dx = __fsub_rn(r.a.x, pxc);
+  dy = add2(dup2(r.a.y), npy);
+  const f32x2 q = fma2(dup2(r.b.x), mul2(dy, dy), dup2(__fmul_rn(r.a.z, __fmul_rn(dx, dx))));
+  const f32x2 pw = fma2(dup2(-0.5f), q, mul2(dup2(-r.a.w), mul2(dup2(dx), dy)));
+  unpack2(pw, power[0], power[1]);
+  // e^p = 2^(p log2 e)
+  float l[2];
+  unpack2(mul2(pw, dup2(1.4426950408889634f)), l[0], l[1]);
+  G = pack2(ex2_approx(l[0]), ex2_approx(l[1]));
 }
 
 // 1: the blends also test a splat's footprint ellipse itself, not only its
@@ -121,9 +141,6 @@ constexpr int kBatchPerThread = GS_BATCH_PER_THREAD;
 constexpr int kFwdBatchDiv = GS_FWD_BATCH_DIV;
 __host__ __device__ __forceinline__ int fwd_batch(const gs_frame& fr, int nthr) {
   return fr.batch ? fr.batch : kBatchPerThread * nthr / kFwdBatchDiv;
-}
-__host__ __device__ __forceinline__ int bwd_batch(const gs_frame& fr, int nthr) {
-  return fr.batch ? fr.batch : kBatchPerThread * nthr;
 }
 // Minimum resident CTAs per SM requested for the forward kernel (0: none), for
 // blocks of 128 threads; blocks of NT threads (tiles of 2 NT pixels) request
@@ -437,54 +454,16 @@ __global__ void GS_FWD_BOUNDS(NT) raster_fwd_kernel(const float4* __restrict__ r
 }
 
 // ------------------------------------------------------------------ reverse
-// The reverse pass stages its batches in a ring of kBwdStages buffers that the
-// warps release one by one, instead of block barriers per batch: a warp moves
-// on to the next batch as soon as it has landed and tests only its own block's
-// visibility, so a warp with little work in a batch does not wait for the
-// others.  The last warp to release a buffer refills it with the batch
-// kBwdStages further on.  At 7 CTAs per SM three stages measured fastest (at
-// 8 CTAs per SM two did: deeper rings took shared memory from L1 or from
-// resident CTAs).
-#ifndef GS_BWD_STAGES
-#define GS_BWD_STAGES 3
-#endif
-constexpr int kBwdStages = GS_BWD_STAGES;
-// ring header: one mbarrier and one release counter per stage, 16-byte aligned
-constexpr size_t kBwdRingHdr = (kBwdStages * (sizeof(uint64_t) + sizeof(uint32_t)) + 15) / 16 * 16;
-__host__ __device__ constexpr size_t bwd_smem_bytes(int batch) {
-  return kBwdRingHdr + (size_t)kBwdStages * batch * (sizeof(Rec) + sizeof(uint32_t)) +
-         ((size_t)kBwdStages * batch + 15) / 16 * 16;  // and the staged block masks, one byte per record
-}
-
-// The calling warp fills ring stage s with batch b of the list (use u of the
-// ring): its lanes store the Gaussian indices (and, given the forward pass's
-// block masks, each record's mask byte) and issue one bulk copy per record,
-// then lane 0 records u as the stage's last fill and arms the stage's barrier
-// with the byte count.  The copies may complete before that arrival (the
-// phase cannot complete while the arrival is pending), and the arrival releases
-// the index stores to the warps that wait on the phase.
-__device__ __forceinline__ void stage_batch_warp(int s, int u, int b, int batch, uint32_t start, int n, int view,
-                                                 int n_pad, const uint32_t* __restrict__ vals,
-                                                 const float4* __restrict__ rec, const uint8_t* __restrict__ masks,
-                                                 Rec* buf, uint32_t* s_idx, uint8_t* s_bits, uint64_t* full,
-                                                 int* fill_use) {
-  const int lane = threadIdx.x & 31;
-  const int cnt = min(batch, n - b * batch);
-  __syncwarp();
-  fence_proxy_async();  // the ring slot's earlier reads come before the copies' writes
-  for (int q = lane; q < cnt; q += 32) {
-    const uint32_t gi = __ldg(vals + start + (uint32_t)(b * batch + q));
-    s_idx[s * batch + q] = gi;
-    if (masks) s_bits[s * batch + q] = __ldg(masks + start + (uint32_t)(b * batch + q));
-    bulk_g2s(&buf[s * batch + q], rec + 3 * ((size_t)view * n_pad + gi), sizeof(Rec), &full[s]);
-  }
-  __syncwarp();
-  if (lane == 0) {
-    fill_use[s] = u;
-    mbar_arrive_expect_tx(&full[s], (uint32_t)(cnt * (int)sizeof(Rec)));
-  }
-}
-
+// The reverse pass runs one warp per CTA, on one 8 x 8 pixel block: the blocks of
+// a tile need nothing from one another, so a warp starts at its own last
+// contributor, stages only the splats its block can see (asynchronous copies
+// into two buffers of 32, whole chunks of 32 list positions at a time) and frees
+// its place on the SM as soon as its own walk ends.  As CTAs of a tile's four
+// warps sharing a ring of TMA-staged batches, staging and the waits for the
+// tile's slowest warp took 0.6 of the 2.6 ms of the blend (1M Gaussians, 8 views
+// of 1080p, two probes): the call went from 3.23 to 2.78 ms, and from 3.40 ms
+// with the warp-wide reduction per splat (no probe 2.29 -> 1.52 ms, one 3.10 ->
+// 2.14 ms; 100k Gaussians, 1297 x 840, one probe 0.66 -> 0.36 ms).
 // True if the splat can reach alpha >= 1/255 at some pixel centre of the 8 x 8
 // block whose first pixel centre is (x0, y0) (the test of warp_block_mask for
 // one block).
@@ -496,76 +475,22 @@ __device__ __forceinline__ bool block_sees(const Rec& r, float x0, float y0) {
          (!GS_EXACT_BLOCK_TEST || footprint_meets_block(r, x0, y0));
 }
 
-// 1: skip the reverse of a lane's first or second pixel when no lane of the
-// warp blends the splat at that pixel.
-#ifndef GS_BWD_SKIP_IDLE_ROW
-#define GS_BWD_SKIP_IDLE_ROW 1
+// Minimum resident CTAs (warps) per SM requested from the compiler for the
+// reverse kernel, by the number of cotangent streams: without a probe 32 (64
+// registers, the most CTAs an SM holds; 28: 1.548 against 1.518 ms per call of
+// 1M Gaussians, 8 views of 1080p), with one 24 (80 registers; 20: 2.320 against
+// 2.144 ms), with two 18 (96 registers and no spills; 16: 2.840, 20: 2.801, 21:
+// 2.877 against 2.775 ms).
+#ifndef GS_BWD_MB1
+#define GS_BWD_MB1 32
 #endif
-// A splat that at most this many lanes of a warp blend is added by those lanes
-// one by one (each its own row of partial derivatives, as float4 atomics)
-// instead of through the warp-wide reduction (0: always reduce).
-#ifndef GS_BWD_SPARSE_LANES
-#define GS_BWD_SPARSE_LANES 8
+#ifndef GS_BWD_MB2
+#define GS_BWD_MB2 24
 #endif
-constexpr int kBwdSparseLanes = GS_BWD_SPARSE_LANES;
-// Minimum resident CTAs per SM requested from the compiler for the reverse
-// kernel (0: no request).
-#ifndef GS_BWD_MIN_BLOCKS
-#define GS_BWD_MIN_BLOCKS 7
+#ifndef GS_BWD_MB3
+#define GS_BWD_MB3 18
 #endif
-#if GS_BWD_MIN_BLOCKS > 0
-#define GS_BWD_BOUNDS(NT) __launch_bounds__(NT, (GS_BWD_MIN_BLOCKS * 128) / (NT))
-#else
-#define GS_BWD_BOUNDS(NT) __launch_bounds__(NT)
-#endif
-
-// Warp sums of v[0..31] delivered as quads: afterwards every lane L with
-// (L & 3) == 0 holds in q[0..3] the warp-wide sums of v[L .. L+3].  Three
-// reduce-scatter stages (lane bits 4, 3, 2) then a butterfly over bits 1, 0.
-__device__ __forceinline__ void warp_reduce_quads32(float (&v)[32], float (&q)[4]) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int o = 16; o >= 4; o >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int i = 0; i < o; ++i) {
-      const float send = up ? v[i] : v[i + o];
-      const float keep = up ? v[i + o] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    float x = v[i];
-    x += __shfl_xor_sync(0xffffffffu, x, 1);
-    x += __shfl_xor_sync(0xffffffffu, x, 2);
-    q[i] = x;
-  }
-}
-// Same for v[0..15] (slots 16..31 unused): lanes L < 16 with (L & 3) == 0 hold
-// the sums of v[L .. L+3].
-__device__ __forceinline__ void warp_reduce_quads16(float (&v)[32], float (&q)[4]) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], 16);
-#pragma unroll
-  for (int o = 8; o >= 4; o >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int i = 0; i < o; ++i) {
-      const float send = up ? v[i] : v[i + o];
-      const float keep = up ? v[i + o] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    float x = v[i];
-    x += __shfl_xor_sync(0xffffffffu, x, 1);
-    x += __shfl_xor_sync(0xffffffffu, x, 2);
-    q[i] = x;
-  }
-}
+__host__ __device__ constexpr int bwd_min_blocks(int S) { return S == 1 ? GS_BWD_MB1 : S == 2 ? GS_BWD_MB2 : GS_BWD_MB3; }
 
 // Row stride (floats) of the per-view 2-D cotangents: 9 per stream, padded to
 // whole float4s so that rows can be added and read as vectors.
@@ -579,334 +504,447 @@ __host__ __device__ constexpr int cot_stride(int streams) { return (9 * streams 
 // buffer, a call that stopped between the blend and the projection reverse)
 // makes the next call clear the rows first; the blend marks the rows dirty
 // when it starts.
+constexpr int kLossSlots = GS_BATCH_MAX;
 struct CotHeader {
   uint64_t magic;         // kCotClear while clear_floats is valid
   uint64_t clear_floats;  // leading floats of the rows known to be zero
   uint32_t done_blocks;   // projection-reverse blocks finished in this call
+  uint32_t reserved;
+  double loss[kLossSlots];  // the objective's partial sums: of each view (a batch), or spread over the slots
 };
 constexpr uint64_t kCotClear = 0x9d2c5680a3b1f4e7ull;
 constexpr size_t kCotHeaderBytes = 256;
+static_assert(sizeof(CotHeader) <= kCotHeaderBytes, "workspace header");
 
 // Zero the first 4 n4 floats of the rows unless the header says they are zero;
 // reset the projection reverse's block count.
 __global__ void cot_prepare_kernel(CotHeader* __restrict__ h, float4* __restrict__ cot, size_t n4) {
   const bool clear = h->magic == kCotClear && h->clear_floats >= 4 * n4;
   if (blockIdx.x == 0 && threadIdx.x == 0) h->done_blocks = 0;
+  if (blockIdx.x == 0 && threadIdx.x < kLossSlots) h->loss[threadIdx.x] = 0.0;
   if (clear) return;
   for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n4; k += (size_t)gridDim.x * blockDim.x)
     cot[k] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
+// The objective's sums onto the caller's: one per view of a batch (loss_views),
+// or all slots onto one value (loss_views 0).
+__device__ __forceinline__ void add_loss(const CotHeader* h, float* loss_out, int loss_views) {
+  double all = 0.0;
+  for (int k = 0; k < kLossSlots; ++k) {
+    if (k < loss_views) atomicAdd(loss_out + k, (float)h->loss[k]);
+    all += h->loss[k];
+  }
+  if (loss_views == 0) atomicAdd(loss_out, (float)all);
+}
+// The same where no projection-reverse block runs (no Gaussians).
+__global__ void add_loss_kernel(const CotHeader* h, float* loss_out, int loss_views) { add_loss(h, loss_out, loss_views); }
+
 // End of a projection-reverse block: after every thread's zeroing stores, the
 // last block to finish records that the first `floats` floats are zero.
-__device__ __forceinline__ void cot_mark_clear(CotHeader* h, uint64_t floats) {
+__device__ __forceinline__ void cot_mark_clear(CotHeader* h, uint64_t floats, float* loss_out, int loss_views) {
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0 && atomicAdd(&h->done_blocks, 1u) == gridDim.x - 1) {
     __threadfence();
+    if (loss_out) add_loss(h, loss_out, loss_views);
     h->clear_floats = floats;
     h->magic = kCotClear;
   }
 }
 
-// 1: the reverse recovers T_i with the fast division intrinsic's reciprocal
-// of 1 - alpha (at most 2 ulps off; 1 - alpha lies in [0.01, 1]) instead of
-// the correctly rounded one, whose slower path also costs registers: about
-// 2.5 ulps per recovered step instead of 1, which over the few hundred splats
-// a pixel walks back stays orders of magnitude inside the gradient and
-// curvature tolerances.
-#ifndef GS_BWD_APPROX_RCP
-#define GS_BWD_APPROX_RCP 1
-#endif
-
-// Reverse-pass state of one pixel: the cotangent dL/dC of each stream, the
-// transmittance being recovered back to front, the colour suffix
-// sum_{j>i} c_j a_j T_j, and the list position after its last blended splat.
-template <int S>
-struct BwdPixel {
-  float w[S][3];
-  float T, suf[3];
-  float pxc, pyc;
-  uint32_t nc;
-};
-
-// The reverse of one splat at one pixel: recover T_i = T_{i+1}/(1 - a),
-// dC/da = c T_i - suffix/(1 - a), and store (FIRST) or add, for every stream,
-// the pixel's terms of the splat's cotangent row in v: the moments
-// (dx g, dy g, dx^2 g, dx dy g, dy^2 g) of g = dL/d(power), then dL/do,
-// dL/d(r, g, b).  power = -(A dx^2 + C dy^2)/2 - B dx dy, so dL/dA = -M2/2,
-// dL/dB = -M3, dL/dC = -M4/2, dL/dmx = -(A M0 + B M1), dL/dmy = -(B M0 + C M1).  A pixel the splat is not blended at passes alpha = G = oG = 0: its state
-// stays as it is and it contributes exact zeros, so the pixels of a thread need
-// no branches.  One reciprocal of 1 - a serves the four quotients.
-template <int S, bool FIRST>
-__device__ __forceinline__ void bwd_accumulate(BwdPixel<S>& p, const Rec& r, float dx, float dy, float G, float oG,
-                                               float alpha, float (&v)[32]) {
-#if GS_BWD_APPROX_RCP
-  const float inv = __fdividef(1.f, 1.f - alpha);
-#else
-  const float inv = __frcp_rn(1.f - alpha);
-#endif
-  const float Ti = p.T * inv;
-  const float rgb0 = r.b.z, rgb1 = r.b.w, rgb2 = r.c.x;
-  const float da0 = rgb0 * Ti - p.suf[0] * inv;
-  const float da1 = rgb1 * Ti - p.suf[1] * inv;
-  const float da2 = rgb2 * Ti - p.suf[2] * inv;
-  const float aT = alpha * Ti;
-  p.suf[0] += rgb0 * aT;
-  p.suf[1] += rgb1 * aT;
-  p.suf[2] += rgb2 * aT;
-  p.T = Ti;
-  // a capped alpha has zero derivative: both of its factors vanish at once
-  const bool capped = oG > kAlphaMax;
-  const float ac = capped ? 0.f : alpha, Gc = capped ? 0.f : G;
-  const float dxx = dx * dx, dxy = dx * dy, dyy = dy * dy;
-#pragma unroll
-  for (int s = 0; s < S; ++s) {
-    const float ga = p.w[s][0] * da0 + p.w[s][1] * da1 + p.w[s][2] * da2;
-    const float gp = ga * ac;  // dL/d(power)
-    // the power's partials are linear in the conic, so the warp sums moments of
-    // (dx, dy) and the projection's reverse pass applies the conic
-    const float c[9] = {dx * gp, dy * gp, dxx * gp, dxy * gp, dyy * gp, ga * Gc,
-                        p.w[s][0] * aT, p.w[s][1] * aT, p.w[s][2] * aT};
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-      if constexpr (FIRST) v[9 * s + q] = c[q];
-      else v[9 * s + q] += c[q];
-    }
-  }
+__device__ __forceinline__ float rcp_approx(float x) {  // at most 1 ulp off
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 }
 
-template <int NU, bool GRAD, bool CB, int NT>
-__global__ void GS_BWD_BOUNDS(NT) raster_bwd_kernel(
+// Reverse-pass state of a thread's two pixels: the cotangent dL/dC of each
+// stream, the transmittance being recovered back to front, per stream the
+// negated suffix -sum_{j>i} a_j T_j (w . c_j), and the list position after each
+// pixel's last blended splat.
+template <int S>
+struct BwdPair {
+  f32x2 w[S][3];
+  f32x2 T, nq[S];
+  f32x2 npy;  // negated pixel centres
+  float pxc;
+  uint32_t nc[2];
+};
+
+// p[0..3] += v, p 16-byte aligned: a reduction, which returns nothing (the
+// atomicAdd on a float4 fetches the old value back).
+__device__ __forceinline__ void red_add4(float* p, float4 v) {
+  asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z),
+               "f"(v.w)
+               : "memory");
+}
+
+// Shared memory of one warp's merge of the partial derivatives (see
+// raster_bwd_kernel): kMergeSlots splats' per-pixel values, S + 1 pairs per
+// lane, and the negated cotangents -w of the warp's pixels, 3 S pairs per lane
+// at a stride (in pairs) that keeps eight consecutive lanes on distinct banks.
+constexpr int kMergeSlots = 4;
+__host__ __device__ constexpr int merge_slot_pairs(int S) { return 32 * (S + 1); }
+__host__ __device__ constexpr int merge_w_stride(int S) { return S == 1 ? 3 : S == 2 ? 6 : 10; }
+__host__ __device__ constexpr int merge_pairs(int S) { return kMergeSlots * merge_slot_pairs(S) + 32 * merge_w_stride(S); }
+
+// The merge of up to kMergeSlots splats of one warp into their cotangent rows.
+// A row's entries per stream are the sums over pixels of (dx, dy, dx^2, dx dy,
+// dy^2, 1) g, g = dL/d(power), and of (w_r, w_g, w_b) a T.  So a pixel needs to
+// hand over only S + 1 values (g of each stream, -a T), not 9 S, and -w stays in
+// shared memory.  power = -(A dx^2 + C dy^2)/2 - B dx dy is linear in the conic,
+// which the projection's reverse pass applies: dL/dA = -M(dx^2)/2, dL/dB =
+// -M(dx dy), dL/dC = -M(dy^2)/2, dL/dmx = -(A M(dx) + B M(dy)), dL/dmy =
+// -(B M(dx) + C M(dy)), dL/d(logit) = M(1) (1 - o).
+// Lanes 8 s .. 8 s + 7 sum splat s, lane & 7 the column of the 8 x 8 block, over
+// four pairs of pixels (y, y + 4); they write their rows over the slots'
+// memory, and lane (s, quad) adds the eight rows of its four values and issues
+// one float4 reduction.  Against a reduce-scatter of the 9 S values over the
+// warp per splat (128 instructions of 290 per splat and block with two
+// probes), a merge costs about 50 per splat; shared-memory bandwidth bounds it
+// (64 % of its peak), most of it the re-read of -w, which eight lanes of four
+// splats each load.  smx, smy, sgi: mean and index of the lane's splat; count:
+// slots in use.
+template <int S>
+__device__ __forceinline__ void merge_slots(f32x2* slots, const f32x2* sw, int count, float wx0, float wy0, float smx,
+                                            float smy, uint32_t sgi, float* __restrict__ cot_view) {
+  constexpr int NVP = cot_stride(S), NQ = NVP / 4;
+  static_assert(NVP * 32 * sizeof(float) <= kMergeSlots * merge_slot_pairs(S) * sizeof(f32x2), "rows fit the slots");
+  const int lane = threadIdx.x & 31, sl = lane >> 3, x = lane & 7;
+  float v[NVP];
+  __syncwarp();
+  const f32x2* my = slots + sl * merge_slot_pairs(S);
+  {
+    f32x2 c[3 * S];
+#pragma unroll
+    for (int k = 0; k < 3 * S; ++k) c[k] = 0ull;
+#pragma unroll(S == 3 ? 2 : 4)
+    for (int r = 0; r < 4; ++r) {
+      const int at = r * 8 + x;
+      const f32x2 naT = S % 2 ? my[32 * (S - 1) + 2 * at + 1] : my[32 * S + at];
+      const f32x2* wp = sw + at * merge_w_stride(S);
+#pragma unroll
+      for (int k = 0; k < 3 * S; k += S == 1 ? 1 : 2) {
+        if (S == 1 || k + 1 >= 3 * S) {
+          c[k] = fma2(naT, wp[k], c[k]);
+        } else {
+          const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(wp + k);
+          c[k] = fma2(naT, t.x, c[k]);
+          c[k + 1] = fma2(naT, t.y, c[k + 1]);
+        }
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < S; ++s)
+#pragma unroll
+      for (int ch = 0; ch < 3; ++ch) v[9 * s + 6 + ch] = sum2(c[3 * s + ch]);
+  }
+  {
+    f32x2 m[S][3];
+#pragma unroll
+    for (int s = 0; s < S; ++s) m[s][0] = m[s][1] = m[s][2] = 0ull;
+#pragma unroll(S == 3 ? 2 : 4)
+    for (int r = 0; r < 4; ++r) {
+      const int at = r * 8 + x;
+      f32x2 gp[S + 1];
+#pragma unroll
+      for (int p = 0; p + 1 < S + 1; p += 2) {
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(my + 32 * p + 2 * at);
+        gp[p] = t.x;
+        gp[p + 1] = t.y;
+      }
+      if constexpr (S % 2 == 0) gp[S] = my[32 * S + at];
+      const f32x2 dy = add2(dup2(smy), pack2(-(wy0 + (float)r), -(wy0 + (float)(r + 4))));
+      const f32x2 dyy = mul2(dy, dy);
+#pragma unroll
+      for (int s = 0; s < S; ++s) {
+        m[s][0] = add2(m[s][0], gp[s]);
+        m[s][1] = fma2(dy, gp[s], m[s][1]);
+        m[s][2] = fma2(dyy, gp[s], m[s][2]);
+      }
+    }
+    const float dx = smx - (wx0 + (float)x);
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      const float m0 = sum2(m[s][0]), m1 = sum2(m[s][1]), m2 = sum2(m[s][2]);
+      v[9 * s + 0] = dx * m0;
+      v[9 * s + 1] = m1;
+      v[9 * s + 2] = dx * dx * m0;
+      v[9 * s + 3] = dx * m1;
+      v[9 * s + 4] = m2;
+      v[9 * s + 5] = m0;
+    }
+  }
+#pragma unroll
+  for (int k = 9 * S; k < NVP; ++k) v[k] = 0.f;
+  __syncwarp();  // every lane has read the slots
+  float* rows = reinterpret_cast<float*>(slots);
+#pragma unroll
+  for (int k = 0; k < NVP; k += 4)
+    *reinterpret_cast<float4*>(rows + lane * NVP + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+  __syncwarp();
+  if (x < NQ && sl < count) {  // quad x of the lane's own splat
+    // neighbours first, as a tree: the sum least changed by its rounding
+    f32x2 a = 0ull, b = 0ull, a4 = 0ull, b4 = 0ull, a2 = 0ull, b2 = 0ull;
+#pragma unroll
+    for (int k = 0; k < 8; k += 2) {
+      const float* at = rows + (sl * 8 + k) * NVP + 4 * x;
+      const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(at), u = *reinterpret_cast<const ulonglong2*>(at + NVP);
+      a = add2(t.x, u.x);
+      b = add2(t.y, u.y);
+      if (k == 2) {
+        a4 = add2(a2, a);
+        b4 = add2(b2, b);
+      } else if (k == 6) {
+        a = add2(a4, add2(a2, a));
+        b = add2(b4, add2(b2, b));
+      }
+      a2 = a;
+      b2 = b;
+    }
+    float4 q;
+    unpack2(a, q.x, q.y);
+    unpack2(b, q.z, q.w);
+    if (q.x != 0.f || q.y != 0.f || q.z != 0.f || q.w != 0.f)
+      red_add4(cot_view + (size_t)sgi * NVP + 4 * x, q);
+  }
+  __syncwarp();  // the slots may be written again
+}
+
+template <int NU, bool GRAD>
+__global__ void __launch_bounds__(32, bwd_min_blocks((GRAD ? 1 : 0) + NU)) raster_bwd_kernel(
     const float4* __restrict__ rec, const uint32_t* __restrict__ vals, const uint32_t* __restrict__ ranges,
-    const uint32_t* __restrict__ order, int n_pad, gs_frame fr, int Tx, int T, const float* __restrict__ image,
-    const float* __restrict__ target,
-    const float* __restrict__ final_T, const uint32_t* __restrict__ n_contrib, const float* __restrict__ image_tan,
-    int loss_kind, float gn_floor, float inv_m, float* __restrict__ cot, float* __restrict__ loss_out,
-    int loss_per_view, CotHeader* cot_hdr, const uint8_t* __restrict__ masks, int32_t* status) {
+    const uint32_t* __restrict__ order, int n_pad, gs_frame fr, int Tx, int T, int log_blocks,
+    const float* __restrict__ image, const float* __restrict__ target, const float* __restrict__ final_T,
+    const uint32_t* __restrict__ n_contrib, const float* __restrict__ image_tan, int loss_kind, float gn_floor,
+    float inv_m, float* __restrict__ cot, bool want_loss, bool loss_per_view, CotHeader* cot_hdr,
+    const uint8_t* __restrict__ masks, const int32_t* status) {
   constexpr int S = (GRAD ? 1 : 0) + NU;  // cotangent streams
   constexpr int NVP = cot_stride(S);      // padded row stride of their 9 S values
   static_assert(NVP <= 32, "streams");
-  static_assert(NT <= 256, "s_loss holds one partial per warp, at most eight");
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int nthr = blockDim.x, nwarps = nthr >> 5, batch = CB ? fr.batch : kBatchPerThread * nthr;
-  constexpr int K = kBwdStages;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem);                     // K phase barriers
-  uint32_t* released = reinterpret_cast<uint32_t*>(smem + K * sizeof(uint64_t));  // K release counters
-  Rec* buf = reinterpret_cast<Rec*>(smem + kBwdRingHdr);
-  uint32_t* s_idx = reinterpret_cast<uint32_t*>(buf + K * batch);
-  uint8_t* s_bits = reinterpret_cast<uint8_t*>(s_idx + K * batch);  // block masks of the staged records
-  __shared__ uint32_t s_max;
-  __shared__ int s_abort;
-  __shared__ float s_loss[8];
-  __shared__ int s_fill_use[kBwdStages];  // ring use of each stage's last fill (-1: none)
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // the merge slots, then the negated cotangents (see merge_slots), and two
+  // buffers of staged records, whose last two words hold the Gaussian index
+  // and the list position instead of the record's radius and extents
+  __shared__ __align__(16) f32x2 slots[merge_pairs(S)];
+  __shared__ Rec buf[2][32];
+  f32x2* s_w = slots + kMergeSlots * merge_slot_pairs(S);
+  const int lane = threadIdx.x;
+  if (blockIdx.x == 0 && lane == 0) cot_hdr->clear_floats = 0;  // the rows are being added into
   // the tile of this block: the heaviest tiles first when an order is given
-  const int blk = order ? (int)min(__ldg(order + blockIdx.x), gridDim.x - 1) : (int)blockIdx.x;
+  const int wb = (int)(blockIdx.x & ((1u << log_blocks) - 1u)), ordinal = (int)(blockIdx.x >> log_blocks);
+  const int blk = order ? (int)min(__ldg(order + ordinal), (gridDim.x >> log_blocks) - 1) : ordinal;
   const int view = blk / T, tile = blk - view * T;
   const int ty = tile / Tx, tx = tile - ty * Tx;
-  int lx, ly;
-  pixel_of(tid, fr.tile_w, lx, ly);
+  const int bx0 = tx * fr.tile_w + (wb % (fr.tile_w >> 3)) * 8, by0 = ty * fr.tile_h + (wb / (fr.tile_w >> 3)) * 8;
+  if (bx0 >= fr.width || by0 >= fr.height) return;
   const size_t tslot = 2 * ((size_t)view * T + tile);
-  const uint32_t start = ranges[tslot], list_len = ranges[tslot + 1] - start;
+  const uint32_t start = __ldg(ranges + tslot), len = __ldg(ranges + tslot + 1) - start;
+  if (len == 0 && !want_loss) return;
   const size_t HW = (size_t)fr.width * fr.height;
-  // first pixel centre of this warp's 8 x 8 block
-  const float wx0 = (float)(tx * fr.tile_w + (warp % (fr.tile_w >> 3)) * 8) + 0.5f;
-  const float wy0 = (float)(ty * fr.tile_h + (warp / (fr.tile_w >> 3)) * 8) + 0.5f;
+  const float wx0 = (float)bx0 + 0.5f, wy0 = (float)by0 + 0.5f;  // the block's first pixel centre
 
   // per-pixel cotangents dL/dC of each stream and the loss
-  BwdPixel<S> pix[kPixPerThread];
+  BwdPair<S> pp;
   float lossp = 0.f;
+  {
+    float wv[kPixPerThread][S][3], Tv[kPixPerThread], pyc[kPixPerThread];
 #pragma unroll
-  for (int q = 0; q < kPixPerThread; ++q) {
-    BwdPixel<S>& p = pix[q];
-    const int px = tx * fr.tile_w + lx, py = ty * fr.tile_h + ly + 4 * q;
-    p.pxc = (float)px + 0.5f;
-    p.pyc = (float)py + 0.5f;
-    p.suf[0] = p.suf[1] = p.suf[2] = 0.f;
-    p.T = 0.f;
-    p.nc = 0;
+    for (int q = 0; q < kPixPerThread; ++q) {
+      const int px = bx0 + (lane & 7), py = by0 + (lane >> 3) + 4 * q;
+      pp.pxc = (float)px + 0.5f;
+      pyc[q] = (float)py + 0.5f;
+      Tv[q] = 0.f;
+      pp.nc[q] = 0;
 #pragma unroll
-    for (int st = 0; st < S; ++st) p.w[st][0] = p.w[st][1] = p.w[st][2] = 0.f;
-    if (!(px < fr.width && py < fr.height)) continue;
-    const size_t at0 = (size_t)py * fr.width + px;
-    p.T = final_T[(size_t)view * HW + at0];
-    p.nc = n_contrib[(size_t)view * HW + at0];
-    if (loss_kind == GS_LOSS_COTANGENT) {  // the caller's cotangent images, one per stream
+      for (int st = 0; st < S; ++st) wv[q][st][0] = wv[q][st][1] = wv[q][st][2] = 0.f;
+      if (!(px < fr.width && py < fr.height)) continue;
+      const size_t at0 = (size_t)py * fr.width + px;
+      if (len) {
+        Tv[q] = final_T[(size_t)view * HW + at0];
+        pp.nc[q] = n_contrib[(size_t)view * HW + at0];
+      }
+      if (loss_kind == GS_LOSS_COTANGENT) {  // the caller's cotangent images, one per stream
 #pragma unroll
-      for (int st = 0; st < S; ++st)
+        for (int st = 0; st < S; ++st)
 #pragma unroll
-        for (int ch = 0; ch < 3; ++ch) p.w[st][ch] = target[(((size_t)st * fr.n_views + view) * 3 + ch) * HW + at0];
-      continue;
-    }
-    if (loss_kind == GS_LOSS_WEIGHTED) {  // dL/dC (gradient stream), then the weights of w . J z_k
-      const float* wimg = target + (GRAD ? (size_t)fr.n_views * 3 * HW : 0);
+          for (int ch = 0; ch < 3; ++ch)
+            wv[q][st][ch] = target[(((size_t)st * fr.n_views + view) * 3 + ch) * HW + at0];
+        continue;
+      }
+      if (loss_kind == GS_LOSS_WEIGHTED) {  // dL/dC (gradient stream), then the weights of w . J z_k
+        const float* wimg = target + (GRAD ? (size_t)fr.n_views * 3 * HW : 0);
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch) {
+          if constexpr (GRAD) wv[q][0][ch] = target[((size_t)view * 3 + ch) * HW + at0];
+          const float wt = wimg[((size_t)view * 3 + ch) * HW + at0];
+#pragma unroll
+          for (int k = 0; k < NU; ++k)
+            wv[q][(GRAD ? 1 : 0) + k][ch] = wt * image_tan[(((size_t)k * fr.n_views + view) * 3 + ch) * HW + at0];
+        }
+        continue;
+      }
 #pragma unroll
       for (int ch = 0; ch < 3; ++ch) {
-        if constexpr (GRAD) p.w[0][ch] = target[((size_t)view * 3 + ch) * HW + at0];
-        const float wv = wimg[((size_t)view * 3 + ch) * HW + at0];
-#pragma unroll
-        for (int k = 0; k < NU; ++k)
-          p.w[(GRAD ? 1 : 0) + k][ch] = wv * image_tan[(((size_t)k * fr.n_views + view) * 3 + ch) * HW + at0];
-      }
-      continue;
-    }
-#pragma unroll
-    for (int ch = 0; ch < 3; ++ch) {
-      const size_t at = ((size_t)view * 3 + ch) * HW + at0;
-      const float r = image[at] - target[at];
-      const float ar = fabsf(r);
-      float lam;
-      if (loss_kind == GS_LOSS_L1) {
-        lossp += 0.5f * inv_m * ar;
-        lam = 0.25f / fmaxf(ar, gn_floor);
-      } else {
-        lossp += 0.5f * inv_m * r * r;
-        lam = 1.f;
-      }
-      if constexpr (GRAD) p.w[0][ch] = (loss_kind == GS_LOSS_L1) ? (0.5f * inv_m) * ((r > 0.f) - (r < 0.f)) : inv_m * r;
-#pragma unroll
-      for (int k = 0; k < NU; ++k)
-        p.w[(GRAD ? 1 : 0) + k][ch] = inv_m * lam * image_tan[(((size_t)k * fr.n_views + view) * 3 + ch) * HW + at0];
-    }
-  }
-  if (tid == 0) {
-    if (blockIdx.x == 0) cot_hdr->clear_floats = 0;  // the rows are being added into
-    s_max = 0;
-    // a stage wait that ran out in an earlier block: skip the list walk
-    s_abort = status ? (*(volatile int32_t*)status & GS_FLAG_TIMEOUT) : 0;
-    for (int k = 0; k < K; ++k) {
-      mbar_init(&full[k], 1);
-      released[k] = 0;
-      s_fill_use[k] = -1;
-    }
-    fence_mbar_init();
-  }
-  __syncthreads();
-  const uint32_t nc_thread = max(pix[0].nc, pix[1].nc);
-  if (nc_thread) atomicMax(&s_max, nc_thread);
-  const uint32_t warp_nc = __reduce_max_sync(0xffffffffu, nc_thread);  // list positions this warp still needs
-  // objective: warp then block reduction, one atomic per CTA
-  if (loss_out) {
-    float lsum = lossp;
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-    if (lane == 0) s_loss[tid >> 5] = lsum;
-  }
-  __syncthreads();
-  if (loss_out && tid == 0) {
-    float tot = 0.f;
-    for (int k = 0; k < nwarps; ++k) tot += s_loss[k];
-    atomicAdd(loss_out + (loss_per_view ? view : 0), tot);
-  }
-  const int n = s_abort ? 0 : (int)min(s_max, list_len);  // n_contrib never exceeds the tile's list
-  const int nb = (n + batch - 1) / batch;
-  // batch b is use u = nb - 1 - b of the ring: stage u % K, its (u / K)-th fill
-  for (int u = warp; u < min(K, nb); u += nwarps)
-    stage_batch_warp(u, u, nb - 1 - u, batch, start, n, view, n_pad, vals, rec, masks, buf, s_idx, s_bits, full,
-                     s_fill_use);
-  bool ok = true;
-  for (int u = 0; u < nb; ++u) {
-    const int st = u % K, b = nb - 1 - u;
-    // every lane waits (bounded) for the stage's phase: each acquires the copies
-    // and indices.  A warp whose wait ran out stops at once: it releases no
-    // further stage, so no later round completes and nothing is refilled
-    // behind it; the other warps run into their own bounded waits.
-    const bool landed = mbar_wait_bounded(&full[st], (uint32_t)((u / K) & 1), status);
-    ok = __all_sync(0xffffffffu, landed) != 0;
-    if (!ok) break;
-    const int cnt = min(batch, n - b * batch);
-    const Rec* bb = buf + st * batch;
-    // the warp walks, back to front, only the splats its block can see (the
-    // forward pass's mask bit when given, else the same footprint test) and
-    // that lie before its last contributor: one ballot per 32 splats
-    const uint8_t* sb = s_bits + st * batch;
-    for (int j0 = ((cnt - 1) & ~31); (uint32_t)(b * batch) < warp_nc && j0 >= 0; j0 -= 32) {
-      const int jl = j0 + lane;
-      uint32_t bits = __ballot_sync(
-          0xffffffffu, jl < cnt && (uint32_t)(b * batch + jl) < warp_nc &&
-                           (masks ? ((sb[jl] >> warp) & 1u) != 0 : block_sees(bb[jl], wx0, wy0)));
-      while (bits) {
-        const int hb = 31 - __clz(bits);
-        bits &= ~(1u << hb);
-        const int j = j0 + hb;
-        const uint32_t pos = (uint32_t)(b * batch + j);
-        const Rec r = bb[j];
-        bool on[kPixPerThread];
-        float dx[kPixPerThread], dy[kPixPerThread], G[kPixPerThread], oG[kPixPerThread], alpha[kPixPerThread];
-#pragma unroll
-        for (int q = 0; q < kPixPerThread; ++q) {
-          dx[q] = __fsub_rn(r.a.x, pix[q].pxc);
-          dy[q] = __fsub_rn(r.a.y, pix[q].pyc);
-          const float power = splat_power(r, dx[q], dy[q]);
-          G[q] = __expf(power);
-          oG[q] = __fmul_rn(r.b.y, G[q]);
-          alpha[q] = fminf(kAlphaMax, oG[q]);
-          on[q] = pos < pix[q].nc && power <= 0.f && alpha[q] >= kAlphaMin;
-          if (!on[q]) G[q] = oG[q] = alpha[q] = 0.f;
-        }
-        const uint32_t act = __ballot_sync(0xffffffffu, on[0] || on[1]);  // lanes that blend the splat
-        if (!act) continue;
-        float v[32];
-#if GS_BWD_SKIP_IDLE_ROW
-        // a pixel row of the block (the lanes' first or second pixels) that no
-        // lane blends the splat at adds exact zeros and keeps its state: skip it
-        const bool any0 = __any_sync(0xffffffffu, on[0]), any1 = __any_sync(0xffffffffu, on[1]);
-        if (any0) {
-          bwd_accumulate<S, true>(pix[0], r, dx[0], dy[0], G[0], oG[0], alpha[0], v);
-          if (any1) bwd_accumulate<S, false>(pix[1], r, dx[1], dy[1], G[1], oG[1], alpha[1], v);
+        const size_t at = ((size_t)view * 3 + ch) * HW + at0;
+        const float r = image[at] - target[at];
+        const float ar = fabsf(r);
+        float lam;
+        if (loss_kind == GS_LOSS_L1) {
+          lossp += 0.5f * inv_m * ar;
+          lam = 0.25f / fmaxf(ar, gn_floor);
         } else {
-          bwd_accumulate<S, true>(pix[1], r, dx[1], dy[1], G[1], oG[1], alpha[1], v);
+          lossp += 0.5f * inv_m * r * r;
+          lam = 1.f;
         }
-#else
-        bwd_accumulate<S, true>(pix[0], r, dx[0], dy[0], G[0], oG[0], alpha[0], v);
-        bwd_accumulate<S, false>(pix[1], r, dx[1], dy[1], G[1], oG[1], alpha[1], v);
-#endif
+        if constexpr (GRAD)
+          wv[q][0][ch] = (loss_kind == GS_LOSS_L1) ? (0.5f * inv_m) * ((r > 0.f) - (r < 0.f)) : inv_m * r;
 #pragma unroll
-        for (int q = 9 * S; q < 32; ++q) v[q] = 0.f;
-        const uint32_t gi = s_idx[st * batch + j];
-        float* dst = cot + ((size_t)view * n_pad + gi) * NVP;
-        if (__popc(act) <= kBwdSparseLanes) {
-          // few lanes blend the splat: each adds its own row instead of the
-          // warp-wide reduction (the other lanes' rows are zero)
-          if (on[0] || on[1]) {
-#pragma unroll
-            for (int q = 0; q < NVP; q += 4)
-              atomicAdd(reinterpret_cast<float4*>(dst + q), make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]));
-          }
-          continue;
-        }
-        float qs[4];
-        if constexpr (NVP <= 16) warp_reduce_quads16(v, qs);
-        else warp_reduce_quads32(v, qs);
-        if ((lane & 3) == 0 && lane < NVP && (qs[0] != 0.f || qs[1] != 0.f || qs[2] != 0.f || qs[3] != 0.f))
-          atomicAdd(reinterpret_cast<float4*>(dst + lane), make_float4(qs[0], qs[1], qs[2], qs[3]));
+        for (int k = 0; len && k < NU; ++k)
+          wv[q][(GRAD ? 1 : 0) + k][ch] =
+              inv_m * lam * image_tan[(((size_t)k * fr.n_views + view) * 3 + ch) * HW + at0];
       }
     }
-    // release the stage: the warp's reads of it are ordered before its count,
-    // and the last warp to count it, ordered after all counts, refills it
-    __syncwarp();
-    uint32_t last = 0;
-    if (lane == 0) {
-      __threadfence_block();
-      last = atomicAdd(&released[st], 1u) == (uint32_t)(nwarps - 1);
-      if (last) {
-        released[st] = 0;
-        __threadfence_block();
+    pp.T = pack2(Tv[0], Tv[1]);
+    pp.npy = pack2(-pyc[0], -pyc[1]);
+#pragma unroll
+    for (int st = 0; st < S; ++st) {
+      pp.nq[st] = 0ull;
+#pragma unroll
+      for (int ch = 0; ch < 3; ++ch) {
+        pp.w[st][ch] = pack2(wv[0][st][ch], wv[1][st][ch]);
+        s_w[lane * merge_w_stride(S) + 3 * st + ch] = pack2(-wv[0][st][ch], -wv[1][st][ch]);
       }
     }
-    last = __shfl_sync(0xffffffffu, last, 0);
-    if (last && u + K < nb)
-      stage_batch_warp(st, u + K, nb - 1 - (u + K), batch, start, n, view, n_pad, vals, rec, masks, buf, s_idx,
-                       s_bits, full, s_fill_use);
   }
-  // Drain after a failed wait: a stage is refilled only by a warp that saw its
-  // previous fill land, so each stage has at most one fill in flight, its last.
-  // One thread per stage waits (bounded) for that fill, so that no bulk copy is
-  // still writing into this block's shared memory, or completing on its
-  // barrier, when the block exits.  Without a failure every fill has landed.
-  if (__syncthreads_or(!ok) && tid < K && s_fill_use[tid] >= 0)
-    mbar_wait_bounded(&full[tid], (uint32_t)((s_fill_use[tid] / K) & 1), status);
+  if (want_loss) {
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) lossp += __shfl_xor_sync(0xffffffffu, lossp, o);
+    if (lane == 0 && lossp != 0.f)
+      atomicAdd(&cot_hdr->loss[loss_per_view ? view : (int)(blockIdx.x % kLossSlots)], (double)lossp);
+  }
+  // list positions this block still needs (n_contrib never exceeds the tile's
+  // list); none after a wait that ran out in an earlier call
+  const uint32_t nw = min(__reduce_max_sync(0xffffffffu, max(pp.nc[0], pp.nc[1])), len);
+  if (__any_sync(0xffffffffu, nw == 0 || (status && (*(volatile const int32_t*)status & GS_FLAG_TIMEOUT)))) return;
+  const int n = (int)nw;
+
+  // Chunks of 32 list positions, back to front: each lane reads the index and
+  // visibility of one position (the forward pass's mask bit when given, else
+  // the footprint test), a chunk ahead of its use.
+  int c = (n - 1) >> 5;
+  uint32_t gi = 0, gi_next = 0;
+  bool see = false, see_next = false;
+  auto fetch = [&](int cc, uint32_t& g, bool& v) {
+    const int p = cc * 32 + lane;
+    v = false;
+    if (cc < 0 || p >= n) return;
+    g = __ldg(vals + start + (uint32_t)p);
+    if (masks) {
+      v = ((__ldg(masks + start + (uint32_t)p) >> wb) & 1u) != 0;
+    } else {
+      const float4* src = rec + 3 * ((size_t)view * n_pad + g);
+      Rec r;
+      r.a = __ldg(src);
+      r.b = __ldg(src + 1);
+      r.c = __ldg(src + 2);
+      v = block_sees(r, wx0, wy0);
+    }
+  };
+  fetch(c, gi, see);
+  fetch(c - 1, gi_next, see_next);
+  // Stages the visible splats of the next chunks, as many whole chunks as fit,
+  // into b (asynchronous copies, one group per call); returns their count.
+  auto fill = [&](Rec* b) {
+    int cnt = 0;
+    while (c >= 0) {
+      const uint32_t bits = __ballot_sync(0xffffffffu, see);
+      const int k = __popc(bits);
+      if (cnt + k > 32) break;
+      if (see) {
+        Rec* d = b + cnt + __popc(bits & (0xfffffffeu << lane));  // the last position first
+        const float4* src = rec + 3 * ((size_t)view * n_pad + gi);
+        cp_async16(&d->a, src);
+        cp_async16(&d->b, src + 1);
+        cp_async4(&d->c.x, src + 2);
+        *reinterpret_cast<uint2*>(&d->c.z) = make_uint2(gi, (uint32_t)(c * 32 + lane));
+      }
+      cnt += k;
+      --c;
+      gi = gi_next;
+      see = see_next;
+      fetch(c - 1, gi_next, see_next);
+    }
+    cp_async_commit();
+    return cnt;
+  };
+
+  int used = 0;  // merge slots filled (warp-uniform)
+  float smx = 0.f, smy = 0.f;
+  uint32_t sgi = 0;
+  float* cot_view = cot + (size_t)view * n_pad * NVP;
+  int cur = 0, cnt = fill(buf[0]);
+  while (cnt > 0) {
+    const int cnt_next = fill(buf[cur ^ 1]);
+    cp_async_wait_prior();  // all but the newest group: this buffer has landed
+    __syncwarp();
+    for (int j = 0; j < cnt; ++j) {
+      const Rec r = buf[cur][j];
+      const uint32_t pos = __float_as_uint(r.c.w);
+      float dx, power[2], oG[2], na[2], ac[2], om[2];
+      f32x2 dy, G;
+      splat_gauss2(r, pp.pxc, pp.npy, dx, dy, power, G);
+      unpack2(mul2(dup2(r.b.y), G), oG[0], oG[1]);
+      bool on[2];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const float al = fminf(kAlphaMax, oG[q]);
+        on[q] = pos < pp.nc[q] && power[q] <= 0.f && al >= kAlphaMin;
+        na[q] = on[q] ? -al : 0.f;
+        ac[q] = on[q] && !(oG[q] > kAlphaMax) ? al : 0.f;  // a capped alpha has zero derivative
+      }
+      if (!__any_sync(0xffffffffu, on[0] || on[1])) continue;
+      // recover T_i = T_{i+1} / (1 - a); with d = w . c and q the stream's
+      // suffix, dL/d(power) = a/(1 - a) (T_{i+1} d - q) per stream.  A pixel
+      // that does not blend the splat has a = 0: its state stays as it is and it
+      // contributes exact zeros.
+      const f32x2 nap = pack2(na[0], na[1]);
+      unpack2(add2(dup2(1.f), nap), om[0], om[1]);
+      const f32x2 inv = pack2(rcp_approx(om[0]), rcp_approx(om[1]));
+      const f32x2 Ti = mul2(pp.T, inv), kk = mul2(inv, pack2(ac[0], ac[1])), naT = mul2(nap, Ti);
+      f32x2 gp[S];
+#pragma unroll
+      for (int s = 0; s < S; ++s) {
+        const f32x2 d = fma2(pp.w[s][2], dup2(r.c.x), fma2(pp.w[s][1], dup2(r.b.w), mul2(pp.w[s][0], dup2(r.b.z))));
+        gp[s] = mul2(kk, fma2(pp.T, d, pp.nq[s]));
+        pp.nq[s] = fma2(naT, d, pp.nq[s]);
+      }
+      pp.T = Ti;
+      // the lane's values of this splat into its merge slot
+      f32x2* my = slots + used * merge_slot_pairs(S);
+      if constexpr (S == 1) {
+        *reinterpret_cast<ulonglong2*>(my + 2 * lane) = make_ulonglong2(gp[0], naT);
+      } else {
+        *reinterpret_cast<ulonglong2*>(my + 2 * lane) = make_ulonglong2(gp[0], gp[1]);
+        if constexpr (S == 2) my[64 + lane] = naT;
+        else *reinterpret_cast<ulonglong2*>(my + 64 + 2 * lane) = make_ulonglong2(gp[S - 1], naT);
+      }
+      if ((lane >> 3) == used) {
+        smx = r.a.x;
+        smy = r.a.y;
+        sgi = __float_as_uint(r.c.z);
+      }
+      if (++used == kMergeSlots) {
+        merge_slots<S>(slots, s_w, kMergeSlots, wx0, wy0, smx, smy, sgi, cot_view);
+        used = 0;
+      }
+
+    }
+    __syncwarp();  // the buffer may be refilled
+    cur ^= 1;
+    cnt = cnt_next;
+  }
+  if (used) merge_slots<S>(slots, s_w, used, wx0, wy0, smx, smy, sgi, cot_view);
 }
 
 // ------------------------------------------------ projection reverse pass
@@ -1026,7 +1064,6 @@ __device__ __forceinline__ void project_bwd_column(const float* __restrict__ P, 
 #pragma unroll
     for (int b = 0; b < 3; ++b) Sg[a][b] = M[a][0] * M[b][0] + M[a][1] * M[b][1] + M[a][2] * M[b][2];
   const float opac = 1.f / (1.f + expf(-ld(10)));
-  const float dsig = opac * (1.f - opac);
 
   // ---- pass 1: geometric rows of every stream
   // g_S: dL/dSigma, symmetric, entries (0,0) (0,1) (0,2) (1,1) (1,2) (2,2)
@@ -1139,7 +1176,7 @@ __device__ __forceinline__ void project_bwd_column(const float* __restrict__ P, 
 #pragma unroll
         for (int e = 0; e < 6; ++e) g_S[st][e] += u[kSymP[e]] * a0[kSymQ[e]] + w[kSymP[e]] * a1[kSymQ[e]];
       }
-      g_ol[st] += mo[5] * dsig;
+      g_ol[st] += mo[5] * (1.f - opac);
     }
     // colour: clamp decisions, and the dependence of colour on mu through the view direction
     float d[3], dn;
@@ -1373,10 +1410,11 @@ template <int DEG, int NU, bool GRAD>
 __global__ void GS_PBWD_BOUNDS project_bwd_kernel(const float* __restrict__ P, int n, int n_pad,
                                                   const gs_camera* __restrict__ cams, gs_frame fr,
                                                   float* __restrict__ cot, ProbeArg pa, float* __restrict__ grad,
-                                                  float* __restrict__ hz, CotHeader* cot_hdr, uint64_t cot_floats) {
+                                                  float* __restrict__ hz, CotHeader* cot_hdr, uint64_t cot_floats,
+                                                  float* loss_out) {
   const int i = blockIdx.x * kPbwdThreads + threadIdx.x;
   project_bwd_column<DEG, NU, GRAD>(P, n, n_pad, i, cams, fr.n_views, fr, cot, n_pad, pa, grad, hz);
-  cot_mark_clear(cot_hdr, cot_floats);
+  cot_mark_clear(cot_hdr, cot_floats, loss_out, 0);
 }
 
 // A batch: item b's share of the grid takes its columns through the reverse of
@@ -1385,7 +1423,7 @@ __global__ void GS_PBWD_BOUNDS project_bwd_kernel(const float* __restrict__ P, i
 template <int DEG, int NU, bool GRAD>
 __global__ void GS_PBWD_BOUNDS project_bwd_batch_kernel(BatchArg ba, gs_frame fr, float* __restrict__ cot,
                                                         int cot_pitch, ProbeArg pa, CotHeader* cot_hdr,
-                                                        uint64_t cot_floats) {
+                                                        uint64_t cot_floats, float* loss_out) {
   constexpr int NVP = cot_stride((GRAD ? 1 : 0) + NU);
   const int b = batch_item(ba, (int)blockIdx.x);
   const int i = ((int)blockIdx.x - ba.first_block[b]) * kPbwdThreads + threadIdx.x;
@@ -1393,7 +1431,7 @@ __global__ void GS_PBWD_BOUNDS project_bwd_batch_kernel(BatchArg ba, gs_frame fr
   pa.t_dev = nullptr;
   project_bwd_column<DEG, NU, GRAD>(ba.P[b], ba.n[b], ba.n_pad[b], i, ba.cam[b], 1, fr,
                                     cot + (size_t)b * cot_pitch * NVP, cot_pitch, pa, ba.grad[b], ba.hz[b]);
-  cot_mark_clear(cot_hdr, cot_floats);
+  cot_mark_clear(cot_hdr, cot_floats, loss_out, ba.n_items);
 }
 
 // ------------------------------------------------------------------ host side
@@ -1462,7 +1500,7 @@ cudaError_t cot_prepare(void* workspace, uint64_t floats, CotWs& ws, cudaStream_
 
 template <int DEG, int NU, bool GRAD>
 void launch_pbwd(const gs_params* x, const gs_camera* cams, gs_frame fr, CotWs ws, const gs_probe* probe,
-                 float* grad, float* hz, cudaStream_t st) {
+                 float* grad, float* hz, float* loss_out, cudaStream_t st) {
   constexpr int S = (GRAD ? 1 : 0) + NU;
   const size_t smem = pbwd_stash_bytes(fr.n_views, S);
   static size_t attr = 0;
@@ -1472,7 +1510,7 @@ void launch_pbwd(const gs_params* x, const gs_camera* cams, gs_frame fr, CotWs w
   }
   const dim3 pg((x->n + kPbwdThreads - 1) / kPbwdThreads), pb(kPbwdThreads);
   project_bwd_kernel<DEG, NU, GRAD><<<pg, pb, smem, st>>>(x->data, x->n, x->n_pad, cams, fr, ws.cot,
-                                                          probe_arg(probe), grad, hz, ws.hdr, ws.floats);
+                                                          probe_arg(probe), grad, hz, ws.hdr, ws.floats, loss_out);
 }
 
 // The reverse blend over the frame, then the projection's reverse pass: of the
@@ -1485,24 +1523,17 @@ void launch_bwd_kernels(const gs_params* x, const BatchArg* ba, int n_pad, int d
                         const gs_probe* probe, gs_loss loss, float* grad, float* hz, float* loss_out, CotWs ws,
                         int32_t* status, cudaStream_t st) {
   const TileGrid g = tile_grid(fr);
-  const int nthr = fr.tile_w * fr.tile_h / kPixPerThread, batch = bwd_batch(fr, nthr);
-  const size_t smem = bwd_smem_bytes(batch);
-  const bool cb = fr.batch != 0, big = blend_threads(nthr) == 256;
-  auto* kern = big ? (cb ? raster_bwd_kernel<NU, GRAD, true, 256> : raster_bwd_kernel<NU, GRAD, false, 256>)
-                   : (cb ? raster_bwd_kernel<NU, GRAD, true, 128> : raster_bwd_kernel<NU, GRAD, false, 128>);
-  static size_t attr[2][2] = {{0, 0}, {0, 0}};
-  if (smem > 48 * 1024 && smem > attr[big][cb]) {
-    if (allow_smem(kern, smem) != cudaSuccess) return;  // the caller reports the error
-    attr[big][cb] = smem;
-  }
   const double views_per_objective = ba ? 1.0 : (double)fr.n_views;
   const float inv_m = (float)(1.0 / (3.0 * (double)fr.width * fr.height * views_per_objective));
-  const unsigned blocks = (unsigned)((size_t)fr.n_views * g.T);
-  kern<<<blocks, nthr, smem, st>>>(
-      reinterpret_cast<const float4*>(proj->rec), sorted->vals, sorted->ranges, sorted->order, n_pad, fr, g.Tx,
-      g.T, image,
-      target, final_T, n_contrib, image_tan, loss.kind, loss.gn_floor, inv_m, ws.cot, loss_out, ba ? 1 : 0, ws.hdr,
-      sorted->masks, status);
+  int log_blocks = 0;  // 8 x 8 blocks per tile
+  while ((64 << log_blocks) < fr.tile_w * fr.tile_h) ++log_blocks;
+  const unsigned blocks = (unsigned)((size_t)fr.n_views * g.T << log_blocks);
+  raster_bwd_kernel<NU, GRAD><<<blocks, 32, 0, st>>>(
+      reinterpret_cast<const float4*>(proj->rec), sorted->vals, sorted->ranges, sorted->order, n_pad, fr, g.Tx, g.T,
+      log_blocks, image, target, final_T, n_contrib, image_tan, loss.kind, loss.gn_floor, inv_m, ws.cot,
+      loss_out != nullptr, ba != nullptr, ws.hdr, sorted->masks, status);
+  if (loss_out && (ba ? ba->first_block[ba->n_items] : x->n) == 0)
+    add_loss_kernel<<<1, 1, 0, st>>>(ws.hdr, loss_out, ba ? ba->n_items : 0);
   if (ba) {
     if (ba->first_block[ba->n_items] == 0) return;
     constexpr int S = (GRAD ? 1 : 0) + NU;
@@ -1517,7 +1548,7 @@ void launch_bwd_kernels(const gs_params* x, const BatchArg* ba, int n_pad, int d
       battr = sm;                                                                                  \
     }                                                                                              \
     project_bwd_batch_kernel<D, NU, GRAD><<<grid, blk, sm, st>>>(*ba, fr, ws.cot, n_pad, pa, ws.hdr, \
-                                                                 ws.floats);                       \
+                                                                 ws.floats, loss_out);             \
   } while (0)
     switch (deg) {
       case 0: GS_PBWD_BATCH(0); break;
@@ -1530,10 +1561,10 @@ void launch_bwd_kernels(const gs_params* x, const BatchArg* ba, int n_pad, int d
   }
   if (x->n == 0) return;
   switch (x->sh_degree) {
-    case 0: launch_pbwd<0, NU, GRAD>(x, cams, fr, ws, probe, grad, hz, st); break;
-    case 1: launch_pbwd<1, NU, GRAD>(x, cams, fr, ws, probe, grad, hz, st); break;
-    case 2: launch_pbwd<2, NU, GRAD>(x, cams, fr, ws, probe, grad, hz, st); break;
-    default: launch_pbwd<3, NU, GRAD>(x, cams, fr, ws, probe, grad, hz, st); break;
+    case 0: launch_pbwd<0, NU, GRAD>(x, cams, fr, ws, probe, grad, hz, loss_out, st); break;
+    case 1: launch_pbwd<1, NU, GRAD>(x, cams, fr, ws, probe, grad, hz, loss_out, st); break;
+    case 2: launch_pbwd<2, NU, GRAD>(x, cams, fr, ws, probe, grad, hz, loss_out, st); break;
+    default: launch_pbwd<3, NU, GRAD>(x, cams, fr, ws, probe, grad, hz, loss_out, st); break;
   }
 }
 

@@ -61,7 +61,7 @@ class TRStep:
         footprint_bins: bin each splat into the tiles its alpha >= 1/255 footprint
         box reaches within its 3DGS tile square (False: the whole square); the
         images and derivatives are the same, the pairs fewer.  batch: records a
-        tile's block stages per step of its list in the blends (0: one per
+        tile's block stages per step of its list in the forward blend (0: one per
         thread; else a multiple of 32 up to 512)."""
         G.load()
         self.n, self.deg, self.V, self.W, self.H, self.nu = n, sh_degree, n_views, width, height, nu

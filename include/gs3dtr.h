@@ -88,14 +88,14 @@ typedef struct gs_camera {
 
 /* Views rendered by one call; every camera of the call has this size.
  * tile_w is 8, 16 or 32, tile_h a power of two >= 8, tile_w * tile_h is 64, 128,
- * 256 or 512 (two pixels per thread; each warp covers an 8 x 8 pixel block).
+ * 256 or 512 (each warp covers an 8 x 8 pixel block).
  * footprint_bins selects the tiles of a splat (see gs_bin_sort): 0 its 3DGS tile
  * square, 1 that square narrowed to its alpha >= 1/255 footprint (its box, then
  * row by row its ellipse).  Both give the same images and derivatives; 1 gives
  * fewer pairs.
- * batch: records a tile's block stages in shared memory per step of its list in
- * the forward blend (gs_raster_fwd): 0 for one per thread, else a multiple of 32
- * from 32 to 512.  It changes speed, not results. */
+ * batch: a hint of how many records the blends stage in shared memory at a time:
+ * 0, or a multiple of 32 from 32 to 512.  It never changes results; the present
+ * kernels choose for themselves. */
 typedef struct gs_frame {
   int32_t n_views, width, height, tile_w, tile_h, footprint_bins, batch;
 } gs_frame;
@@ -152,9 +152,10 @@ typedef struct gs_projected {
  *             (lengths grouped in steps of 1/8 of a power of two, any order
  *             within a group); the blends then start the heaviest tiles first.
  *             It changes when a tile runs, never its result.
- *   masks:    NULL, or capacity bytes.  gs_raster_fwd writes, for every pair it
- *             stages, which 8 x 8 pixel blocks of the pair's tile the splat's
- *             footprint reaches (bit w: the block of warp w, see gs_frame);
+ *   masks:    NULL, or capacity bytes.  gs_raster_fwd writes (over the whole
+ *             array), for every pair, which 8 x 8 pixel blocks of the pair's tile
+ *             walk as far as the pair and are reached by the splat's footprint
+ *             (bit w: the block of warp w, see gs_frame);
  *             gs_raster_bwd, gs_hvp_diag and gs_raster_bwd_batch then read those
  *             bits instead of testing the footprint again.  The bits of a pair
  *             are valid once gs_raster_fwd has run on these sorted pairs with the
@@ -415,11 +416,11 @@ gs_status gs_raster_bwd_batch(const gs_batch_item* items, int32_t n_items, int32
 gs_status gs_tr_update_batch(const gs_batch_item* items, int32_t n_items, const gs_tr_config* cfg, int32_t* status,
                              void* stream);
 
-/* Diagnostics (no paper counterpart): runs, in one warp, the bounded wait that
- * every kernel uses on its asynchronous copies, on an mbarrier that nothing
- * completes, giving up after `limit` tries (1 <= limit <= 2^20).  Raises
- * GS_FLAG_TIMEOUT in *status (device int32) as a kernel does when a staged copy
- * never lands; the kernel then returns and the context stays usable.  Lets
+/* Diagnostics (no paper counterpart): runs, in one warp, a bounded wait on an
+ * mbarrier that nothing completes, giving up after `limit` tries
+ * (1 <= limit <= 2^20).  Raises GS_FLAG_TIMEOUT in *status (device int32) as a
+ * kernel does whose wait runs out; the kernel then returns and the context
+ * stays usable.  Lets
  * the failure path be tested without a fault. */
 gs_status gs_wait_check(uint32_t limit, int32_t* status, void* stream);
 

@@ -26,10 +26,9 @@ gs_status check_launch(const char* what) {
 }
 
 namespace {
-// One warp waits, as the kernels' bounded wait (mbar_wait_bounded) does but
-// with `limit` tries, on an mbarrier that nothing arrives at and no copy
-// completes: every lane gives up and raises GS_FLAG_TIMEOUT, as a kernel does
-// when a staged copy never lands.
+// One warp waits, with `limit` tries, on an mbarrier that nothing arrives at and
+// no copy completes: every lane gives up and raises GS_FLAG_TIMEOUT, as a kernel
+// does whose bounded wait runs out.
 __global__ void wait_check_kernel(uint32_t limit, int32_t* status) {
   __shared__ __align__(8) uint64_t bar;
   if (threadIdx.x == 0) {

@@ -500,7 +500,7 @@ __device__ __forceinline__ uint32_t foot_count(const FootRows& f, int tw, int th
   return n;
 }
 
-// ------------------------------------------------- async copies (TMA bulk)
+// ------------------------------------------------- barriers, async copies
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }
@@ -509,22 +509,6 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
 }
 __device__ __forceinline__ void fence_mbar_init() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-__device__ __forceinline__ void fence_proxy_async() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-               : "memory");
-}
-// One non-multicast bulk copy global -> this CTA's shared memory, completing on bar.
-// dst, src and bytes must be multiples of 16.
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
 }
 // Per-thread asynchronous copies global -> shared (16 or 4 bytes), in groups.
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
@@ -536,6 +520,7 @@ __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 // Waits for all of the calling thread's groups but the newest.
 __device__ __forceinline__ void cp_async_wait_prior() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -545,20 +530,11 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Bounded wait for phase `parity` of bar.  Returns false (and raises
-// GS_FLAG_TIMEOUT) if the phase did not complete within the limit.
-constexpr uint32_t kWaitLimit = 1u << 22;
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, int32_t* status) {
-  for (uint32_t it = 0; it < kWaitLimit; ++it)
-    if (mbar_try_wait(bar, parity)) return true;
-  if (status) atomicOr(status, GS_FLAG_TIMEOUT);
-  return false;
-}
 
 // ---------------------------------------------------------- frames
-// Tile shapes the kernels support: two pixels per thread and warps covering
-// 8 x 8 pixel blocks, so tile_w is 8, 16 or 32, tile_h a power of two >= 8, and
-// tile_w * tile_h is 64, 128, 256 or 512 (at most eight warps per tile).
+// Tile shapes the kernels support: warps covering 8 x 8 pixel blocks, so tile_w is
+// 8, 16 or 32, tile_h a power of two >= 8, and tile_w * tile_h is 64, 128, 256 or
+// 512 (at most eight blocks per tile, one bit each in the masks).
 inline bool frame_ok(gs_frame fr) {
   auto pow2 = [](int v) { return v > 0 && (v & (v - 1)) == 0; };
   const int tt = fr.tile_w * fr.tile_h;

@@ -7,14 +7,12 @@
 //                  in the same sweep, the Gauss-Newton products J^T diag(w) J z_k
 //   gs_hvp_diag    the Gauss-Newton products alone
 //
-// Forward: one CTA renders one tile of one view with two pixels per thread;
-// each warp owns an 8 x 8 pixel block.  The tile's splat records are staged
-// through shared memory in batches (one record per pixel of the tile), each
-// record moved by a TMA bulk copy (cp.async.bulk, no multicast) completing on an
-// mbarrier, double-buffered so that the next batch lands while the current one
-// is blended.  Per batch every splat gets a mask of the warp blocks its
-// alpha >= 1/255 footprint can reach, and each warp walks only its own visible
-// splats (one ballot per 32).  Reverse: one warp per CTA and 8 x 8 block.  It
+// Both blends run one warp per CTA on one 8 x 8 pixel block of a tile, two pixels
+// per thread held as a packed FP32 pair.  A warp walks its tile's list in
+// chunks of 32 positions, keeps the splats whose alpha >= 1/255 footprint can
+// reach its block, and stages those records in shared memory by asynchronous
+// copies, one buffer ahead of the one it blends.  Nothing is shared with the
+// tile's other blocks, so no block waits for another.  The reverse pass
 // walks the list back to front, recovers T_i = T_{i+1} / (1 - a_i) from the final
 // transmittance (nothing per pair is stored), merges each splat's 9 x streams
 // partial derivatives over the block's 64 pixels, four splats at a time, and
@@ -33,13 +31,6 @@ struct alignas(16) Rec {
 };
 static_assert(sizeof(Rec) == 48, "record size");
 
-// Power and alpha of a splat at a pixel with a fixed rounding sequence, so that
-// the forward and reverse kernels take identical decisions.
-__device__ __forceinline__ float splat_power(const Rec& r, float dx, float dy) {
-  const float q = __fmaf_rn(r.b.x, __fmul_rn(dy, dy), __fmul_rn(r.a.z, __fmul_rn(dx, dx)));
-  return __fmaf_rn(-0.5f, q, -__fmul_rn(r.a.w, __fmul_rn(dx, dy)));
-}
-
 __device__ __forceinline__ float ex2_approx(float x) {
   float r;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -47,7 +38,8 @@ __device__ __forceinline__ float ex2_approx(float x) {
 }
 // The splat at a thread's two pixels, which share their column: dx and the
 // negated centres -py of the pair give dy, then power and exp(power) per pixel.
-// Each lane rounds exactly as splat_power does.
+// One function with a fixed rounding sequence, so that the forward and reverse
+// kernels take identical decisions.
 __device__ __forceinline__ void splat_gauss2(const Rec& r, float pxc, f32x2 npy, float& dx, f32x2& dy,
                                              float (&power)[2], f32x2& G) {
   dx = __fsub_rn(r.a.x, pxc);
@@ -97,376 +89,39 @@ __device__ __forceinline__ bool footprint_meets_block(const Rec& r, float x0, fl
   return qmin <= thr + slack;
 }
 
-// Stage batch b of a tile list (records [b * batch, b * batch + batch)) into
-// buffer (b & 1): one bulk copy per splat, of its record alone (NT = 0, from
-// rec) or of its record and NT probe tangent records (from tan, where they are
-// adjacent; staged as [batch][1 + NT]), issued by the block's threads in turn,
-// all completing on the buffer's mbarrier.
-template <int NT>
-__device__ __forceinline__ void stage_batch(int b, int batch, uint32_t start, int n, int view, int n_pad,
-                                            const uint32_t* __restrict__ vals, const float4* __restrict__ rec,
-                                            const float4* __restrict__ tan, Rec* buf, uint32_t* s_idx,
-                                            uint64_t* bars) {
-  const int bi = b & 1;
-  const int cnt = min(batch, n - b * batch);
-  if (threadIdx.x == 0) mbar_arrive_expect_tx(&bars[bi], (uint32_t)(cnt * (int)sizeof(Rec) * (1 + NT)));
-  fence_proxy_async();
-  for (int q = threadIdx.x; q < cnt; q += blockDim.x) {
-    const uint32_t gi = vals[start + (uint32_t)(b * batch + q)];
-    if (s_idx) s_idx[bi * batch + q] = gi;
-    if (NT > 0)  // the record and its NT probe tangent records, adjacent in tan: one copy
-      bulk_g2s(&buf[((size_t)bi * batch + q) * (1 + NT)], tan + 3 * ((size_t)view * n_pad + gi) * (1 + NT),
-               (1 + NT) * sizeof(Rec), &bars[bi]);
-    else
-      bulk_g2s(&buf[bi * batch + q], rec + 3 * ((size_t)view * n_pad + gi), sizeof(Rec), &bars[bi]);
-  }
-}
-
 // ------------------------------------------------------------ pixel blocks
-// A tile has tile_w x tile_h pixels and half as many threads: each warp covers
-// an 8 x 8 pixel block, warp w the block (w % (tile_w/8), w / (tile_w/8)), and
-// its lane renders pixels (lx, ly) and (lx, ly + 4) of it.  Compact blocks meet
-// few splats; two pixels per thread halve the per-splat warp overheads.
+// A tile is cut into 8 x 8 pixel blocks, block w at (w % (tile_w/8), w / (tile_w/8)),
+// and a lane renders pixels (lx, ly) and (lx, ly + 4) of its warp's block.
+// Compact blocks meet few splats; two pixels per thread halve the per-splat
+// overheads and share a column.
 constexpr int kPixPerThread = 2;
-// Records staged per batch, per thread (when the frame leaves the batch at 0).
-#ifndef GS_BATCH_PER_THREAD
-#define GS_BATCH_PER_THREAD 1
-#endif
-constexpr int kBatchPerThread = GS_BATCH_PER_THREAD;
-// The forward pass stages nthr / kFwdBatchDiv records per batch (its tangent
-// records triple the shared memory of a batch).
-#ifndef GS_FWD_BATCH_DIV
-#define GS_FWD_BATCH_DIV 1
-#endif
-constexpr int kFwdBatchDiv = GS_FWD_BATCH_DIV;
-__host__ __device__ __forceinline__ int fwd_batch(const gs_frame& fr, int nthr) {
-  return fr.batch ? fr.batch : kBatchPerThread * nthr / kFwdBatchDiv;
-}
-// Minimum resident CTAs per SM requested for the forward kernel (0: none), for
-// blocks of 128 threads; blocks of NT threads (tiles of 2 NT pixels) request
-// the same threads per SM.  Six (80 registers, a few bytes spilled) measured
-// 9 % faster than the five that 93 unbounded registers allow; seven spilled
-// more and gained less.
-#ifndef GS_FWD_MIN_BLOCKS
-#define GS_FWD_MIN_BLOCKS 6
-#endif
-#if GS_FWD_MIN_BLOCKS > 0
-#define GS_FWD_BOUNDS(NT) __launch_bounds__(NT, (GS_FWD_MIN_BLOCKS * 128) / (NT))
-#else
-#define GS_FWD_BOUNDS(NT) __launch_bounds__(NT)
-#endif
-// Threads per block the blends are built for: tiles of up to 256 pixels run
-// as blocks of at most 128 threads, tiles of 512 pixels as blocks of 256.
-__host__ __device__ constexpr int blend_threads(int nthr) { return nthr <= 128 ? 128 : 256; }
 
-__device__ __forceinline__ void pixel_of(int tid, int tile_w, int& lx, int& ly) {
-  const int warp = tid >> 5, lane = tid & 31, bxn = tile_w >> 3;
-  lx = (warp % bxn) * 8 + (lane & 7);
-  ly = (warp / bxn) * 8 + (lane >> 3);
-}
-
-// Bit w is set if the splat can reach alpha >= 1/255 at some pixel centre of
-// warp block w.  The record's last word holds the half-extents of the bounding
-// box of that footprint, widened and rounded up by the projection
-// (footprint_extents); a block inside the box is then tested against the
-// ellipse (footprint_meets_block).  Both tests are conservative, so a cleared
-// bit skips only pairs that every pixel of the block skips anyway: results are
-// unchanged.
-__device__ __forceinline__ uint32_t warp_block_mask(const Rec& r, float tile_x0, float tile_y0, int tile_w,
-                                                    int nwarps) {
-  const uint32_t e = __float_as_uint(r.c.w);
-  const float hx = __half2float(__ushort_as_half((unsigned short)(e & 0xffffu)));
-  const float hy = __half2float(__ushort_as_half((unsigned short)(e >> 16)));
-  const int bxn = tile_w >> 3;
-  uint32_t m = 0;
-  for (int w = 0; w < nwarps; ++w) {
-    const float x0 = tile_x0 + (float)((w % bxn) * 8) + 0.5f, x1 = x0 + 7.f;
-    const float y0 = tile_y0 + (float)((w / bxn) * 8) + 0.5f, y1 = y0 + 7.f;
-    if (r.a.x + hx >= x0 && r.a.x - hx <= x1 && r.a.y + hy >= y0 && r.a.y - hy <= y1 &&
-        (!GS_EXACT_BLOCK_TEST || footprint_meets_block(r, x0, y0)))
-      m |= 1u << w;
-  }
-  return m;
-}
-
-// ------------------------------------------------------------------ forward
-// Blend state of one pixel: colour, transmittance, the probe tangents of both,
-// and the list position after the last blended splat.
-template <int NU>
-struct FwdPixel {
-  float C[3], T;
-  float Cd[NU > 0 ? NU : 1][3], Td[NU > 0 ? NU : 1];
-  float pxc, pyc;
-  uint32_t last;
-  bool done;
+// The 8 x 8 block of a one-warp CTA: its view and tile (the heaviest tiles first
+// when an order is given), its number w in the tile and its first pixel.
+struct PixelBlock {
+  int view, tile, w, x0, y0;
 };
-
-// The splat at one pixel: offsets, Gaussian, alpha, and whether it is blended
-// there (a done pixel blends nothing).
-template <int NU>
-__device__ __forceinline__ bool fwd_eval(const FwdPixel<NU>& p, const Rec& r, float& dx, float& dy, float& G,
-                                         float& oG, float& alpha) {
-  dx = __fsub_rn(r.a.x, p.pxc);
-  dy = __fsub_rn(r.a.y, p.pyc);
-  const float power = splat_power(r, dx, dy);
-  G = __expf(power);
-  oG = __fmul_rn(r.b.y, G);
-  alpha = fminf(kAlphaMax, oG);
-  return !p.done && power <= 0.f && alpha >= kAlphaMin;
+__device__ __forceinline__ PixelBlock pixel_block(const uint32_t* __restrict__ order, const gs_frame& fr, int Tx, int T,
+                                                  int log_blocks) {
+  PixelBlock p;
+  p.w = (int)(blockIdx.x & ((1u << log_blocks) - 1u));
+  const int ordinal = (int)(blockIdx.x >> log_blocks);
+  const int blk = order ? (int)min(__ldg(order + ordinal), (gridDim.x >> log_blocks) - 1) : ordinal;
+  p.view = blk / T;
+  p.tile = blk - p.view * T;
+  const int ty = p.tile / Tx, tx = p.tile - ty * Tx, bw = fr.tile_w >> 3;
+  p.x0 = tx * fr.tile_w + (p.w % bw) * 8;
+  p.y0 = ty * fr.tile_h + (p.w / bw) * 8;
+  return p;
 }
 
-// The splat's front-to-back update of one pixel, with the decisions as
-// selects: a pixel that does not blend the splat (on false, or the splat would
-// take T below kTMin, which ends the pixel instead) adds exact zeros and keeps
-// T, its tangents and its last position.  `t0` points at the splat's first
-// rewritten tangent record; the records of further probes follow at stride
-// `tstride`.  With the power's tangent pd, a blended pixel gets
-// C += c a T, C' += c' a T + c (a' T + a T'), T' <- T' (1 - a) - T a', T <- T (1 - a),
-// a' = o' G + a pd (0 for a capped alpha).
-template <int NU>
-__device__ __forceinline__ void fwd_apply(FwdPixel<NU>& p, const Rec& r, const Rec* t0, int tstride, uint32_t pos,
-                                          bool on, float dx, float dy, float G, float oG, float alpha) {
-  const float Tn = p.T * (1.f - alpha);
-  const bool term = on && Tn < kTMin;
-  const bool bl = on && !term;
-  p.done = p.done || term;
-  const float a = bl ? alpha : 0.f;
-  const float w = a * p.T;
-  if constexpr (NU > 0) {
-    const bool live = bl && !(oG > kAlphaMax);  // a capped alpha has no tangent
-#pragma unroll
-    for (int k = 0; k < NU; ++k) {
-      const Rec t = t0[k * tstride];
-      const float pd = dx * (t.a.x * dx + t.a.y * dy + t.a.w) + dy * (t.a.z * dy + t.b.x);
-      const float ad = live ? (t.b.y * G + alpha * pd) : 0.f;
-      const float sk = ad * p.T + a * p.Td[k];
-      p.Cd[k][0] += t.b.z * w + r.b.z * sk;
-      p.Cd[k][1] += t.b.w * w + r.b.w * sk;
-      p.Cd[k][2] += t.c.x * w + r.c.x * sk;
-      p.Td[k] = p.Td[k] * (1.f - a) - p.T * ad;
-    }
-  }
-  p.C[0] += r.b.z * w;
-  p.C[1] += r.b.w * w;
-  p.C[2] += r.c.x * w;
-  p.T = bl ? Tn : p.T;
-  p.last = bl ? pos + 1 : p.last;
-}
-
-// 1: when a batch holds at most one record per thread, each thread reads the
-// Gaussian index of its record in the batch after next one iteration ahead, so
-// that staging a batch does not wait on that read.
-#ifndef GS_FWD_PREFETCH_VALS
-#define GS_FWD_PREFETCH_VALS 1
-#endif
-
-// stage_batch for a batch of at most blockDim.x records, the calling thread's
-// record (threadIdx.x) being splat gi.
-template <int NT>
-__device__ __forceinline__ void stage_batch_one(int b, int batch, int n, int view, int n_pad, uint32_t gi,
-                                                const float4* __restrict__ rec, const float4* __restrict__ tan,
-                                                Rec* buf, uint64_t* bars) {
-  const int bi = b & 1;
-  const int cnt = min(batch, n - b * batch);
-  if (threadIdx.x == 0) mbar_arrive_expect_tx(&bars[bi], (uint32_t)(cnt * (int)sizeof(Rec) * (1 + NT)));
-  fence_proxy_async();
-  const int q = threadIdx.x;
-  if (q < cnt) {
-    if (NT > 0)  // the record and its NT probe tangent records, adjacent in tan: one copy
-      bulk_g2s(&buf[((size_t)bi * batch + q) * (1 + NT)], tan + 3 * ((size_t)view * n_pad + gi) * (1 + NT),
-               (1 + NT) * sizeof(Rec), &bars[bi]);
-    else
-      bulk_g2s(&buf[bi * batch + q], rec + 3 * ((size_t)view * n_pad + gi), sizeof(Rec), &bars[bi]);
-  }
-}
-
-// CB: the frame sets its own batch (else one record per thread, known to the
-// compiler as the block size).
-template <int NU, bool CB, int NT>
-__global__ void GS_FWD_BOUNDS(NT) raster_fwd_kernel(const float4* __restrict__ rec, const float4* __restrict__ tan,
-                                                         const uint32_t* __restrict__ vals,
-                                                         const uint32_t* __restrict__ ranges,
-                                                         const uint32_t* __restrict__ order, int n_pad, gs_frame fr,
-                                                         int Tx, int T, float* __restrict__ image,
-                                                         float* __restrict__ final_T, uint32_t* __restrict__ n_contrib,
-                                                         float* __restrict__ image_tan, uint8_t* __restrict__ masks,
-                                                         int32_t* status) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int nthr = blockDim.x, nwarps = nthr >> 5, batch = CB ? fr.batch : kBatchPerThread * nthr / kFwdBatchDiv;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem);
-  Rec* buf = reinterpret_cast<Rec*>(smem + 16);
-  uint32_t* s_mask = reinterpret_cast<uint32_t*>(buf + 2 * (1 + NU) * batch);  // after both buffers
-  const int tid = threadIdx.x, lane = tid & 31;
-  const uint32_t wbit = 1u << (tid >> 5);
-  // the tile of this block: the heaviest tiles first when an order is given
-  const int blk = order ? (int)min(__ldg(order + blockIdx.x), gridDim.x - 1) : (int)blockIdx.x;
-  const int view = blk / T, tile = blk - view * T;
-  const int ty = tile / Tx, tx = tile - ty * Tx;
-  int lx, ly;
-  pixel_of(tid, fr.tile_w, lx, ly);
-  const float tile_x0 = (float)(tx * fr.tile_w), tile_y0 = (float)(ty * fr.tile_h);
-  const size_t tslot = 2 * ((size_t)view * T + tile);
-  const uint32_t start = ranges[tslot], end = ranges[tslot + 1];
-  const int n = (int)(end - start);
-  if (tid == 0) {
-    mbar_init(&bars[0], 1);
-    mbar_init(&bars[1], 1);
-    fence_mbar_init();
-  }
-  FwdPixel<NU> pix[kPixPerThread];
-  int px[kPixPerThread], py[kPixPerThread];
-#pragma unroll
-  for (int q = 0; q < kPixPerThread; ++q) {
-    px[q] = tx * fr.tile_w + lx;
-    py[q] = ty * fr.tile_h + ly + 4 * q;
-    FwdPixel<NU>& p = pix[q];
-    p.C[0] = p.C[1] = p.C[2] = 0.f;
-    p.T = 1.f;
-#pragma unroll
-    for (int k = 0; k < NU; ++k) p.Cd[k][0] = p.Cd[k][1] = p.Cd[k][2] = p.Td[k] = 0.f;
-    p.pxc = (float)px[q] + 0.5f;
-    p.pyc = (float)py[q] + 0.5f;
-    p.last = 0;
-    p.done = !(px[q] < fr.width && py[q] < fr.height);
-  }
-  __syncthreads();
-
-  const int nb = (n + batch - 1) / batch;
-  int issued = 0;  // batches staged so far (block-uniform)
-  // with at most one record per thread and batch, the index of this thread's
-  // record in batch bb (0 past the list), read one batch ahead of its staging
-  const bool one = GS_FWD_PREFETCH_VALS && batch <= nthr;
-  auto index_of = [&](int bb) -> uint32_t {
-    const int q = bb * batch + tid;
-    return (bb < nb && tid < batch && q < n) ? __ldg(vals + start + (uint32_t)q) : 0u;
-  };
-  uint32_t gi_next = 0;
-  if (nb > 0) {
-    if (one) {
-      stage_batch_one<NU>(0, batch, n, view, n_pad, index_of(0), rec, tan, buf, bars);
-      gi_next = index_of(1);
-    } else {
-      stage_batch<NU>(0, batch, start, n, view, n_pad, vals, rec, tan, buf, nullptr, bars);
-    }
-    issued = 1;
-  }
-  for (int b = 0; b < nb; ++b) {
-    if (b + 1 < nb) {
-      if (one) {
-        stage_batch_one<NU>(b + 1, batch, n, view, n_pad, gi_next, rec, tan, buf, bars);
-        gi_next = index_of(b + 2);
-      } else {
-        stage_batch<NU>(b + 1, batch, start, n, view, n_pad, vals, rec, tan, buf, nullptr, bars);
-      }
-      issued = b + 2;
-    }
-    const int bi = b & 1;
-    const bool ok = mbar_wait_bounded(&bars[bi], (uint32_t)((b >> 1) & 1), status);
-    const int cnt = min(batch, n - b * batch);
-    // record q of the batch; its probe tangent records follow it (NU > 0)
-    auto recp = [&](int q) -> Rec* {
-      return NU > 0 ? &buf[((size_t)bi * batch + q) * (1 + NU)] : &buf[bi * batch + q];
-    };
-    // per splat: which warps it can reach, and the probe tangents of its power
-    // rewritten as the quadratic form pd = dx (a dx + b dy + d) + dy (c dy + e)
-    for (int q = tid; q < cnt; q += nthr) {
-      const Rec r = *recp(q);
-      s_mask[q] = ok ? warp_block_mask(r, tile_x0, tile_y0, fr.tile_w, nwarps) : 0u;
-      if (masks) masks[start + (uint32_t)(b * batch + q)] = (uint8_t)s_mask[q];  // for the reverse passes
-#pragma unroll
-      for (int k = 0; k < NU; ++k) {
-        Rec* tp = recp(q) + 1 + k;
-        const float4 ta = tp->a;  // dmx, dmy, dA, dB
-        const float dC = tp->b.x;
-        tp->a = make_float4(-0.5f * ta.z, -ta.w, -0.5f * dC, -(r.a.z * ta.x + r.a.w * ta.y));
-        tp->b.x = -(r.b.x * ta.y + r.a.w * ta.x);
-      }
-    }
-    __syncthreads();
-    if (!ok) {
-#pragma unroll
-      for (int q = 0; q < kPixPerThread; ++q) pix[q].done = true;
-    }
-    // The warp walks only the splats its block can see: one ballot per 32
-    // splats, then the set bits in list order.
-    for (int j0 = 0; j0 < cnt; j0 += 32) {
-      if (__all_sync(0xffffffffu, pix[0].done && pix[1].done)) break;
-      uint32_t bits = __ballot_sync(0xffffffffu, j0 + lane < cnt && (s_mask[j0 + lane] & wbit));
-      while (bits) {
-        const int j = j0 + __ffs(bits) - 1;
-        bits &= bits - 1;
-        const Rec r = *recp(j);
-        const Rec* t0 = recp(j) + 1;
-        const uint32_t pos = (uint32_t)(b * batch + j);
-        float dx[kPixPerThread], dy[kPixPerThread], G[kPixPerThread], oG[kPixPerThread], al[kPixPerThread];
-        bool on[kPixPerThread];
-#pragma unroll
-        for (int q = 0; q < kPixPerThread; ++q) on[q] = fwd_eval<NU>(pix[q], r, dx[q], dy[q], G[q], oG[q], al[q]);
-        // a pixel row (the lanes' first or second pixels) that no lane blends
-        // the splat at is skipped as a whole; the splat's probe tangent records
-        // are read once for both rows
-        bool rows[kPixPerThread];
-        bool anyrow = false;
-#pragma unroll
-        for (int q = 0; q < kPixPerThread; ++q) {
-          rows[q] = __any_sync(0xffffffffu, on[q]);
-          anyrow = anyrow || rows[q];
-        }
-        if (!anyrow) continue;
-        Rec tk[NU > 0 ? NU : 1];
-#pragma unroll
-        for (int k = 0; k < NU; ++k) tk[k] = t0[k];
-#pragma unroll
-        for (int q = 0; q < kPixPerThread; ++q)
-          if (rows[q]) fwd_apply<NU>(pix[q], r, tk, 1, pos, on[q], dx[q], dy[q], G[q], oG[q], al[q]);
-      }
-    }
-    if (__syncthreads_count(pix[0].done && pix[1].done) == nthr) break;
-  }
-  // Drain: a buffer is refilled only after a barrier that follows every
-  // thread's wait on its previous fill, and only when some wait saw that fill
-  // land, so each buffer has at most one fill in flight, its last.  Thread 0
-  // waits (bounded) for the last fill of both buffers, so that no bulk copy is
-  // still writing into this block's shared memory when it exits: the batch
-  // staged ahead of an early finish, or a fill whose waits ran out.
-  if (tid == 0) {
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      const int last = issued - 1 - (((issued - 1) ^ s) & 1);  // largest batch < issued in buffer s
-      if (last >= 0) mbar_wait_bounded(&bars[s], (uint32_t)((last >> 1) & 1), status);
-    }
-  }
-  const size_t HW = (size_t)fr.width * fr.height;
-#pragma unroll
-  for (int q = 0; q < kPixPerThread; ++q) {
-    if (!(px[q] < fr.width && py[q] < fr.height)) continue;
-    const FwdPixel<NU>& p = pix[q];
-    const size_t at = (size_t)py[q] * fr.width + px[q];
-#pragma unroll
-    for (int ch = 0; ch < 3; ++ch) image[((size_t)view * 3 + ch) * HW + at] = p.C[ch];
-    final_T[(size_t)view * HW + at] = p.T;
-    n_contrib[(size_t)view * HW + at] = p.last;
-#pragma unroll
-    for (int k = 0; k < NU; ++k)
-#pragma unroll
-      for (int ch = 0; ch < 3; ++ch) image_tan[(((size_t)k * fr.n_views + view) * 3 + ch) * HW + at] = p.Cd[k][ch];
-  }
-}
-
-// ------------------------------------------------------------------ reverse
-// The reverse pass runs one warp per CTA, on one 8 x 8 pixel block: the blocks of
-// a tile need nothing from one another, so a warp starts at its own last
-// contributor, stages only the splats its block can see (asynchronous copies
-// into two buffers of 32, whole chunks of 32 list positions at a time) and frees
-// its place on the SM as soon as its own walk ends.  As CTAs of a tile's four
-// warps sharing a ring of TMA-staged batches, staging and the waits for the
-// tile's slowest warp took 0.6 of the 2.6 ms of the blend (1M Gaussians, 8 views
-// of 1080p, two probes): the call went from 3.23 to 2.78 ms, and from 3.40 ms
-// with the warp-wide reduction per splat (no probe 2.29 -> 1.52 ms, one 3.10 ->
-// 2.14 ms; 100k Gaussians, 1297 x 840, one probe 0.66 -> 0.36 ms).
 // True if the splat can reach alpha >= 1/255 at some pixel centre of the 8 x 8
-// block whose first pixel centre is (x0, y0) (the test of warp_block_mask for
-// one block).
+// block whose first pixel centre is (x0, y0).  The record's last word holds the
+// half-extents of the bounding box of that footprint, widened and rounded up by
+// the projection (footprint_extents); a block inside the box is then tested
+// against the ellipse (footprint_meets_block).  Both tests are conservative, so a
+// block that fails them skips only splats that every pixel of it skips anyway:
+// results are unchanged.
 __device__ __forceinline__ bool block_sees(const Rec& r, float x0, float y0) {
   const uint32_t e = __float_as_uint(r.c.w);
   const float hx = __half2float(__ushort_as_half((unsigned short)(e & 0xffffu)));
@@ -475,6 +130,264 @@ __device__ __forceinline__ bool block_sees(const Rec& r, float x0, float y0) {
          (!GS_EXACT_BLOCK_TEST || footprint_meets_block(r, x0, y0));
 }
 
+// ------------------------------------------------------------------ forward
+// Blend state of a thread's two pixels: colour, transmittance, the probe tangents
+// of both, and each pixel's list position after its last blended splat.
+template <int NU>
+struct FwdPair {
+  f32x2 C[3], T;
+  f32x2 Cd[NU > 0 ? NU : 1][3], Td[NU > 0 ? NU : 1];
+  f32x2 npy;  // negated pixel centres
+  float pxc;
+  uint32_t last[2];
+  bool done[2];
+};
+
+// One splat's front-to-back update of the two pixels, with the decisions as
+// selects: a pixel that does not blend the splat (it is done or skips it, or the
+// splat would take T below kTMin, which ends the pixel instead) adds exact
+// zeros and keeps T, its tangents and its last position.  tk: the splat's
+// rewritten tangent records (see raster_fwd_kernel).  With the power's tangent
+// pd, a blended pixel gets C += c a T, C' += c' a T + c (a' T + a T'),
+// T' <- T' (1 - a) - T a', T <- T (1 - a), a' = a (o'/o + pd) (0 for a capped alpha).
+template <int NU>
+__device__ __forceinline__ void fwd_visit(FwdPair<NU>& p, const Rec& r, const Rec* tk, uint32_t pos) {
+  float dx, power[2], oG[2], al[2], Tn[2];
+  f32x2 dy, G;
+  splat_gauss2(r, p.pxc, p.npy, dx, dy, power, G);
+  unpack2(mul2(dup2(r.b.y), G), oG[0], oG[1]);
+  bool on[2], bl[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    al[q] = fminf(kAlphaMax, oG[q]);
+    on[q] = !p.done[q] && power[q] <= 0.f && al[q] >= kAlphaMin;
+  }
+  if (!__any_sync(0xffffffffu, on[0] || on[1])) return;
+  const f32x2 alp = pack2(al[0], al[1]);
+  unpack2(mul2(p.T, fma2(alp, dup2(-1.f), dup2(1.f))), Tn[0], Tn[1]);
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    bl[q] = on[q] && !(Tn[q] < kTMin);
+    p.done[q] = p.done[q] || (on[q] && !bl[q]);
+    p.last[q] = bl[q] ? pos + 1 : p.last[q];
+  }
+  const f32x2 a = pack2(bl[0] ? al[0] : 0.f, bl[1] ? al[1] : 0.f);
+  const f32x2 om = fma2(a, dup2(-1.f), dup2(1.f)), w = mul2(a, p.T);
+  if constexpr (NU > 0) {
+    const bool live0 = bl[0] && !(oG[0] > kAlphaMax), live1 = bl[1] && !(oG[1] > kAlphaMax);
+#pragma unroll
+    for (int k = 0; k < NU; ++k) {
+      const Rec t = tk[k];
+      const float p0 = fmaf(dx, fmaf(t.a.x, dx, t.a.w), t.b.y), p1 = fmaf(t.a.y, dx, t.b.x);
+      float ad0, ad1;
+      unpack2(mul2(alp, fma2(dy, fma2(dy, dup2(t.a.z), dup2(p1)), dup2(p0))), ad0, ad1);
+      const f32x2 adT = mul2(pack2(live0 ? ad0 : 0.f, live1 ? ad1 : 0.f), p.T);
+      const f32x2 sk = fma2(a, p.Td[k], adT);
+      p.Cd[k][0] = fma2(dup2(r.b.z), sk, fma2(dup2(t.b.z), w, p.Cd[k][0]));
+      p.Cd[k][1] = fma2(dup2(r.b.w), sk, fma2(dup2(t.b.w), w, p.Cd[k][1]));
+      p.Cd[k][2] = fma2(dup2(r.c.x), sk, fma2(dup2(t.c.x), w, p.Cd[k][2]));
+      p.Td[k] = fma2(adT, dup2(-1.f), mul2(p.Td[k], om));
+    }
+  }
+  p.C[0] = fma2(dup2(r.b.z), w, p.C[0]);
+  p.C[1] = fma2(dup2(r.b.w), w, p.C[1]);
+  p.C[2] = fma2(dup2(r.c.x), w, p.C[2]);
+  p.T = mul2(p.T, om);  // a pixel that blends nothing has om = 1
+}
+
+// Minimum resident CTAs (warps) per SM requested from the compiler for the
+// forward kernel, by the number of probes, and the splats per staging buffer
+// (larger buffers pause less often, smaller ones leave room for more warps).
+// Measured on 1M Gaussians, 8 views of 1080p: without a probe 32 CTAs and
+// buffers of 32 (0.762 ms; 28 CTAs 0.821, buffers of 16 0.790), with one 30 and
+// 16 (1.053; 24 CTAs 1.165), with two 21 and 24 (80 registers, so 24 CTAs run;
+// 1.370; 20 CTAs and 16 1.487, 25 CTAs 1.486, buffers of 16 1.399, of 32 1.432).
+#ifndef GS_FWD_MB0
+#define GS_FWD_MB0 32
+#endif
+#ifndef GS_FWD_MB1
+#define GS_FWD_MB1 30
+#endif
+#ifndef GS_FWD_MB2
+#define GS_FWD_MB2 21
+#endif
+#ifndef GS_FWD_BUF0
+#define GS_FWD_BUF0 32
+#endif
+#ifndef GS_FWD_BUF1
+#define GS_FWD_BUF1 16
+#endif
+#ifndef GS_FWD_BUF2
+#define GS_FWD_BUF2 24
+#endif
+// Splats per staging buffer, at most 32.
+__host__ __device__ constexpr int fwd_buffer(int nu) { return nu == 0 ? GS_FWD_BUF0 : nu == 1 ? GS_FWD_BUF1 : GS_FWD_BUF2; }
+__host__ __device__ constexpr int fwd_min_blocks(int nu) { return nu == 0 ? GS_FWD_MB0 : nu == 1 ? GS_FWD_MB1 : GS_FWD_MB2; }
+
+// The kernel is bound by issue slots (65 %) and the FMA pipe (50 %).  As CTAs of a
+// tile's four warps that met at two barriers per staged batch, with scalar
+// pixels, it took 1.702 ms with two probes (now 1.370), 1.414 with one (1.053)
+// and 1.085 without (0.762); 100k Gaussians, 1297 x 840, one probe 0.293 ms
+// (0.243).  Instructions per launch of two views: 411M, now 293M.
+// mask_words: the masks as 32-bit words, cleared before the launch (the blocks of
+// a tile set their own bits of the same bytes).
+template <int NU>
+__global__ void __launch_bounds__(32, fwd_min_blocks(NU)) raster_fwd_kernel(
+    const float4* __restrict__ rec, const float4* __restrict__ tan, const uint32_t* __restrict__ vals,
+    const uint32_t* __restrict__ ranges, const uint32_t* __restrict__ order, int n_pad, gs_frame fr, int Tx, int T,
+    int log_blocks, float* __restrict__ image, float* __restrict__ final_T, uint32_t* __restrict__ n_contrib,
+    float* __restrict__ image_tan, uint32_t* __restrict__ mask_words) {
+  constexpr int kFwdBuf = fwd_buffer(NU);
+  constexpr int kPieces = 3 * (1 + NU);  // 16-byte pieces of a splat's record and tangents
+  // two buffers of staged splats (the record, whose radius word is replaced by
+  // the list position, then its tangents), and the splats' indices and positions
+  __shared__ Rec buf[2][kFwdBuf * (1 + NU)];
+  __shared__ uint2 s_who[2][kFwdBuf];
+  const int lane = threadIdx.x;
+  const PixelBlock pb = pixel_block(order, fr, Tx, T, log_blocks);
+  const int view = pb.view;
+  if (pb.x0 >= fr.width || pb.y0 >= fr.height) return;
+  const size_t tslot = 2 * ((size_t)view * T + pb.tile);
+  const uint32_t start = __ldg(ranges + tslot);
+  const int n = (int)(__ldg(ranges + tslot + 1) - start), nc = (n + 31) >> 5;
+  const float wx0 = (float)pb.x0 + 0.5f, wy0 = (float)pb.y0 + 0.5f;  // the block's first pixel centre
+  const int px = pb.x0 + (lane & 7), py = pb.y0 + (lane >> 3);       // and (px, py + 4)
+
+  FwdPair<NU> p;
+  p.C[0] = p.C[1] = p.C[2] = 0ull;
+  p.T = dup2(1.f);
+#pragma unroll
+  for (int k = 0; k < NU; ++k) p.Cd[k][0] = p.Cd[k][1] = p.Cd[k][2] = p.Td[k] = 0ull;
+  p.pxc = (float)px + 0.5f;
+  p.npy = pack2(-((float)py + 0.5f), -((float)(py + 4) + 0.5f));
+  p.last[0] = p.last[1] = 0;
+  p.done[0] = !(px < fr.width && py < fr.height);
+  p.done[1] = !(px < fr.width && py + 4 < fr.height);
+
+  // Chunks of 32 list positions, front to back: a lane holds one position's
+  // index two chunks ahead and its record one chunk ahead of the test whether
+  // the splat can reach this block.
+  const float4* vrec = rec + 3 * (size_t)view * n_pad;
+  int c = 0;
+  auto index_of = [&](int cc) -> uint32_t {
+    const int q = cc * 32 + lane;
+    return q < n ? __ldg(vals + start + (uint32_t)q) : 0xffffffffu;
+  };
+  auto record_of = [&](uint32_t g, Rec& r) {
+    if (g == 0xffffffffu) return;
+    const float4* src = vrec + 3 * (size_t)g;  // what block_sees reads
+    r.a = __ldg(src);
+    const float2 Co = __ldg(reinterpret_cast<const float2*>(src + 1));
+    r.b.x = Co.x;
+    r.b.y = Co.y;
+    r.c.w = __ldg(reinterpret_cast<const float*>(src + 2) + 3);
+  };
+  uint32_t gi = index_of(0), gi1 = index_of(1), gi2 = 0, bits = 0;
+  Rec rn{};
+  record_of(gi, rn);
+  // tests chunk c (index gi, record rn), marks its visible pairs, and starts the
+  // loads of the chunks after it
+  auto test = [&]() {
+    bits = 0;
+    if (c >= nc) return;
+    bits = __ballot_sync(0xffffffffu, gi != 0xffffffffu && block_sees(rn, wx0, wy0));
+    if (mask_words && lane <= 8) {
+      // byte q of the masks is pair q's: the chunk's bits, shifted to the words'
+      // boundaries, four at a time spread over a word's bytes at bit w
+      const uint32_t at = start + (uint32_t)(c * 32);
+      const uint32_t nib = (uint32_t)(((uint64_t)bits << (at & 3u)) >> (4 * lane)) & 15u;
+      if (nib) atomicOr(mask_words + (at >> 2) + lane, ((nib * 0x204081u) & 0x01010101u) << pb.w);
+    }
+    record_of(gi1, rn);
+    gi2 = index_of(c + 2);
+  };
+  test();
+  auto fill = [&](int b) {
+    int cnt = 0;
+    while (c < nc) {
+      const int at = cnt + __popc(bits & ((1u << lane) - 1u));
+      const bool mine = ((bits >> lane) & 1u) && at < kFwdBuf;
+      if (mine) s_who[b][at] = make_uint2(gi, (uint32_t)(c * 32 + lane));
+      cnt += __popc(bits);
+      if (cnt > kFwdBuf) {  // the rest of the chunk goes to the next buffer
+        bits &= ~__ballot_sync(0xffffffffu, mine);
+        cnt = kFwdBuf;
+        break;
+      }
+      ++c;
+      gi = gi1;
+      gi1 = gi2;
+      test();
+    }
+    __syncwarp();
+    const float4* src = NU > 0 ? tan + (size_t)kPieces * ((size_t)view * n_pad) : vrec;
+    for (int q = lane; q < cnt * kPieces; q += 32) {
+      const int e = q / kPieces;
+      cp_async16(reinterpret_cast<float4*>(buf[b]) + q, src + (size_t)kPieces * s_who[b][e].x + (q - e * kPieces));
+    }
+    cp_async_commit();
+    return cnt;
+  };
+
+  int cur = 0, cnt = fill(0);
+  while (cnt > 0) {
+    const int cnt_next = fill(cur ^ 1);
+    cp_async_wait_prior();  // all but the newest group: this buffer has landed
+    __syncwarp();
+    if (lane < cnt) {
+      // the list position, and the probe tangents of the splat's power and
+      // opacity rewritten as pd + o'/o = (a dx + d) dx + f + (b dx + e) dy + c dy^2
+      Rec* rp = &buf[cur][lane * (1 + NU)];
+      const float4 ra = rp->a;
+      const float rC = rp->b.x, o = rp->b.y;
+      rp->c.z = __uint_as_float(s_who[cur][lane].y);
+#pragma unroll
+      for (int k = 0; k < NU; ++k) {
+        Rec* tp = rp + 1 + k;
+        const float4 ta = tp->a;  // dmx, dmy, dA, dB
+        const float dC = tp->b.x;
+        tp->a = make_float4(-0.5f * ta.z, -ta.w, -0.5f * dC, -(ra.z * ta.x + ra.w * ta.y));
+        tp->b.x = -(rC * ta.y + ra.w * ta.x);
+        tp->b.y = __fdividef(tp->b.y, o);
+      }
+    }
+    __syncwarp();
+    for (int j = 0; j < cnt; ++j) {
+      const Rec r = buf[cur][j * (1 + NU)];
+      fwd_visit<NU>(p, r, &buf[cur][j * (1 + NU) + 1], __float_as_uint(r.c.z));
+    }
+    if (__all_sync(0xffffffffu, p.done[0] && p.done[1])) break;
+    __syncwarp();  // the buffer may be refilled
+    cur ^= 1;
+    cnt = cnt_next;
+  }
+  cp_async_wait_all();  // a buffer staged ahead of an early end lands before the CTA does
+
+  const size_t HW = (size_t)fr.width * fr.height, at = (size_t)py * fr.width + px;
+  auto store = [&](float* plane, f32x2 v) {
+    float lo, hi;
+    unpack2(v, lo, hi);
+    if (px < fr.width && py < fr.height) plane[at] = lo;
+    if (px < fr.width && py + 4 < fr.height) plane[at + 4 * (size_t)fr.width] = hi;
+  };
+#pragma unroll
+  for (int ch = 0; ch < 3; ++ch) store(image + ((size_t)view * 3 + ch) * HW, p.C[ch]);
+  store(final_T + (size_t)view * HW, p.T);
+  store(reinterpret_cast<float*>(n_contrib) + (size_t)view * HW,
+        pack2(__uint_as_float(p.last[0]), __uint_as_float(p.last[1])));
+#pragma unroll
+  for (int k = 0; k < NU; ++k)
+#pragma unroll
+    for (int ch = 0; ch < 3; ++ch) store(image_tan + (((size_t)k * fr.n_views + view) * 3 + ch) * HW, p.Cd[k][ch]);
+}
+
+// ------------------------------------------------------------------ reverse
+// Against CTAs of a tile's four warps sharing a ring of TMA-staged batches, where
+// staging and the waits for the tile's slowest warp took 0.6 of the blend's 2.6
+// ms (1M Gaussians, 8 views of 1080p, two probes), one warp per CTA took the call
+// from 3.23 to 2.78 ms; with the merge below it was 3.40 ms before (no probe
+// 2.29 -> 1.52 ms, one 3.10 -> 2.14 ms; 100k Gaussians, 1297 x 840, one probe 0.66
+// -> 0.36 ms).
 // Minimum resident CTAs (warps) per SM requested from the compiler for the
 // reverse kernel, by the number of cotangent streams: without a probe 32 (64
 // registers, the most CTAs an SM holds; 28: 1.548 against 1.518 ms per call of
@@ -731,14 +644,10 @@ __global__ void __launch_bounds__(32, bwd_min_blocks((GRAD ? 1 : 0) + NU)) raste
   f32x2* s_w = slots + kMergeSlots * merge_slot_pairs(S);
   const int lane = threadIdx.x;
   if (blockIdx.x == 0 && lane == 0) cot_hdr->clear_floats = 0;  // the rows are being added into
-  // the tile of this block: the heaviest tiles first when an order is given
-  const int wb = (int)(blockIdx.x & ((1u << log_blocks) - 1u)), ordinal = (int)(blockIdx.x >> log_blocks);
-  const int blk = order ? (int)min(__ldg(order + ordinal), (gridDim.x >> log_blocks) - 1) : ordinal;
-  const int view = blk / T, tile = blk - view * T;
-  const int ty = tile / Tx, tx = tile - ty * Tx;
-  const int bx0 = tx * fr.tile_w + (wb % (fr.tile_w >> 3)) * 8, by0 = ty * fr.tile_h + (wb / (fr.tile_w >> 3)) * 8;
+  const PixelBlock pb = pixel_block(order, fr, Tx, T, log_blocks);
+  const int view = pb.view, wb = pb.w, bx0 = pb.x0, by0 = pb.y0;
   if (bx0 >= fr.width || by0 >= fr.height) return;
-  const size_t tslot = 2 * ((size_t)view * T + tile);
+  const size_t tslot = 2 * ((size_t)view * T + pb.tile);
   const uint32_t start = __ldg(ranges + tslot), len = __ldg(ranges + tslot + 1) - start;
   if (len == 0 && !want_loss) return;
   const size_t HW = (size_t)fr.width * fr.height;
@@ -1446,6 +1355,12 @@ TileGrid tile_grid(gs_frame fr) {
   return g;
 }
 
+int log_tile_blocks(gs_frame fr) {  // 8 x 8 blocks per tile, a power of two
+  int b = 0;
+  while ((64 << b) < fr.tile_w * fr.tile_h) ++b;
+  return b;
+}
+
 template <class F>
 cudaError_t allow_smem(F* f, size_t bytes) {
   return cudaFuncSetAttribute((const void*)f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
@@ -1453,24 +1368,16 @@ cudaError_t allow_smem(F* f, size_t bytes) {
 
 template <int NU>
 gs_status launch_fwd(const gs_projected* proj, const gs_sorted* sorted, int n_pad, gs_frame fr, float* image,
-                     float* final_T, uint32_t* n_contrib, float* image_tan, int32_t* status, cudaStream_t st) {
+                     float* final_T, uint32_t* n_contrib, float* image_tan, cudaStream_t st) {
   const TileGrid g = tile_grid(fr);
-  const int nthr = fr.tile_w * fr.tile_h / kPixPerThread, batch = fwd_batch(fr, nthr);
-  const size_t smem = 16 + (size_t)batch * (2 * sizeof(Rec) * (1 + NU) + sizeof(uint32_t));
-  // the dynamic shared-memory limit, raised as far as a launch needs
-  const bool cb = fr.batch != 0, big = blend_threads(nthr) == 256;
-  auto* kern = big ? (cb ? raster_fwd_kernel<NU, true, 256> : raster_fwd_kernel<NU, false, 256>)
-                   : (cb ? raster_fwd_kernel<NU, true, 128> : raster_fwd_kernel<NU, false, 128>);
-  static size_t attr[2][2] = {{0, 0}, {0, 0}};
-  if (smem > attr[big][cb]) {
-    if (allow_smem(kern, smem) != cudaSuccess) return check_launch("gs_raster_fwd: smem attribute");
-    attr[big][cb] = smem;
-  }
-  const unsigned blocks = (unsigned)((size_t)fr.n_views * g.T);
-  kern<<<blocks, nthr, smem, st>>>(reinterpret_cast<const float4*>(proj->rec),
-                                   reinterpret_cast<const float4*>(proj->tangent), sorted->vals, sorted->ranges,
-                                   sorted->order, n_pad,
-                                   fr, g.Tx, g.T, image, final_T, n_contrib, image_tan, sorted->masks, status);
+  if (sorted->masks && cudaMemsetAsync(sorted->masks, 0, sorted->capacity, st) != cudaSuccess)
+    return check_launch("gs_raster_fwd: memset");
+  const int log_blocks = log_tile_blocks(fr);
+  const unsigned blocks = (unsigned)((size_t)fr.n_views * g.T << log_blocks);
+  raster_fwd_kernel<NU><<<blocks, 32, 0, st>>>(
+      reinterpret_cast<const float4*>(proj->rec), reinterpret_cast<const float4*>(proj->tangent), sorted->vals,
+      sorted->ranges, sorted->order, n_pad, fr, g.Tx, g.T, log_blocks, image, final_T, n_contrib, image_tan,
+      reinterpret_cast<uint32_t*>(sorted->masks));
   return check_launch("gs_raster_fwd");
 }
 
@@ -1525,8 +1432,7 @@ void launch_bwd_kernels(const gs_params* x, const BatchArg* ba, int n_pad, int d
   const TileGrid g = tile_grid(fr);
   const double views_per_objective = ba ? 1.0 : (double)fr.n_views;
   const float inv_m = (float)(1.0 / (3.0 * (double)fr.width * fr.height * views_per_objective));
-  int log_blocks = 0;  // 8 x 8 blocks per tile
-  while ((64 << log_blocks) < fr.tile_w * fr.tile_h) ++log_blocks;
+  const int log_blocks = log_tile_blocks(fr);
   const unsigned blocks = (unsigned)((size_t)fr.n_views * g.T << log_blocks);
   raster_bwd_kernel<NU, GRAD><<<blocks, 32, 0, st>>>(
       reinterpret_cast<const float4*>(proj->rec), sorted->vals, sorted->ranges, sorted->order, n_pad, fr, g.Tx, g.T,
@@ -1636,6 +1542,7 @@ extern "C" gs_status gs_raster_fwd(const gs_projected* proj, const gs_sorted* so
                                    const gs_probe* probe, float* image, float* final_T, uint32_t* n_contrib,
                                    float* image_tangent, int32_t* status, void* stream) {
   using namespace gs;
+  (void)status;
   GS_REQUIRE(proj && sorted && proj->rec && sorted->vals && sorted->ranges, "gs_raster_fwd: null argument");
   GS_REQUIRE(image && final_T && n_contrib, "gs_raster_fwd: null output");
   GS_REQUIRE(frame_ok(frame), "gs_raster_fwd: bad frame (tile %dx%d)", frame.tile_w, frame.tile_h);
@@ -1647,9 +1554,9 @@ extern "C" gs_status gs_raster_fwd(const gs_projected* proj, const gs_sorted* so
   }
   GS_REQUIRE(nu == 0 || proj->tangent, "gs_raster_fwd: probes given but proj->tangent is NULL");
   cudaStream_t st = (cudaStream_t)stream;
-  if (nu == 0) return launch_fwd<0>(proj, sorted, n_pad, frame, image, final_T, n_contrib, nullptr, status, st);
-  if (nu == 1) return launch_fwd<1>(proj, sorted, n_pad, frame, image, final_T, n_contrib, image_tangent, status, st);
-  return launch_fwd<2>(proj, sorted, n_pad, frame, image, final_T, n_contrib, image_tangent, status, st);
+  if (nu == 0) return launch_fwd<0>(proj, sorted, n_pad, frame, image, final_T, n_contrib, nullptr, st);
+  if (nu == 1) return launch_fwd<1>(proj, sorted, n_pad, frame, image, final_T, n_contrib, image_tangent, st);
+  return launch_fwd<2>(proj, sorted, n_pad, frame, image, final_T, n_contrib, image_tangent, st);
 }
 
 extern "C" size_t gs_raster_bwd_workspace_size(int32_t n_pad, gs_frame frame, int32_t nu) {

@@ -11,10 +11,20 @@
 //   A[a] = G*(a dS/dmx) + 2 x G*(a dS/dEx2) + y G*(a dS/dExy)   (G is symmetric)
 //   dS[d] = dS/dmx G*d + dS/dEx2 G*(2 x d) + dS/dExy G*(y d)
 //
-// Every pass works on 32 x 32 output tiles of one (view, channel) plane: the
-// inputs of the tile and its 5-pixel halo go to shared memory (zero outside
-// the image), the products are filtered horizontally into shared memory, then
-// vertically, and an epilogue combines the filtered values at each pixel.
+// Two kernels: the first filters the image, the target and the probes' tangents
+// and writes the SSIM map's partials and each probe's weighted derivative; the
+// second filters those and writes the cotangents of all streams.  Both work on
+// 32 x 32 output tiles of one (view, channel) plane: the inputs of the tile and
+// its 5-pixel halo go to shared memory by asynchronous copies (zero outside the
+// image), up to three pairs of products at a time are filtered horizontally into
+// shared memory, then vertically into registers, and an epilogue combines the
+// filtered values at each pixel.  Packing the products that are filtered alike
+// (image and target, the two probes) and running two kernels instead of four
+// (S is no longer stored, the partials are read once) took 8 views of 1080p with
+// two probes from 3.31 to 2.17 ms: issue slots 61-66 %, shared memory 70 % of
+// its bandwidth.  Three blocks of 256 threads run per SM; with 2 x 4 pixels of
+// row pairs per thread and all products of a tile filtered at once, two blocks of
+// 192 fitted and the loads' latency showed (3.47 ms).
 #include <cmath>
 
 #include "common.cuh"
@@ -25,91 +35,107 @@ namespace {
 constexpr int kR = 5, kTile = 32, kIn = kTile + 2 * kR;  // 42
 constexpr int kSsimThreads = 256;
 constexpr float kC1 = 1e-4f, kC2 = 9e-4f;
-__constant__ float c_win[2 * kR + 1];
 
 struct Plane {
   int W, H, planes;  // planes = views x 3
 };
+struct Window {  // the symmetric window: w[|d|] for offsets d = -5..5
+  float w[kR + 1];
+};
 
-// inputs of the tile (with halo) of NIN planes into s_in[NIN][kIn][kIn]
-template <int NIN>
-__device__ __forceinline__ void load_tile(const float* const (&src)[NIN], size_t plane_off, int W, int H, int x0,
-                                          int y0, float (*s_in)[kIn][kIn]) {
-  for (int q = threadIdx.x; q < kIn * kIn; q += blockDim.x) {
+// Shared memory.  Two quantities that are filtered alike are held as pairs, so
+// that a packed instruction filters both.  Rows are an odd number of pairs long:
+// the horizontal pass gives consecutive lanes consecutive rows.
+constexpr int kInRow = 43, kInPlane = kIn * kInRow;    // staged inputs, [kIn][kInRow]
+constexpr int kHRow = 33, kHPlane = kIn * kHRow;       // horizontal sums, [kIn][kHRow]
+constexpr int kGroup = 3;                              // pairs filtered at a time
+
+// Starts the copies of a plane's tile (with halo) into dst[(ty * kInRow + tx) * stride].
+__device__ __forceinline__ void load_tile(const float* __restrict__ src, int W, int H, int x0, int y0, float* dst,
+                                          int stride) {
+#pragma unroll
+  for (int n = 0; n < (kIn * kIn + kSsimThreads - 1) / kSsimThreads; ++n) {
+    const int q = n * kSsimThreads + (int)threadIdx.x;
+    if (q >= kIn * kIn) break;
     const int ty = q / kIn, tx = q - ty * kIn;
     const int gx = x0 - kR + tx, gy = y0 - kR + ty;
     const bool in = gx >= 0 && gx < W && gy >= 0 && gy < H;
-    const size_t at = plane_off + (size_t)(in ? gy : 0) * W + (in ? gx : 0);
-#pragma unroll
-    for (int k = 0; k < NIN; ++k) s_in[k][ty][tx] = in ? src[k][at] : 0.f;
+    cp_async4_or_zero(dst + (ty * kInRow + tx) * stride, in ? src + (size_t)gy * W + gx : src, in);
   }
 }
 
-// Horizontal window sums of NOUT products (prod of the NIN inputs at (ty, tx))
-// for all kIn rows and the kTile output columns.  A thread covers kCols adjacent
-// columns of one row and reads each input value once; every sum still adds its
-// 11 terms in window order.
+// Horizontal window sums of NPAIR pairs of products (prod(at, p) of the inputs at
+// index `at`) for all kIn rows and kTile columns.  A thread covers kCols columns
+// of one row and forms each product once; every sum adds its 11 terms in window
+// order.
 constexpr int kCols = 4, kRows = 4;
-template <int NIN, int NOUT, class Prod>
-__device__ __forceinline__ void filter_tile(float (*s_in)[kIn][kIn], float (*s_h)[kIn][kTile], Prod prod) {
-  for (int q = threadIdx.x; q < kIn * (kTile / kCols); q += blockDim.x) {
-    const int ty = q / (kTile / kCols), ox0 = (q - ty * (kTile / kCols)) * kCols;
-    float acc[NOUT][kCols];
+template <int NPAIR, class Prod>
+__device__ __forceinline__ void filter_rows(f32x2* s_h, const Window& win, Prod prod) {
+  for (int q = threadIdx.x; q < kIn * (kTile / kCols); q += kSsimThreads) {
+    const int cg = q / kIn, row = q - cg * kIn;
+    f32x2 acc[NPAIR][kCols];
 #pragma unroll
-    for (int o = 0; o < NOUT; ++o)
+    for (int o = 0; o < NPAIR; ++o)
 #pragma unroll
-      for (int j = 0; j < kCols; ++j) acc[o][j] = 0.f;
+      for (int j = 0; j < kCols; ++j) acc[o][j] = 0ull;
 #pragma unroll
     for (int c = 0; c < kCols + 2 * kR; ++c) {
-      float v[NIN];
-#pragma unroll
-      for (int k = 0; k < NIN; ++k) v[k] = s_in[k][ty][ox0 + c];
-      float p[NOUT];
-      prod(v, p);
+      f32x2 p[NPAIR];
+      prod(row * kInRow + cg * kCols + c, p);
 #pragma unroll
       for (int j = 0; j < kCols; ++j) {
         const int dd = c - j;
         if (dd >= 0 && dd <= 2 * kR) {
+          const f32x2 w = dup2(win.w[dd < kR ? kR - dd : dd - kR]);
 #pragma unroll
-          for (int o = 0; o < NOUT; ++o) acc[o][j] += c_win[dd] * p[o];
+          for (int o = 0; o < NPAIR; ++o) acc[o][j] = fma2(w, p[o], acc[o][j]);
         }
       }
     }
 #pragma unroll
-    for (int o = 0; o < NOUT; ++o)
+    for (int o = 0; o < NPAIR; ++o)
 #pragma unroll
-      for (int j = 0; j < kCols; ++j) s_h[o][ty][ox0 + j] = acc[o][j];
+      for (int j = 0; j < kCols; ++j) s_h[o * kHPlane + row * kHRow + cg * kCols + j] = acc[o][j];
   }
 }
 
-// Vertical window sums at output rows oy0 .. oy0 + kRows - 1 of column ox, each
-// horizontal sum read once.
-template <int NOUT>
-__device__ __forceinline__ void vertical(float (*s_h)[kIn][kTile], int oy0, int ox, float (&out)[NOUT][kRows]) {
+// Vertical window sums at the thread's pixels: rows oy0 .. oy0 + kRows - 1 of
+// column ox, each horizontal sum read once.
+template <int NPAIR>
+__device__ __forceinline__ void filter_columns(const f32x2* s_h, const Window& win, int oy0, int ox,
+                                               f32x2 (&out)[NPAIR][kRows]) {
 #pragma unroll
-  for (int o = 0; o < NOUT; ++o)
+  for (int o = 0; o < NPAIR; ++o) {
 #pragma unroll
-    for (int j = 0; j < kRows; ++j) out[o][j] = 0.f;
+    for (int j = 0; j < kRows; ++j) out[o][j] = 0ull;
 #pragma unroll
-  for (int c = 0; c < kRows + 2 * kR; ++c) {
-#pragma unroll
-    for (int o = 0; o < NOUT; ++o) {
-      const float hv = s_h[o][oy0 + c][ox];
+    for (int c = 0; c < kRows + 2 * kR; ++c) {
+      const f32x2 h = s_h[o * kHPlane + (oy0 + c) * kHRow + ox];
 #pragma unroll
       for (int j = 0; j < kRows; ++j) {
         const int dd = c - j;
-        if (dd >= 0 && dd <= 2 * kR) out[o][j] += c_win[dd] * hv;
+        if (dd >= 0 && dd <= 2 * kR) out[o][j] = fma2(dup2(win.w[dd < kR ? kR - dd : dd - kR]), h, out[o][j]);
       }
     }
   }
 }
-
-// The output pixels of a thread: rows oy0 .. oy0 + kRows - 1 of column ox.
+// The output pixels of a thread.
 __device__ __forceinline__ void out_block(int& oy0, int& ox) {
   ox = threadIdx.x % kTile;
   oy0 = (threadIdx.x / kTile) * kRows;
 }
 static_assert(kSsimThreads * kRows == kTile * kTile, "one block of kRows pixels per thread");
+
+__device__ __forceinline__ float lo2(f32x2 v) {
+  float a, b;
+  unpack2(v, a, b);
+  return a;
+}
+__device__ __forceinline__ float hi2(f32x2 v) {
+  float a, b;
+  unpack2(v, a, b);
+  return b;
+}
 
 // SSIM and its partials by the raw window moments at one pixel
 __device__ __forceinline__ void ssim_at(float mx, float my, float ex2, float ey2, float exy, float& S, float& dmx,
@@ -127,48 +153,85 @@ __device__ __forceinline__ void ssim_at(float mx, float my, float ex2, float ey2
   dexy = d_sxy;
 }
 
-// pass 1: S and its partials per pixel; the objective's sum
-__global__ void __launch_bounds__(kSsimThreads) ssim_stats_kernel(const float* __restrict__ img,
-                                                                  const float* __restrict__ tgt, Plane pl, float lambda,
-                                                                  float inv_2m, float* __restrict__ S,
-                                                                  float* __restrict__ P1, float* __restrict__ P2,
-                                                                  float* __restrict__ P3, float* __restrict__ loss) {
-  extern __shared__ __align__(16) float smem[];
-  float(*s_in)[kIn][kIn] = reinterpret_cast<float(*)[kIn][kIn]>(smem);
-  float(*s_h)[kIn][kTile] = reinterpret_cast<float(*)[kIn][kTile]>(smem + 2 * kIn * kIn);
+// The SSIM map's partials P1..P3 by the window moments, the objective's sum, and
+// for each of NP probes a_k = lambda/(4 max(1 - S, floor))/m . dS[d_k].  The
+// planes of d and a are `stride` floats apart.
+template <int NP>
+__global__ void __launch_bounds__(kSsimThreads, 3) ssim_map_kernel(
+    const float* __restrict__ img, const float* __restrict__ tgt, const float* __restrict__ d, Plane pl, size_t stride,
+    Window win, float lambda, float inv_2m, float wscale, float floor_, float* __restrict__ P1, float* __restrict__ P2,
+    float* __restrict__ P3, float* __restrict__ a, float* __restrict__ loss) {
+  extern __shared__ __align__(16) f32x2 smem2[];
+  f32x2* s_xy = smem2;             // (image, target)
+  f32x2* s_d = s_xy + kInPlane;    // the probes' tangents
+  f32x2* s_h = smem2 + (NP > 0 ? 2 : 1) * kInPlane;
   __shared__ float s_red[kSsimThreads / 32];
   const int x0 = blockIdx.x * kTile, y0 = blockIdx.y * kTile;
   const size_t off = (size_t)blockIdx.z * pl.W * pl.H;
-  const float* src[2] = {img, tgt};
-  load_tile<2>(src, off, pl.W, pl.H, x0, y0, s_in);
+  load_tile(img + off, pl.W, pl.H, x0, y0, reinterpret_cast<float*>(s_xy), 2);
+  load_tile(tgt + off, pl.W, pl.H, x0, y0, reinterpret_cast<float*>(s_xy) + 1, 2);
+#pragma unroll
+  for (int k = 0; k < NP; ++k)
+    load_tile(d + (size_t)k * stride + off, pl.W, pl.H, x0, y0, reinterpret_cast<float*>(s_d) + k, 2);
+  cp_async_wait_all();
   __syncthreads();
-  filter_tile<2, 5>(s_in, s_h, [](const float (&v)[2], float (&p)[5]) {
-    p[0] = v[0];
-    p[1] = v[1];
-    p[2] = v[0] * v[0];
-    p[3] = v[1] * v[1];
-    p[4] = v[0] * v[1];
-  });
-  __syncthreads();
-  float lsum = 0.f;
   int oy0, ox;
   out_block(oy0, ox);
-  float fb[5][kRows];
-  vertical<5>(s_h, oy0, ox, fb);
+  float lsum = 0.f, g1[kRows], g2[kRows], g3[kRows], wv[kRows];
+  {
+    filter_rows<3>(s_h, win, [&](int at, f32x2 (&p)[3]) {
+      p[0] = s_xy[at];
+      p[1] = mul2(p[0], p[0]);
+      p[2] = pack2(lo2(p[0]) * hi2(p[0]), 0.f);
+    });
+    __syncthreads();
+    f32x2 f[3][kRows];
+    filter_columns<3>(s_h, win, oy0, ox, f);
 #pragma unroll
-  for (int j = 0; j < kRows; ++j) {
-    const int oy = oy0 + j;
-    const int gx = x0 + ox, gy = y0 + oy;
-    if (gx >= pl.W || gy >= pl.H) continue;
-    float s, d1, d2, d3;
-    ssim_at(fb[0][j], fb[1][j], fb[2][j], fb[3][j], fb[4][j], s, d1, d2, d3);
-    const size_t at = off + (size_t)gy * pl.W + gx;
-    S[at] = s;
-    P1[at] = d1;
-    P2[at] = d2;
-    P3[at] = d3;
-    const float r = s_in[0][oy + kR][ox + kR] - s_in[1][oy + kR][ox + kR];
-    lsum += ((1.f - lambda) * fabsf(r) + lambda * (1.f - s)) * inv_2m;
+    for (int j = 0; j < kRows; ++j) {
+      float s;
+      ssim_at(lo2(f[0][j]), hi2(f[0][j]), lo2(f[1][j]), hi2(f[1][j]), lo2(f[2][j]), s, g1[j], g2[j], g3[j]);
+      const int gx = x0 + ox, gy = y0 + oy0 + j;
+      wv[j] = wscale / (4.f * fmaxf(1.f - s, floor_));
+      if (gx >= pl.W || gy >= pl.H) continue;
+      const size_t at = off + (size_t)gy * pl.W + gx;
+      P1[at] = g1[j];
+      P2[at] = g2[j];
+      P3[at] = g3[j];
+      const f32x2 xy = s_xy[(oy0 + j + kR) * kInRow + ox + kR];
+      lsum += ((1.f - lambda) * fabsf(lo2(xy) - hi2(xy)) + lambda * (1.f - s)) * inv_2m;
+    }
+  }
+  if constexpr (NP > 0) {
+    constexpr int NPAIR = NP == 2 ? 3 : 2;
+    __syncthreads();  // the sums have been read
+    filter_rows<NPAIR>(s_h, win, [&](int at, f32x2 (&p)[NPAIR]) {
+      const f32x2 xy = s_xy[at], dk = s_d[at];
+      const float x2 = 2.f * lo2(xy), y = hi2(xy);
+      if constexpr (NP == 2) {
+        p[0] = dk;
+        p[1] = mul2(dup2(x2), dk);
+        p[2] = mul2(dup2(y), dk);
+      } else {
+        p[0] = pack2(lo2(dk), x2 * lo2(dk));
+        p[1] = pack2(y * lo2(dk), 0.f);
+      }
+    });
+    __syncthreads();
+    f32x2 f[NPAIR][kRows];
+    filter_columns<NPAIR>(s_h, win, oy0, ox, f);
+#pragma unroll
+    for (int j = 0; j < kRows; ++j) {
+      const int gx = x0 + ox, gy = y0 + oy0 + j;
+      if (gx >= pl.W || gy >= pl.H) continue;
+      const size_t at = off + (size_t)gy * pl.W + gx;
+      if constexpr (NP == 2) {
+        a[at] = wv[j] * (g1[j] * lo2(f[0][j]) + g2[j] * lo2(f[1][j]) + g3[j] * lo2(f[2][j]));
+        a[stride + at] = wv[j] * (g1[j] * hi2(f[0][j]) + g2[j] * hi2(f[1][j]) + g3[j] * hi2(f[2][j]));
+      } else {
+        a[at] = wv[j] * (g1[j] * lo2(f[0][j]) + g2[j] * hi2(f[0][j]) + g3[j] * lo2(f[1][j]));
+      }
+    }
   }
   if (loss) {
 #pragma unroll
@@ -183,148 +246,153 @@ __global__ void __launch_bounds__(kSsimThreads) ssim_stats_kernel(const float* _
   }
 }
 
-// pass 2, all NP probes of the step in one launch (the image, target, S and
-// partials read once): a_k = lambda/(4 max(1 - S, floor))/m . dS[d_k]; the
-// probes' planes are `stride` floats apart
-template <int NP>
-__global__ void __launch_bounds__(kSsimThreads) ssim_jvp_kernel(const float* __restrict__ d,
-                                                                const float* __restrict__ img,
-                                                                const float* __restrict__ tgt, Plane pl, size_t stride,
-                                                                const float* __restrict__ S,
-                                                                const float* __restrict__ P1,
-                                                                const float* __restrict__ P2,
-                                                                const float* __restrict__ P3, float wscale,
-                                                                float floor_, float* __restrict__ a) {
-  extern __shared__ __align__(16) float smem[];
-  float(*s_in)[kIn][kIn] = reinterpret_cast<float(*)[kIn][kIn]>(smem);
-  float(*s_h)[kIn][kTile] = reinterpret_cast<float(*)[kIn][kTile]>(smem + (NP + 2) * kIn * kIn);
+// The cotangent images: the gradient stream (GRAD; the map's adjoint with
+// weights all 1) and NA probe streams (the adjoint of the weight planes a_k),
+// each with its L1 part.  The planes of a, d and cot are `stride` floats apart.
+template <int NA, bool GRAD>
+__global__ void __launch_bounds__(kSsimThreads, 3) ssim_cot_kernel(
+    const float* __restrict__ a, const float* __restrict__ img, const float* __restrict__ tgt, Plane pl, size_t stride,
+    Window win, const float* __restrict__ P1, const float* __restrict__ P2, const float* __restrict__ P3,
+    const float* __restrict__ d, float lambda, float inv_m, float floor_, float* __restrict__ cot) {
+  extern __shared__ __align__(16) f32x2 smem2[];
+  f32x2* s_p = smem2;                // (P1, P2)
+  f32x2* s_a = s_p + kInPlane;       // the probes' weights
+  f32x2* s_h = s_p + (NA > 0 ? 2 : 1) * kInPlane;
+  float* s_p3 = reinterpret_cast<float*>(s_h + kGroup * kHPlane);
   const int x0 = blockIdx.x * kTile, y0 = blockIdx.y * kTile;
   const size_t off = (size_t)blockIdx.z * pl.W * pl.H;
-  const float* src[NP + 2];
+  load_tile(P1 + off, pl.W, pl.H, x0, y0, reinterpret_cast<float*>(s_p), 2);
+  load_tile(P2 + off, pl.W, pl.H, x0, y0, reinterpret_cast<float*>(s_p) + 1, 2);
+  load_tile(P3 + off, pl.W, pl.H, x0, y0, s_p3, 1);
 #pragma unroll
-  for (int k = 0; k < NP; ++k) src[k] = d + (size_t)k * stride;
-  src[NP] = img;
-  src[NP + 1] = tgt;
-  load_tile<NP + 2>(src, off, pl.W, pl.H, x0, y0, s_in);
-  __syncthreads();
-  filter_tile<NP + 2, 3 * NP>(s_in, s_h, [](const float (&v)[NP + 2], float (&p)[3 * NP]) {
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-      p[3 * k] = v[k];
-      p[3 * k + 1] = 2.f * v[NP] * v[k];
-      p[3 * k + 2] = v[NP + 1] * v[k];
-    }
-  });
-  __syncthreads();
+  for (int k = 0; k < NA; ++k)
+    load_tile(a + (size_t)k * stride + off, pl.W, pl.H, x0, y0, reinterpret_cast<float*>(s_a) + k, 2);
   int oy0, ox;
   out_block(oy0, ox);
-  float fb[3 * NP][kRows];
-  vertical<3 * NP>(s_h, oy0, ox, fb);
+  float x[kRows], y[kRows];
+  const int gx = x0 + ox, gy0 = y0 + oy0;
+  const size_t at0 = off + (size_t)gy0 * pl.W + gx;
 #pragma unroll
   for (int j = 0; j < kRows; ++j) {
-    const int oy = oy0 + j;
-    const int gx = x0 + ox, gy = y0 + oy;
-    if (gx >= pl.W || gy >= pl.H) continue;
-    const size_t at = off + (size_t)gy * pl.W + gx;
-    const float p1 = P1[at], p2 = P2[at], p3 = P3[at];
-    const float w = wscale / (4.f * fmaxf(1.f - S[at], floor_));
-#pragma unroll
-    for (int k = 0; k < NP; ++k)
-      a[(size_t)k * stride + at] = w * (p1 * fb[3 * k][j] + p2 * fb[3 * k + 1][j] + p3 * fb[3 * k + 2][j]);
+    const bool in = gx < pl.W && gy0 + j < pl.H;
+    x[j] = in ? __ldg(img + at0 + (size_t)j * pl.W) : 0.f;
+    y[j] = in ? __ldg(tgt + at0 + (size_t)j * pl.W) : 0.f;
   }
-}
-
-// pass 3: the adjoint of NA weight planes a_k (NA = 0: one stream with weights
-// all 1, the gradient) plus the L1 part, into NA (or 1) cotangent images; the
-// planes of a, d and cot are `stride` floats apart
-template <int NA>
-__global__ void __launch_bounds__(kSsimThreads) ssim_vjp_kernel(const float* __restrict__ a,
-                                                                const float* __restrict__ img,
-                                                                const float* __restrict__ tgt, Plane pl, size_t stride,
-                                                                const float* __restrict__ P1,
-                                                                const float* __restrict__ P2,
-                                                                const float* __restrict__ P3,
-                                                                const float* __restrict__ d, float lambda,
-                                                                float inv_m, float floor_, float* __restrict__ cot) {
-  constexpr int NS = NA > 0 ? NA : 1;  // output streams
-  constexpr int NIN = NA + 3;
-  extern __shared__ __align__(16) float smem[];
-  float(*s_in)[kIn][kIn] = reinterpret_cast<float(*)[kIn][kIn]>(smem);
-  float(*s_h)[kIn][kTile] = reinterpret_cast<float(*)[kIn][kTile]>(smem + NIN * kIn * kIn);
-  const int x0 = blockIdx.x * kTile, y0 = blockIdx.y * kTile;
-  const size_t off = (size_t)blockIdx.z * pl.W * pl.H;
-  const float* src[NIN];
-#pragma unroll
-  for (int k = 0; k < NA; ++k) src[k] = a + (size_t)k * stride;
-  src[NA] = P1;
-  src[NA + 1] = P2;
-  src[NA + 2] = P3;
-  load_tile<NIN>(src, off, pl.W, pl.H, x0, y0, s_in);
+  cp_async_wait_all();
   __syncthreads();
-  filter_tile<NIN, 3 * NS>(s_in, s_h, [](const float (&v)[NIN], float (&p)[3 * NS]) {
+  if constexpr (GRAD) {
+    filter_rows<2>(s_h, win, [&](int at, f32x2 (&p)[2]) {
+      p[0] = s_p[at];
+      p[1] = pack2(s_p3[at], 0.f);
+    });
+    __syncthreads();
+    f32x2 f[2][kRows];
+    filter_columns<2>(s_h, win, oy0, ox, f);
 #pragma unroll
-    for (int k = 0; k < NS; ++k) {
-      const float wk = NA > 0 ? v[k] : 1.f;  // weights all 1: the products are the partials
-      p[3 * k] = wk * v[NA];
-      p[3 * k + 1] = wk * v[NA + 1];
-      p[3 * k + 2] = wk * v[NA + 2];
+    for (int j = 0; j < kRows; ++j) {
+      if (gx >= pl.W || gy0 + j >= pl.H) continue;
+      const float r = x[j] - y[j], A = lo2(f[0][j]) + 2.f * x[j] * hi2(f[0][j]) + y[j] * lo2(f[1][j]);
+      cot[at0 + (size_t)j * pl.W] = 0.5f * inv_m * ((1.f - lambda) * (float)((r > 0.f) - (r < 0.f)) - lambda * A);
     }
-  });
-  __syncthreads();
-  int oy0, ox;
-  out_block(oy0, ox);
-  float fb[3 * NS][kRows];
-  vertical<3 * NS>(s_h, oy0, ox, fb);
+  }
+  if constexpr (NA > 0) {
+    constexpr int NPAIR = NA == 2 ? 3 : 2;
+    float* out = cot + (GRAD ? stride : 0);
+    float dv[NA][kRows];
 #pragma unroll
-  for (int j = 0; j < kRows; ++j) {
-    const int oy = oy0 + j;
-    const int gx = x0 + ox, gy = y0 + oy;
-    if (gx >= pl.W || gy >= pl.H) continue;
-    const size_t at = off + (size_t)gy * pl.W + gx;
-    const float x = img[at], y = tgt[at], r = x - y;
+    for (int k = 0; k < NA; ++k)
 #pragma unroll
-    for (int k = 0; k < NS; ++k) {
-      const float A = fb[3 * k][j] + 2.f * x * fb[3 * k + 1][j] + y * fb[3 * k + 2][j];
-      if (NA == 0)
-        cot[at] = 0.5f * inv_m * ((1.f - lambda) * (float)((r > 0.f) - (r < 0.f)) - lambda * A);
-      else
-        cot[(size_t)k * stride + at] =
-            (1.f - lambda) * inv_m / (4.f * fmaxf(fabsf(r), floor_)) * d[(size_t)k * stride + at] + A;
+      for (int j = 0; j < kRows; ++j)
+        dv[k][j] = gx < pl.W && gy0 + j < pl.H ? __ldg(d + (size_t)k * stride + at0 + (size_t)j * pl.W) : 0.f;
+    if (GRAD) __syncthreads();  // the sums have been read
+    filter_rows<NPAIR>(s_h, win, [&](int at, f32x2 (&p)[NPAIR]) {
+      const f32x2 p12 = s_p[at], ak = s_a[at];
+      const float p3 = s_p3[at];
+      if constexpr (NA == 2) {
+        p[0] = mul2(ak, dup2(lo2(p12)));
+        p[1] = mul2(ak, dup2(hi2(p12)));
+        p[2] = mul2(ak, dup2(p3));
+      } else {
+        p[0] = mul2(dup2(lo2(ak)), p12);
+        p[1] = pack2(lo2(ak) * p3, 0.f);
+      }
+    });
+    __syncthreads();
+    f32x2 f[NPAIR][kRows];
+    filter_columns<NPAIR>(s_h, win, oy0, ox, f);
+#pragma unroll
+    for (int j = 0; j < kRows; ++j) {
+      if (gx >= pl.W || gy0 + j >= pl.H) continue;
+      const float l1 = (1.f - lambda) * inv_m / (4.f * fmaxf(fabsf(x[j] - y[j]), floor_));
+#pragma unroll
+      for (int k = 0; k < NA; ++k) {
+        float f0, f1, f2;
+        if constexpr (NA == 2) {
+          f0 = k ? hi2(f[0][j]) : lo2(f[0][j]);
+          f1 = k ? hi2(f[1][j]) : lo2(f[1][j]);
+          f2 = k ? hi2(f[2][j]) : lo2(f[2][j]);
+        } else {
+          f0 = lo2(f[0][j]);
+          f1 = hi2(f[0][j]);
+          f2 = lo2(f[1][j]);
+        }
+        out[(size_t)k * stride + at0 + (size_t)j * pl.W] = l1 * dv[k][j] + (f0 + 2.f * x[j] * f1 + y[j] * f2);
+      }
     }
   }
 }
 
-size_t smem_bytes(int nin, int nout) { return sizeof(float) * ((size_t)nin * kIn * kIn + (size_t)nout * kIn * kTile); }
+// Shared memory of the kernels: their pair planes, the sums of a group, and P3.
+size_t map_smem(int np) { return sizeof(f32x2) * ((np > 0 ? 2 : 1) * kInPlane + kGroup * kHPlane); }
+size_t cot_smem(int na) { return map_smem(na) + sizeof(float) * kInPlane; }
 
-cudaError_t set_window() {
-  static bool done = false;
+Window window() {
+  double g[kR + 1], s = 0.0;
+  for (int i = 0; i <= kR; ++i) g[i] = std::exp(-(double)(i * i) / (2.0 * 1.5 * 1.5));
+  for (int i = -kR; i <= kR; ++i) s += g[i < 0 ? -i : i];
+  Window w;
+  for (int i = 0; i <= kR; ++i) w.w[i] = (float)(g[i] / s);
+  return w;
+}
+
+template <class F>
+cudaError_t allow_smem(F* f, size_t bytes, bool& done) {
   if (done) return cudaSuccess;
-  double g[2 * kR + 1], s = 0.0;
-  for (int i = -kR; i <= kR; ++i) s += g[i + kR] = std::exp(-(double)(i * i) / (2.0 * 1.5 * 1.5));
-  float gf[2 * kR + 1];
-  for (int i = 0; i <= 2 * kR; ++i) gf[i] = (float)(g[i] / s);
-  cudaError_t e = cudaMemcpyToSymbol(c_win, gf, sizeof(gf));
-  if (e == cudaSuccess) {
-    e = cudaFuncSetAttribute((const void*)ssim_stats_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem_bytes(2, 5));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute((const void*)ssim_jvp_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem_bytes(3, 3));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute((const void*)ssim_jvp_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem_bytes(4, 6));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute((const void*)ssim_vjp_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem_bytes(3, 3));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute((const void*)ssim_vjp_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem_bytes(4, 3));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute((const void*)ssim_vjp_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem_bytes(5, 6));
-  }
+  const cudaError_t e = cudaFuncSetAttribute((const void*)f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   done = e == cudaSuccess;
   return e;
+}
+
+// Planes of the call and where they are.
+struct SsimArgs {
+  Plane pl;
+  size_t stride;
+  Window win;
+  const float *img, *tgt, *d;
+  float lambda, inv_m, floor_;
+  float *P1, *P2, *P3, *a, *cot, *loss;
+};
+
+template <int NP>
+cudaError_t launch_ssim(const SsimArgs& s, bool grad, cudaStream_t st) {
+  const dim3 grid((s.pl.W + kTile - 1) / kTile, (s.pl.H + kTile - 1) / kTile, s.pl.planes);
+  const size_t sm_map = map_smem(NP), sm_cot = cot_smem(NP);
+  static bool map_done = false, cot_done[2] = {false, false};
+  cudaError_t e = allow_smem(ssim_map_kernel<NP>, sm_map, map_done);
+  if (e != cudaSuccess) return e;
+  ssim_map_kernel<NP><<<grid, kSsimThreads, sm_map, st>>>(s.img, s.tgt, s.d, s.pl, s.stride, s.win, s.lambda,
+                                                          0.5f * s.inv_m, s.lambda * s.inv_m, s.floor_, s.P1, s.P2,
+                                                          s.P3, s.a, s.loss);
+  if (grad) {
+    if ((e = allow_smem(ssim_cot_kernel<NP, true>, sm_cot, cot_done[1])) != cudaSuccess) return e;
+    ssim_cot_kernel<NP, true><<<grid, kSsimThreads, sm_cot, st>>>(s.a, s.img, s.tgt, s.pl, s.stride, s.win, s.P1, s.P2,
+                                                                  s.P3, s.d, s.lambda, s.inv_m, s.floor_, s.cot);
+  } else if constexpr (NP > 0) {
+    if ((e = allow_smem(ssim_cot_kernel<NP, false>, sm_cot, cot_done[0])) != cudaSuccess) return e;
+    ssim_cot_kernel<NP, false><<<grid, kSsimThreads, sm_cot, st>>>(s.a, s.img, s.tgt, s.pl, s.stride, s.win, s.P1,
+                                                                   s.P2, s.P3, s.d, s.lambda, s.inv_m, s.floor_, s.cot);
+  }
+  return cudaSuccess;
 }
 
 }  // namespace
@@ -333,7 +401,7 @@ cudaError_t set_window() {
 extern "C" size_t gs_dssim_workspace_size(gs_frame frame, int32_t nu) {
   if (frame.n_views < 1 || frame.width < 1 || frame.height < 1 || nu < 0 || nu > 2) return 0;
   const size_t plane = (size_t)frame.n_views * 3 * frame.width * frame.height;
-  return plane * sizeof(float) * (4 + (size_t)nu);  // S, three partials, one weight map per probe
+  return plane * sizeof(float) * (4 + (size_t)nu);  // three partials, one weight map per probe (and one plane spare)
 }
 
 extern "C" gs_status gs_dssim_cotangents(gs_frame frame, const float* image, const float* target,
@@ -350,34 +418,26 @@ extern "C" gs_status gs_dssim_cotangents(gs_frame frame, const float* image, con
   const size_t need = gs_dssim_workspace_size(frame, nu);
   GS_REQUIRE(workspace && workspace_bytes >= need, "gs_dssim_cotangents: workspace needs %zu bytes, got %zu", need,
              workspace_bytes);
-  if (set_window() != cudaSuccess) return check_launch("gs_dssim_cotangents: window");
   cudaStream_t st = (cudaStream_t)stream;
-  const Plane pl{frame.width, frame.height, frame.n_views * 3};
-  const size_t plane = (size_t)pl.planes * pl.W * pl.H;
+  SsimArgs a;
+  a.pl = Plane{frame.width, frame.height, frame.n_views * 3};
+  const size_t plane = a.stride = (size_t)a.pl.planes * a.pl.W * a.pl.H;
   float* ws = (float*)workspace;
-  float *S = ws, *P1 = ws + plane, *P2 = ws + 2 * plane, *P3 = ws + 3 * plane, *A = ws + 4 * plane;
-  const double m = 6.0 * frame.width * frame.height * frame.n_views;
-  const float inv_m = (float)(1.0 / m), inv_2m = (float)(0.5 / m);
-  const dim3 grid((pl.W + kTile - 1) / kTile, (pl.H + kTile - 1) / kTile, pl.planes);
-  ssim_stats_kernel<<<grid, kSsimThreads, smem_bytes(2, 5), st>>>(image, target, pl, lambda, inv_2m, S, P1, P2, P3,
-                                                                   loss_out);
-  if (nu == 1)
-    ssim_jvp_kernel<1><<<grid, kSsimThreads, smem_bytes(3, 3), st>>>(image_tangent, image, target, pl, plane, S, P1,
-                                                                      P2, P3, lambda * inv_m, gn_floor, A);
-  else if (nu == 2)
-    ssim_jvp_kernel<2><<<grid, kSsimThreads, smem_bytes(4, 6), st>>>(image_tangent, image, target, pl, plane, S, P1,
-                                                                      P2, P3, lambda * inv_m, gn_floor, A);
-  float* cot_p = cot;
-  if (want_grad) {
-    ssim_vjp_kernel<0><<<grid, kSsimThreads, smem_bytes(3, 3), st>>>(nullptr, image, target, pl, plane, P1, P2, P3,
-                                                                      nullptr, lambda, inv_m, gn_floor, cot_p);
-    cot_p += plane;
-  }
-  if (nu == 1)
-    ssim_vjp_kernel<1><<<grid, kSsimThreads, smem_bytes(4, 3), st>>>(A, image, target, pl, plane, P1, P2, P3,
-                                                                      image_tangent, lambda, inv_m, gn_floor, cot_p);
-  else if (nu == 2)
-    ssim_vjp_kernel<2><<<grid, kSsimThreads, smem_bytes(5, 6), st>>>(A, image, target, pl, plane, P1, P2, P3,
-                                                                      image_tangent, lambda, inv_m, gn_floor, cot_p);
+  a.win = window();
+  a.img = image;
+  a.tgt = target;
+  a.d = image_tangent;
+  a.lambda = lambda;
+  a.inv_m = (float)(1.0 / (6.0 * frame.width * frame.height * frame.n_views));
+  a.floor_ = gn_floor;
+  a.P1 = ws;
+  a.P2 = ws + plane;
+  a.P3 = ws + 2 * plane;
+  a.a = ws + 3 * plane;
+  a.cot = cot;
+  a.loss = loss_out;
+  const cudaError_t e = nu == 0 ? launch_ssim<0>(a, want_grad != 0, st)
+                        : nu == 1 ? launch_ssim<1>(a, want_grad != 0, st) : launch_ssim<2>(a, want_grad != 0, st);
+  if (e != cudaSuccess) return check_launch("gs_dssim_cotangents: smem attribute");
   return check_launch("gs_dssim_cotangents");
 }

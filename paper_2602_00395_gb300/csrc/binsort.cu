@@ -15,11 +15,13 @@
 //            within a tile is the emission order, so no depth bits are moved
 //   ranges   [start, end) of every tile
 //
-// Each radix pass is a per-block digit histogram, a device-wide scan of the
-// histograms, and a scatter that ranks each block's keys stably in shared
-// memory and writes every digit's run contiguously; no block waits on another.
-// The result is the total order (key, splat index).  Grids are sized by the
-// pair capacity and read P from device memory, so the call needs no host
+// A radix pass cuts its segment into one contiguous range per resident block: a
+// kernel counts each range's digits, another turns the counts into first output
+// positions (for many ranges), and the scatter walks its range tile by tile,
+// ranks each tile's keys stably in shared memory and writes every digit's run
+// contiguously, carrying the positions from tile to tile; no block waits on
+// another.  The result is the total order (key, splat index).  Grids are sized
+// for the chip and read P from device memory, so the call needs no host
 // synchronisation (and can be captured in a graph).
 #include "common.cuh"
 
@@ -29,17 +31,13 @@ namespace {
 constexpr int kScanThreads = 256;
 constexpr int kScanItems = 8;
 constexpr int kScanChunk = kScanThreads * kScanItems;  // 2048
-// Items per thread of a radix tile, and the scatter's resident blocks per SM
-// (its launch bound); overridable at build time for sweeps.
-#ifndef GS_RADIX_ITEMS
-#define GS_RADIX_ITEMS 8
-#endif
-#ifndef GS_RADIX_MIN_BLOCKS
-#define GS_RADIX_MIN_BLOCKS 4
-#endif
+// A radix tile is kRadixThreads x ITEMS items.  ITEMS is 16 where digits are many
+// and the input fills the chip (longer runs per digit; 2 resident blocks per SM),
+// else 8 (3 blocks): 12.2M pairs, random low digits 87 against 102 us, high digits
+// with few values per warp 69 against 58 us.
 constexpr int kRadixThreads = 256;
-constexpr int kRadixItems = GS_RADIX_ITEMS;
-constexpr int kRadixTile = kRadixThreads * kRadixItems;  // 2048 by default
+__host__ __device__ constexpr int radix_tile(int items) { return kRadixThreads * items; }
+__host__ __device__ constexpr int radix_blocks(int items) { return items == 16 ? 2 : 3; }
 constexpr int kRadixWarps = kRadixThreads / 32;
 
 __device__ __forceinline__ uint32_t lanemask_lt() {
@@ -91,8 +89,8 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t& t
 }
 
 // ------------------------------------------------------------------ records
-// Per record g: counts[g] = its pairs; rkeys[g] = bits(depth) (then sorted
-// within each view's segment); rvals[g] = g; and its row table for the emit:
+// Per record g: rkeys[g] = bits(depth) (then sorted within each view's segment,
+// the first pass taking g itself as the value); and its row table for the emit:
 // one entry per row of its rectangle, (pairs in the rows above, first tile),
 // allocated from `rows` by one atomic per block, and the header
 // hdr[g] = (bits(depth), first row | rows << 16, table offset, pairs).  The
@@ -100,8 +98,7 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t& t
 // are contiguous), so rows_cap = pair capacity + 2 x records overflows only with
 // the pairs; then the record keeps no table and GS_FLAG_CAPACITY is raised.
 __global__ void record_keys_kernel(const float4* __restrict__ rec, int n_pad, gs_frame fr, int Tx, int Ty,
-                                   uint32_t* __restrict__ counts, uint32_t* __restrict__ rkeys,
-                                   uint32_t* __restrict__ rvals, uint4* __restrict__ hdr, uint2* __restrict__ rows,
+                                   uint32_t* __restrict__ rkeys, uint4* __restrict__ hdr, uint2* __restrict__ rows,
                                    uint64_t rows_cap, uint32_t* __restrict__ rows_used, int32_t* __restrict__ status) {
   __shared__ uint32_t s_warp[32];
   __shared__ uint32_t s_base;
@@ -141,40 +138,30 @@ __global__ void record_keys_kernel(const float4* __restrict__ rec, int n_pad, gs
     R = 0;
     if (status) atomicOr(status, GS_FLAG_CAPACITY);
   }
-  counts[g] = cnt;
   hdr[g] = make_uint4(__float_as_uint(depth), (uint32_t)f.y0 | (R << 16), off, cnt);
   rkeys[g] = __float_as_uint(depth);
-  rvals[g] = (uint32_t)g;
-}
-
-// scnt[p] = counts of the record at sorted position p
-__global__ void gather_counts_kernel(const uint32_t* __restrict__ order, const uint32_t* __restrict__ counts,
-                                     uint32_t* __restrict__ scnt, size_t items) {
-  const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p < items) scnt[p] = counts[order[p]];
 }
 
 // ------------------------------------------------------------------- scan
-// Length of a scan: n, or, when `pairs` is given, the radix histogram length
-// 256 * ceil(min(*pairs, capacity) / tile) of the pairs in use.
-__device__ __forceinline__ size_t scan_length(size_t n, const uint32_t* pairs, uint64_t capacity) {
-  if (!pairs) return n;
-  const uint64_t p = *pairs < capacity ? *pairs : capacity;
-  return (size_t)256 * (size_t)((p + kRadixTile - 1) / kRadixTile);
-}
-
-__global__ void __launch_bounds__(kScanThreads) scan_reduce_kernel(const uint32_t* __restrict__ in, size_t n_host,
-                                                                   const uint32_t* pairs, uint64_t capacity,
-                                                                   uint32_t* __restrict__ block_sums) {
+// scnt[p] = the pairs of the record at sorted position p, and the sum of each
+// chunk of kScanChunk of them.
+__global__ void __launch_bounds__(kScanThreads) gather_counts_kernel(const uint32_t* __restrict__ order,
+                                                                     const uint4* __restrict__ hdr,
+                                                                     uint32_t* __restrict__ scnt, size_t items,
+                                                                     uint32_t* __restrict__ block_sums) {
   __shared__ uint32_t s_warp[32];
-  const size_t n = scan_length(n_host, pairs, capacity);
   const size_t base = (size_t)blockIdx.x * kScanChunk;
-  if (base >= n) return;
-  uint32_t s = 0;
+  uint32_t c[kScanItems], s = 0;
 #pragma unroll
   for (int k = 0; k < kScanItems; ++k) {
-    size_t idx = base + (size_t)k * kScanThreads + threadIdx.x;
-    if (idx < n) s += in[idx];
+    const size_t p = base + (size_t)k * kScanThreads + threadIdx.x;
+    c[k] = p < items ? __ldg(&hdr[__ldg(order + p)].w) : 0u;
+  }
+#pragma unroll
+  for (int k = 0; k < kScanItems; ++k) {
+    const size_t p = base + (size_t)k * kScanThreads + threadIdx.x;
+    if (p < items) scnt[p] = c[k];
+    s += c[k];
   }
   uint32_t total;
   block_exclusive_scan(s, total, s_warp);
@@ -182,109 +169,88 @@ __global__ void __launch_bounds__(kScanThreads) scan_reduce_kernel(const uint32_
 }
 
 // One block: exclusive scan of the block sums; the grand total goes to *total
-// (and, if capacity is non-zero, GS_FLAG_CAPACITY is raised when it exceeds it).
-__global__ void __launch_bounds__(1024) scan_blocks_kernel(uint32_t* __restrict__ sums, size_t n_host,
-                                                           const uint32_t* pairs, uint64_t pair_capacity,
+// (GS_FLAG_CAPACITY is raised when it exceeds the capacity).
+__global__ void __launch_bounds__(1024) scan_blocks_kernel(uint32_t* __restrict__ sums, int nb,
                                                            uint32_t* __restrict__ total, uint64_t capacity,
                                                            int32_t* __restrict__ status) {
   __shared__ uint32_t s_warp[32];
-  __shared__ uint32_t s_carry;
-  const int nb = (int)((scan_length(n_host, pairs, pair_capacity) + kScanChunk - 1) / kScanChunk);
-  if (threadIdx.x == 0) s_carry = 0;
-  __syncthreads();
-  for (int base = 0; base < nb; base += blockDim.x) {
-    const int idx = base + threadIdx.x;
-    const uint32_t v = idx < nb ? sums[idx] : 0;
-    uint32_t chunk_total;
-    const uint32_t ex = block_exclusive_scan(v, chunk_total, s_warp);
-    const uint32_t carry = s_carry;
-    if (idx < nb) sums[idx] = carry + ex;
-    __syncthreads();
-    if (threadIdx.x == 0) s_carry = carry + chunk_total;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    if (total) *total = s_carry;
-    if (capacity && (uint64_t)s_carry > capacity && status) atomicOr(status, GS_FLAG_CAPACITY);
-  }
-}
-
-__global__ void __launch_bounds__(kScanThreads) scan_apply_kernel(const uint32_t* in, uint32_t* out, size_t n_host,
-                                                                  const uint32_t* pairs, uint64_t capacity,
-                                                                  const uint32_t* __restrict__ block_sums) {
-  __shared__ uint32_t s_warp[32];
-  const size_t n = scan_length(n_host, pairs, capacity);
-  if ((size_t)blockIdx.x * kScanChunk >= n) return;
-  const size_t base = (size_t)blockIdx.x * kScanChunk + (size_t)threadIdx.x * kScanItems;
-  uint32_t v[kScanItems];
-  uint32_t s = 0;
-#pragma unroll
-  for (int k = 0; k < kScanItems; ++k) {
-    v[k] = (base + k < n) ? in[base + k] : 0u;
-    s += v[k];
-  }
-  uint32_t total;
-  uint32_t run = block_exclusive_scan(s, total, s_warp) + block_sums[blockIdx.x];
-#pragma unroll
-  for (int k = 0; k < kScanItems; ++k) {
-    if (base + k < n) out[base + k] = run;
-    run += v[k];
-  }
-}
-
-// The whole scan in one block of 1024 threads (chunks of 8192 entries with a
-// carried total), for lengths where three dependent launches would cost more
-// than the work: the short histograms of small scenes.
-constexpr size_t kSingleScanMax = 65536;
-__global__ void __launch_bounds__(1024) scan_single_kernel(const uint32_t* in, uint32_t* out, size_t n_host,
-                                                           const uint32_t* pairs, uint64_t pair_capacity,
-                                                           uint32_t* __restrict__ total, uint64_t capacity,
-                                                           int32_t* __restrict__ status) {
-  __shared__ uint32_t s_warp[32];
-  const size_t n = scan_length(n_host, pairs, pair_capacity);
   uint32_t carry = 0;
-  for (size_t base = 0; base < n; base += (size_t)1024 * kScanItems) {
-    const size_t b = base + (size_t)threadIdx.x * kScanItems;
-    uint32_t v[kScanItems];
-    uint32_t s = 0;
+  for (int base = 0; base < nb; base += (int)blockDim.x * kScanItems) {
+    const int b = base + (int)threadIdx.x * kScanItems;
+    uint32_t v[kScanItems], s = 0;
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
-      v[k] = b + k < n ? in[b + k] : 0u;
+      v[k] = b + k < nb ? sums[b + k] : 0u;
       s += v[k];
     }
     uint32_t tot;
     uint32_t run = block_exclusive_scan(s, tot, s_warp) + carry;
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
-      if (b + k < n) out[b + k] = run;
+      if (b + k < nb) sums[b + k] = run;
       run += v[k];
     }
     carry += tot;
   }
   if (threadIdx.x == 0) {
-    if (total) *total = carry;
-    if (capacity && (uint64_t)carry > capacity && status) atomicOr(status, GS_FLAG_CAPACITY);
+    *total = carry;
+    if ((uint64_t)carry > capacity && status) atomicOr(status, GS_FLAG_CAPACITY);
+  }
+}
+
+// In place: the exclusive scan of n entries, given the scanned sums of its chunks.
+__global__ void __launch_bounds__(kScanThreads) scan_apply_kernel(uint32_t* __restrict__ v_all, size_t n,
+                                                                  const uint32_t* __restrict__ block_sums) {
+  __shared__ uint32_t s_warp[32];
+  const size_t base = (size_t)blockIdx.x * kScanChunk + (size_t)threadIdx.x * kScanItems;
+  uint32_t v[kScanItems];
+  uint32_t s = 0;
+#pragma unroll
+  for (int k = 0; k < kScanItems; ++k) {
+    v[k] = (base + k < n) ? v_all[base + k] : 0u;
+    s += v[k];
+  }
+  uint32_t total;
+  uint32_t run = block_exclusive_scan(s, total, s_warp) + block_sums[blockIdx.x];
+#pragma unroll
+  for (int k = 0; k < kScanItems; ++k) {
+    if (base + k < n) v_all[base + k] = run;
+    run += v[k];
+  }
+}
+
+// Gather, scan and total in one block, for up to kSmallScan records: one launch
+// where three would each cost more than the work.
+constexpr size_t kSmallScan = 16384;
+__global__ void __launch_bounds__(1024) small_offsets_kernel(const uint32_t* __restrict__ order,
+                                                             const uint4* __restrict__ hdr, uint32_t* __restrict__ scnt,
+                                                             int items, uint32_t* __restrict__ total, uint64_t capacity,
+                                                             int32_t* __restrict__ status) {
+  __shared__ uint32_t s_warp[32];
+  uint32_t carry = 0;
+  for (int base = 0; base < items; base += 1024 * kScanItems) {
+    const int p = base + (int)threadIdx.x * kScanItems;
+    uint32_t v[kScanItems], s = 0;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) v[k] = p + k < items ? __ldg(&hdr[__ldg(order + p + k)].w) : 0u;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) s += v[k];
+    uint32_t tot;
+    uint32_t run = block_exclusive_scan(s, tot, s_warp) + carry;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+      if (p + k < items) scnt[p + k] = run;
+      run += v[k];
+    }
+    carry += tot;
+  }
+  if (threadIdx.x == 0) {
+    *total = carry;
+    if ((uint64_t)carry > capacity && status) atomicOr(status, GS_FLAG_CAPACITY);
   }
 }
 
 inline int scan_blocks(size_t n) { return (int)((n + kScanChunk - 1) / kScanChunk); }
-
-// in -> out exclusive scan of n_max entries (in may equal out).  If `pairs` is
-// given, only the radix histogram of the pairs in use is scanned (n_max bounds
-// it).  The grand total goes to *total; GS_FLAG_CAPACITY is raised when it
-// exceeds a non-zero `capacity`.
-void exclusive_scan(const uint32_t* in, uint32_t* out, size_t n_max, const uint32_t* pairs, uint64_t pair_capacity,
-                    uint32_t* block_sums, uint32_t* total, uint64_t capacity, int32_t* status, cudaStream_t st) {
-  const int nb = scan_blocks(n_max);
-  if (nb == 0) return;
-  if (n_max <= kSingleScanMax) {
-    scan_single_kernel<<<1, 1024, 0, st>>>(in, out, n_max, pairs, pair_capacity, total, capacity, status);
-    return;
-  }
-  scan_reduce_kernel<<<nb, kScanThreads, 0, st>>>(in, n_max, pairs, pair_capacity, block_sums);
-  scan_blocks_kernel<<<1, 1024, 0, st>>>(block_sums, n_max, pairs, pair_capacity, total, capacity, status);
-  scan_apply_kernel<<<nb, kScanThreads, 0, st>>>(in, out, n_max, pairs, pair_capacity, block_sums);
-}
 
 // ------------------------------------------------------------------- emit
 // One warp emits the pairs of 32 consecutive records in (view, depth) order.
@@ -292,10 +258,15 @@ void exclusive_scan(const uint32_t* in, uint32_t* out, size_t n_max, const uint3
 // order), so the warp writes its whole range with consecutive lanes on
 // consecutive pairs; each lane finds the record that owns its pair by a binary
 // search over the warp's prefix sums, and the pair's row by a binary search
-// over that record's row table (see record_keys_kernel).
-__global__ void emit_kernel(const uint4* __restrict__ hdr, const uint2* __restrict__ rows, int n_pad, gs_frame fr,
-                            int Tx, int Ty, const uint32_t* __restrict__ order, const uint32_t* __restrict__ offsets,
-                            uint64_t capacity, uint32_t* __restrict__ keys, uint32_t* __restrict__ vals) {
+// over that record's row table (see record_keys_kernel), N pairs per lane at
+// once: two where records have few pairs (8 blocks per SM; four: 286 against
+// 246 us for 45M pairs of 8M records), four where they have many (61k records
+// of 64 pairs: 76 against 101 us with one).
+template <int N>
+__global__ void __launch_bounds__(256, N == 2 ? 8 : 5) emit_kernel(
+    const uint4* __restrict__ hdr, const uint2* __restrict__ rows, int n_pad, gs_frame fr, int Tx, int Ty,
+    const uint32_t* __restrict__ order, const uint32_t* __restrict__ offsets, uint64_t capacity,
+    uint32_t* __restrict__ keys, uint32_t* __restrict__ vals) {
   const size_t G = (size_t)fr.n_views * n_pad;
   const size_t p0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;  // sorted record position
   const size_t w0 = p0 - (threadIdx.x & 31);
@@ -322,46 +293,63 @@ __global__ void emit_kernel(const uint4* __restrict__ hdr, const uint2* __restri
   const uint32_t start = incl - cnt;
   const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
   const uint64_t base = offsets[w0];
-  const uint32_t rounds = (total + 31) / 32;
-  for (uint32_t rd = 0; rd < rounds; ++rd) {
-    const uint32_t p = rd * 32 + lane;
+  const uint32_t max_rows = __reduce_max_sync(0xffffffffu, h.y >> 16);
+  // N pairs per lane at once, so that their searches' loads overlap
+  for (uint32_t p0r = 0; p0r < total; p0r += 32 * N) {
+    int lo[N];
+    uint32_t a[N], b[N], q[N], off[N];
+#pragma unroll
+    for (int u = 0; u < N; ++u) lo[u] = 0;
     // owner = largest lane whose start <= p (lanes with no pairs never win over the next lane)
-    int lo = 0;
 #pragma unroll
     for (int step = 16; step >= 1; step >>= 1) {
-      const int cand = lo + step;
-      const uint32_t sc = __shfl_sync(0xffffffffu, start, cand & 31);
-      if (cand < 32 && sc <= p) lo = cand;
-    }
-    const uint32_t o_start = __shfl_sync(0xffffffffu, start, lo);
-    const uint32_t okey0 = __shfl_sync(0xffffffffu, gkey0, lo);
-    const uint32_t osplat = __shfl_sync(0xffffffffu, gsplat, lo);
-    const uint32_t oyr = __shfl_sync(0xffffffffu, h.y, lo);
-    const uint32_t ooff = __shfl_sync(0xffffffffu, h.z, lo);
-    const uint32_t R = oyr >> 16;
-    const uint64_t at = base + p;
-    if (p < total && at < capacity) {
-      uint32_t tile = okey0;
-      if (R > 0) {
-        const uint32_t q = p - o_start;
-        // last row whose pairs above are <= q (empty rows repeat the count before them)
-        uint32_t a = 0, b = R - 1;
-        while (a < b) {
-          const uint32_t mid = (a + b + 1) >> 1;
-          if (__ldg(&rows[(size_t)ooff + mid].x) <= q) a = mid; else b = mid - 1;
-        }
-        const uint2 e = __ldg(&rows[(size_t)ooff + a]);
-        // q - e.x < the row's pairs, so txx stays in the row; the clamp only
-        // keeps every tile index inside the view if that ever failed
-        const uint32_t txx = min(e.y + (q - e.x), (uint32_t)(Tx - 1));
-        tile += ((oyr & 0xffffu) + a) * (uint32_t)Tx + txx;
+#pragma unroll
+      for (int u = 0; u < N; ++u) {
+        const int cand = lo[u] + step;
+        const uint32_t sc = __shfl_sync(0xffffffffu, start, cand & 31);
+        if (cand < 32 && sc <= p0r + 32 * u + lane) lo[u] = cand;
       }
-      // (R == 0 with pairs: the record's row table did not fit, which happens
-      // only when the pairs exceed the capacity and GS_FLAG_CAPACITY is raised;
-      // its slots still get a valid tile and splat so that every slot below the
-      // capacity holds an in-range pair)
-      keys[at] = tile;
-      vals[at] = osplat;
+    }
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+      const uint32_t R = __shfl_sync(0xffffffffu, h.y, lo[u]) >> 16;
+      q[u] = p0r + 32 * u + lane - __shfl_sync(0xffffffffu, start, lo[u]);
+      off[u] = __shfl_sync(0xffffffffu, h.z, lo[u]);
+      a[u] = 0;
+      b[u] = R && p0r + 32 * u + lane < total ? R - 1 : 0;
+    }
+    // last row whose pairs above are <= q (empty rows repeat the count before them)
+    for (uint32_t span = max_rows; span > 1; span = (span + 1) >> 1) {
+#pragma unroll
+      for (int u = 0; u < N; ++u) {
+        const uint32_t mid = (a[u] + b[u] + 1) >> 1;
+        if (a[u] < b[u]) {
+          if (__ldg(&rows[(size_t)off[u] + mid].x) <= q[u]) a[u] = mid; else b[u] = mid - 1;
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+      const uint32_t p = p0r + 32 * u + lane;
+      uint32_t tile = __shfl_sync(0xffffffffu, gkey0, lo[u]);
+      const uint32_t osplat = __shfl_sync(0xffffffffu, gsplat, lo[u]);
+      const uint32_t oyr = __shfl_sync(0xffffffffu, h.y, lo[u]);
+      const uint64_t at = base + p;
+      if (p < total && at < capacity) {
+        if (oyr >> 16) {
+          const uint2 e = __ldg(&rows[(size_t)off[u] + a[u]]);
+          // q - e.x < the row's pairs, so txx stays in the row; the clamp only
+          // keeps every tile index inside the view if that ever failed
+          const uint32_t txx = min(e.y + (q[u] - e.x), (uint32_t)(Tx - 1));
+          tile += ((oyr & 0xffffu) + a[u]) * (uint32_t)Tx + txx;
+        }
+        // (no rows but pairs: the record's row table did not fit, which happens
+        // only when the pairs exceed the capacity and GS_FLAG_CAPACITY is
+        // raised; its slots still get a valid tile and splat so that every slot
+        // below the capacity holds an in-range pair)
+        keys[at] = tile;
+        vals[at] = osplat;
+      }
     }
   }
 }
@@ -370,12 +358,13 @@ __global__ void emit_kernel(const uint4* __restrict__ hdr, const uint2* __restri
 // A pass sorts nseg segments independently and stably on one 8-bit digit.
 // Segment g holds items [g * stride, g * stride + len): the record sort has one
 // segment per view (len = stride = n_pad), the pair sort one segment whose
-// length is the pair count P in device memory.  Each segment is cut into
-// tiles of kRadixTile items, tile t of segment g handled by block g * bpg + t
-// (blocks past the segment's tiles return).  The digit histograms are stored
-// segment-major, then digit, then tile: hist[(g * 256 + d) * bps + t], so that
-// one exclusive scan of all of them gives every (segment, digit, tile) its
-// first output position.
+// length is the pair count P in device memory.  A segment is cut into tiles (see
+// radix_tile) and its tiles into bps contiguous ranges of equal length,
+// one per block (g * bps + b).  hist[(g * bps + b) * 256 + d] counts digit d in a
+// range; the first output position of a range's digit follows from the ranges
+// before it and the totals of the smaller digits.  With one histogram per tile of
+// 2048 instead, the histograms of the 45M pairs of 8 views of 1080p took a
+// 22 MB scan of three kernels per pass.
 struct Seg {
   const uint32_t* len_dev;  // device length of the single segment, or null
   uint64_t cap;             // clamp of *len_dev
@@ -394,138 +383,249 @@ __device__ __forceinline__ uint32_t digit_of(K key, int shift) {
   return (uint32_t)(key >> shift) & 255u;
 }
 
-// Digit counts of one tile.  A thread counts kRadixItems consecutive keys (read
-// as 16-byte vectors) and adds each run of equal digits to the block's
-// counters with one shared atomic: a splat's pairs are adjacent and share their
-// high tile digit, so runs are common.
-template <typename K>
-__device__ __forceinline__ void load_run(const K* p, K (&kk)[kRadixItems]) {
-  static_assert((kRadixItems * sizeof(K)) % 16 == 0, "vector loads");
-  const uint4* q = reinterpret_cast<const uint4*>(p);
-#pragma unroll
-  for (int v = 0; v < (int)(kRadixItems * sizeof(K) / 16); ++v) {
-    const uint4 w = __ldg(q + v);
-    memcpy(reinterpret_cast<char*>(kk) + 16 * v, &w, 16);
-  }
+__device__ __forceinline__ uint32_t digit_of(uint32_t key, int shift) { return (key >> shift) & 255u; }
+
+// The items [begin, end) of range b of a segment of len items.
+template <int ITEMS>
+__device__ __forceinline__ void range_of(uint32_t len, int bps, int b, uint32_t& begin, uint32_t& end) {
+  constexpr uint32_t kTile = radix_tile(ITEMS);
+  const uint32_t tiles = len / kTile + (len % kTile != 0), per = tiles / (uint32_t)bps, extra = tiles % (uint32_t)bps;
+  const uint32_t t0 = (uint32_t)b * per + min((uint32_t)b, extra), n = per + ((uint32_t)b < extra);
+  begin = t0 * kTile;  // below len + kTile, and only used where below len
+  end = t0 + n >= tiles ? len : (t0 + n) * kTile;
+  if (n == 0) end = begin;
 }
 
-template <typename K>
-__global__ void __launch_bounds__(kRadixThreads) radix_hist_kernel(const K* __restrict__ keys, Seg sg, int bpg,
+// The lanes of the warp that hold the same digit (256: no item).  The match
+// instruction takes longer the more distinct digits the warp holds; nine ballots
+// take the same time always.  FEW: the digits of a warp are mostly alike.
+template <bool FEW>
+__device__ __forceinline__ uint32_t digit_peers(uint32_t d) {
+  if constexpr (FEW) return __match_any_sync(0xffffffffu, d);
+  uint32_t m = 0xffffffffu;
+#pragma unroll
+  for (int b = 0; b < 9; ++b) {
+    const bool one = (d >> b) & 1u;
+    const uint32_t v = __ballot_sync(0xffffffffu, one);
+    m &= one ? v : ~v;
+  }
+  return m;
+}
+
+// Digit counts of one range.  A thread counts ITEMS consecutive keys (read
+// as 16-byte vectors) and adds each run of equal digits to its warp's counters
+// with one shared atomic: a splat's pairs are adjacent and share their high tile
+// digit, so runs are common.
+template <int ITEMS>
+__global__ void __launch_bounds__(kRadixThreads) radix_hist_kernel(const uint32_t* __restrict__ keys, Seg sg, int bps,
                                                                    int shift, uint32_t* __restrict__ hist) {
-  __shared__ uint32_t s_cnt[256];
-  const uint32_t len = seg_len(sg);
-  const int g = blockIdx.x / bpg, t = blockIdx.x - g * bpg;
-  const uint32_t bps = (len + kRadixTile - 1) / kRadixTile;
-  if ((uint32_t)t >= bps) return;
-  s_cnt[threadIdx.x] = 0;
+  __shared__ uint32_t s_cnt[kRadixWarps][256];
+  const int g = blockIdx.x / bps, b = blockIdx.x - g * bps, tid = threadIdx.x, warp = tid >> 5;
+  uint32_t begin, end;
+  range_of<ITEMS>(seg_len(sg), bps, b, begin, end);
+#pragma unroll
+  for (int w = 0; w < kRadixWarps; ++w) s_cnt[w][tid] = 0;
   __syncthreads();
-  const K* kin = keys + (size_t)g * sg.stride;
-  const uint32_t base = (uint32_t)t * kRadixTile + threadIdx.x * kRadixItems;
-  K kk[kRadixItems];
-  if (base + kRadixItems <= len) {
-    load_run(kin + base, kk);
-  } else {
+  const uint32_t* kin = keys + (size_t)g * sg.stride;
+  for (uint32_t base = begin; base < end; base += radix_tile(ITEMS)) {
+    const uint32_t at = base + (uint32_t)tid * ITEMS;
+    uint32_t kk[ITEMS];
+    if (at + ITEMS <= end) {
 #pragma unroll
-    for (int k = 0; k < kRadixItems; ++k) kk[k] = base + k < len ? kin[base + k] : (K)0;
-  }
-  uint32_t prev = 256u, run = 0;
+      for (int v = 0; v < ITEMS; v += 4) {
+        const uint4 w = __ldg(reinterpret_cast<const uint4*>(kin + at + v));
+        kk[v] = w.x; kk[v + 1] = w.y; kk[v + 2] = w.z; kk[v + 3] = w.w;
+      }
+    } else {
 #pragma unroll
-  for (int k = 0; k < kRadixItems; ++k) {
-    const uint32_t d = base + k < len ? digit_of(kk[k], shift) : 256u;
-    if (d != prev) {
-      if (run) atomicAdd(&s_cnt[prev], run);
-      prev = d;
-      run = 0;
+      for (int k = 0; k < ITEMS; ++k) kk[k] = at + k < end ? kin[at + k] : 0u;
     }
-    run += d < 256u;
+    uint32_t prev = 256u, run = 0;
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) {
+      const uint32_t d = at + k < end ? digit_of(kk[k], shift) : 256u;
+      if (d != prev) {
+        if (run) atomicAdd(&s_cnt[warp][prev], run);
+        prev = d;
+        run = 0;
+      }
+      run += d < 256u;
+    }
+    if (run) atomicAdd(&s_cnt[warp][prev], run);
   }
-  if (run) atomicAdd(&s_cnt[prev], run);
   __syncthreads();
-  hist[((size_t)g * 256 + threadIdx.x) * bps + t] = s_cnt[threadIdx.x];
+  uint32_t c = 0;
+#pragma unroll
+  for (int w = 0; w < kRadixWarps; ++w) c += s_cnt[w][tid];
+  hist[(size_t)blockIdx.x * 256 + tid] = c;
 }
 
-// Stable scatter of one tile.  Warp w owns the tile's items
-// [w * 32 * kRadixItems, (w + 1) * 32 * kRadixItems), item k of lane L at
+// For segments of many ranges: hist becomes, per digit, the exclusive prefix over
+// the segment's ranges, and totals its digits' totals.  A block takes 32 digits
+// of one segment, a warp every 32nd part of its ranges, a lane one digit.
+__global__ void __launch_bounds__(1024) radix_prefix_kernel(uint32_t* __restrict__ hist, uint32_t* __restrict__ totals,
+                                                            int bps) {
+  __shared__ uint32_t s_sum[32][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, d = blockIdx.x * 32 + lane, g = blockIdx.y;
+  uint32_t* h = hist + (size_t)g * bps * 256 + d;
+  const int per = (bps + 31) / 32, b0 = min(warp * per, bps), b1 = min(b0 + per, bps);
+  uint32_t s = 0;
+#pragma unroll 4
+  for (int b = b0; b < b1; ++b) s += h[(size_t)b * 256];
+  s_sum[warp][lane] = s;
+  __syncthreads();
+  uint32_t run = 0;
+  for (int w = 0; w < warp; ++w) run += s_sum[w][lane];
+  if (warp == 31) totals[(size_t)g * 256 + d] = run + s;
+#pragma unroll 4
+  for (int b = b0; b < b1; ++b) {
+    const uint32_t c = h[(size_t)b * 256];
+    h[(size_t)b * 256] = run;
+    run += c;
+  }
+}
+// Up to this many ranges a scatter block sums the ranges' counts itself, which
+// spares the kernel above (small inputs are bound by their launches).
+constexpr int kDirectRanges = 32;
+
+// Stable scatter of one range, tile by tile.  Warp w owns a tile's items
+// [w * 32 * ITEMS, (w + 1) * 32 * ITEMS), item k of lane L at
 // offset k * 32 + L, so the warps' strips and the items within a strip are in
 // input order.  Each warp ranks its strip against private digit counters (one
 // match per item, no block barrier); the per-digit prefix over the warps and
 // the tile's digit starts follow from one block scan; the keys are reordered by
 // (digit, rank) in shared memory and each digit's run written contiguously.
-template <typename K>
-__global__ void __launch_bounds__(kRadixThreads, GS_RADIX_MIN_BLOCKS) radix_scatter_kernel(const K* __restrict__ kin_all,
-                                                                      const uint32_t* __restrict__ vin_all,
-                                                                      K* __restrict__ kout, uint32_t* __restrict__ vout,
-                                                                      Seg sg, int bpg, int shift,
-                                                                      const uint32_t* __restrict__ hist_scanned) {
-  __shared__ K s_keys[kRadixTile];
-  __shared__ uint32_t s_vals[kRadixTile];
-  __shared__ uint32_t s_wc[kRadixWarps][256];  // per-warp digit counts, then their prefix over warps
-  __shared__ uint32_t s_start[256];           // first tile position of each digit
+// Measured on 12.2M pairs (2 views of 1080p): low digits 87 us, high digits 58 us;
+// the chain of dependent steps per tile bounds it (the stores cost 30 us of it,
+// loads are a tile ahead).  With a tile per block and a histogram per tile the
+// whole sort of 8 views took 1.78 ms, now 1.53 ms (45M pairs, 8M records); a
+// render of 61k large splats 0.50 -> 0.35 ms, a step of 1k Gaussians 0.27 -> 0.20.
+// totals null: hist holds plain counts (see kDirectRanges).  vin null: the
+// values are the items' positions.
+template <bool FEW, int ITEMS>
+__global__ void __launch_bounds__(kRadixThreads, radix_blocks(ITEMS)) radix_scatter_kernel(
+    const uint32_t* __restrict__ kin_all, const uint32_t* __restrict__ vin_all, uint32_t* __restrict__ kout,
+    uint32_t* __restrict__ vout, Seg sg, int bps, int shift, const uint32_t* __restrict__ hist,
+    const uint32_t* __restrict__ totals) {
+  constexpr int kTile = radix_tile(ITEMS);
+  __shared__ uint32_t s_keys[kTile];
+  __shared__ uint32_t s_vals[kTile];
+  __shared__ uint32_t s_wc[kRadixWarps][256];  // per-warp digit counts, then their first tile positions
   __shared__ uint32_t s_gofs[256];            // output position minus tile position, per digit
   __shared__ uint32_t s_warp[32];
-  const uint32_t len = seg_len(sg);
-  const int g = blockIdx.x / bpg, t = blockIdx.x - g * bpg;
-  const uint32_t bps = (len + kRadixTile - 1) / kRadixTile;
-  if ((uint32_t)t >= bps) return;
+  const int g = blockIdx.x / bps, b = blockIdx.x - g * bps;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint32_t begin, end;
+  range_of<ITEMS>(seg_len(sg), bps, b, begin, end);
+  if (begin >= end) return;
   const uint32_t lt = lanemask_lt();
-  const K* kin = kin_all + (size_t)g * sg.stride;
-  const uint32_t* vin = vin_all + (size_t)g * sg.stride;
-  const uint32_t base = (uint32_t)t * kRadixTile + (uint32_t)warp * 32 * kRadixItems + lane;
-  K key[kRadixItems];
-  uint32_t vv[kRadixItems], rank[kRadixItems], dg[kRadixItems];
-#pragma unroll
-  for (int k = 0; k < kRadixItems; ++k) {
-    const uint32_t idx = base + (uint32_t)k * 32;
-    key[k] = idx < len ? kin[idx] : (K)0;
-    vv[k] = idx < len ? vin[idx] : 0u;
-  }
-#pragma unroll
-  for (int q = lane; q < 256; q += 32) s_wc[warp][q] = 0;
-  __syncwarp();
-#pragma unroll
-  for (int k = 0; k < kRadixItems; ++k) {
-    const bool ok = base + (uint32_t)k * 32 < len;
-    const uint32_t d = ok ? digit_of(key[k], shift) : 256u;
-    dg[k] = d;
-    const uint32_t peers = __match_any_sync(0xffffffffu, d);
-    const uint32_t before = ok ? s_wc[warp][d] : 0u;
-    rank[k] = before + (uint32_t)__popc(peers & lt);
-    __syncwarp();
-    if (ok && (peers & lt) == 0) s_wc[warp][d] = before + (uint32_t)__popc(peers);
-    __syncwarp();
-  }
-  __syncthreads();
-  // digit tid: prefix of the warps' counts, the tile's count, its start
-  uint32_t run = 0;
-#pragma unroll
-  for (int w = 0; w < kRadixWarps; ++w) {
-    const uint32_t c = s_wc[w][tid];
-    s_wc[w][tid] = run;
-    run += c;
-  }
-  uint32_t tot;
-  const uint32_t start = block_exclusive_scan(run, tot, s_warp);
-  s_start[tid] = start;
-  s_gofs[tid] = hist_scanned[((size_t)g * 256 + tid) * bps + t] - start;
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < kRadixItems; ++k) {
-    if (dg[k] < 256u) {
-      const uint32_t pos = s_start[dg[k]] + s_wc[warp][dg[k]] + rank[k];
-      s_keys[pos] = key[k];
-      s_vals[pos] = vv[k];
+  // first output position of digit tid in this range
+  uint32_t next;
+  {
+    const uint32_t* h = hist + (size_t)g * bps * 256 + tid;
+    uint32_t before = 0, all = 0, tot;
+    if (totals) {
+      before = h[(size_t)b * 256];
+      all = totals[(size_t)g * 256 + tid];
+    } else {
+#pragma unroll 8
+      for (int q = 0; q < bps; ++q) {
+        const uint32_t c = h[(size_t)q * 256];
+        if (q < b) before += c;
+        all += c;
+      }
     }
+    next = block_exclusive_scan(all, tot, s_warp) + before + (uint32_t)g * sg.stride;
   }
-  __syncthreads();
+  const uint32_t* kin = kin_all + (size_t)g * sg.stride;
+  const uint32_t* vin = vin_all ? vin_all + (size_t)g * sg.stride : nullptr;
+  // the next tile's items are loaded while this one is ranked
+  uint32_t key[ITEMS], vv[ITEMS], nkey[ITEMS], nval[ITEMS];
+  const uint32_t mine = (uint32_t)warp * 32 * ITEMS + lane;
+  auto load = [&](uint32_t tile) {
 #pragma unroll
-  for (int k = 0; k < kRadixItems; ++k) {
-    const uint32_t p = (uint32_t)k * kRadixThreads + tid;
-    if (p < tot) {
-      const K kk = s_keys[p];
-      const size_t at = (size_t)s_gofs[digit_of(kk, shift)] + p;
-      kout[at] = kk;
-      vout[at] = s_vals[p];
+    for (int k = 0; k < ITEMS; ++k) {
+      const uint32_t idx = tile + mine + (uint32_t)k * 32;
+      nkey[k] = idx < end ? __ldg(kin + idx) : 0u;
+      nval[k] = idx < end ? (vin ? __ldg(vin + idx) : (uint32_t)g * sg.stride + idx) : 0u;
+    }
+  };
+  load(begin);
+  for (uint32_t tile = begin; tile < end; tile += kTile) {
+    const uint32_t base = tile + mine;
+    uint32_t rank[ITEMS], peers[ITEMS];
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) {
+      key[k] = nkey[k];
+      vv[k] = nval[k];
+    }
+    if (tile + kTile < end) load(tile + kTile);
+    auto digit = [&](int k) { return base + (uint32_t)k * 32 < end ? digit_of(key[k], shift) : 256u; };
+#pragma unroll
+    for (int q = lane; q < 256; q += 32) s_wc[warp][q] = 0;
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) peers[k] = digit_peers<FEW>(digit(k));
+    // the first lane of each digit takes the digit's next ranks for all its
+    // peers; the items' atomics follow one another without waiting
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) {
+      const uint32_t d = digit(k);
+      rank[k] = 0;
+      if (d < 256u && (peers[k] & lt) == 0) rank[k] = atomicAdd(&s_wc[warp][d], (uint32_t)__popc(peers[k]));
+      __syncwarp();
+    }
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k)
+      rank[k] = __shfl_sync(0xffffffffu, rank[k], __ffs(peers[k]) - 1) + (uint32_t)__popc(peers[k] & lt);
+    __syncthreads();
+    // digit tid: the tile's count, its start, and the warps' first positions
+    uint32_t cw[kRadixWarps], count = 0;
+#pragma unroll
+    for (int w = 0; w < kRadixWarps; ++w) {
+      cw[w] = s_wc[w][tid];
+      count += cw[w];
+    }
+    uint32_t incl = count;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    uint32_t start = incl - count;
+#pragma unroll
+    for (int w = 0; w < kRadixWarps; ++w) start += w < warp ? s_warp[w] : 0u;
+    s_gofs[tid] = next - start;
+    next += count;
+#pragma unroll
+    for (int w = 0; w < kRadixWarps; ++w) {
+      s_wc[w][tid] = start;
+      start += cw[w];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) {
+      const uint32_t d = digit(k);
+      if (d < 256u) {
+        const uint32_t pos = s_wc[warp][d] + rank[k];
+        s_keys[pos] = key[k];
+        s_vals[pos] = vv[k];
+      }
+    }
+    __syncthreads();
+    // (what is read below is written again only after two more barriers)
+    const uint32_t tot = min((uint32_t)kTile, end - tile);
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) {
+      const uint32_t p = (uint32_t)k * kRadixThreads + tid;
+      if (p < tot) {
+        const uint32_t kk = s_keys[p];
+        const size_t at = (size_t)(s_gofs[digit_of(kk, shift)] + p);
+        kout[at] = kk;
+        vout[at] = s_vals[p];
+      }
     }
   }
 }
@@ -612,8 +712,44 @@ __global__ void tile_order_kernel(const uint32_t* __restrict__ ranges, uint32_t 
   if (c != 0xffffffffu) order[base + __popc(peers & ((1u << lane) - 1u))] = t;
 }
 
+// The whole order in one block, for few tiles.
+constexpr uint32_t kSmallOrder = 8192;
+__global__ void __launch_bounds__(1024) small_tile_order_kernel(const uint32_t* __restrict__ ranges, uint32_t n_tiles,
+                                                                uint32_t* __restrict__ order) {
+  __shared__ uint32_t s_next[256], s_warp[32];
+  const uint32_t tid = threadIdx.x, lane = tid & 31;
+  if (tid < 256) s_next[tid] = 0;
+  __syncthreads();
+  for (uint32_t t0 = 0; t0 < n_tiles; t0 += 1024) {
+    const uint32_t t = t0 + tid;
+    const uint32_t c = t < n_tiles ? tile_class(ranges[2 * t + 1] - ranges[2 * t]) : 256u;
+    const uint32_t peers = __match_any_sync(0xffffffffu, c);
+    if (c < 256u && (peers & ((1u << lane) - 1u)) == 0) atomicAdd(&s_next[c], (uint32_t)__popc(peers));
+  }
+  __syncthreads();
+  const uint32_t mine = tid < 256 ? s_next[255 - tid] : 0u;  // thread k holds class 255 - k
+  uint32_t total;
+  const uint32_t first = block_exclusive_scan(mine, total, s_warp);
+  if (tid < 256) s_next[255 - tid] = first;
+  __syncthreads();
+  for (uint32_t t0 = 0; t0 < n_tiles; t0 += 1024) {
+    const uint32_t t = t0 + tid;
+    const uint32_t c = t < n_tiles ? tile_class(ranges[2 * t + 1] - ranges[2 * t]) : 256u;
+    const uint32_t peers = __match_any_sync(0xffffffffu, c);
+    const int leader = __ffs(peers) - 1;
+    uint32_t base = 0;
+    if ((int)lane == leader && c < 256u) base = atomicAdd(&s_next[c], (uint32_t)__popc(peers));
+    base = __shfl_sync(0xffffffffu, base, leader);
+    if (c < 256u) order[base + __popc(peers & ((1u << lane) - 1u))] = t;
+  }
+}
+
 void fill_tile_order(const uint32_t* ranges, uint32_t n_tiles, uint32_t* cls, uint32_t* order, cudaStream_t st) {
   const unsigned tb = (n_tiles + 255) / 256;
+  if (n_tiles <= kSmallOrder) {
+    if (n_tiles) small_tile_order_kernel<<<1, 1024, 0, st>>>(ranges, n_tiles, order);
+    return;
+  }
   if (tb == 0 || cudaMemsetAsync(cls, 0, 256 * sizeof(uint32_t), st) != cudaSuccess) return;  // reported by the caller
   tile_class_count_kernel<<<tb, 256, 0, st>>>(ranges, n_tiles, cls);
   tile_class_starts_kernel<<<1, 256, 0, st>>>(cls);
@@ -624,10 +760,10 @@ void fill_tile_order(const uint32_t* ranges, uint32_t n_tiles, uint32_t* cls, ui
 inline size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 struct SortPlan {
-  int Tx, Ty, rec_pass, pair_pass, nb_pairs, rec_bps;
+  int Tx, Ty, rec_pass, pair_pass;
   size_t n_items;  // views x n_pad
-  size_t off_counts, off_scnt, off_sums, off_rk0, off_rk1, off_rv0, off_rv1, off_keys, off_vals, off_hist, off_hdr,
-      off_rows, off_used, off_cls, total;
+  size_t off_scnt, off_sums, off_rk0, off_rk1, off_rv0, off_rv1, off_keys, off_vals, off_hist, off_tot, off_hdr, off_rows,
+      off_used, off_cls, total;
   uint64_t rows_cap;
 };
 
@@ -635,6 +771,20 @@ inline int bits_for(uint64_t v) {  // smallest b with 2^b >= v
   int b = 0;
   while ((1ull << b) < v) ++b;
   return b;
+}
+
+// Items per thread of a pass over at most `len` items in each of nseg segments:
+// 16 where the digits are many and there are two large tiles for every resident
+// block.
+inline int radix_items(uint64_t len, int nseg, bool few) {
+  return !few && len * (uint64_t)nseg >= (uint64_t)2 * 152 * radix_blocks(16) * radix_tile(16) ? 16 : 8;
+}
+// Ranges (blocks) of a segment of at most `len` items when nseg segments share
+// the chip: one per resident scatter block, at most one per tile.
+inline int ranges_per_segment(uint64_t len, int nseg, int items) {
+  const uint64_t tiles = std::max<uint64_t>(1, (len + radix_tile(items) - 1) / radix_tile(items));
+  const uint64_t fair = (uint64_t)(152 * radix_blocks(items) + nseg - 1) / nseg;
+  return (int)std::min<uint64_t>(tiles, std::max<uint64_t>(1, fair));
 }
 
 SortPlan plan_sort(int32_t n_pad, gs_frame fr, uint64_t capacity) {
@@ -645,12 +795,11 @@ SortPlan plan_sort(int32_t n_pad, gs_frame fr, uint64_t capacity) {
   p.pair_pass = std::max(1, (bits_for(tiles) + 7) / 8);
   p.rec_pass = 4;  // 32 depth bits within each view
   p.n_items = (size_t)fr.n_views * n_pad;
-  p.nb_pairs = (int)((capacity + kRadixTile - 1) / kRadixTile);
-  p.rec_bps = (int)(((size_t)n_pad + kRadixTile - 1) / kRadixTile);
-  const size_t hist_n = (size_t)256 * std::max((size_t)p.nb_pairs, (size_t)fr.n_views * p.rec_bps);
-  const size_t sums_n = (size_t)std::max(scan_blocks(p.n_items), scan_blocks(hist_n)) + 1;
+  // (a pass of 8 items per thread has the most ranges)
+  const size_t hist_n = (size_t)256 * std::max((size_t)ranges_per_segment(capacity, 1, 8),
+                                               (size_t)fr.n_views * ranges_per_segment((uint64_t)n_pad, fr.n_views, 8));
+  const size_t sums_n = (size_t)scan_blocks(p.n_items) + 1;
   size_t o = 0;
-  p.off_counts = o; o += align256(p.n_items * 4);
   p.off_scnt = o;   o += align256(p.n_items * 4);
   p.off_sums = o;   o += align256(sums_n * 4);
   p.off_rk0 = o;    o += align256(p.n_items * 4);
@@ -660,6 +809,7 @@ SortPlan plan_sort(int32_t n_pad, gs_frame fr, uint64_t capacity) {
   p.off_keys = o;   o += align256(capacity * 4);
   p.off_vals = o;   o += align256(capacity * 4);
   p.off_hist = o;   o += align256(hist_n * 4);
+  p.off_tot = o;    o += align256((size_t)256 * std::max(1, fr.n_views) * 4);
   p.rows_cap = std::min<uint64_t>(capacity + 2 * (uint64_t)p.n_items, 0xffffffffull);
   p.off_hdr = o;    o += align256(p.n_items * 16);
   p.off_rows = o;   o += align256(p.rows_cap * 8);
@@ -669,22 +819,33 @@ SortPlan plan_sort(int32_t n_pad, gs_frame fr, uint64_t capacity) {
   return p;
 }
 
-// Stable LSD passes over 8-bit digits starting at `shift0` on nseg segments of
-// bpg tiles each (see Seg); the keys/values ping-pong between buffer 0 and 1
-// starting in `cur`, which is updated.  The histogram scan runs over
-// nseg x 256 x bpg entries, or over the pairs in use when the length is on the
-// device.
-template <typename K>
-void radix_passes(K** kbuf, uint32_t** vbuf, int& cur, int npass, int shift0, Seg sg, int nseg, int bpg,
-                  uint32_t* hist, uint32_t* sums, cudaStream_t st) {
-  const size_t hist_n = (size_t)nseg * 256 * bpg;
-  const unsigned grid = (unsigned)((size_t)nseg * bpg);
+// One stable pass (see Seg) over at most len_max items per segment; vin null: the
+// values are the items' positions.
+template <bool FEW, int ITEMS>
+void radix_pass(const uint32_t* kin, const uint32_t* vin, uint32_t* kout, uint32_t* vout, int shift, Seg sg, int nseg,
+                uint64_t len_max, uint32_t* hist, uint32_t* totals, cudaStream_t st) {
+  const int bps = ranges_per_segment(len_max, nseg, ITEMS);
+  const unsigned grid = (unsigned)((size_t)nseg * bps);
+  const bool direct = bps <= kDirectRanges;
+  radix_hist_kernel<ITEMS><<<grid, kRadixThreads, 0, st>>>(kin, sg, bps, shift, hist);
+  if (!direct) radix_prefix_kernel<<<dim3(256 / 32, nseg), 1024, 0, st>>>(hist, totals, bps);
+  radix_scatter_kernel<FEW, ITEMS><<<grid, kRadixThreads, 0, st>>>(kin, vin, kout, vout, sg, bps, shift, hist,
+                                                                   direct ? nullptr : totals);
+}
+
+// Stable LSD passes over 8-bit digits from bit 0; the keys/values ping-pong
+// between buffer 0 and 1 starting in `cur`, which is updated.  iota: the first
+// pass's values are the items' positions instead of vbuf[cur].  The last digit
+// (the exponents of the depths, the views and upper rows of the tiles) takes few
+// values within a warp.
+void radix_passes(uint32_t** kbuf, uint32_t** vbuf, int& cur, int npass, bool iota, Seg sg, int nseg, uint64_t len_max,
+                  uint32_t* hist, uint32_t* totals, cudaStream_t st) {
   for (int pass = 0; pass < npass; ++pass) {
-    const int shift = shift0 + 8 * pass;
-    radix_hist_kernel<K><<<grid, kRadixThreads, 0, st>>>(kbuf[cur], sg, bpg, shift, hist);
-    exclusive_scan(hist, hist, hist_n, sg.len_dev, sg.cap, sums, nullptr, 0, nullptr, st);
-    radix_scatter_kernel<K><<<grid, kRadixThreads, 0, st>>>(kbuf[cur], vbuf[cur], kbuf[cur ^ 1], vbuf[cur ^ 1], sg,
-                                                            bpg, shift, hist);
+    const bool few = npass > 1 && pass + 1 == npass;
+    auto* run = few ? radix_pass<true, 8>
+                    : radix_items(len_max, nseg, few) == 16 ? radix_pass<false, 16> : radix_pass<false, 8>;
+    run(kbuf[cur], iota && pass == 0 ? nullptr : vbuf[cur], kbuf[cur ^ 1], vbuf[cur ^ 1], 8 * pass, sg, nseg, len_max,
+        hist, totals, st);
     cur ^= 1;
   }
 }
@@ -712,10 +873,10 @@ extern "C" gs_status gs_bin_sort(const gs_projected* proj, int32_t n_pad, gs_fra
              workspace_bytes);
   cudaStream_t st = (cudaStream_t)stream;
   char* ws = (char*)workspace;
-  uint32_t* counts = (uint32_t*)(ws + p.off_counts);
   uint32_t* scnt = (uint32_t*)(ws + p.off_scnt);
   uint32_t* sums = (uint32_t*)(ws + p.off_sums);
   uint32_t* hist = (uint32_t*)(ws + p.off_hist);
+  uint32_t* totals = (uint32_t*)(ws + p.off_tot);
   const float4* rec = reinterpret_cast<const float4*>(proj->rec);
   const uint64_t T = (uint64_t)p.Tx * p.Ty;
 
@@ -723,7 +884,7 @@ extern "C" gs_status gs_bin_sort(const gs_projected* proj, int32_t n_pad, gs_fra
   uint2* rows = (uint2*)(ws + p.off_rows);
   uint32_t* rows_used = (uint32_t*)(ws + p.off_used);
   if (cudaMemsetAsync(out->ranges, 0, (size_t)frame.n_views * T * 2 * sizeof(uint32_t), st) != cudaSuccess ||
-      cudaMemsetAsync(out->n_pairs, 0, sizeof(uint32_t), st) != cudaSuccess ||
+      (p.n_items == 0 && cudaMemsetAsync(out->n_pairs, 0, sizeof(uint32_t), st) != cudaSuccess) ||
       cudaMemsetAsync(rows_used, 0, sizeof(uint32_t), st) != cudaSuccess)
     return check_launch("gs_bin_sort: memset");
   if (p.n_items == 0) {  // no splats: every range is empty
@@ -734,23 +895,31 @@ extern "C" gs_status gs_bin_sort(const gs_projected* proj, int32_t n_pad, gs_fra
   // records sorted by depth within each view's segment
   uint32_t* rk[2] = {(uint32_t*)(ws + p.off_rk0), (uint32_t*)(ws + p.off_rk1)};
   uint32_t* rv[2] = {(uint32_t*)(ws + p.off_rv0), (uint32_t*)(ws + p.off_rv1)};
-  record_keys_kernel<<<eb, 256, 0, st>>>(rec, n_pad, frame, p.Tx, p.Ty, counts, rk[0], rv[0], hdr, rows, p.rows_cap,
-                                         rows_used, status);
+  record_keys_kernel<<<eb, 256, 0, st>>>(rec, n_pad, frame, p.Tx, p.Ty, rk[0], hdr, rows, p.rows_cap, rows_used,
+                                         status);
   int rcur = 0;
   const Seg rseg{nullptr, 0, (uint32_t)n_pad, (uint32_t)n_pad};
-  radix_passes<uint32_t>(rk, rv, rcur, p.rec_pass, 0, rseg, frame.n_views, p.rec_bps, hist, sums, st);
+  radix_passes(rk, rv, rcur, p.rec_pass, true, rseg, frame.n_views, (uint64_t)n_pad, hist, totals, st);
   // emission offsets in that order, and the pair count
-  gather_counts_kernel<<<eb, 256, 0, st>>>(rv[rcur], counts, scnt, p.n_items);
-  exclusive_scan(scnt, scnt, p.n_items, nullptr, 0, sums, out->n_pairs, out->capacity, status, st);
+  if (p.n_items <= kSmallScan) {
+    small_offsets_kernel<<<1, 1024, 0, st>>>(rv[rcur], hdr, scnt, (int)p.n_items, out->n_pairs, out->capacity, status);
+  } else {
+    const int sb = scan_blocks(p.n_items);
+    gather_counts_kernel<<<sb, kScanThreads, 0, st>>>(rv[rcur], hdr, scnt, p.n_items, sums);
+    scan_blocks_kernel<<<1, 1024, 0, st>>>(sums, sb, out->n_pairs, out->capacity, status);
+    scan_apply_kernel<<<sb, kScanThreads, 0, st>>>(scnt, p.n_items, sums);
+  }
   // pairs in (view, depth, splat) order, then stable passes on their tile keys;
   // the last pass must land in the caller's arrays
   uint32_t* kbuf[2] = {out->keys, (uint32_t*)(ws + p.off_keys)};
   uint32_t* vbuf[2] = {out->vals, (uint32_t*)(ws + p.off_vals)};
   int cur = (p.pair_pass % 2 == 0) ? 0 : 1;
-  emit_kernel<<<eb, 256, 0, st>>>(hdr, rows, n_pad, frame, p.Tx, p.Ty, rv[rcur], scnt, out->capacity, kbuf[cur],
+  // many pairs per record: more rounds at once, on fewer resident warps
+  auto* emit = out->capacity >= 16 * (uint64_t)p.n_items ? emit_kernel<4> : emit_kernel<2>;
+  emit<<<eb, 256, 0, st>>>(hdr, rows, n_pad, frame, p.Tx, p.Ty, rv[rcur], scnt, out->capacity, kbuf[cur],
                                   vbuf[cur]);
   const Seg pseg{out->n_pairs, out->capacity, 0, 0};
-  radix_passes<uint32_t>(kbuf, vbuf, cur, p.pair_pass, 0, pseg, 1, p.nb_pairs, hist, sums, st);
+  radix_passes(kbuf, vbuf, cur, p.pair_pass, false, pseg, 1, out->capacity, hist, totals, st);
   const int rb = (int)std::min<uint64_t>((out->capacity + 255) / 256, 152 * 16);
   ranges_kernel<<<rb, 256, 0, st>>>(out->keys, out->n_pairs, out->capacity, (uint64_t)frame.n_views * T,
                                     out->ranges);

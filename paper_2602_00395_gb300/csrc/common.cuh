@@ -411,15 +411,16 @@ __device__ __forceinline__ void tile_rect(float mx, float my, int r, uint32_t ex
                                           int& x0, int& x1, int& y0, int& y1) {
   const float hx = __half2float(__ushort_as_half((unsigned short)(ext & 0xffffu)));
   const float hy = __half2float(__ushort_as_half((unsigned short)(ext >> 16)));
-  const float ftw = (float)tw, fth = (float)th;
-  x0 = max(clamp_floor(floorf(__fdiv_rn(__fsub_rn(mx, (float)r), ftw)), Tx),
-           clamp_floor(floorf(__fdiv_rn(__fsub_rn(mx, hx), ftw)), Tx));
-  x1 = min(clamp_floor(floorf(__fdiv_rn(__fadd_rn(mx, (float)(r + tw - 1)), ftw)), Tx),
-           clamp_floor(__fadd_rn(floorf(__fdiv_rn(__fadd_rn(mx, hx), ftw)), 1.0f), Tx));
-  y0 = max(clamp_floor(floorf(__fdiv_rn(__fsub_rn(my, (float)r), fth)), Ty),
-           clamp_floor(floorf(__fdiv_rn(__fsub_rn(my, hy), fth)), Ty));
-  y1 = min(clamp_floor(floorf(__fdiv_rn(__fadd_rn(my, (float)(r + th - 1)), fth)), Ty),
-           clamp_floor(__fadd_rn(floorf(__fdiv_rn(__fadd_rn(my, hy), fth)), 1.0f), Ty));
+  // tw and th are powers of two: x / tw is the exact product by 1 / tw
+  const float itw = 1.0f / (float)tw, ith = 1.0f / (float)th;
+  x0 = max(clamp_floor(floorf(__fmul_rn(__fsub_rn(mx, (float)r), itw)), Tx),
+           clamp_floor(floorf(__fmul_rn(__fsub_rn(mx, hx), itw)), Tx));
+  x1 = min(clamp_floor(floorf(__fmul_rn(__fadd_rn(mx, (float)(r + tw - 1)), itw)), Tx),
+           clamp_floor(__fadd_rn(floorf(__fmul_rn(__fadd_rn(mx, hx), itw)), 1.0f), Tx));
+  y0 = max(clamp_floor(floorf(__fmul_rn(__fsub_rn(my, (float)r), ith)), Ty),
+           clamp_floor(floorf(__fmul_rn(__fsub_rn(my, hy), ith)), Ty));
+  y1 = min(clamp_floor(floorf(__fmul_rn(__fadd_rn(my, (float)(r + th - 1)), ith)), Ty),
+           clamp_floor(__fadd_rn(floorf(__fmul_rn(__fadd_rn(my, hy), ith)), 1.0f), Ty));
 }
 
 // ------------------------------------------------------- per-row tile spans

@@ -1,0 +1,60 @@
+"""gs_bin_sort at the sizes where its passes change shape.
+
+The radix passes run on tiles of 2048 items, or 4096 when the input fills the
+chip, cut into one range per resident block, whose prefix the scatter sums itself
+up to 32 ranges; offsets and the tile order take one block for small inputs.  The
+sizes here lie on both sides of each change, with ragged ends, duplicate depths
+and one or several views.  The result is checked against the definition, exactly:
+the pairs are strictly increasing in (key, depth, splat), every pair's tile lies
+in its splat's 3DGS square, and their number is the squares' area, so that no pair
+is missing, doubled or out of place; ranges and order follow from the keys.
+"""
+import pytest
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.mark.parametrize("n,V,W,H", [(31, 1, 40, 24), (2049, 3, 257, 130), (4097, 4, 320, 200), (9001, 1, 1600, 1500),
+                                     (61003, 1, 800, 600), (70001, 3, 640, 480), (1300007, 2, 1920, 1080)])
+def test_pairs_ranges_and_order(n, V, W, H):
+    from paper_2602_00395_gb300.engine import TRStep
+    e = TRStep(n, 0, V, W, H, nu=0, footprint_bins=False)
+    g = torch.Generator(device="cuda").manual_seed(n)
+    rnd = lambda: torch.rand(V, n, generator=g, device="cuda")
+    mx, my = rnd() * (W + 60) - 30, rnd() * (H + 60) - 30
+    radius = (rnd() * 12).int()  # 0: culled
+    depth = (rnd() * 4000).floor() / 100 + 0.25  # many ties
+    rec = e.rec.view(V, e.n_pad, 12)
+    rec.zero_()
+    rec[:, :n, 0], rec[:, :n, 1], rec[:, :n, 9] = mx, my, depth
+    rec.view(torch.int32)[:, :n, 10] = radius
+    rec.view(torch.int32)[:, :n, 11] = 0x7C007C00
+    r = radius.float()
+    lo = lambda m, T: torch.floor((m - r) / 16).clamp(0, T).long()
+    hi = lambda m, T: torch.floor((m + (r + 15)) / 16).clamp(0, T).long()
+    x0, x1, y0, y1 = lo(mx, e.Tx), hi(mx, e.Tx), lo(my, e.Ty), hi(my, e.Ty)
+    area = (x1 - x0).clamp(min=0) * (y1 - y0).clamp(min=0) * (radius > 0)
+    P = int(area.sum())
+    if P > e.capacity:
+        e._alloc_pairs(P)
+    for _ in range(2):  # the second call finds the first one's workspace
+        e.bin_sort()
+    torch.cuda.synchronize()
+    assert e.read_status() == 0 and int(e.n_pairs.item()) == P
+    key, val = e.keys[:P].long(), e.vals[:P].long()
+    T = e.Tx * e.Ty
+    view, tile = key // T, key % T
+    d = depth[view, val]
+    k0, k1, d0, d1, v0, v1 = key[:-1], key[1:], d[:-1], d[1:], val[:-1], val[1:]
+    assert bool(((k0 < k1) | ((k0 == k1) & ((d0 < d1) | ((d0 == d1) & (v0 < v1))))).all())
+    tx, ty = tile % e.Tx, tile // e.Tx
+    assert bool(((tx >= x0[view, val]) & (tx < x1[view, val]) & (ty >= y0[view, val]) & (ty < y1[view, val])).all())
+    cnt = torch.bincount(key, minlength=V * T)
+    rng = e.ranges.view(-1, 2).long()
+    assert torch.equal(rng[:, 1] - rng[:, 0], cnt)
+    assert torch.equal(rng[cnt > 0, 0], (torch.cumsum(cnt, 0) - cnt)[cnt > 0])
+    order = e.order.long()
+    assert torch.equal(torch.sort(order).values, torch.arange(V * T, device="cuda"))
+    lens = cnt[order].double()
+    assert bool((lens[1:] <= torch.clamp(lens[:-1], min=1) * 1.125 + 1).all())  # heaviest classes of 1/8 first

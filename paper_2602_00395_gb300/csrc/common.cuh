@@ -123,6 +123,41 @@ __device__ __forceinline__ uint64_t probe_signs(uint64_t seed, int64_t t, int k,
   return rows >= 64 ? bits : (bits & ((1ull << rows) - 1ull));
 }
 
+// ------------------------------------------------------ pairs of FP32 values
+// Two FP32 values in one 64-bit register: Blackwell's packed instructions do
+// both lanes in one issue slot, each rounded as the scalar instruction rounds.
+// The blends hold a thread's two pixels as a pair.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ f32x2 dup2(float v) { return pack2(v, v); }
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ float sum2(f32x2 v) {
+  float lo, hi;
+  unpack2(v, lo, hi);
+  return lo + hi;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
 // ------------------------------------------------ forward-mode dual numbers
 // Value plus N tangents; used to push the Rademacher directions through the
 // projection (the "forward-mode AD" half of the Hessian-vector product).
@@ -130,6 +165,13 @@ template <int N>
 struct Dn {
   float v;
   float d[N];
+};
+
+// Two tangents as a pair: every tangent operation is one packed instruction.
+template <>
+struct Dn<2> {
+  float v;
+  f32x2 d;
 };
 
 template <class S>
@@ -245,48 +287,60 @@ __device__ __forceinline__ Dn<N> ssqrt(const Dn<N>& a) {
   return r;
 }
 
+using D2 = Dn<2>;
+template <>
+__device__ __forceinline__ D2 cst<2>(float v) {
+  return D2{v, 0ull};
+}
+__device__ __forceinline__ D2 operator+(const D2& a, const D2& b) { return D2{a.v + b.v, add2(a.d, b.d)}; }
+__device__ __forceinline__ D2 operator-(const D2& a, const D2& b) {
+  return D2{a.v - b.v, fma2(b.d, dup2(-1.f), a.d)};
+}
+__device__ __forceinline__ D2 operator-(const D2& a) { return D2{-a.v, mul2(a.d, dup2(-1.f))}; }
+__device__ __forceinline__ D2 operator*(const D2& a, const D2& b) {
+  return D2{a.v * b.v, fma2(a.d, dup2(b.v), mul2(dup2(a.v), b.d))};
+}
+__device__ __forceinline__ D2 operator/(const D2& a, const D2& b) {
+  const float ib = 1.0f / b.v, q = a.v * ib;
+  return D2{q, mul2(fma2(dup2(-q), b.d, a.d), dup2(ib))};
+}
+__device__ __forceinline__ D2 operator+(const D2& a, float b) { return D2{a.v + b, a.d}; }
+__device__ __forceinline__ D2 operator+(float b, const D2& a) { return a + b; }
+__device__ __forceinline__ D2 operator-(const D2& a, float b) { return D2{a.v - b, a.d}; }
+__device__ __forceinline__ D2 operator-(float b, const D2& a) { return D2{-a.v + b, mul2(a.d, dup2(-1.f))}; }
+__device__ __forceinline__ D2 operator*(const D2& a, float b) { return D2{a.v * b, mul2(a.d, dup2(b))}; }
+__device__ __forceinline__ D2 operator*(float b, const D2& a) { return a * b; }
+__device__ __forceinline__ D2 operator/(const D2& a, float b) { return a * (1.0f / b); }
+__device__ __forceinline__ D2 operator/(float a, const D2& b) {
+  const float ib = 1.0f / b.v, q = a * ib;
+  return D2{q, mul2(b.d, dup2(-q * ib))};
+}
+__device__ __forceinline__ D2 sexp(const D2& a) {
+  const float e = expf(a.v);
+  return D2{e, mul2(a.d, dup2(e))};
+}
+__device__ __forceinline__ D2 ssqrt(const D2& a) {
+  const float r = sqrtf(a.v);
+  return D2{r, mul2(a.d, dup2(0.5f / r))};
+}
+// Tangent k of x.
+template <int N>
+__device__ __forceinline__ float tangent(const Dn<N>& x, int k) {
+  return x.d[k];
+}
+__device__ __forceinline__ float tangent(const D2& x, int k) {
+  float a, b;
+  unpack2(x.d, a, b);
+  return k ? b : a;
+}
+
 template <class S>
 __device__ __forceinline__ S constant(float v) {
   if constexpr (is_dual<S>::value) {
-    return cst<sizeof(S::d) / sizeof(float)>(v);
+    return cst<std::is_same<S, D2>::value ? 2 : 1>(v);
   } else {
     return v;
   }
-}
-
-// ------------------------------------------------------ pairs of FP32 values
-// Two FP32 values in one 64-bit register: Blackwell's packed instructions do
-// both lanes in one issue slot, each rounded as the scalar instruction rounds.
-// The blends hold a thread's two pixels as a pair.
-using f32x2 = unsigned long long;
-__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ f32x2 dup2(float v) { return pack2(v, v); }
-__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ float sum2(f32x2 v) {
-  float lo, hi;
-  unpack2(v, lo, hi);
-  return lo + hi;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
 }
 
 // ------------------------------------------------------------ SH basis
@@ -511,6 +565,17 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
 __device__ __forceinline__ void fence_mbar_init() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
+// Bulk copies shared -> global of the calling thread, in groups; both addresses and
+// the size are multiples of 16.  Generic writes to the source come before
+// fence_proxy_async.
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ void bulk_s2g(void* dst, const void* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)), "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// Waits until the calling thread's bulk copies have read their sources.
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 // Per-thread asynchronous copies global -> shared (16 or 4 bytes), in groups.
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
@@ -534,6 +599,26 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "r"(smem_u32(bar)), "r"(parity)
       : "memory");
   return ok != 0;
+}
+
+// Starts the copies of ROWS rows of 32 columns (pitch n_pad floats, the first
+// column c0 a multiple of 32) of the calling warp into dst[row * dst_pitch + lane],
+// 16 bytes per lane; columns past the pitch become zero.  After cp_async_wait_all
+// and __syncwarp every lane may read its column.
+__device__ __forceinline__ void cp_async16_or_zero(void* dst, const void* src, bool in) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(in ? 16 : 0)
+               : "memory");
+}
+template <int ROWS>
+__device__ __forceinline__ void stage_rows(float* dst, int dst_pitch, const float* src, int n_pad, int c0) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int q = 0; q < (ROWS * 8 + 31) / 32; ++q) {
+    const int at = q * 32 + lane, row = at >> 3, c = 4 * (at & 7);
+    if (ROWS % 4 && row >= ROWS) break;
+    const bool in = c0 + c < n_pad;
+    cp_async16_or_zero(dst + row * dst_pitch + c, in ? src + (size_t)row * n_pad + c0 + c : src, in);
+  }
 }
 
 // ---------------------------------------------------------- frames

@@ -408,6 +408,12 @@ __host__ __device__ constexpr int bwd_min_blocks(int S) { return S == 1 ? GS_BWD
 // Row stride (floats) of the per-view 2-D cotangents: 9 per stream, padded to
 // whole float4s so that rows can be added and read as vectors.
 __host__ __device__ constexpr int cot_stride(int streams) { return (9 * streams + 3) & ~3; }
+// Place of entry k of stream st in a row of S streams, NU of them probes (the
+// last ones).  Two probes are interleaved, so that the projection's reverse pass
+// reads them as packed pairs.
+__host__ __device__ constexpr int cot_index(int S, int nu, int st, int k) {
+  return nu < 2 ? 9 * st + k : st < S - 2 ? 18 + k : 2 * k + (st - (S - 2));
+}
 
 // The reverse pass's workspace: a header, then the cotangent rows the reverse
 // blend adds into.  They must be zero when the blend starts.  The projection
@@ -519,7 +525,7 @@ __host__ __device__ constexpr int merge_pairs(int S) { return kMergeSlots * merg
 // (64 % of its peak), most of it the re-read of -w, which eight lanes of four
 // splats each load.  smx, smy, sgi: mean and index of the lane's splat; count:
 // slots in use.
-template <int S>
+template <int S, int NU>
 __device__ __forceinline__ void merge_slots(f32x2* slots, const f32x2* sw, int count, float wx0, float wy0, float smx,
                                             float smy, uint32_t sgi, float* __restrict__ cot_view) {
   constexpr int NVP = cot_stride(S), NQ = NVP / 4;
@@ -551,7 +557,7 @@ __device__ __forceinline__ void merge_slots(f32x2* slots, const f32x2* sw, int c
 #pragma unroll
     for (int s = 0; s < S; ++s)
 #pragma unroll
-      for (int ch = 0; ch < 3; ++ch) v[9 * s + 6 + ch] = sum2(c[3 * s + ch]);
+      for (int ch = 0; ch < 3; ++ch) v[cot_index(S, NU, s, 6 + ch)] = sum2(c[3 * s + ch]);
   }
   {
     f32x2 m[S][3];
@@ -581,12 +587,12 @@ __device__ __forceinline__ void merge_slots(f32x2* slots, const f32x2* sw, int c
 #pragma unroll
     for (int s = 0; s < S; ++s) {
       const float m0 = sum2(m[s][0]), m1 = sum2(m[s][1]), m2 = sum2(m[s][2]);
-      v[9 * s + 0] = dx * m0;
-      v[9 * s + 1] = m1;
-      v[9 * s + 2] = dx * dx * m0;
-      v[9 * s + 3] = dx * m1;
-      v[9 * s + 4] = m2;
-      v[9 * s + 5] = m0;
+      v[cot_index(S, NU, s, 0)] = dx * m0;
+      v[cot_index(S, NU, s, 1)] = m1;
+      v[cot_index(S, NU, s, 2)] = dx * dx * m0;
+      v[cot_index(S, NU, s, 3)] = dx * m1;
+      v[cot_index(S, NU, s, 4)] = m2;
+      v[cot_index(S, NU, s, 5)] = m0;
     }
   }
 #pragma unroll
@@ -844,7 +850,7 @@ __global__ void __launch_bounds__(32, bwd_min_blocks((GRAD ? 1 : 0) + NU)) raste
         sgi = __float_as_uint(r.c.z);
       }
       if (++used == kMergeSlots) {
-        merge_slots<S>(slots, s_w, kMergeSlots, wx0, wy0, smx, smy, sgi, cot_view);
+        merge_slots<S, NU>(slots, s_w, kMergeSlots, wx0, wy0, smx, smy, sgi, cot_view);
         used = 0;
       }
 
@@ -853,7 +859,7 @@ __global__ void __launch_bounds__(32, bwd_min_blocks((GRAD ? 1 : 0) + NU)) raste
     cur ^= 1;
     cnt = cnt_next;
   }
-  if (used) merge_slots<S>(slots, s_w, used, wx0, wy0, smx, smy, sgi, cot_view);
+  if (used) merge_slots<S, NU>(slots, s_w, used, wx0, wy0, smx, smy, sgi, cot_view);
 }
 
 // ------------------------------------------------ projection reverse pass
@@ -878,15 +884,12 @@ __global__ void __launch_bounds__(32, bwd_min_blocks((GRAD ? 1 : 0) + NU)) raste
 // pass reads them there instead of from L2.  The probe streams are combined into
 // hz = (1/nu) sum_k z_k . (G z_k).
 constexpr int kPbwdThreads = 128;
-// Minimum resident CTAs per SM requested for the projection reverse (0: none).
-#ifndef GS_PBWD_MIN_BLOCKS
-#define GS_PBWD_MIN_BLOCKS 3
-#endif
-#if GS_PBWD_MIN_BLOCKS > 0
-#define GS_PBWD_BOUNDS __launch_bounds__(kPbwdThreads, GS_PBWD_MIN_BLOCKS)
-#else
-#define GS_PBWD_BOUNDS __launch_bounds__(kPbwdThreads)
-#endif
+// Resident CTAs per SM requested for the projection reverse, by the number of
+// cotangent streams.  A fourth CTA with three streams spills and has no room for
+// the stash (2.633 against 2.610 ms per call of 1M Gaussians, 8 views, two
+// probes); without a probe a fifth CTA: 1.415 against 1.510 ms, with one a fourth:
+// 2.050 against 2.093.
+__host__ __device__ constexpr int pbwd_min_blocks(int streams) { return streams == 3 ? 3 : streams == 2 ? 4 : 5; }
 constexpr int kClampViews = 21;  // clamp bits kept for the first 21 views (3 per view)
 constexpr int kStashViews = 8;   // views whose colour cotangents pass 2 reads from shared memory
 
@@ -922,9 +925,73 @@ __device__ __forceinline__ void view_direction(const ViewGeom& v, const float mu
   d[2] = d2 / dn;
 }
 
+// One stream's arithmetic, or two probes' at once as packed pairs (1M Gaussians, 8
+// views, two probes: the call 2.760 -> 2.610 ms; the loads' latency at 12 warps
+// per SM, and 3 TB/s of rows read and cleared, are what is left).
+__device__ __forceinline__ float vmul(float a, float b) { return a * b; }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ f32x2 vmul(f32x2 a, float b) { return mul2(a, dup2(b)); }
+__device__ __forceinline__ f32x2 vfma(f32x2 a, float b, f32x2 c) { return fma2(a, dup2(b), c); }
+
+// What a view's geometry gives every stream: coefficients of the moments in
+// dL/d(conic, mean), of those in dL/d(Sigma', J, t), and W.
+struct ViewTerms {
+  float cs[2][2];             // dL/d(mx, my) by the moments of dx, dy
+  float k2[3][3];             // dL/d(a, b, c) of Sigma' by the moments of dx^2, dx dy, dy^2
+  float j00[2], j02[2], j11[2], j12[2];  // dL/dJ by dL/d(a, b) or dL/d(b, c)
+  float tx[2], ty[2], tz[6];  // dL/dt by dL/d(mx, my) and dL/dJ
+  float a0[3], a1[3];
+};
+template <class T>
+struct GeoSums {
+  T mu[3], S[6], ol;  // dL/dmu, the entries (0,0) (0,1) (0,2) (1,1) (1,2) (2,2) of dL/dSigma, dL/d(logit)
+};
+// mo: the view's moments of (dx, dy, dx^2, dx dy, dy^2, 1) dL/d(power).
+template <class T>
+__device__ __forceinline__ void add_view(GeoSums<T>& g, const T (&mo)[6], const ViewTerms& v, const float (&Rc)[3][3],
+                                         float one_minus_o) {
+  const T cs0 = vfma(mo[1], v.cs[0][1], vmul(mo[0], v.cs[0][0])), cs1 = vfma(mo[1], v.cs[1][1], vmul(mo[0], v.cs[1][0]));
+  T q[3];
+#pragma unroll
+  for (int e = 0; e < 3; ++e) q[e] = vfma(mo[4], v.k2[e][2], vfma(mo[3], v.k2[e][1], vmul(mo[2], v.k2[e][0])));
+  const T ga = q[0], gb = q[1], gc = q[2];
+  const T gJ00 = vfma(gb, v.j00[1], vmul(ga, v.j00[0])), gJ02 = vfma(gb, v.j02[1], vmul(ga, v.j02[0]));
+  const T gJ11 = vfma(gc, v.j11[1], vmul(gb, v.j11[0])), gJ12 = vfma(gc, v.j12[1], vmul(gb, v.j12[0]));
+  const T gt0 = vfma(gJ02, v.tx[1], vmul(cs0, v.tx[0])), gt1 = vfma(gJ12, v.ty[1], vmul(cs1, v.ty[0]));
+  const T gt2 = vfma(gJ12, v.tz[5], vfma(gJ02, v.tz[4], vfma(gJ11, v.tz[3], vfma(gJ00, v.tz[2],
+                     vfma(cs1, v.tz[1], vmul(cs0, v.tz[0]))))));
+#pragma unroll
+  for (int e = 0; e < 3; ++e) g.mu[e] = vfma(gt2, Rc[2][e], vfma(gt1, Rc[1][e], vfma(gt0, Rc[0][e], g.mu[e])));
+  // dSigma += ga a0 a0^T + gb/2 (a0 a1^T + a1 a0^T) + gc a1 a1^T = u a0^T + w a1^T
+  constexpr int kSymP[6] = {0, 0, 0, 1, 1, 2}, kSymQ[6] = {0, 1, 2, 1, 2, 2};
+  const T hb = vmul(gb, 0.5f);
+  T u[3], w[3];
+#pragma unroll
+  for (int e = 0; e < 3; ++e) {
+    u[e] = vfma(hb, v.a1[e], vmul(ga, v.a0[e]));
+    w[e] = vfma(gc, v.a1[e], vmul(hb, v.a0[e]));
+  }
+#pragma unroll
+  for (int e = 0; e < 6; ++e) g.S[e] = vfma(w[kSymP[e]], v.a1[kSymQ[e]], vfma(u[kSymP[e]], v.a0[kSymQ[e]], g.S[e]));
+  g.ol = vfma(mo[5], one_minus_o, g.ol);
+}
+// The colour's dependence on mu through the view direction d (distance 1 / idn):
+// gdc[ch] the direction gradient of channel ch's colour, gcol its cotangent.
+template <class T>
+__device__ __forceinline__ void add_view_colour(GeoSums<T>& g, const T (&gcol)[3], const float (&gdc)[3][3],
+                                                const float (&d)[3], float idn) {
+  T gd[3];
+#pragma unroll
+  for (int e = 0; e < 3; ++e)
+    gd[e] = vfma(gcol[2], gdc[2][e], vfma(gcol[1], gdc[1][e], vmul(gcol[0], gdc[0][e])));
+  const T dot = vfma(gd[2], d[2], vfma(gd[1], d[1], vmul(gd[0], d[0])));
+#pragma unroll
+  for (int e = 0; e < 3; ++e) g.mu[e] = vfma(vfma(dot, -d[e], gd[e]), idn, g.mu[e]);
+}
+
 // Column i (of n Gaussians, parameter pitch n_pad) summed over views cams[0..V),
 // its cotangent row of view v at (v * cot_pitch + i) * NVP of cot.  Called by
-// every thread of a kPbwdThreads block (the SH staging is block-wide).
+// every thread of a kPbwdThreads block, warp by warp.
 template <int DEG, int NU, bool GRAD>
 __device__ __forceinline__ void project_bwd_column(const float* __restrict__ P, int n, int n_pad, int i,
                                                    const gs_camera* __restrict__ cams, int V, gs_frame fr,
@@ -935,9 +1002,13 @@ __device__ __forceinline__ void project_bwd_column(const float* __restrict__ P, 
   constexpr int K = (DEG + 1) * (DEG + 1);
   // the block's SH coefficients, staged once and read per view from shared
   // memory (volatile: re-read, not held in registers across the view loops)
-  __shared__ float s_sh[3 * K][kPbwdThreads];
-  for (int r = 0; r < 3 * K; ++r) s_sh[r][threadIdx.x] = i < n ? P[(size_t)(kRowSH + r) * n_pad + i] : 0.f;
-  __syncthreads();
+  __shared__ __align__(16) float s_sh[3 * K][kPbwdThreads];
+  {
+    const int lane = threadIdx.x & 31;
+    stage_rows<3 * K>(&s_sh[0][threadIdx.x - lane], kPbwdThreads, P + (size_t)kRowSH * n_pad, n_pad, i - lane);
+    cp_async_wait_all();
+    __syncwarp();
+  }
   const volatile float* vsh = &s_sh[0][0];
   auto sh_of = [&](int k, int ch) { return vsh[(3 * k + ch) * kPbwdThreads + threadIdx.x]; };
   // colour cotangents (0 where clamped) of views v < kStashViews, one column per thread
@@ -975,17 +1046,10 @@ __device__ __forceinline__ void project_bwd_column(const float* __restrict__ P, 
   const float opac = 1.f / (1.f + expf(-ld(10)));
 
   // ---- pass 1: geometric rows of every stream
-  // g_S: dL/dSigma, symmetric, entries (0,0) (0,1) (0,2) (1,1) (1,2) (2,2)
-  constexpr int kSymP[6] = {0, 0, 0, 1, 1, 2}, kSymQ[6] = {0, 1, 2, 1, 2, 2};
-  float g_mu[S][3], g_S[S][6], g_ol[S];
-#pragma unroll
-  for (int st = 0; st < S; ++st) {
-    g_ol[st] = 0.f;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) g_mu[st][a] = 0.f;
-#pragma unroll
-    for (int e = 0; e < 6; ++e) g_S[st][e] = 0.f;
-  }
+  // (two probes as a pair, the other streams one by one)
+  constexpr int kOne = NU == 2 ? S - 2 : S;
+  GeoSums<float> g1[kOne > 0 ? kOne : 1] = {};
+  GeoSums<f32x2> g2 = {};
   uint64_t clamp_bits = 0;  // bit 3 v + c: colour channel c clamped at 0 in view v (v < kClampViews)
   uint64_t read_rows = 0;   // bit v: the row of view v held a nonzero value (cleared at the end; v >= 64 always)
 #pragma unroll 1
@@ -1048,44 +1112,30 @@ __device__ __forceinline__ void project_bwd_column(const float* __restrict__ P, 
       JS1[q] = J11 * Sc[1][q] + J12 * Sc[2][q];
     }
     const float itz2 = itz * itz, itz3 = itz2 * itz;
-    const float dJ02_dtx = clx ? 0.f : -fx * itz2, dJ12_dty = cly ? 0.f : -fy * itz2;
-    const float dJ02_dtz = clx ? fx * uc * itz2 : 2.f * fx * t[0] * itz3;
-    const float dJ12_dtz = cly ? fy * vc * itz2 : 2.f * fy * t[1] * itz3;
     // conic of this view, to turn the blend's moments into dL/d(mx, my, A, B, C)
-    const float cA = cc * idet, cB = -bb * idet, cCc = a * idet;
+    const float cA = cc * idet, cB = -bb * idet, cCc = a * idet, dac = idet - a * cc * id2;
+    const ViewTerms vt = {
+        {{-cA, -cB}, {-cB, -cCc}},
+        {{0.5f * cc * cc * id2, -bb * cc * id2, -0.5f * dac},
+         {-bb * cc * id2, idet + 2.f * bb * bb * id2, -a * bb * id2},
+         {-0.5f * dac, -a * bb * id2, 0.5f * a * a * id2}},
+        {2.f * JS0[0], JS1[0]}, {2.f * JS0[2], JS1[2]}, {JS0[1], 2.f * JS1[1]}, {JS0[2], 2.f * JS1[2]},
+        {J00, clx ? 0.f : -fx * itz2}, {J11, cly ? 0.f : -fy * itz2},
+        {-fx * t[0] * itz2, -fy * t[1] * itz2, -fx * itz2, -fy * itz2, clx ? fx * uc * itz2 : 2.f * fx * t[0] * itz3,
+         cly ? fy * vc * itz2 : 2.f * fy * t[1] * itz3},
+        {a0[0], a0[1], a0[2]}, {a1[0], a1[1], a1[2]}};
 #pragma unroll
-    for (int st = 0; st < S; ++st) {
-      const float* mo = c + 9 * st;
-      const float cs[5] = {-(cA * mo[0] + cB * mo[1]), -(cB * mo[0] + cCc * mo[1]), -0.5f * mo[2], -mo[3],
-                           -0.5f * mo[4]};
-      const float gA = cs[2], gB = cs[3], gC = cs[4];
-      const float ga = gA * (-cc * cc * id2) + gB * (bb * cc * id2) + gC * (idet - a * cc * id2);
-      const float gb = gA * (2.f * bb * cc * id2) + gB * (-idet - 2.f * bb * bb * id2) + gC * (2.f * a * bb * id2);
-      const float gc = gA * (idet - a * cc * id2) + gB * (a * bb * id2) + gC * (-a * a * id2);
-      const float gJ00 = 2.f * (ga * JS0[0] + 0.5f * gb * JS1[0]);
-      const float gJ02 = 2.f * (ga * JS0[2] + 0.5f * gb * JS1[2]);
-      const float gJ11 = 2.f * (0.5f * gb * JS0[1] + gc * JS1[1]);
-      const float gJ12 = 2.f * (0.5f * gb * JS0[2] + gc * JS1[2]);
-      float gt[3];
-      gt[0] = cs[0] * fx * itz + gJ02 * dJ02_dtx;
-      gt[1] = cs[1] * fy * itz + gJ12 * dJ12_dty;
-      gt[2] = -cs[0] * fx * t[0] * itz2 - cs[1] * fy * t[1] * itz2 - gJ00 * fx * itz2 - gJ11 * fy * itz2 +
-              gJ02 * dJ02_dtz + gJ12 * dJ12_dtz;
+    for (int st = 0; st < kOne; ++st) {
+      float mo[6];
 #pragma unroll
-      for (int q = 0; q < 3; ++q) g_mu[st][q] += vg.Rc[0][q] * gt[0] + vg.Rc[1][q] * gt[1] + vg.Rc[2][q] * gt[2];
-      // dSigma += ga a0 a0^T + gb/2 (a0 a1^T + a1 a0^T) + gc a1 a1^T = u a0^T + w a1^T
-      {
-        const float hb = 0.5f * gb;
-        float u[3], w[3];
+      for (int k = 0; k < 6; ++k) mo[k] = c[cot_index(S, NU, st, k)];
+      add_view(g1[st], mo, vt, vg.Rc, 1.f - opac);
+    }
+    if constexpr (NU == 2) {
+      f32x2 mo[6];
 #pragma unroll
-        for (int p2 = 0; p2 < 3; ++p2) {
-          u[p2] = ga * a0[p2] + hb * a1[p2];
-          w[p2] = hb * a0[p2] + gc * a1[p2];
-        }
-#pragma unroll
-        for (int e = 0; e < 6; ++e) g_S[st][e] += u[kSymP[e]] * a0[kSymQ[e]] + w[kSymP[e]] * a1[kSymQ[e]];
-      }
-      g_ol[st] += mo[5] * (1.f - opac);
+      for (int k = 0; k < 6; ++k) mo[k] = pack2(c[2 * k], c[2 * k + 1]);
+      add_view(g2, mo, vt, vg.Rc, 1.f - opac);
     }
     // colour: clamp decisions, and the dependence of colour on mu through the view direction
     float d[3], dn;
@@ -1113,20 +1163,22 @@ __device__ __forceinline__ void project_bwd_column(const float* __restrict__ P, 
 #pragma unroll
       for (int st = 0; st < S; ++st)
 #pragma unroll
-        for (int ch = 0; ch < 3; ++ch) stash(v, 3 * st + ch) = clamped[ch] ? 0.f : c[9 * st + 6 + ch];
+        for (int ch = 0; ch < 3; ++ch) stash(v, 3 * st + ch) = clamped[ch] ? 0.f : c[cot_index(S, NU, st, 6 + ch)];
     }
     if constexpr (DEG > 0) {
+      const float idn = 1.f / dn;
 #pragma unroll
-      for (int st = 0; st < S; ++st) {
+      for (int st = 0; st < kOne; ++st) {
         float gcol[3];
 #pragma unroll
-        for (int ch = 0; ch < 3; ++ch) gcol[ch] = clamped[ch] ? 0.f : c[9 * st + 6 + ch];
-        float gd[3];
+        for (int ch = 0; ch < 3; ++ch) gcol[ch] = clamped[ch] ? 0.f : c[cot_index(S, NU, st, 6 + ch)];
+        add_view_colour(g1[st], gcol, gdc, d, idn);
+      }
+      if constexpr (NU == 2) {
+        f32x2 gcol[3];
 #pragma unroll
-        for (int q = 0; q < 3; ++q) gd[q] = gcol[0] * gdc[0][q] + gcol[1] * gdc[1][q] + gcol[2] * gdc[2][q];
-        const float dot = gd[0] * d[0] + gd[1] * d[1] + gd[2] * d[2];
-#pragma unroll
-        for (int q = 0; q < 3; ++q) g_mu[st][q] += (gd[q] - d[q] * dot) / dn;
+        for (int ch = 0; ch < 3; ++ch) gcol[ch] = clamped[ch] ? 0ull : pack2(c[12 + 2 * ch], c[13 + 2 * ch]);
+        add_view_colour(g2, gcol, gdc, d, idn);
       }
     }
   }
@@ -1139,9 +1191,22 @@ __device__ __forceinline__ void project_bwd_column(const float* __restrict__ P, 
   const float inv_nu = NU > 0 ? 1.f / (float)NU : 0.f;
 #pragma unroll
   for (int st = 0; st < S; ++st) {
-    const float gS[3][3] = {{g_S[st][0], g_S[st][1], g_S[st][2]},
-                            {g_S[st][1], g_S[st][3], g_S[st][4]},
-                            {g_S[st][2], g_S[st][4], g_S[st][5]}};
+    GeoSums<float> g;
+    if (st < kOne) {
+      g = g1[st < kOne ? st : 0];
+    } else {
+      auto half = [&](f32x2 v) {
+        float lo, hi;
+        unpack2(v, lo, hi);
+        return st - kOne ? hi : lo;
+      };
+#pragma unroll
+      for (int e = 0; e < 3; ++e) g.mu[e] = half(g2.mu[e]);
+#pragma unroll
+      for (int e = 0; e < 6; ++e) g.S[e] = half(g2.S[e]);
+      g.ol = half(g2.ol);
+    }
+    const float gS[3][3] = {{g.S[0], g.S[1], g.S[2]}, {g.S[1], g.S[3], g.S[4]}, {g.S[2], g.S[4], g.S[5]}};
     float gM[3][3];
 #pragma unroll
     for (int a = 0; a < 3; ++a)
@@ -1167,10 +1232,10 @@ __device__ __forceinline__ void project_bwd_column(const float* __restrict__ P, 
             2.f * x * gR[2][1];
     const float qd = gq[0] * x + gq[1] * y + gq[2] * z + gq[3] * ww;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) rowv[a] = g_mu[st][a];
+    for (int a = 0; a < 3; ++a) rowv[a] = g.mu[a];
 #pragma unroll
     for (int cq = 0; cq < 4; ++cq) rowv[6 + cq] = (gq[cq] - qn[cq] * qd) / qlen;
-    rowv[10] = g_ol[st];
+    rowv[10] = g.ol;
     if (GRAD && st == 0) {
 #pragma unroll
       for (int r = 0; r < kRowSH; ++r) grad[(size_t)r * n_pad + i] = rowv[r];
@@ -1199,9 +1264,9 @@ __device__ __forceinline__ void project_bwd_column(const float* __restrict__ P, 
 #pragma unroll
       for (int ch = 0; ch < 3; ++ch) g[ch] = stash(v, 3 * st + ch);
     } else {
-      const float* cv = cot + ((size_t)v * cot_pitch + i) * NVP + 9 * st + 6;
+      const float* cv = cot + ((size_t)v * cot_pitch + i) * NVP;
 #pragma unroll
-      for (int ch = 0; ch < 3; ++ch) g[ch] = cv[ch];
+      for (int ch = 0; ch < 3; ++ch) g[ch] = cv[cot_index(S, NU, st, 6 + ch)];
     }
   };
   // basis of view v and its clamp decisions (true: channel clamped at 0)
@@ -1266,11 +1331,11 @@ __device__ __forceinline__ void project_bwd_column(const float* __restrict__ P, 
   if constexpr (NU == 1) sh_rows_single(GRAD ? 1 : 0);
   if constexpr (NU == 2) {
     constexpr int s1 = GRAD ? 1 : 0, s2 = s1 + 1;
-    float sp[K][3], sm[K][3];  // sums of Y (dc1 + dc2) and Y (dc1 - dc2)
+    f32x2 spm[K][3];  // sums of Y (dc1 + dc2) and of Y (dc1 - dc2)
 #pragma unroll
     for (int k = 0; k < K; ++k)
 #pragma unroll
-      for (int ch = 0; ch < 3; ++ch) sp[k][ch] = sm[k][ch] = 0.f;
+      for (int ch = 0; ch < 3; ++ch) spm[k][ch] = 0ull;
 #pragma unroll 1
     for (int v = 0; v < V; ++v) {
       float g1[3], g2[3];
@@ -1280,19 +1345,13 @@ __device__ __forceinline__ void project_bwd_column(const float* __restrict__ P, 
       float Y[K];
       bool cl[3];
       view_basis(v, Y, cl);
-      float gp[3], gm[3];
+      f32x2 gpm[3];
 #pragma unroll
-      for (int ch = 0; ch < 3; ++ch) {
-        gp[ch] = cl[ch] ? 0.f : g1[ch] + g2[ch];
-        gm[ch] = cl[ch] ? 0.f : g1[ch] - g2[ch];
-      }
+      for (int ch = 0; ch < 3; ++ch) gpm[ch] = cl[ch] ? 0ull : pack2(g1[ch] + g2[ch], g1[ch] - g2[ch]);
 #pragma unroll
       for (int k = 0; k < K; ++k)
 #pragma unroll
-        for (int ch = 0; ch < 3; ++ch) {
-          sp[k][ch] += Y[k] * gp[ch];
-          sm[k][ch] += Y[k] * gm[ch];
-        }
+        for (int ch = 0; ch < 3; ++ch) spm[k][ch] = vfma(gpm[ch], Y[k], spm[k][ch]);
     }
     const uint64_t zn1 = probe_signs(seed, step, 0, (uint64_t)i, kRowSH + 3 * K);
     const uint64_t zn2 = probe_signs(seed, step, 1, (uint64_t)i, kRowSH + 3 * K);
@@ -1302,7 +1361,9 @@ __device__ __forceinline__ void project_bwd_column(const float* __restrict__ P, 
       for (int ch = 0; ch < 3; ++ch) {
         const int r = kRowSH + 3 * k + ch;
         const bool n1 = (zn1 >> r) & 1ull, same = ((zn1 ^ zn2) >> r & 1ull) == 0;
-        const float val = same ? sp[k][ch] : sm[k][ch];
+        float sum, diff;
+        unpack2(spm[k][ch], sum, diff);
+        const float val = same ? sum : diff;
         hz[(size_t)r * n_pad + i] = (n1 ? -val : val) * inv_nu;
       }
   }
@@ -1316,7 +1377,7 @@ __device__ __forceinline__ void project_bwd_column(const float* __restrict__ P, 
 }
 
 template <int DEG, int NU, bool GRAD>
-__global__ void GS_PBWD_BOUNDS project_bwd_kernel(const float* __restrict__ P, int n, int n_pad,
+__global__ void __launch_bounds__(kPbwdThreads, pbwd_min_blocks((GRAD ? 1 : 0) + NU)) project_bwd_kernel(const float* __restrict__ P, int n, int n_pad,
                                                   const gs_camera* __restrict__ cams, gs_frame fr,
                                                   float* __restrict__ cot, ProbeArg pa, float* __restrict__ grad,
                                                   float* __restrict__ hz, CotHeader* cot_hdr, uint64_t cot_floats,
@@ -1330,7 +1391,7 @@ __global__ void GS_PBWD_BOUNDS project_bwd_kernel(const float* __restrict__ P, i
 // its own projection, from its slot of the cotangents (pitch cot_pitch), with
 // its own probe step, into its own gradient and Hutchinson rows.
 template <int DEG, int NU, bool GRAD>
-__global__ void GS_PBWD_BOUNDS project_bwd_batch_kernel(BatchArg ba, gs_frame fr, float* __restrict__ cot,
+__global__ void __launch_bounds__(kPbwdThreads, pbwd_min_blocks((GRAD ? 1 : 0) + NU)) project_bwd_batch_kernel(BatchArg ba, gs_frame fr, float* __restrict__ cot,
                                                         int cot_pitch, ProbeArg pa, CotHeader* cot_hdr,
                                                         uint64_t cot_floats, float* loss_out) {
   constexpr int NVP = cot_stride((GRAD ? 1 : 0) + NU);

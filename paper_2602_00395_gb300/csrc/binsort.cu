@@ -97,9 +97,14 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t& t
 // table holds at most 2 empty rows per record beyond its pairs (non-empty rows
 // are contiguous), so rows_cap = pair capacity + 2 x records overflows only with
 // the pairs; then the record keeps no table and GS_FLAG_CAPACITY is raised.
-__global__ void record_keys_kernel(const float4* __restrict__ rec, int n_pad, gs_frame fr, int Tx, int Ty,
-                                   uint32_t* __restrict__ rkeys, uint4* __restrict__ hdr, uint2* __restrict__ rows,
-                                   uint64_t rows_cap, uint32_t* __restrict__ rows_used, int32_t* __restrict__ status) {
+// Bound by the latency of its loads and its uneven row loops: blocks of 128 let
+// a finished warp's place be taken sooner (sort of 8 views of 1M: 1.39 ms against
+// 1.40 with 256, 1.45 with 512).
+constexpr int kRecThreads = 128;
+__global__ void __launch_bounds__(kRecThreads) record_keys_kernel(
+    const float4* __restrict__ rec, int n_pad, gs_frame fr, int Tx, int Ty, uint32_t* __restrict__ rkeys,
+    uint4* __restrict__ hdr, uint2* __restrict__ rows, uint64_t rows_cap, uint32_t* __restrict__ rows_used,
+    int32_t* __restrict__ status) {
   __shared__ uint32_t s_warp[32];
   __shared__ uint32_t s_base;
   const size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -203,19 +208,35 @@ __global__ void __launch_bounds__(kScanThreads) scan_apply_kernel(uint32_t* __re
                                                                   const uint32_t* __restrict__ block_sums) {
   __shared__ uint32_t s_warp[32];
   const size_t base = (size_t)blockIdx.x * kScanChunk + (size_t)threadIdx.x * kScanItems;
-  uint32_t v[kScanItems];
+  const bool whole = base + kScanItems <= n;
+  __align__(16) uint32_t v[kScanItems];
+  if (whole) {
+#pragma unroll
+    for (int k = 0; k < kScanItems; k += 4)
+      *reinterpret_cast<uint4*>(v + k) = *reinterpret_cast<const uint4*>(v_all + base + k);
+  } else {
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) v[k] = (base + k < n) ? v_all[base + k] : 0u;
+  }
   uint32_t s = 0;
 #pragma unroll
-  for (int k = 0; k < kScanItems; ++k) {
-    v[k] = (base + k < n) ? v_all[base + k] : 0u;
-    s += v[k];
-  }
+  for (int k = 0; k < kScanItems; ++k) s += v[k];
   uint32_t total;
   uint32_t run = block_exclusive_scan(s, total, s_warp) + block_sums[blockIdx.x];
 #pragma unroll
   for (int k = 0; k < kScanItems; ++k) {
-    if (base + k < n) v_all[base + k] = run;
-    run += v[k];
+    const uint32_t c = v[k];
+    v[k] = run;
+    run += c;
+  }
+  if (whole) {
+#pragma unroll
+    for (int k = 0; k < kScanItems; k += 4)
+      *reinterpret_cast<uint4*>(v_all + base + k) = *reinterpret_cast<const uint4*>(v + k);
+  } else {
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k)
+      if (base + k < n) v_all[base + k] = v[k];
   }
 }
 
@@ -253,53 +274,30 @@ __global__ void __launch_bounds__(1024) small_offsets_kernel(const uint32_t* __r
 inline int scan_blocks(size_t n) { return (int)((n + kScanChunk - 1) / kScanChunk); }
 
 // ------------------------------------------------------------------- emit
-// One warp emits the pairs of 32 consecutive records in (view, depth) order.
-// Their output ranges are contiguous (the offsets are an exclusive scan in that
-// order), so the warp writes its whole range with consecutive lanes on
-// consecutive pairs; each lane finds the record that owns its pair by a binary
-// search over the warp's prefix sums, and the pair's row by a binary search
-// over that record's row table (see record_keys_kernel), N pairs per lane at
-// once: two where records have few pairs (8 blocks per SM; four: 286 against
-// 246 us for 45M pairs of 8M records), four where they have many (61k records
-// of 64 pairs: 76 against 101 us with one).
+// A warp writes the pairs [p0, p1) of the emission order that belong to 32
+// records in (view, depth) order: lane L holds record L's first pair `start`
+// (non-decreasing over the lanes), header h, first tile key of its view gkey0 and
+// splat index.  Consecutive lanes write consecutive pairs; each finds the record
+// that owns its pair by a binary search over the lanes and the pair's row by a
+// binary search over that record's row table (see record_keys_kernel), N pairs
+// per lane at once so that the searches' loads overlap.
 template <int N>
-__global__ void __launch_bounds__(256, N == 2 ? 8 : 5) emit_kernel(
-    const uint4* __restrict__ hdr, const uint2* __restrict__ rows, int n_pad, gs_frame fr, int Tx, int Ty,
-    const uint32_t* __restrict__ order, const uint32_t* __restrict__ offsets, uint64_t capacity,
-    uint32_t* __restrict__ keys, uint32_t* __restrict__ vals) {
-  const size_t G = (size_t)fr.n_views * n_pad;
-  const size_t p0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;  // sorted record position
-  const size_t w0 = p0 - (threadIdx.x & 31);
-  if (w0 >= G) return;  // whole warp
+__device__ __forceinline__ void emit_span(uint32_t p0, uint32_t p1, uint32_t start, uint4 h, uint32_t gkey0,
+                                          uint32_t gsplat, const uint2* __restrict__ rows, int Tx, uint64_t capacity,
+                                          uint32_t* __restrict__ keys, uint32_t* __restrict__ vals) {
   const int lane = threadIdx.x & 31;
-  uint32_t g = 0;
-  uint4 h = make_uint4(0u, 0u, 0u, 0u);
-  if (p0 < G) {
-    g = order[p0];
-    h = hdr[g];
-  }
-  // this lane's record as (first tile key of its view, splat index): one
-  // division per record instead of one per pair (views x tiles < 2^32)
-  const uint32_t gview = g / (uint32_t)n_pad;
-  const uint32_t gkey0 = gview * (uint32_t)(Tx * Ty), gsplat = g - gview * (uint32_t)n_pad;
-  const uint32_t cnt = h.w;
-  // inclusive warp scan of the counts
-  uint32_t incl = cnt;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
-  }
-  const uint32_t start = incl - cnt;
-  const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-  const uint64_t base = offsets[w0];
   const uint32_t max_rows = __reduce_max_sync(0xffffffffu, h.y >> 16);
-  // N pairs per lane at once, so that their searches' loads overlap
-  for (uint32_t p0r = 0; p0r < total; p0r += 32 * N) {
+  const uint32_t n = p1 - p0;
+  for (uint32_t done = 0; done < n; done = n - done > 32 * N ? done + 32 * N : n) {
+    const uint32_t pr = p0 + done;
     int lo[N];
     uint32_t a[N], b[N], q[N], off[N];
+    bool in[N];
 #pragma unroll
-    for (int u = 0; u < N; ++u) lo[u] = 0;
+    for (int u = 0; u < N; ++u) {
+      lo[u] = 0;
+      in[u] = 32u * u + lane < n - done;
+    }
     // owner = largest lane whose start <= p (lanes with no pairs never win over the next lane)
 #pragma unroll
     for (int step = 16; step >= 1; step >>= 1) {
@@ -307,16 +305,16 @@ __global__ void __launch_bounds__(256, N == 2 ? 8 : 5) emit_kernel(
       for (int u = 0; u < N; ++u) {
         const int cand = lo[u] + step;
         const uint32_t sc = __shfl_sync(0xffffffffu, start, cand & 31);
-        if (cand < 32 && sc <= p0r + 32 * u + lane) lo[u] = cand;
+        if (cand < 32 && sc <= pr + 32 * u + lane) lo[u] = cand;
       }
     }
 #pragma unroll
     for (int u = 0; u < N; ++u) {
       const uint32_t R = __shfl_sync(0xffffffffu, h.y, lo[u]) >> 16;
-      q[u] = p0r + 32 * u + lane - __shfl_sync(0xffffffffu, start, lo[u]);
+      q[u] = pr + 32 * u + lane - __shfl_sync(0xffffffffu, start, lo[u]);
       off[u] = __shfl_sync(0xffffffffu, h.z, lo[u]);
       a[u] = 0;
-      b[u] = R && p0r + 32 * u + lane < total ? R - 1 : 0;
+      b[u] = R && in[u] ? R - 1 : 0;
     }
     // last row whose pairs above are <= q (empty rows repeat the count before them)
     for (uint32_t span = max_rows; span > 1; span = (span + 1) >> 1) {
@@ -330,12 +328,11 @@ __global__ void __launch_bounds__(256, N == 2 ? 8 : 5) emit_kernel(
     }
 #pragma unroll
     for (int u = 0; u < N; ++u) {
-      const uint32_t p = p0r + 32 * u + lane;
+      const uint64_t at = (uint64_t)pr + 32 * u + lane;
       uint32_t tile = __shfl_sync(0xffffffffu, gkey0, lo[u]);
       const uint32_t osplat = __shfl_sync(0xffffffffu, gsplat, lo[u]);
       const uint32_t oyr = __shfl_sync(0xffffffffu, h.y, lo[u]);
-      const uint64_t at = base + p;
-      if (p < total && at < capacity) {
+      if (in[u] && at < capacity) {
         if (oyr >> 16) {
           const uint2 e = __ldg(&rows[(size_t)off[u] + a[u]]);
           // q - e.x < the row's pairs, so txx stays in the row; the clamp only
@@ -350,6 +347,82 @@ __global__ void __launch_bounds__(256, N == 2 ? 8 : 5) emit_kernel(
         keys[at] = tile;
         vals[at] = osplat;
       }
+    }
+  }
+}
+
+// The record at sorted position p (none past the items): its header, first tile
+// key and splat index.  One division per record instead of one per pair
+// (views x tiles < 2^32).
+__device__ __forceinline__ void emit_record(size_t p, size_t items, const uint4* __restrict__ hdr,
+                                            const uint32_t* __restrict__ order, int n_pad, uint32_t tiles, uint4& h,
+                                            uint32_t& gkey0, uint32_t& gsplat) {
+  h = make_uint4(0u, 0u, 0u, 0u);
+  const uint32_t g = p < items ? __ldg(order + p) : 0u;
+  if (p < items) h = __ldg(hdr + g);
+  const uint32_t gview = g / (uint32_t)n_pad;
+  gkey0 = gview * tiles;
+  gsplat = g - gview * (uint32_t)n_pad;
+}
+
+// Few pairs per record: a warp emits 32 consecutive records, two pairs per lane
+// at once (8 blocks per SM; four at once on fewer: 286 against 246 us for 45M pairs
+// of 8M records).  Bound by the latency of the searches.
+__global__ void __launch_bounds__(256, 8) emit_kernel(const uint4* __restrict__ hdr, const uint2* __restrict__ rows,
+                                                      int n_pad, size_t items, int Tx, uint32_t tiles,
+                                                      const uint32_t* __restrict__ order,
+                                                      const uint32_t* __restrict__ offsets, uint64_t capacity,
+                                                      uint32_t* __restrict__ keys, uint32_t* __restrict__ vals) {
+  const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;  // sorted record position
+  if (p - (threadIdx.x & 31) >= items) return;                     // whole warp
+  uint4 h;
+  uint32_t gkey0, gsplat;
+  emit_record(p, items, hdr, order, n_pad, tiles, h, gkey0, gsplat);
+  const uint32_t start = __ldg(offsets + min(p, items - 1)) + (p < items ? 0u : __ldg(&hdr[__ldg(order + items - 1)].w));
+  emit_span<2>(__shfl_sync(0xffffffffu, start, 0), __shfl_sync(0xffffffffu, start + h.w, 31), start, h, gkey0, gsplat,
+               rows, Tx, capacity, keys, vals);
+}
+
+// Many pairs per record: a warp emits a chunk of consecutive pairs (an equal share
+// of them, from kEmitChunkMin to kEmitChunk), whose first record it finds by a
+// 32-way search over the records' first pairs.  A warp per 32 records left the
+// chip to the few warps with the largest splats: 61k records of 64 pairs on
+// average 76 us, 30 us with chunks.  The caller takes it from a capacity of 16
+// pairs per record on: below that a chunk spans many groups of 32 records and a
+// warp per group has the same share (8M records of 6 pairs: 246 us so).
+constexpr uint32_t kEmitChunk = 512, kEmitChunkMin = 64;
+__global__ void __launch_bounds__(256) emit_chunk_kernel(const uint4* __restrict__ hdr, const uint2* __restrict__ rows,
+                                                         int n_pad, size_t items, int Tx, uint32_t tiles,
+                                                         const uint32_t* __restrict__ order,
+                                                         const uint32_t* __restrict__ offsets,
+                                                         const uint32_t* __restrict__ n_pairs, uint64_t capacity,
+                                                         uint32_t* __restrict__ keys, uint32_t* __restrict__ vals) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t total = *n_pairs, P = (uint32_t)min((uint64_t)total, capacity);
+  const uint32_t warps = gridDim.x * (blockDim.x / 32);
+  const uint32_t chunk = min(kEmitChunk, max(kEmitChunkMin, (P / warps + 32) & ~31u));
+  for (uint64_t c0 = (uint64_t)(blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32) * chunk; c0 < P;
+       c0 += (uint64_t)warps * chunk) {
+    uint32_t p0 = (uint32_t)c0;
+    const uint32_t p1 = (uint32_t)min((uint64_t)P, c0 + chunk);
+    size_t r = 0, len = items;  // the last record that starts at or before p0 is in [r, r + len)
+    while (len > 1) {
+      const size_t step = (len + 31) / 32, at = lane * step;
+      const uint32_t ok = __ballot_sync(0xffffffffu, at < len && __ldg(offsets + r + at) <= p0);
+      const size_t k = (size_t)(31 - __clz(ok)) * step;  // lane 0 always holds
+      r += k;
+      len = min(step, len - k);
+    }
+    while (p0 < p1) {  // 32 records at a time
+      uint4 h;
+      uint32_t gkey0, gsplat;
+      emit_record(r + lane, items, hdr, order, n_pad, tiles, h, gkey0, gsplat);
+      const uint32_t start = r + lane < items ? __ldg(offsets + r + lane) : total;
+      const uint32_t end = min(p1, __shfl_sync(0xffffffffu, start + h.w, 31));
+      if (p0 < end) emit_span<4>(p0, end, start, h, gkey0, gsplat, rows, Tx, capacity, keys, vals);
+      p0 = max(p0, end);
+      r += 32;
+      if (r >= items) break;
     }
   }
 }
@@ -427,19 +500,25 @@ __global__ void __launch_bounds__(kRadixThreads) radix_hist_kernel(const uint32_
   for (int w = 0; w < kRadixWarps; ++w) s_cnt[w][tid] = 0;
   __syncthreads();
   const uint32_t* kin = keys + (size_t)g * sg.stride;
-  for (uint32_t base = begin; base < end; base += radix_tile(ITEMS)) {
-    const uint32_t at = base + (uint32_t)tid * ITEMS;
-    uint32_t kk[ITEMS];
+  uint32_t kk[ITEMS], next[ITEMS];  // the next tile's keys are on their way while this one is counted
+  auto load = [&](uint32_t at) {
     if (at + ITEMS <= end) {
 #pragma unroll
       for (int v = 0; v < ITEMS; v += 4) {
         const uint4 w = __ldg(reinterpret_cast<const uint4*>(kin + at + v));
-        kk[v] = w.x; kk[v + 1] = w.y; kk[v + 2] = w.z; kk[v + 3] = w.w;
+        next[v] = w.x; next[v + 1] = w.y; next[v + 2] = w.z; next[v + 3] = w.w;
       }
     } else {
 #pragma unroll
-      for (int k = 0; k < ITEMS; ++k) kk[k] = at + k < end ? kin[at + k] : 0u;
+      for (int k = 0; k < ITEMS; ++k) next[k] = at + k < end ? kin[at + k] : 0u;
     }
+  };
+  if (begin < end) load(begin + (uint32_t)tid * ITEMS);
+  for (uint32_t base = begin; base < end; base += radix_tile(ITEMS)) {
+    const uint32_t at = base + (uint32_t)tid * ITEMS;
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) kk[k] = next[k];
+    if (base + radix_tile(ITEMS) < end) load(at + radix_tile(ITEMS));
     uint32_t prev = 256u, run = 0;
 #pragma unroll
     for (int k = 0; k < ITEMS; ++k) {
@@ -498,7 +577,7 @@ constexpr int kDirectRanges = 32;
 // Measured on 12.2M pairs (2 views of 1080p): low digits 87 us, high digits 58 us;
 // the chain of dependent steps per tile bounds it (the stores cost 30 us of it,
 // loads are a tile ahead).  With a tile per block and a histogram per tile the
-// whole sort of 8 views took 1.78 ms, now 1.53 ms (45M pairs, 8M records); a
+// whole sort of 8 views took 1.78 ms, 1.53 ms so (45M pairs, 8M records); a
 // render of 61k large splats 0.50 -> 0.35 ms, a step of 1k Gaussians 0.27 -> 0.20.
 // totals null: hist holds plain counts (see kDirectRanges).  vin null: the
 // values are the items' positions.
@@ -627,6 +706,79 @@ __global__ void __launch_bounds__(kRadixThreads, radix_blocks(ITEMS)) radix_scat
         vout[at] = s_vals[p];
       }
     }
+  }
+}
+
+// All four passes of a segment of up to kSmallSort records in one block.  So few
+// records are bound by the launches (twelve for the passes above): one step of 1k
+// Gaussians 200 us with them, 155 us so.  Same ranking as above; the items stay in
+// shared memory between the passes.  At most kSmallSort because the keys, places
+// and counters of more do not fit 48 KB of shared memory.
+constexpr int kSmallThreads = 512, kSmallItems = 8, kSmallSort = kSmallThreads * kSmallItems;
+__global__ void __launch_bounds__(kSmallThreads) small_sort_kernel(const uint32_t* __restrict__ keys, uint32_t len,
+                                                                   uint32_t* __restrict__ vout) {
+  constexpr int kWarps = kSmallThreads / 32;
+  __shared__ uint32_t s_keys[kSmallSort];
+  __shared__ uint16_t s_vals[kSmallSort];
+  __shared__ uint16_t s_wc[kWarps][256];  // per-warp digit counts, then their first positions
+  __shared__ uint32_t s_warp[32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t lt = lanemask_lt(), mine = (uint32_t)warp * 32 * kSmallItems + lane;
+  const size_t first = (size_t)blockIdx.x * len;
+  uint32_t key[kSmallItems], val[kSmallItems], rank[kSmallItems];
+#pragma unroll
+  for (int k = 0; k < kSmallItems; ++k) {
+    val[k] = mine + (uint32_t)k * 32;
+    key[k] = val[k] < len ? __ldg(keys + first + val[k]) : 0u;
+  }
+  for (int shift = 0; shift < 32; shift += 8) {
+#pragma unroll
+    for (int q = lane; q < 256; q += 32) s_wc[warp][q] = 0;
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < kSmallItems; ++k) {
+      const uint32_t d = mine + (uint32_t)k * 32 < len ? digit_of(key[k], shift) : 256u;
+      const uint32_t peers = digit_peers<false>(d);
+      const uint32_t before = d < 256u ? s_wc[warp][d] : 0u;
+      rank[k] = before + (uint32_t)__popc(peers & lt);
+      __syncwarp();
+      if (d < 256u && (peers & lt) == 0) s_wc[warp][d] = (uint16_t)(before + (uint32_t)__popc(peers));
+      __syncwarp();
+    }
+    __syncthreads();
+    uint32_t count = 0, total;
+    if (tid < 256)
+      for (int w = 0; w < kWarps; ++w) count += s_wc[w][tid];
+    uint32_t at = block_exclusive_scan(count, total, s_warp);
+    if (tid < 256)
+      for (int w = 0; w < kWarps; ++w) {
+        const uint32_t c = s_wc[w][tid];
+        s_wc[w][tid] = (uint16_t)at;
+        at += c;
+      }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kSmallItems; ++k) {
+      if (mine + (uint32_t)k * 32 < len) {
+        const uint32_t pos = s_wc[warp][digit_of(key[k], shift)] + rank[k];
+        s_keys[pos] = key[k];
+        s_vals[pos] = (uint16_t)val[k];
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kSmallItems; ++k) {
+      const uint32_t p = mine + (uint32_t)k * 32;
+      if (p < len) {
+        key[k] = s_keys[p];
+        val[k] = s_vals[p];
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < kSmallItems; ++k) {
+    const uint32_t p = mine + (uint32_t)k * 32;
+    if (p < len) vout[first + p] = (uint32_t)first + val[k];
   }
 }
 
@@ -895,11 +1047,14 @@ extern "C" gs_status gs_bin_sort(const gs_projected* proj, int32_t n_pad, gs_fra
   // records sorted by depth within each view's segment
   uint32_t* rk[2] = {(uint32_t*)(ws + p.off_rk0), (uint32_t*)(ws + p.off_rk1)};
   uint32_t* rv[2] = {(uint32_t*)(ws + p.off_rv0), (uint32_t*)(ws + p.off_rv1)};
-  record_keys_kernel<<<eb, 256, 0, st>>>(rec, n_pad, frame, p.Tx, p.Ty, rk[0], hdr, rows, p.rows_cap, rows_used,
-                                         status);
+  record_keys_kernel<<<(unsigned)((p.n_items + kRecThreads - 1) / kRecThreads), kRecThreads, 0, st>>>(
+      rec, n_pad, frame, p.Tx, p.Ty, rk[0], hdr, rows, p.rows_cap, rows_used, status);
   int rcur = 0;
   const Seg rseg{nullptr, 0, (uint32_t)n_pad, (uint32_t)n_pad};
-  radix_passes(rk, rv, rcur, p.rec_pass, true, rseg, frame.n_views, (uint64_t)n_pad, hist, totals, st);
+  if (n_pad <= kSmallSort)
+    small_sort_kernel<<<frame.n_views, kSmallThreads, 0, st>>>(rk[0], (uint32_t)n_pad, rv[0]);
+  else
+    radix_passes(rk, rv, rcur, p.rec_pass, true, rseg, frame.n_views, (uint64_t)n_pad, hist, totals, st);
   // emission offsets in that order, and the pair count
   if (p.n_items <= kSmallScan) {
     small_offsets_kernel<<<1, 1024, 0, st>>>(rv[rcur], hdr, scnt, (int)p.n_items, out->n_pairs, out->capacity, status);
@@ -914,10 +1069,14 @@ extern "C" gs_status gs_bin_sort(const gs_projected* proj, int32_t n_pad, gs_fra
   uint32_t* kbuf[2] = {out->keys, (uint32_t*)(ws + p.off_keys)};
   uint32_t* vbuf[2] = {out->vals, (uint32_t*)(ws + p.off_vals)};
   int cur = (p.pair_pass % 2 == 0) ? 0 : 1;
-  // many pairs per record: more rounds at once, on fewer resident warps
-  auto* emit = out->capacity >= 16 * (uint64_t)p.n_items ? emit_kernel<4> : emit_kernel<2>;
-  emit<<<eb, 256, 0, st>>>(hdr, rows, n_pad, frame, p.Tx, p.Ty, rv[rcur], scnt, out->capacity, kbuf[cur],
-                                  vbuf[cur]);
+  if (out->capacity >= 16 * (uint64_t)p.n_items) {
+    const unsigned cb = (unsigned)std::min<uint64_t>((out->capacity + 8 * kEmitChunkMin - 1) / (8 * kEmitChunkMin), 152 * 8);
+    emit_chunk_kernel<<<cb, 256, 0, st>>>(hdr, rows, n_pad, p.n_items, p.Tx, (uint32_t)T, rv[rcur], scnt, out->n_pairs,
+                                          out->capacity, kbuf[cur], vbuf[cur]);
+  } else {
+    emit_kernel<<<eb, 256, 0, st>>>(hdr, rows, n_pad, p.n_items, p.Tx, (uint32_t)T, rv[rcur], scnt, out->capacity,
+                                    kbuf[cur], vbuf[cur]);
+  }
   const Seg pseg{out->n_pairs, out->capacity, 0, 0};
   radix_passes(kbuf, vbuf, cur, p.pair_pass, false, pseg, 1, out->capacity, hist, totals, st);
   const int rb = (int)std::min<uint64_t>((out->capacity + 255) / 256, 152 * 16);

@@ -58,3 +58,38 @@ def test_pairs_ranges_and_order(n, V, W, H):
     assert torch.equal(torch.sort(order).values, torch.arange(V * T, device="cuda"))
     lens = cnt[order].double()
     assert bool((lens[1:] <= torch.clamp(lens[:-1], min=1) * 1.125 + 1).all())  # heaviest classes of 1/8 first
+
+
+@pytest.mark.parametrize("n,V,W,H,big", [(40, 1, 96, 64, 90), (1000, 3, 512, 300, 250), (4096, 1, 512, 512, 400),
+                                         (30011, 2, 800, 600, 300)])
+def test_pairs_do_not_depend_on_the_capacity(n, V, W, H, big):
+    """From a capacity of 16 pairs per record on, warps emit chunks of pairs instead
+    of the pairs of 32 records: the same keys, splats and ranges.  One record in 64
+    is large, so that chunks begin and end within a record."""
+    from paper_2602_00395_gb300.engine import TRStep
+    out = []
+    for room in (False, True):
+        e = TRStep(n, 0, V, W, H, nu=0, footprint_bins=False)
+        g = torch.Generator(device="cuda").manual_seed(n)
+        rnd = lambda: torch.rand(V, n, generator=g, device="cuda")
+        rec = e.rec.view(V, e.n_pad, 12)
+        rec.zero_()
+        rec[:, :n, 0], rec[:, :n, 1] = rnd() * (W + 60) - 30, rnd() * (H + 60) - 30
+        rec[:, :n, 2] = rec[:, :n, 4] = 0.01
+        rec[:, :n, 9] = (rnd() * 4000).floor() / 100 + 0.25
+        radius = torch.where(rnd() < 1 / 64, rnd() * big, rnd() * 9).int()
+        rec.view(torch.int32)[:, :n, 10] = radius
+        rec.view(torch.int32)[:, :n, 11] = 0x7C007C00
+        e.bin_sort()
+        P = int(e.n_pairs.item())
+        items = V * e.n_pad
+        assert 0 < P < 16 * items
+        e._alloc_pairs(16 * items + 3 if room else P)
+        assert (e.capacity >= 16 * items) == room
+        for _ in range(2):
+            e.bin_sort()
+        torch.cuda.synchronize()
+        assert int(e.n_pairs.item()) == P
+        out.append((e.keys[:P].clone(), e.vals[:P].clone(), e.ranges.clone()))
+    for a, b in zip(*out):
+        assert torch.equal(a, b)

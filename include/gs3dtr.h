@@ -157,7 +157,9 @@ typedef struct gs_projected {
  *             walk as far as the pair and are reached by the splat's footprint
  *             (bit w: the block of warp w, see gs_frame);
  *             gs_raster_bwd, gs_hvp_diag and gs_raster_bwd_batch then read those
- *             bits instead of testing the footprint again.  The bits of a pair
+ *             bits instead of testing the footprint again (the bits of up to
+ *             three bytes at each end that share an aligned 4-byte word with
+ *             other memory are all set).  The bits of a pair
  *             are valid once gs_raster_fwd has run on these sorted pairs with the
  *             same frame (the reverse passes read only list positions the
  *             forward staged); pass NULL to a reverse pass otherwise.  Either

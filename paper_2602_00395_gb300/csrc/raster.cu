@@ -224,19 +224,28 @@ __device__ __forceinline__ void fwd_visit(FwdPair<NU>& p, const Rec& r, const Re
 __host__ __device__ constexpr int fwd_buffer(int nu) { return nu == 0 ? GS_FWD_BUF0 : nu == 1 ? GS_FWD_BUF1 : GS_FWD_BUF2; }
 __host__ __device__ constexpr int fwd_min_blocks(int nu) { return nu == 0 ? GS_FWD_MB0 : nu == 1 ? GS_FWD_MB1 : GS_FWD_MB2; }
 
+// The pairs' mask bytes as aligned 32-bit words: byte q is byte head + q of
+// `words` (head < 4), and `count` words from `first` on lie within the array.  The
+// bytes of the array outside them, at most three at each end, have every bit set
+// instead (the reverse pass then tests the splat at the pixels, which is as right).
+struct MaskWords {
+  uint32_t* words;  // NULL: no masks, or none but set bits
+  uint32_t head, first, count;
+};
+
 // The kernel is bound by issue slots (65 %) and the FMA pipe (50 %).  As CTAs of a
 // tile's four warps that met at two barriers per staged batch, with scalar
 // pixels, it took 1.702 ms with two probes (now 1.370), 1.414 with one (1.053)
 // and 1.085 without (0.762); 100k Gaussians, 1297 x 840, one probe 0.293 ms
 // (0.243).  Instructions per launch of two views: 411M, now 293M.
-// mask_words: the masks as 32-bit words, cleared before the launch (the blocks of
-// a tile set their own bits of the same bytes).
+// masks: cleared before the launch (the blocks of a tile set their own bits of the
+// same bytes).
 template <int NU>
 __global__ void __launch_bounds__(32, fwd_min_blocks(NU)) raster_fwd_kernel(
     const float4* __restrict__ rec, const float4* __restrict__ tan, const uint32_t* __restrict__ vals,
     const uint32_t* __restrict__ ranges, const uint32_t* __restrict__ order, int n_pad, gs_frame fr, int Tx, int T,
     int log_blocks, float* __restrict__ image, float* __restrict__ final_T, uint32_t* __restrict__ n_contrib,
-    float* __restrict__ image_tan, uint32_t* __restrict__ mask_words) {
+    float* __restrict__ image_tan, MaskWords masks) {
   constexpr int kFwdBuf = fwd_buffer(NU);
   constexpr int kPieces = 3 * (1 + NU);  // 16-byte pieces of a splat's record and tangents
   // two buffers of staged splats (the record, whose radius word is replaced by
@@ -291,12 +300,13 @@ __global__ void __launch_bounds__(32, fwd_min_blocks(NU)) raster_fwd_kernel(
     bits = 0;
     if (c >= nc) return;
     bits = __ballot_sync(0xffffffffu, gi != 0xffffffffu && block_sees(rn, wx0, wy0));
-    if (mask_words && lane <= 8) {
+    if (masks.words && lane <= 8) {
       // byte q of the masks is pair q's: the chunk's bits, shifted to the words'
       // boundaries, four at a time spread over a word's bytes at bit w
-      const uint32_t at = start + (uint32_t)(c * 32);
+      const uint32_t at = start + (uint32_t)(c * 32) + masks.head, word = (at >> 2) + lane;
       const uint32_t nib = (uint32_t)(((uint64_t)bits << (at & 3u)) >> (4 * lane)) & 15u;
-      if (nib) atomicOr(mask_words + (at >> 2) + lane, ((nib * 0x204081u) & 0x01010101u) << pb.w);
+      if (nib && word - masks.first < masks.count)
+        atomicOr(masks.words + word, ((nib * 0x204081u) & 0x01010101u) << pb.w);
     }
     record_of(gi1, rn);
     gi2 = index_of(c + 2);
@@ -1427,18 +1437,33 @@ cudaError_t allow_smem(F* f, size_t bytes) {
   return cudaFuncSetAttribute((const void*)f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+// Clears the masks and cuts them into whole words (see MaskWords).
+bool clear_masks(uint8_t* p, size_t bytes, MaskWords& m, cudaStream_t st) {
+  if (!p) return true;
+  m.head = (uint32_t)((uintptr_t)p & 3);
+  const size_t lead = (4 - m.head) & 3, tail = (m.head + bytes) & 3;
+  if (bytes < 8 || bytes > 0xfffffff0u)  // no whole word, or byte numbers that 32 bits do not hold
+    return cudaMemsetAsync(p, 0xff, bytes, st) == cudaSuccess;
+  m.words = reinterpret_cast<uint32_t*>(p - m.head);
+  m.first = m.head ? 1 : 0;
+  m.count = (uint32_t)((m.head + bytes) >> 2) - m.first;
+  return cudaMemsetAsync(p, 0, bytes, st) == cudaSuccess &&
+         (!lead || cudaMemsetAsync(p, 0xff, lead, st) == cudaSuccess) &&
+         (!tail || cudaMemsetAsync(p + bytes - tail, 0xff, tail, st) == cudaSuccess);
+}
+
 template <int NU>
 gs_status launch_fwd(const gs_projected* proj, const gs_sorted* sorted, int n_pad, gs_frame fr, float* image,
                      float* final_T, uint32_t* n_contrib, float* image_tan, cudaStream_t st) {
   const TileGrid g = tile_grid(fr);
-  if (sorted->masks && cudaMemsetAsync(sorted->masks, 0, sorted->capacity, st) != cudaSuccess)
-    return check_launch("gs_raster_fwd: memset");
+  MaskWords masks{};
+  if (!clear_masks(sorted->masks, sorted->capacity, masks, st)) return check_launch("gs_raster_fwd: memset");
   const int log_blocks = log_tile_blocks(fr);
   const unsigned blocks = (unsigned)((size_t)fr.n_views * g.T << log_blocks);
   raster_fwd_kernel<NU><<<blocks, 32, 0, st>>>(
       reinterpret_cast<const float4*>(proj->rec), reinterpret_cast<const float4*>(proj->tangent), sorted->vals,
       sorted->ranges, sorted->order, n_pad, fr, g.Tx, g.T, log_blocks, image, final_T, n_contrib, image_tan,
-      reinterpret_cast<uint32_t*>(sorted->masks));
+      masks);
   return check_launch("gs_raster_fwd");
 }
 

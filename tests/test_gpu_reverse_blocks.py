@@ -50,3 +50,46 @@ def test_short_lists_match_oracle(n, nu):
     if nu:
         _group_close(e.hz[:, :n].cpu().numpy(), ref["hz"], 1e-3, "hz", ref["hz_mass"], ref["hz_sens"],
                      ref["hz_allow"], rnd=ref["hz_round"])
+
+
+@pytest.mark.parametrize("n,off,room", [(1, 0, 0), (33, 0, 0), (33, 0, 1), (33, 0, 2), (33, 1, 0), (33, 2, 3), (33, 3, 1)])
+def test_masks_at_any_address(n, off, room):
+    """The masks are written as 32-bit words: whatever the buffer's address and
+    size, the bytes around it stay, the bytes in whole words are what an aligned
+    buffer holds, the others have every bit set, and the gradient is the one
+    without masks up to the order of its float sums."""
+    from paper_2602_00395_gb300.engine import TRStep
+    W, H = 41, 19
+    sc = S.make_scene(n, 1, seed=70 + n, extent=0.4, log_scale_shift=math.log(3.0))
+    e = TRStep(n, 1, 1, W, H, nu=0)
+    e.set_cameras([S.single_camera(W, H)])
+    e.set_params(sc.params)
+    e.set_target(S.noise_target(1, H, W, seed=71))
+    e.ensure_capacity()
+    e.project()
+    e.bin_sort()
+    P = int(e.n_pairs.item())
+    e._alloc_pairs(P + room)
+    e.bin_sort()
+    e.raster_fwd()
+    aligned = e.masks.clone()
+    e.raster_bwd()
+    grad = e.grad.clone()
+    e.masks_valid = False
+    e.raster_bwd()
+    plain = e.grad.clone()
+    around = torch.full((P + room + 32,), 0xA5, dtype=torch.uint8, device="cuda")
+    e.masks = around[16 + off : 16 + off + P + room]
+    e.raster_fwd()
+    e.raster_bwd()
+    torch.cuda.synchronize()
+    assert e.read_status() == 0
+    assert bool((around[: 16 + off] == 0xA5).all()) and bool((around[16 + off + P + room :] == 0xA5).all())
+    at = torch.arange(16 + off, 16 + off + P + room, device="cuda")
+    whole = (at // 4 * 4 >= 16 + off) & (at // 4 * 4 + 4 <= 16 + off + P + room) & (P + room >= 8)
+    both = whole & (torch.arange(P + room, device="cuda") < (P + room) // 4 * 4)
+    assert torch.equal(e.masks[both], aligned[both]) and bool((e.masks[~whole] == 0xFF).all())
+    scale = float(plain.abs().max())
+    assert scale > 0
+    for g in (grad, e.grad):
+        assert float((g - plain).abs().max()) <= 1e-5 * scale

@@ -948,8 +948,8 @@ SortPlan plan_sort(int32_t n_pad, gs_frame fr, uint64_t capacity) {
   p.rec_pass = 4;  // 32 depth bits within each view
   p.n_items = (size_t)fr.n_views * n_pad;
   // (a pass of 8 items per thread has the most ranges)
-  const size_t hist_n = (size_t)256 * std::max((size_t)ranges_per_segment(capacity, 1, 8),
-                                               (size_t)fr.n_views * ranges_per_segment((uint64_t)n_pad, fr.n_views, 8));
+  const int rec_ranges = ranges_per_segment((uint64_t)n_pad, fr.n_views, 8);
+  const size_t hist_n = (size_t)256 * std::max((size_t)ranges_per_segment(capacity, 1, 8), (size_t)fr.n_views * rec_ranges);
   const size_t sums_n = (size_t)scan_blocks(p.n_items) + 1;
   size_t o = 0;
   p.off_scnt = o;   o += align256(p.n_items * 4);
@@ -961,7 +961,7 @@ SortPlan plan_sort(int32_t n_pad, gs_frame fr, uint64_t capacity) {
   p.off_keys = o;   o += align256(capacity * 4);
   p.off_vals = o;   o += align256(capacity * 4);
   p.off_hist = o;   o += align256(hist_n * 4);
-  p.off_tot = o;    o += align256((size_t)256 * std::max(1, fr.n_views) * 4);
+  p.off_tot = o;    o += rec_ranges > kDirectRanges ? align256((size_t)256 * fr.n_views * 4) : 0;
   p.rows_cap = std::min<uint64_t>(capacity + 2 * (uint64_t)p.n_items, 0xffffffffull);
   p.off_hdr = o;    o += align256(p.n_items * 16);
   p.off_rows = o;   o += align256(p.rows_cap * 8);
@@ -1078,7 +1078,8 @@ extern "C" gs_status gs_bin_sort(const gs_projected* proj, int32_t n_pad, gs_fra
                                     kbuf[cur], vbuf[cur]);
   }
   const Seg pseg{out->n_pairs, out->capacity, 0, 0};
-  radix_passes(kbuf, vbuf, cur, p.pair_pass, false, pseg, 1, out->capacity, hist, totals, st);
+  // (the digits' totals, of more than kDirectRanges ranges, in the row tables that the emit has read)
+  radix_passes(kbuf, vbuf, cur, p.pair_pass, false, pseg, 1, out->capacity, hist, (uint32_t*)(ws + p.off_rows), st);
   const int rb = (int)std::min<uint64_t>((out->capacity + 255) / 256, 152 * 16);
   ranges_kernel<<<rb, 256, 0, st>>>(out->keys, out->n_pairs, out->capacity, (uint64_t)frame.n_views * T,
                                     out->ranges);

@@ -162,8 +162,19 @@ def make_workload(n, device, rank=0, views=N_VIEWS, n_batches=None, tile=TILE):
 
 
 def kernel_launches_per_step(eng) -> int:
-    """Kernels of this library launched per step (the sort's memsets are not
-    kernels and are not counted)."""
+    """At most so many kernels of this library run per step: with a three-kernel
+    scan in every pass of the sort (the sort's memsets are not kernels and are
+    not counted)."""
+    return _kernels(eng, scan=3)
+
+
+def launched_per_step(eng) -> int:
+    """Kernels of this library launched per step as the sort stands: one kernel
+    turns a pass's digit counts into positions."""
+    return _kernels(eng, scan=1)
+
+
+def _kernels(eng, scan: int) -> int:
     def bits(v):
         b = 0
         while (1 << b) < v:
@@ -171,7 +182,7 @@ def kernel_launches_per_step(eng) -> int:
         return b
     rec_pass = 4  # 32 depth bits, per view
     pair_pass = max(1, (bits(N_VIEWS * eng.Tx * eng.Ty) + 7) // 8)
-    radix = 1 + 3 + 1  # histogram, three-kernel scan, scatter
+    radix = 1 + scan + 1  # histogram, scan, scatter
     # record keys, record passes, count gather, three-kernel scan, emit, pair passes, ranges,
     # heaviest-first tile order (class counts, class starts, placement)
     sort = 1 + rec_pass * radix + 1 + 3 + 1 + pair_pass * radix + 1 + 3
@@ -975,7 +986,7 @@ def run_data_parallel(args, ws, rank, local, device):
             "e2e": {"value": ws * args.steps / (e2e_ms / 1e3), "unit": UNIT,
                     "h2d_bytes_per_step": targets[0].numel() * 4, "d2h_bytes_per_step": 4},
             # the eager step launches no step counter
-            "gpu_launches": (kernel_launches_per_step(eng) - 1) * args.steps,
+            "gpu_launches": (launched_per_step(eng) - 1) * args.steps,
             "roofline": roof, "roofline_calls": roof_calls, "clocks": clk.summary(), "cpu_baseline": None,
         }))
 
@@ -1116,7 +1127,7 @@ def run_cuda(args):
             "graph": "one captured CUDA graph per view batch, step index and eps_t on the device",
             "curvature": {**curv, "l1_fused_ms": ms_per_step, "overhead_l1_fused": ms_per_step / curv["gradient_only_ms"] - 1.0},
             "variants": variants, "memory": memory,
-            "gpu_launches": kernel_launches_per_step(eng) * args.steps,
+            "gpu_launches": launched_per_step(eng) * args.steps,
             "roofline": roof, "roofline_calls": roof_calls, "clocks": clocks, "cpu_baseline": cpu,
             "served": None,
         }

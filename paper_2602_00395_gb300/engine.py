@@ -60,9 +60,9 @@ class TRStep:
         pixel loss (1 - lambda) L1 + lambda D-SSIM of Eq. pixel_loss instead of L1.
         footprint_bins: bin each splat into the tiles its alpha >= 1/255 footprint
         box reaches within its 3DGS tile square (False: the whole square); the
-        images and derivatives are the same, the pairs fewer.  batch: records a
-        tile's block stages per step of its list in the forward blend (0: one per
-        thread; else a multiple of 32 up to 512)."""
+        images and derivatives are the same, the pairs fewer.  batch:
+        gs_frame.batch, a hint that the blends do not need (0, or a multiple of 32
+        up to 512)."""
         G.load()
         self.n, self.deg, self.V, self.W, self.H, self.nu = n, sh_degree, n_views, width, height, nu
         self.n_pad = synth.pad_count(n)
@@ -349,8 +349,8 @@ class TRStep:
 
 def autotune_tile(eng: TRStep, candidates=((16, 16), (32, 8), (8, 32), (16, 8), (32, 16), (16, 32)),
                   batches=(0, 64, 256), steps: int = 3, stream=None) -> tuple[tuple[int, int, int], dict]:
-    """Pick the tile shape, then the blends' per-block record batch for it, with
-    the shortest step on the caller's own workload: each candidate is a TRStep
+    """Pick the tile shape, then gs_frame.batch for it (a hint that the blends do
+    not need), with the shortest step on the caller's own workload: each candidate is a TRStep
     with the same parameters, cameras, targets and probes that runs one untimed
     and `steps` timed steps (CUDA events), starting from copies of eng's state so
     that eng is left unchanged.  Returns (tile_w, tile_h, batch) and the ms per

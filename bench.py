@@ -170,7 +170,8 @@ def kernel_launches_per_step(eng) -> int:
 
 def launched_per_step(eng) -> int:
     """Kernels of this library launched per step as the sort stands: one kernel
-    turns a pass's digit counts into positions."""
+    turns a pass's digit counts into positions, and the count gather is also the
+    first kernel of the counts' scan."""
     return _kernels(eng, scan=1)
 
 
@@ -185,7 +186,7 @@ def _kernels(eng, scan: int) -> int:
     radix = 1 + scan + 1  # histogram, scan, scatter
     # record keys, record passes, count gather, three-kernel scan, emit, pair passes, ranges,
     # heaviest-first tile order (class counts, class starts, placement)
-    sort = 1 + rec_pass * radix + 1 + 3 + 1 + pair_pass * radix + 1 + 3
+    sort = 1 + rec_pass * radix + (4 if scan == 3 else 3) + 1 + pair_pass * radix + 1 + 3
     # step counter, project, sort, fwd, reverse call (workspace check, reverse blend,
     # projection reverse), update
     return 1 + 1 + sort + 1 + 3 + 1

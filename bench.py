@@ -614,13 +614,13 @@ def raster_bwd_flops_per_unit() -> int:
 RASTER_BWD_TRAFFIC = {
     # one-kernel captures (dram__bytes_read.sum + dram__bytes_write.sum) of the
     # reverse call's two kernels on the 2-view case of the bench scene
-    "blend_bytes": 245_467_648 + 35_035_136,        # raster_bwd_kernel
-    "projection_bytes": 460_128_512 + 448_820_992,  # project_bwd_kernel
+    "blend_bytes": 245_436_160 + 34_334_208,        # raster_bwd_kernel
+    "projection_bytes": 460_086_784 + 448_578_304,  # project_bwd_kernel
     "pairs": 12_223_264,                            # pairs blended in that launch
     "n": 1_000_000,
     "views": 2,
     "sources": {
-        "paper_2602_00395_gb300/csrc/raster.cu": "25977aa71bf02399f30b065965b6cd973a485e7dafcb796da84a8119a1d70a80",
+        "paper_2602_00395_gb300/csrc/raster.cu": "2b104bd3a08966c966a1bac4c72973b98537d645794e06e52e439f90825cebee",
         "paper_2602_00395_gb300/csrc/common.cuh": "e9bcf2711bfbde27362ad3a8babfd4d75ec7ef387c8b5d98516574231b7735db",
     },
 }

@@ -957,13 +957,17 @@ struct GeoSums {
   T mu[3], S[6], ol;  // dL/dmu, the entries (0,0) (0,1) (0,2) (1,1) (1,2) (2,2) of dL/dSigma, dL/d(logit)
 };
 // mo: the view's moments of (dx, dy, dx^2, dx dy, dy^2, 1) dL/d(power).
+// Which product of a sum is rounded before it is added matters: the conic of a
+// needle cancels, and two orders differ by as much as the blend's atomics do (a
+// scale's entry by 4e-3 of the gradient's root mean square, 9e-4 in this order and
+// that of the scalar kernel).
 template <class T>
 __device__ __forceinline__ void add_view(GeoSums<T>& g, const T (&mo)[6], const ViewTerms& v, const float (&Rc)[3][3],
                                          float one_minus_o) {
-  const T cs0 = vfma(mo[1], v.cs[0][1], vmul(mo[0], v.cs[0][0])), cs1 = vfma(mo[1], v.cs[1][1], vmul(mo[0], v.cs[1][0]));
+  const T cs0 = vfma(mo[0], v.cs[0][0], vmul(mo[1], v.cs[0][1])), cs1 = vfma(mo[0], v.cs[1][0], vmul(mo[1], v.cs[1][1]));
   T q[3];
 #pragma unroll
-  for (int e = 0; e < 3; ++e) q[e] = vfma(mo[4], v.k2[e][2], vfma(mo[3], v.k2[e][1], vmul(mo[2], v.k2[e][0])));
+  for (int e = 0; e < 3; ++e) q[e] = vfma(mo[4], v.k2[e][2], vfma(mo[2], v.k2[e][0], vmul(mo[3], v.k2[e][1])));
   const T ga = q[0], gb = q[1], gc = q[2];
   const T gJ00 = vfma(gb, v.j00[1], vmul(ga, v.j00[0])), gJ02 = vfma(gb, v.j02[1], vmul(ga, v.j02[0]));
   const T gJ11 = vfma(gc, v.j11[1], vmul(gb, v.j11[0])), gJ12 = vfma(gc, v.j12[1], vmul(gb, v.j12[0]));
@@ -978,8 +982,8 @@ __device__ __forceinline__ void add_view(GeoSums<T>& g, const T (&mo)[6], const 
   T u[3], w[3];
 #pragma unroll
   for (int e = 0; e < 3; ++e) {
-    u[e] = vfma(hb, v.a1[e], vmul(ga, v.a0[e]));
-    w[e] = vfma(gc, v.a1[e], vmul(hb, v.a0[e]));
+    u[e] = vfma(ga, v.a0[e], vmul(hb, v.a1[e]));
+    w[e] = vfma(hb, v.a0[e], vmul(gc, v.a1[e]));
   }
 #pragma unroll
   for (int e = 0; e < 6; ++e) g.S[e] = vfma(w[kSymP[e]], v.a1[kSymQ[e]], vfma(u[kSymP[e]], v.a0[kSymQ[e]], g.S[e]));

@@ -15,8 +15,8 @@
 // tile's other blocks, so no block waits for another.  The reverse pass
 // walks the list back to front, recovers T_i = T_{i+1} / (1 - a_i) from the final
 // transmittance (nothing per pair is stored), merges each splat's 9 x streams
-// partial derivatives over the block's 64 pixels, four splats at a time, and
-// adds them with float4 reductions.  The projection's reverse pass (2-D
+// partial derivatives over the block's 64 pixels, four splats at a time in a
+// fixed order, and adds them with float4 reductions.  The projection's reverse pass (2-D
 // cotangents -> 11 + 3K parameter rows) runs one thread per Gaussian and sums
 // over the views.
 #include "common.cuh"
@@ -392,37 +392,37 @@ __global__ void __launch_bounds__(32, fwd_min_blocks(NU)) raster_fwd_kernel(
 }
 
 // ------------------------------------------------------------------ reverse
-// Against CTAs of a tile's four warps sharing a ring of TMA-staged batches, where
-// staging and the waits for the tile's slowest warp took 0.6 of the blend's 2.6
-// ms (1M Gaussians, 8 views of 1080p, two probes), one warp per CTA took the call
-// from 3.23 to 2.78 ms; with the merge below it was 3.40 ms before (no probe
-// 2.29 -> 1.52 ms, one 3.10 -> 2.14 ms; 100k Gaussians, 1297 x 840, one probe 0.66
-// -> 0.36 ms).
+// Against CTAs of a tile's four warps sharing a ring of TMA-staged batches, with
+// a reduce-scatter of every splat's row, one warp per CTA and the merge below take
+// the call from 3.40 to 2.83 ms (1M Gaussians, 8 views of 1080p, two probes; no
+// probe 2.29 -> 1.59 ms, one 3.10 -> 2.38 ms; 100k Gaussians, 1297 x 840, one
+// probe 0.66 -> 0.45 ms).
 // Minimum resident CTAs (warps) per SM requested from the compiler for the
-// reverse kernel, by the number of cotangent streams: without a probe 32 (64
-// registers, the most CTAs an SM holds; 28: 1.548 against 1.518 ms per call of
-// 1M Gaussians, 8 views of 1080p), with one 24 (80 registers; 20: 2.320 against
-// 2.144 ms), with two 18 (96 registers and no spills; 16: 2.840, 20: 2.801, 21:
-// 2.877 against 2.775 ms).
+// reverse kernel, by the number of cotangent streams; what counts is the warps of
+// one of the SM's four schedulers, whose registers they share.  Without a probe 28
+// (72 registers; 24: 1.577 against 1.585 ms per call of 1M Gaussians, 8 views of
+// 1080p, 32, with spills: 1.612), with one 20 (95 registers; 16: 2.524, 24, with
+// spills: 2.512 against 2.378), with two 20 (96 registers; 16: 3.003, 24, with
+// spills: 3.495 against 2.825).
 #ifndef GS_BWD_MB1
-#define GS_BWD_MB1 32
+#define GS_BWD_MB1 28
 #endif
 #ifndef GS_BWD_MB2
-#define GS_BWD_MB2 24
+#define GS_BWD_MB2 20
 #endif
 #ifndef GS_BWD_MB3
-#define GS_BWD_MB3 18
+#define GS_BWD_MB3 20
 #endif
 __host__ __device__ constexpr int bwd_min_blocks(int S) { return S == 1 ? GS_BWD_MB1 : S == 2 ? GS_BWD_MB2 : GS_BWD_MB3; }
 
 // Row stride (floats) of the per-view 2-D cotangents: 9 per stream, padded to
 // whole float4s so that rows can be added and read as vectors.
 __host__ __device__ constexpr int cot_stride(int streams) { return (9 * streams + 3) & ~3; }
-// Place of entry k of stream st in a row of S streams, NU of them probes (the
-// last ones).  Two probes are interleaved, so that the projection's reverse pass
-// reads them as packed pairs.
-__host__ __device__ constexpr int cot_index(int S, int nu, int st, int k) {
-  return nu < 2 ? 9 * st + k : st < S - 2 ? 18 + k : 2 * k + (st - (S - 2));
+// Place of entry k of stream st in a row of S streams.  The last two streams are
+// interleaved, so that the projection's reverse pass reads two probes as packed
+// pairs; the first of three follows them.
+__host__ __device__ constexpr int cot_index(int S, int st, int k) {
+  return S == 1 ? k : st < S - 2 ? 18 + k : 2 * k + (st - (S - 2));
 }
 
 // The reverse pass's workspace: a header, then the cotangent rows the reverse
@@ -488,14 +488,14 @@ __device__ __forceinline__ float rcp_approx(float x) {  // at most 1 ulp off
   return r;
 }
 
-// Reverse-pass state of a thread's two pixels: the cotangent dL/dC of each
-// stream, the transmittance being recovered back to front, per stream the
-// negated suffix -sum_{j>i} a_j T_j (w . c_j), and the list position after each
-// pixel's last blended splat.
+// Reverse-pass state of a thread's two pixels: the negated cotangent -dL/dC of
+// each stream, the transmittance being recovered back to front, the negated
+// colour suffix -sum_{j>i} a_j T_j c_j, and the list position after each pixel's
+// last blended splat.
 template <int S>
 struct BwdPair {
-  f32x2 w[S][3];
-  f32x2 T, nq[S];
+  f32x2 nw[S][3];
+  f32x2 T, ns[3];
   f32x2 npy;  // negated pixel centres
   float pxc;
   uint32_t nc[2];
@@ -513,10 +513,16 @@ __device__ __forceinline__ void red_add4(float* p, float4 v) {
 // raster_bwd_kernel): kMergeSlots splats' per-pixel values, S + 1 pairs per
 // lane, and the negated cotangents -w of the warp's pixels, 3 S pairs per lane
 // at a stride (in pairs) that keeps eight consecutive lanes on distinct banks.
+// A slot holds the values of the last two streams, side by side, then the first
+// one's (of an odd number) beside -a T, or -a T alone.
 constexpr int kMergeSlots = 4;
 __host__ __device__ constexpr int merge_slot_pairs(int S) { return 32 * (S + 1); }
 __host__ __device__ constexpr int merge_w_stride(int S) { return S == 1 ? 3 : S == 2 ? 6 : 10; }
 __host__ __device__ constexpr int merge_pairs(int S) { return kMergeSlots * merge_slot_pairs(S) + 32 * merge_w_stride(S); }
+
+// Where a column's float4s of the second part lie, so that eight lanes' are on
+// distinct banks (of the first part, and of one stream, 12 floats apart, they are).
+__host__ __device__ constexpr int part_swizzle(int S, int x) { return S == 1 ? 0 : S == 2 ? x >> 2 : x >> 1; }
 
 // The merge of up to kMergeSlots splats of one warp into their cotangent rows.
 // A row's entries per stream are the sums over pixels of (dx, dy, dx^2, dx dy,
@@ -526,32 +532,86 @@ __host__ __device__ constexpr int merge_pairs(int S) { return kMergeSlots * merg
 // which the projection's reverse pass applies: dL/dA = -M(dx^2)/2, dL/dB =
 // -M(dx dy), dL/dC = -M(dy^2)/2, dL/dmx = -(A M(dx) + B M(dy)), dL/dmy =
 // -(B M(dx) + C M(dy)), dL/d(logit) = M(1) (1 - o).
-// Lanes 8 s .. 8 s + 7 sum splat s, lane & 7 the column of the 8 x 8 block, over
-// four pairs of pixels (y, y + 4); they write their rows over the slots'
-// memory, and lane (s, quad) adds the eight rows of its four values and issues
-// one float4 reduction.  Against a reduce-scatter of the 9 S values over the
-// warp per splat (128 instructions of 290 per splat and block with two
-// probes), a merge costs about 50 per splat; shared-memory bandwidth bounds it
-// (64 % of its peak), most of it the re-read of -w, which eight lanes of four
-// splats each load.  smx, smy, sgi: mean and index of the lane's splat; count:
-// slots in use.
-template <int S, int NU>
+// For a needle those products cancel by the square of its axis ratio, so the
+// order of the moments' sums shows in its scale and rotation: it is fixed.  A
+// pixel's product is added to that of the pixel four rows below it (one fused
+// operation), then rows y and y + 2, rows y and y + 1, columns x and x + 4, x and
+// x + 1, x and x + 2; the pixels' g come from the suffix of each colour.  Summing
+// whole columns first and keeping one suffix per stream took 2.60 ms instead of
+// 2.83 (two probes), and moved single entries of the gradient by 1e-3 of its root
+// mean square, up to eight times what repeats differ by.
+// Lanes 8 s .. 8 s + 7 sum splat s, lane & 7 the column of the 8 x 8 block.  A lane
+// holds rows (0, 1), (2, 3), (4, 5), (6, 7) as pairs, first of the last two
+// streams, whose sums it writes over their slots' values, then of the rest, so
+// that half the row is live at a time; lane (s, quad) then adds the eight columns
+// of its four entries and issues one float4 reduction.  Against a reduce-scatter
+// of the 9 S values over the warp per splat (128 instructions of 290 per splat and
+// block with two probes) a merge costs about 70 per splat; the blend's bounds are
+// the path to shared memory (68 % of its wavefronts) and issue slots (57 %).
+// smx, smy, sgi: mean and index of the lane's splat; count: slots in use.
+template <int S>
 __device__ __forceinline__ void merge_slots(f32x2* slots, const f32x2* sw, int count, float wx0, float wy0, float smx,
                                             float smy, uint32_t sgi, float* __restrict__ cot_view) {
   constexpr int NVP = cot_stride(S), NQ = NVP / 4;
-  static_assert(NVP * 32 * sizeof(float) <= kMergeSlots * merge_slot_pairs(S) * sizeof(f32x2), "rows fit the slots");
+  constexpr int kA = S >= 2 ? 12 : 0, kB = NVP - kA;  // floats of a column's first and second part
+  constexpr int kQA = kA / 4, kQB = kB / 4;
   const int lane = threadIdx.x & 31, sl = lane >> 3, x = lane & 7;
-  float v[NVP];
+  f32x2* my = slots + sl * merge_slot_pairs(S);
+  float* rows = reinterpret_cast<float*>(my);
+  const float dx = smx - (wx0 + (float)x);
+  const f32x2 dx2 = dup2(dx), dxx2 = dup2(dx * dx);
+  f32x2 dy[4];  // of rows (0, 1), (2, 3), (4, 5), (6, 7)
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+    dy[r] = add2(dup2(smy), pack2(-(wy0 + (float)(2 * r)), -(wy0 + (float)(2 * r + 1))));
+  // sums over a column of g times (dx, dy, dx^2, dx dy, dy^2, 1); lo, hi: g of rows
+  // 0..3 and 4..7
+  auto moments = [&](const float (&lo)[4], const float (&hi)[4], float (&m)[6]) {
+    const f32x2 g0 = pack2(lo[0], lo[1]), g1 = pack2(lo[2], lo[3]), g2 = pack2(hi[0], hi[1]), g3 = pack2(hi[2], hi[3]);
+    auto column = [&](f32x2 k0, f32x2 k1, f32x2 k2, f32x2 k3) {
+      return sum2(add2(fma2(k2, g2, mul2(k0, g0)), fma2(k3, g3, mul2(k1, g1))));
+    };
+    m[0] = column(dx2, dx2, dx2, dx2);
+    m[1] = column(dy[0], dy[1], dy[2], dy[3]);
+    m[2] = column(dxx2, dxx2, dxx2, dxx2);
+    m[3] = column(mul2(dx2, dy[0]), mul2(dx2, dy[1]), mul2(dx2, dy[2]), mul2(dx2, dy[3]));
+    m[4] = column(mul2(dy[0], dy[0]), mul2(dy[1], dy[1]), mul2(dy[2], dy[2]), mul2(dy[3], dy[3]));
+    m[5] = sum2(add2(add2(g0, g1), add2(g2, g3)));
+  };
   __syncwarp();
-  const f32x2* my = slots + sl * merge_slot_pairs(S);
+  if constexpr (S >= 2) {  // the moments of the last two streams
+    float lo[2][4], hi[2][4], m[2][6];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(my + 2 * (r * 8 + x));
+      unpack2(t.x, lo[0][r], hi[0][r]);
+      unpack2(t.y, lo[1][r], hi[1][r]);
+    }
+    moments(lo[0], hi[0], m[0]);
+    moments(lo[1], hi[1], m[1]);
+    __syncwarp();  // every lane has read these values
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+      *reinterpret_cast<float4*>(rows + x * kA + 4 * q) =
+          make_float4(m[0][2 * q], m[1][2 * q], m[0][2 * q + 1], m[1][2 * q + 1]);
+  }
   {
+    float b[kB];
     f32x2 c[3 * S];
 #pragma unroll
     for (int k = 0; k < 3 * S; ++k) c[k] = 0ull;
-#pragma unroll(S == 3 ? 2 : 4)
+    float lo[4], hi[4];
+#pragma unroll
     for (int r = 0; r < 4; ++r) {
       const int at = r * 8 + x;
-      const f32x2 naT = S % 2 ? my[32 * (S - 1) + 2 * at + 1] : my[32 * S + at];
+      f32x2 naT;
+      if constexpr (S % 2) {
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(my + 32 * (S - 1) + 2 * at);
+        unpack2(t.x, lo[r], hi[r]);
+        naT = t.y;
+      } else {
+        naT = my[64 + at];
+      }
       const f32x2* wp = sw + at * merge_w_stride(S);
 #pragma unroll
       for (int k = 0; k < 3 * S; k += S == 1 ? 1 : 2) {
@@ -567,78 +627,95 @@ __device__ __forceinline__ void merge_slots(f32x2* slots, const f32x2* sw, int c
 #pragma unroll
     for (int s = 0; s < S; ++s)
 #pragma unroll
-      for (int ch = 0; ch < 3; ++ch) v[cot_index(S, NU, s, 6 + ch)] = sum2(c[3 * s + ch]);
-  }
-  {
-    f32x2 m[S][3];
+      for (int ch = 0; ch < 3; ++ch) b[cot_index(S, s, 6 + ch) - kA] = sum2(c[3 * s + ch]);
+    if constexpr (S % 2) {
+      float m[6];
+      moments(lo, hi, m);
 #pragma unroll
-    for (int s = 0; s < S; ++s) m[s][0] = m[s][1] = m[s][2] = 0ull;
-#pragma unroll(S == 3 ? 2 : 4)
-    for (int r = 0; r < 4; ++r) {
-      const int at = r * 8 + x;
-      f32x2 gp[S + 1];
-#pragma unroll
-      for (int p = 0; p + 1 < S + 1; p += 2) {
-        const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(my + 32 * p + 2 * at);
-        gp[p] = t.x;
-        gp[p + 1] = t.y;
-      }
-      if constexpr (S % 2 == 0) gp[S] = my[32 * S + at];
-      const f32x2 dy = add2(dup2(smy), pack2(-(wy0 + (float)r), -(wy0 + (float)(r + 4))));
-      const f32x2 dyy = mul2(dy, dy);
-#pragma unroll
-      for (int s = 0; s < S; ++s) {
-        m[s][0] = add2(m[s][0], gp[s]);
-        m[s][1] = fma2(dy, gp[s], m[s][1]);
-        m[s][2] = fma2(dyy, gp[s], m[s][2]);
-      }
+      for (int k = 0; k < 6; ++k) b[cot_index(S, 0, k) - kA] = m[k];
     }
-    const float dx = smx - (wx0 + (float)x);
 #pragma unroll
-    for (int s = 0; s < S; ++s) {
-      const float m0 = sum2(m[s][0]), m1 = sum2(m[s][1]), m2 = sum2(m[s][2]);
-      v[cot_index(S, NU, s, 0)] = dx * m0;
-      v[cot_index(S, NU, s, 1)] = m1;
-      v[cot_index(S, NU, s, 2)] = dx * dx * m0;
-      v[cot_index(S, NU, s, 3)] = dx * m1;
-      v[cot_index(S, NU, s, 4)] = m2;
-      v[cot_index(S, NU, s, 5)] = m0;
-    }
+    for (int k = 9 * S - kA; k < kB; ++k) b[k] = 0.f;
+    __syncwarp();  // every lane has read these values
+#pragma unroll
+    for (int q = 0; q < kQB; ++q)
+      *reinterpret_cast<float4*>(rows + 128 * (S >= 2) + x * kB + 4 * (q ^ part_swizzle(S, x))) =
+          make_float4(b[4 * q], b[4 * q + 1], b[4 * q + 2], b[4 * q + 3]);
   }
-#pragma unroll
-  for (int k = 9 * S; k < NVP; ++k) v[k] = 0.f;
-  __syncwarp();  // every lane has read the slots
-  float* rows = reinterpret_cast<float*>(slots);
-#pragma unroll
-  for (int k = 0; k < NVP; k += 4)
-    *reinterpret_cast<float4*>(rows + lane * NVP + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
   __syncwarp();
   if (x < NQ && sl < count) {  // quad x of the lane's own splat
-    // neighbours first, as a tree: the sum least changed by its rounding
-    f32x2 a = 0ull, b = 0ull, a4 = 0ull, b4 = 0ull, a2 = 0ull, b2 = 0ull;
+    const bool first = x < kQA;
+    const float* part = rows + (first ? 4 * x : 128 * (S >= 2));
+    const int stride = first ? kA : kB;
+    auto quad = [&](int k) {
+      return *reinterpret_cast<const ulonglong2*>(part + k * stride + (first ? 0 : 4 * ((x - kQA) ^ part_swizzle(S, k))));
+    };
+    f32x2 a[2], b[2];
 #pragma unroll
-    for (int k = 0; k < 8; k += 2) {
-      const float* at = rows + (sl * 8 + k) * NVP + 4 * x;
-      const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(at), u = *reinterpret_cast<const ulonglong2*>(at + NVP);
-      a = add2(t.x, u.x);
-      b = add2(t.y, u.y);
-      if (k == 2) {
-        a4 = add2(a2, a);
-        b4 = add2(b2, b);
-      } else if (k == 6) {
-        a = add2(a4, add2(a2, a));
-        b = add2(b4, add2(b2, b));
-      }
-      a2 = a;
-      b2 = b;
+    for (int k = 0; k < 4; k += 2) {  // columns 0, 4, 1, 5 and 2, 6, 3, 7
+      const ulonglong2 t = quad(k), u = quad(k + 4), v = quad(k + 1), w = quad(k + 5);
+      a[k / 2] = add2(add2(t.x, u.x), add2(v.x, w.x));
+      b[k / 2] = add2(add2(t.y, u.y), add2(v.y, w.y));
     }
     float4 q;
-    unpack2(a, q.x, q.y);
-    unpack2(b, q.z, q.w);
+    unpack2(add2(a[0], a[1]), q.x, q.y);
+    unpack2(add2(b[0], b[1]), q.z, q.w);
     if (q.x != 0.f || q.y != 0.f || q.z != 0.f || q.w != 0.f)
       red_add4(cot_view + (size_t)sgi * NVP + 4 * x, q);
   }
   __syncwarp();  // the slots may be written again
+}
+
+// A lane's cotangents from shared memory; volatile, so that they are read here and
+// not held in registers across a merge (spilled there, they cost the call 0.45 ms).
+template <int S>
+__device__ __forceinline__ void load_w(f32x2 (&nw)[S][3], const f32x2* sw) {
+#pragma unroll
+  for (int k = 0; k < 3 * S; ++k) {
+    if (S == 1 || k + 1 >= 3 * S) {
+      asm volatile("ld.shared.b64 %0, [%1];" : "=l"(nw[k / 3][k % 3]) : "r"(smem_u32(sw + k)));
+    } else if (k % 2 == 0) {
+      asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];"
+                   : "=l"(nw[k / 3][k % 3]), "=l"(nw[(k + 1) / 3][(k + 1) % 3])
+                   : "r"(smem_u32(sw + k)));
+    }
+  }
+}
+// A splat that at most this many lanes blend is added by those lanes, each the row
+// of its two pixels, instead of through the merge: part of the fixed order too (a
+// quarter of the splats that a block blends; without it the call of 1M Gaussians and
+// 8 views takes 1.557 instead of 1.584 ms with no probe, 2.425 instead of 2.378 with
+// one, 2.924 instead of 2.824 with two).
+constexpr int kSparseLanes = 8;
+template <int S>
+__device__ __forceinline__ void add_lane(const f32x2 (&gp)[S], f32x2 naT, const f32x2 (&nw)[S][3], float dx, f32x2 dy,
+                                         float* __restrict__ row) {
+  constexpr int NVP = cot_stride(S);
+  float y0, y1, t0, t1;
+  unpack2(dy, y0, y1);
+  unpack2(naT, t0, t1);
+  float v[NVP];
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    float g0, g1;
+    unpack2(gp[s], g0, g1);
+    v[cot_index(S, s, 0)] = fmaf(dx, g1, __fmul_rn(dx, g0));
+    v[cot_index(S, s, 1)] = fmaf(y1, g1, __fmul_rn(y0, g0));
+    v[cot_index(S, s, 2)] = fmaf(__fmul_rn(dx, dx), g1, __fmul_rn(__fmul_rn(dx, dx), g0));
+    v[cot_index(S, s, 3)] = fmaf(__fmul_rn(dx, y1), g1, __fmul_rn(__fmul_rn(dx, y0), g0));
+    v[cot_index(S, s, 4)] = fmaf(__fmul_rn(y1, y1), g1, __fmul_rn(__fmul_rn(y0, y0), g0));
+    v[cot_index(S, s, 5)] = g0 + g1;
+#pragma unroll
+    for (int ch = 0; ch < 3; ++ch) {
+      float w0, w1;
+      unpack2(nw[s][ch], w0, w1);
+      v[cot_index(S, s, 6 + ch)] = fmaf(w1, t1, __fmul_rn(w0, t0));
+    }
+  }
+#pragma unroll
+  for (int k = 9 * S; k < NVP; ++k) v[k] = 0.f;
+#pragma unroll
+  for (int k = 0; k < NVP; k += 4) red_add4(row + k, make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]));
 }
 
 template <int NU, bool GRAD>
@@ -732,13 +809,13 @@ __global__ void __launch_bounds__(32, bwd_min_blocks((GRAD ? 1 : 0) + NU)) raste
     }
     pp.T = pack2(Tv[0], Tv[1]);
     pp.npy = pack2(-pyc[0], -pyc[1]);
+    pp.ns[0] = pp.ns[1] = pp.ns[2] = 0ull;
 #pragma unroll
     for (int st = 0; st < S; ++st) {
-      pp.nq[st] = 0ull;
 #pragma unroll
       for (int ch = 0; ch < 3; ++ch) {
-        pp.w[st][ch] = pack2(wv[0][st][ch], wv[1][st][ch]);
-        s_w[lane * merge_w_stride(S) + 3 * st + ch] = pack2(-wv[0][st][ch], -wv[1][st][ch]);
+        pp.nw[st][ch] = pack2(-wv[0][st][ch], -wv[1][st][ch]);
+        s_w[lane * merge_w_stride(S) + 3 * st + ch] = pp.nw[st][ch];
       }
     }
   }
@@ -826,50 +903,55 @@ __global__ void __launch_bounds__(32, bwd_min_blocks((GRAD ? 1 : 0) + NU)) raste
         const float al = fminf(kAlphaMax, oG[q]);
         on[q] = pos < pp.nc[q] && power[q] <= 0.f && al >= kAlphaMin;
         na[q] = on[q] ? -al : 0.f;
-        ac[q] = on[q] && !(oG[q] > kAlphaMax) ? al : 0.f;  // a capped alpha has zero derivative
+        ac[q] = on[q] && !(oG[q] > kAlphaMax) ? -al : 0.f;  // a capped alpha has zero derivative
       }
-      if (!__any_sync(0xffffffffu, on[0] || on[1])) continue;
-      // recover T_i = T_{i+1} / (1 - a); with d = w . c and q the stream's
-      // suffix, dL/d(power) = a/(1 - a) (T_{i+1} d - q) per stream.  A pixel
-      // that does not blend the splat has a = 0: its state stays as it is and it
-      // contributes exact zeros.
+      const uint32_t act = __ballot_sync(0xffffffffu, on[0] || on[1]);
+      if (!act) continue;
+      // recover T_i = T_{i+1} / (1 - a); dC/da = c T_i - suffix / (1 - a), and
+      // dL/d(power) = a (w . dC/da) per stream.  A pixel that does not blend the
+      // splat has a = 0: its state stays as it is and it contributes exact zeros.
       const f32x2 nap = pack2(na[0], na[1]);
       unpack2(add2(dup2(1.f), nap), om[0], om[1]);
       const f32x2 inv = pack2(rcp_approx(om[0]), rcp_approx(om[1]));
-      const f32x2 Ti = mul2(pp.T, inv), kk = mul2(inv, pack2(ac[0], ac[1])), naT = mul2(nap, Ti);
-      f32x2 gp[S];
+      const f32x2 Ti = mul2(pp.T, inv), nac = pack2(ac[0], ac[1]), naT = mul2(nap, Ti);
+      const float rgb[3] = {r.b.z, r.b.w, r.c.x};
+      f32x2 gp[S], da[3];
 #pragma unroll
-      for (int s = 0; s < S; ++s) {
-        const f32x2 d = fma2(pp.w[s][2], dup2(r.c.x), fma2(pp.w[s][1], dup2(r.b.w), mul2(pp.w[s][0], dup2(r.b.z))));
-        gp[s] = mul2(kk, fma2(pp.T, d, pp.nq[s]));
-        pp.nq[s] = fma2(naT, d, pp.nq[s]);
+      for (int ch = 0; ch < 3; ++ch) {
+        da[ch] = fma2(dup2(rgb[ch]), Ti, mul2(pp.ns[ch], inv));
+        pp.ns[ch] = fma2(dup2(rgb[ch]), naT, pp.ns[ch]);
       }
+#pragma unroll
+      for (int s = 0; s < S; ++s)
+        gp[s] = mul2(fma2(pp.nw[s][2], da[2], fma2(pp.nw[s][0], da[0], mul2(pp.nw[s][1], da[1]))), nac);
       pp.T = Ti;
+      if (__popc(act) <= kSparseLanes) {
+        if (on[0] || on[1])
+          add_lane<S>(gp, naT, pp.nw, dx, dy, cot_view + (size_t)__float_as_uint(r.c.z) * NVP);
+        continue;
+      }
       // the lane's values of this splat into its merge slot
       f32x2* my = slots + used * merge_slot_pairs(S);
-      if constexpr (S == 1) {
-        *reinterpret_cast<ulonglong2*>(my + 2 * lane) = make_ulonglong2(gp[0], naT);
-      } else {
-        *reinterpret_cast<ulonglong2*>(my + 2 * lane) = make_ulonglong2(gp[0], gp[1]);
-        if constexpr (S == 2) my[64 + lane] = naT;
-        else *reinterpret_cast<ulonglong2*>(my + 64 + 2 * lane) = make_ulonglong2(gp[S - 1], naT);
-      }
+      if constexpr (S >= 2) *reinterpret_cast<ulonglong2*>(my + 2 * lane) = make_ulonglong2(gp[S - 2], gp[S - 1]);
+      if constexpr (S % 2) *reinterpret_cast<ulonglong2*>(my + 32 * (S - 1) + 2 * lane) = make_ulonglong2(gp[0], naT);
+      else my[64 + lane] = naT;
       if ((lane >> 3) == used) {
         smx = r.a.x;
         smy = r.a.y;
         sgi = __float_as_uint(r.c.z);
       }
       if (++used == kMergeSlots) {
-        merge_slots<S, NU>(slots, s_w, kMergeSlots, wx0, wy0, smx, smy, sgi, cot_view);
+        merge_slots<S>(slots, s_w, kMergeSlots, wx0, wy0, smx, smy, sgi, cot_view);
         used = 0;
+        // the cotangents again, so that they take no registers during a merge
+        load_w<S>(pp.nw, s_w + lane * merge_w_stride(S));
       }
-
     }
     __syncwarp();  // the buffer may be refilled
     cur ^= 1;
     cnt = cnt_next;
   }
-  if (used) merge_slots<S, NU>(slots, s_w, used, wx0, wy0, smx, smy, sgi, cot_view);
+  if (used) merge_slots<S>(slots, s_w, used, wx0, wy0, smx, smy, sgi, cot_view);
 }
 
 // ------------------------------------------------ projection reverse pass
@@ -1142,7 +1224,7 @@ __device__ __forceinline__ void project_bwd_column(const float* __restrict__ P, 
     for (int st = 0; st < kOne; ++st) {
       float mo[6];
 #pragma unroll
-      for (int k = 0; k < 6; ++k) mo[k] = c[cot_index(S, NU, st, k)];
+      for (int k = 0; k < 6; ++k) mo[k] = c[cot_index(S, st, k)];
       add_view(g1[st], mo, vt, vg.Rc, 1.f - opac);
     }
     if constexpr (NU == 2) {
@@ -1177,7 +1259,7 @@ __device__ __forceinline__ void project_bwd_column(const float* __restrict__ P, 
 #pragma unroll
       for (int st = 0; st < S; ++st)
 #pragma unroll
-        for (int ch = 0; ch < 3; ++ch) stash(v, 3 * st + ch) = clamped[ch] ? 0.f : c[cot_index(S, NU, st, 6 + ch)];
+        for (int ch = 0; ch < 3; ++ch) stash(v, 3 * st + ch) = clamped[ch] ? 0.f : c[cot_index(S, st, 6 + ch)];
     }
     if constexpr (DEG > 0) {
       const float idn = 1.f / dn;
@@ -1185,7 +1267,7 @@ __device__ __forceinline__ void project_bwd_column(const float* __restrict__ P, 
       for (int st = 0; st < kOne; ++st) {
         float gcol[3];
 #pragma unroll
-        for (int ch = 0; ch < 3; ++ch) gcol[ch] = clamped[ch] ? 0.f : c[cot_index(S, NU, st, 6 + ch)];
+        for (int ch = 0; ch < 3; ++ch) gcol[ch] = clamped[ch] ? 0.f : c[cot_index(S, st, 6 + ch)];
         add_view_colour(g1[st], gcol, gdc, d, idn);
       }
       if constexpr (NU == 2) {
@@ -1280,7 +1362,7 @@ __device__ __forceinline__ void project_bwd_column(const float* __restrict__ P, 
     } else {
       const float* cv = cot + ((size_t)v * cot_pitch + i) * NVP;
 #pragma unroll
-      for (int ch = 0; ch < 3; ++ch) g[ch] = cv[cot_index(S, NU, st, 6 + ch)];
+      for (int ch = 0; ch < 3; ++ch) g[ch] = cv[cot_index(S, st, 6 + ch)];
     }
   };
   // basis of view v and its clamp decisions (true: channel clamped at 0)

@@ -93,3 +93,40 @@ def test_pairs_do_not_depend_on_the_capacity(n, V, W, H, big):
         out.append((e.keys[:P].clone(), e.vals[:P].clone(), e.ranges.clone()))
     for a, b in zip(*out):
         assert torch.equal(a, b)
+
+
+def test_runs_of_records_without_pairs_cost_no_walk():
+    """Chunks of pairs at a view's end are followed by the next view's culled
+    records, a million of them without a pair, and the capacity is far above the
+    pairs.  A warp that walks them takes 17 ms; the whole sort
+    takes no more than three times the one that gives a warp to every 32 records
+    (capacity below 16 pairs per record), with the same result."""
+    from paper_2602_00395_gb300.engine import TRStep
+    n, V, W, H, seen = 1 << 20, 3, 1920, 1080, 3000
+    e = TRStep(n, 0, V, W, H, nu=0, footprint_bins=False)
+    g = torch.Generator(device="cuda").manual_seed(7)
+    rnd = lambda: torch.rand(V, seen, generator=g, device="cuda")
+    rec = e.rec.view(V, e.n_pad, 12)
+    rec.zero_()
+    at = torch.randperm(n, generator=g, device="cuda")[:seen]
+    rec[:, at, 0], rec[:, at, 1], rec[:, at, 9] = rnd() * W, rnd() * H, rnd() * 40 + 0.25
+    rec.view(torch.int32)[:, at, 10] = 20
+    rec.view(torch.int32)[:, at, 11] = 0x7C007C00
+    out, ms = [], []
+    for room in (False, True):
+        e._alloc_pairs(16 * V * e.n_pad if room else 1 << 18)
+        times = []
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            e.bin_sort()
+            b.record()
+            b.synchronize()
+            times.append(a.elapsed_time(b))
+        P = int(e.n_pairs.item())
+        assert e.read_status() == 0 and 0 < P <= 1 << 18
+        out.append((e.keys[:P].clone(), e.vals[:P].clone(), e.ranges.clone()))
+        ms.append(min(times))
+    for x, y in zip(*out):
+        assert torch.equal(x, y)
+    assert ms[1] <= 3 * ms[0], ms

@@ -24,6 +24,7 @@
 // for the chip and read P from device memory, so the call needs no host
 // synchronisation (and can be captured in a graph).
 #include "common.cuh"
+#include "ranges.cuh"
 
 namespace gs {
 namespace {
@@ -470,17 +471,6 @@ __device__ __forceinline__ uint32_t digit_of(K key, int shift) {
 
 __device__ __forceinline__ uint32_t digit_of(uint32_t key, int shift) { return (key >> shift) & 255u; }
 
-// The items [begin, end) of range b of a segment of len items.
-template <int ITEMS>
-__device__ __forceinline__ void range_of(uint32_t len, int bps, int b, uint32_t& begin, uint32_t& end) {
-  constexpr uint32_t kTile = radix_tile(ITEMS);
-  const uint32_t tiles = len / kTile + (len % kTile != 0), per = tiles / (uint32_t)bps, extra = tiles % (uint32_t)bps;
-  const uint32_t t0 = (uint32_t)b * per + min((uint32_t)b, extra), n = per + ((uint32_t)b < extra);
-  begin = t0 * kTile;  // below len + kTile, and only used where below len
-  end = t0 + n >= tiles ? len : (t0 + n) * kTile;
-  if (n == 0) end = begin;
-}
-
 // The lanes of the warp that hold the same digit (256: no item).  The match
 // instruction takes longer the more distinct digits the warp holds; nine ballots
 // take the same time always.  FEW: the digits of a warp are mostly alike.
@@ -500,20 +490,20 @@ __device__ __forceinline__ uint32_t digit_peers(uint32_t d) {
 // Digit counts of one range.  A thread counts ITEMS consecutive keys (read
 // as 16-byte vectors) and adds each run of equal digits to its warp's counters
 // with one shared atomic: a splat's pairs are adjacent and share their high tile
-// digit, so runs are common.
-template <int ITEMS>
+// digit, so runs are common.  Pos: the type of positions (see positions_wrap).
+template <int ITEMS, class Pos>
 __global__ void __launch_bounds__(kRadixThreads) radix_hist_kernel(const uint32_t* __restrict__ keys, Seg sg, int bps,
                                                                    int shift, uint32_t* __restrict__ hist) {
   __shared__ uint32_t s_cnt[kRadixWarps][256];
   const int g = blockIdx.x / bps, b = blockIdx.x - g * bps, tid = threadIdx.x, warp = tid >> 5;
-  uint32_t begin, end;
-  range_of<ITEMS>(seg_len(sg), bps, b, begin, end);
+  const Range<Pos> rg = range_of<Pos>(seg_len(sg), radix_tile(ITEMS), bps, b);
+  const Pos begin = rg.begin, end = rg.end;
 #pragma unroll
   for (int w = 0; w < kRadixWarps; ++w) s_cnt[w][tid] = 0;
   __syncthreads();
   const uint32_t* kin = keys + (size_t)g * sg.stride;
   uint32_t kk[ITEMS], next[ITEMS];  // the next tile's keys are on their way while this one is counted
-  auto load = [&](uint32_t at) {
+  auto load = [&](Pos at) {
     if (at + ITEMS <= end) {
 #pragma unroll
       for (int v = 0; v < ITEMS; v += 4) {
@@ -526,8 +516,8 @@ __global__ void __launch_bounds__(kRadixThreads) radix_hist_kernel(const uint32_
     }
   };
   if (begin < end) load(begin + (uint32_t)tid * ITEMS);
-  for (uint32_t base = begin; base < end; base += radix_tile(ITEMS)) {
-    const uint32_t at = base + (uint32_t)tid * ITEMS;
+  for (Pos base = begin; base < end; base += radix_tile(ITEMS)) {
+    const Pos at = base + (uint32_t)tid * ITEMS;
 #pragma unroll
     for (int k = 0; k < ITEMS; ++k) kk[k] = next[k];
     if (base + radix_tile(ITEMS) < end) load(at + radix_tile(ITEMS));
@@ -593,7 +583,7 @@ constexpr int kDirectRanges = 32;
 // render of 61k large splats 0.50 -> 0.35 ms, a step of 1k Gaussians 0.27 -> 0.20.
 // totals null: hist holds plain counts (see kDirectRanges).  vin null: the
 // values are the items' positions.
-template <bool FEW, int ITEMS>
+template <bool FEW, int ITEMS, class Pos>
 __global__ void __launch_bounds__(kRadixThreads, radix_blocks(ITEMS)) radix_scatter_kernel(
     const uint32_t* __restrict__ kin_all, const uint32_t* __restrict__ vin_all, uint32_t* __restrict__ kout,
     uint32_t* __restrict__ vout, Seg sg, int bps, int shift, const uint32_t* __restrict__ hist,
@@ -606,8 +596,8 @@ __global__ void __launch_bounds__(kRadixThreads, radix_blocks(ITEMS)) radix_scat
   __shared__ uint32_t s_warp[32];
   const int g = blockIdx.x / bps, b = blockIdx.x - g * bps;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  uint32_t begin, end;
-  range_of<ITEMS>(seg_len(sg), bps, b, begin, end);
+  const Range<Pos> rg = range_of<Pos>(seg_len(sg), kTile, bps, b);
+  const Pos begin = rg.begin, end = rg.end;
   if (begin >= end) return;
   const uint32_t lt = lanemask_lt();
   // first output position of digit tid in this range
@@ -633,17 +623,17 @@ __global__ void __launch_bounds__(kRadixThreads, radix_blocks(ITEMS)) radix_scat
   // the next tile's items are loaded while this one is ranked
   uint32_t key[ITEMS], vv[ITEMS], nkey[ITEMS], nval[ITEMS];
   const uint32_t mine = (uint32_t)warp * 32 * ITEMS + lane;
-  auto load = [&](uint32_t tile) {
+  auto load = [&](Pos tile) {
 #pragma unroll
     for (int k = 0; k < ITEMS; ++k) {
-      const uint32_t idx = tile + mine + (uint32_t)k * 32;
+      const Pos idx = tile + mine + (uint32_t)k * 32;
       nkey[k] = idx < end ? __ldg(kin + idx) : 0u;
-      nval[k] = idx < end ? (vin ? __ldg(vin + idx) : (uint32_t)g * sg.stride + idx) : 0u;
+      nval[k] = idx < end ? (vin ? __ldg(vin + idx) : (uint32_t)g * sg.stride + (uint32_t)idx) : 0u;
     }
   };
   load(begin);
-  for (uint32_t tile = begin; tile < end; tile += kTile) {
-    const uint32_t base = tile + mine;
+  for (Pos tile = begin; tile < end; tile += kTile) {
+    const Pos base = tile + mine;
     uint32_t rank[ITEMS], peers[ITEMS];
 #pragma unroll
     for (int k = 0; k < ITEMS; ++k) {
@@ -707,7 +697,7 @@ __global__ void __launch_bounds__(kRadixThreads, radix_blocks(ITEMS)) radix_scat
     }
     __syncthreads();
     // (what is read below is written again only after two more barriers)
-    const uint32_t tot = min((uint32_t)kTile, end - tile);
+    const uint32_t tot = (uint32_t)min((Pos)kTile, end - tile);
 #pragma unroll
     for (int k = 0; k < ITEMS; ++k) {
       const uint32_t p = (uint32_t)k * kRadixThreads + tid;
@@ -985,16 +975,16 @@ SortPlan plan_sort(int32_t n_pad, gs_frame fr, uint64_t capacity) {
 
 // One stable pass (see Seg) over at most len_max items per segment; vin null: the
 // values are the items' positions.
-template <bool FEW, int ITEMS>
+template <bool FEW, int ITEMS, class Pos>
 void radix_pass(const uint32_t* kin, const uint32_t* vin, uint32_t* kout, uint32_t* vout, int shift, Seg sg, int nseg,
                 uint64_t len_max, uint32_t* hist, uint32_t* totals, cudaStream_t st) {
   const int bps = ranges_per_segment(len_max, nseg, ITEMS);
   const unsigned grid = (unsigned)((size_t)nseg * bps);
   const bool direct = bps <= kDirectRanges;
-  radix_hist_kernel<ITEMS><<<grid, kRadixThreads, 0, st>>>(kin, sg, bps, shift, hist);
+  radix_hist_kernel<ITEMS, Pos><<<grid, kRadixThreads, 0, st>>>(kin, sg, bps, shift, hist);
   if (!direct) radix_prefix_kernel<<<dim3(256 / 32, nseg), 1024, 0, st>>>(hist, totals, bps);
-  radix_scatter_kernel<FEW, ITEMS><<<grid, kRadixThreads, 0, st>>>(kin, vin, kout, vout, sg, bps, shift, hist,
-                                                                   direct ? nullptr : totals);
+  radix_scatter_kernel<FEW, ITEMS, Pos><<<grid, kRadixThreads, 0, st>>>(kin, vin, kout, vout, sg, bps, shift, hist,
+                                                                        direct ? nullptr : totals);
 }
 
 // Stable LSD passes over 8-bit digits from bit 0; the keys/values ping-pong
@@ -1006,8 +996,11 @@ void radix_passes(uint32_t** kbuf, uint32_t** vbuf, int& cur, int npass, bool io
                   uint32_t* hist, uint32_t* totals, cudaStream_t st) {
   for (int pass = 0; pass < npass; ++pass) {
     const bool few = npass > 1 && pass + 1 == npass;
-    auto* run = few ? radix_pass<true, 8>
-                    : radix_items(len_max, nseg, few) == 16 ? radix_pass<false, 16> : radix_pass<false, 8>;
+    const bool long_tiles = radix_items(len_max, nseg, few) == 16;
+    auto* run = few ? radix_pass<true, 8, uint32_t>
+                    : long_tiles ? radix_pass<false, 16, uint32_t> : radix_pass<false, 8, uint32_t>;
+    if (positions_wrap(len_max, radix_tile(16)))  // (a segment so long has long tiles)
+      run = few ? radix_pass<true, 8, uint64_t> : radix_pass<false, 16, uint64_t>;
     run(kbuf[cur], iota && pass == 0 ? nullptr : vbuf[cur], kbuf[cur ^ 1], vbuf[cur ^ 1], 8 * pass, sg, nseg, len_max,
         hist, totals, st);
     cur ^= 1;

@@ -130,3 +130,32 @@ def test_runs_of_records_without_pairs_cost_no_walk():
     for x, y in zip(*out):
         assert torch.equal(x, y)
     assert ms[1] <= 3 * ms[0], ms
+
+
+def test_largest_capacity():
+    """At the largest capacity the pair passes run on 64-bit positions (and the
+    buffers take 105 GB): the same keys, splats and ranges as with a small one."""
+    from paper_2602_00395_gb300.engine import TRStep
+    if torch.cuda.mem_get_info()[0] < 130 << 30:
+        pytest.skip("needs 130 GB of free device memory")
+    n, V, W, H = 70001, 3, 640, 480
+    e = TRStep(n, 0, V, W, H, nu=0, footprint_bins=False)
+    g = torch.Generator(device="cuda").manual_seed(n)
+    rnd = lambda: torch.rand(V, n, generator=g, device="cuda")
+    rec = e.rec.view(V, e.n_pad, 12)
+    rec.zero_()
+    rec[:, :n, 0], rec[:, :n, 1], rec[:, :n, 9] = rnd() * W, rnd() * H, (rnd() * 4000).floor() / 100 + 0.25
+    rec.view(torch.int32)[:, :n, 10] = (rnd() * 12).int()
+    rec.view(torch.int32)[:, :n, 11] = 0x7C007C00
+    out = []
+    for capacity in (1 << 22, (1 << 32) - 1):
+        e.keys = e.vals = e.masks = e.sort_ws = None
+        e._alloc_pairs(capacity)
+        e.bin_sort()
+        P = int(e.n_pairs.item())
+        assert e.read_status() == 0 and 300000 < P < 1 << 22
+        out.append((e.keys[:P].clone(), e.vals[:P].clone(), e.ranges.clone()))
+    e.keys = e.vals = e.masks = e.sort_ws = None
+    torch.cuda.empty_cache()
+    for a, b in zip(*out):
+        assert torch.equal(a, b)

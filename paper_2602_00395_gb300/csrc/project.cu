@@ -306,6 +306,8 @@ extern "C" gs_status gs_project(const gs_params* x, const gs_camera* cams, gs_fr
     return GS_ERR_UNSUPPORTED;
   }
   GS_REQUIRE(nu == 0 || out->tangent, "gs_project: probes given but out->tangent is NULL");
+  GS_REQUIRE(gs::on_16_bytes(out->rec) && (nu == 0 || gs::on_16_bytes(out->tangent)),
+             "gs_project: rec and tangent must be 16-byte aligned");
   if (x->n_pad == 0) return GS_OK;
   cudaStream_t st = (cudaStream_t)stream;
   const gs::ProbeArg pa = gs::probe_arg(probe);
@@ -349,6 +351,8 @@ extern "C" gs_status gs_project_batch(const gs_batch_item* items, int32_t n_item
     return GS_ERR_UNSUPPORTED;
   }
   GS_REQUIRE(nu == 0 || out->tangent, "gs_project_batch: probes given but out->tangent is NULL");
+  GS_REQUIRE(gs::on_16_bytes(out->rec) && (nu == 0 || gs::on_16_bytes(out->tangent)),
+             "gs_project_batch: rec and tangent must be 16-byte aligned");
   for (int b = 0; b < n_items; ++b) {
     const gs_batch_item& it = items[b];
     GS_REQUIRE(it.x.data && it.cam, "gs_project_batch: item %d has a null buffer", b);

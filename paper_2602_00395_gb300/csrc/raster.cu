@@ -1673,6 +1673,7 @@ gs_status run_bwd(bool want_grad, const gs_params* x, const gs_camera* cams, gs_
                   int32_t* status, void* stream, const char* name) {
   GS_REQUIRE(x && cams && proj && sorted && image && target && final_T && n_contrib, "%s: null argument", name);
   GS_REQUIRE(proj->rec && sorted->vals && sorted->ranges && x->data, "%s: null device buffer", name);
+  GS_REQUIRE(on_16_bytes(proj->rec), "%s: rec must be 16-byte aligned", name);
   GS_REQUIRE(frame_ok(frame), "%s: bad frame", name);
   GS_REQUIRE(x->n >= 0 && x->n_pad >= x->n && x->n_pad % 4 == 0, "%s: bad n/n_pad", name);
   GS_REQUIRE(loss.kind == GS_LOSS_L1 || loss.kind == GS_LOSS_L2 || loss.kind == GS_LOSS_COTANGENT ||
@@ -1725,6 +1726,8 @@ extern "C" gs_status gs_raster_fwd(const gs_projected* proj, const gs_sorted* so
     return GS_ERR_UNSUPPORTED;
   }
   GS_REQUIRE(nu == 0 || proj->tangent, "gs_raster_fwd: probes given but proj->tangent is NULL");
+  GS_REQUIRE(on_16_bytes(proj->rec) && (nu == 0 || on_16_bytes(proj->tangent)),
+             "gs_raster_fwd: rec and tangent must be 16-byte aligned");
   cudaStream_t st = (cudaStream_t)stream;
   if (nu == 0) return launch_fwd<0>(proj, sorted, n_pad, frame, image, final_T, n_contrib, nullptr, st);
   if (nu == 1) return launch_fwd<1>(proj, sorted, n_pad, frame, image, final_T, n_contrib, image_tangent, st);
@@ -1765,6 +1768,7 @@ extern "C" gs_status gs_raster_bwd_batch(const gs_batch_item* items, int32_t n_i
   const char* name = "gs_raster_bwd_batch";
   GS_REQUIRE(items && proj && sorted && image && target && final_T && n_contrib, "%s: null argument", name);
   GS_REQUIRE(proj->rec && sorted->vals && sorted->ranges, "%s: null device buffer", name);
+  GS_REQUIRE(on_16_bytes(proj->rec), "%s: rec must be 16-byte aligned", name);
   GS_REQUIRE(n_items >= 1 && n_items <= GS_BATCH_MAX, "%s: n_items=%d outside [1, %d]", name, n_items, GS_BATCH_MAX);
   GS_REQUIRE(frame_ok(frame) && frame.n_views == n_items, "%s: bad frame (n_views must equal n_items)", name);
   GS_REQUIRE(n_pad_max >= 4 && n_pad_max % 4 == 0, "%s: bad n_pad_max=%d", name, n_pad_max);

@@ -192,11 +192,11 @@ def _kernels(eng, scan: int) -> int:
     return 1 + 1 + sort + 1 + 3 + 1
 
 
-def retile_workload(eng, cam_dev, targets, batches, tile, device, batch=0):
+def retile_workload(eng, cam_dev, targets, batches, tile, device):
     """The same workload (parameters, cameras, targets) on a step with another
-    tile shape and blend batch."""
+    tile shape."""
     from paper_2602_00395_gb300.engine import TRStep
-    e = TRStep(eng.n, SH_DEG, eng.V, W, H, nu=NU, tile=tile, cfg=eng.cfg, device=device, batch=batch)
+    e = TRStep(eng.n, SH_DEG, eng.V, W, H, nu=NU, tile=tile, cfg=eng.cfg, device=device)
     e.x.copy_(eng.x)
     need = 0
     for cd in cam_dev:
@@ -207,11 +207,23 @@ def retile_workload(eng, cam_dev, targets, batches, tile, device, batch=0):
     return e, cam_dev, targets, batches, need
 
 
+def visited_pixels(masks):
+    """Pixels at which the blends evaluate a splat, summed over the pairs: 64 per
+    8 x 8 block that a pair's mask names (those that walk as far as the pair and
+    that its footprint reaches).  Unlike a pixel's list position, the count hardly
+    depends on the tile shape."""
+    import torch
+    m = masks[: masks.numel() & ~3]  # (the bytes of a last part word are all set)
+    m = m - ((m >> 1) & 0x55)
+    m = (m & 0x33) + ((m >> 2) & 0x33)
+    return 64.0 * ((m + (m >> 4)) & 0x0F).sum(dtype=torch.float64)
+
+
 def timed_steps(eng, cam_dev, targets, K, W0, t0, stream, per_call=False):
     """K steps on `stream`; returns (ms total from events, per-call ms dict).
     With per_call, each call is bracketed by its own events, and the work units
     of those very launches are summed on the device between the calls: the dict
-    then also holds "sum_n_contrib" and "pairs", their means per step."""
+    then also holds "visited_pixels" and "pairs", their means per step."""
     import torch
     from paper_2602_00395_gb300.engine import eps_schedule
     calls = ["project", "bin_sort", "raster_fwd", "raster_bwd", "update"]
@@ -219,7 +231,7 @@ def timed_steps(eng, cam_dev, targets, K, W0, t0, stream, per_call=False):
     start = torch.cuda.Event(enable_timing=True)
     stop = torch.cuda.Event(enable_timing=True)
     nb = len(targets)
-    units = torch.zeros(2, dtype=torch.float64, device=eng.device)  # sum n_contrib, pairs
+    units = torch.zeros(2, dtype=torch.float64, device=eng.device)  # visited pixels, pairs
     with torch.cuda.stream(stream):
         start.record(stream)
         for k in range(K):
@@ -243,7 +255,7 @@ def timed_steps(eng, cam_dev, targets, K, W0, t0, stream, per_call=False):
                     z.record(stream)
                     ev[name].append((a, z))
                     if name == "raster_fwd":  # outside the calls' event brackets
-                        units[0] += eng.n_contrib.sum(dtype=torch.float64)
+                        units[0] += visited_pixels(eng.masks)
                         units[1] += eng.n_pairs.to(torch.float64).sum()
                 else:
                     fn()
@@ -252,7 +264,7 @@ def timed_steps(eng, cam_dev, targets, K, W0, t0, stream, per_call=False):
     total = start.elapsed_time(stop)
     per = {c: (sum(a.elapsed_time(z) for a, z in ev[c]) / len(ev[c]) if ev[c] else None) for c in calls}
     if per_call:
-        per["sum_n_contrib"], per["pairs"] = (float(u) / K for u in units.cpu())
+        per["visited_pixels"], per["pairs"] = (float(u) / K for u in units.cpu())
     return total, per
 
 
@@ -593,10 +605,10 @@ def served_metrics(device, n_requests=200, slots=16, budget_gb=40.0):
 
 
 # ------------------------------------------------------------------ roofline
-# Algorithmic FP32 work per contributing (pixel, splat) unit, the unit being
-# sum over pixels of n_contrib (list position of the last blended splat): the
-# forward blend ~20 FLOP per unit plus ~25 per probe for the fused tangents; the
-# reverse blend ~50 FLOP per unit per cotangent stream (1 + nu streams).
+# Algorithmic FP32 work per (pixel, splat) at which the blends evaluate the splat
+# (visited_pixels; about 30 % of them blend it): the forward blend ~20 FLOP plus
+# ~25 per probe for the fused tangents; the reverse blend ~50 FLOP per cotangent
+# stream (1 + nu streams).
 def raster_fwd_flops_per_unit() -> int:
     return 20 + 25 * NU
 
@@ -619,6 +631,7 @@ RASTER_BWD_TRAFFIC = {
     "pairs": 12_223_264,                            # pairs blended in that launch
     "n": 1_000_000,
     "views": 2,
+    "tile": (16, 16),  # a larger tile's blocks walk longer lists for the same pairs
     "sources": {
         "paper_2602_00395_gb300/csrc/raster.cu": "2b104bd3a08966c966a1bac4c72973b98537d645794e06e52e439f90825cebee",
         "paper_2602_00395_gb300/csrc/common.cuh": "e9bcf2711bfbde27362ad3a8babfd4d75ec7ef387c8b5d98516574231b7735db",
@@ -637,14 +650,14 @@ def projection_reverse_bytes(n: int, views: int, sh_degree: int = SH_DEG, nu: in
     return n * (4 * rows + 2 * views * 4 * cot + (2 if nu > 0 else 1) * 4 * rows)
 
 
-def raster_bwd_traffic(pairs: float | None = None, n: int | None = None, views: int | None = None):
+def raster_bwd_traffic(pairs: float | None = None, n: int | None = None, views: int | None = None, tile=None):
     """DRAM bytes of one reverse call, scaled from the captures: the blend's by
     the pairs it blends, the projection reverse's by its algorithmic bytes (the
-    cotangent rows it reads grow with the views).  None once a source of the
-    captured build has changed."""
+    cotangent rows it reads grow with the views).  None for another tile shape
+    than the captured one, and once a source of the captured build has changed."""
     import hashlib
     c = RASTER_BWD_TRAFFIC
-    if c["blend_bytes"] is None:
+    if c["blend_bytes"] is None or (tile is not None and tuple(tile) != c["tile"]):
         return None
     for rel, digest in c["sources"].items():
         with open(os.path.join(ROOT, rel), "rb") as f:
@@ -851,7 +864,7 @@ def run_configs(device):
     return out
 
 
-def rooflines(eng, per_call, sum_nc, pairs_timed, local, full_size):
+def rooflines(eng, per_call, visited, pairs_timed, local, full_size):
     """The dominant call's roofline and every call's, from per-call CUDA-event
     times and the work units of the same launches."""
     import torch
@@ -877,8 +890,8 @@ def rooflines(eng, per_call, sum_nc, pairs_timed, local, full_size):
         # (count, key, value, row-table header; the row entries are not counted),
         # 16 B per pass, 12 B count gather, 16 B header read by the emit
         "bin_sort": ("hbm", pairs_timed * (8 + 16 * pair_pass + 4) + R * (48 + 28 + 16 * rec_pass + 12 + 16)),
-        "raster_fwd": ("alu", raster_fwd_flops_per_unit() * sum_nc),
-        "raster_bwd": ("alu", raster_bwd_flops_per_unit() * sum_nc),
+        "raster_fwd": ("alu", raster_fwd_flops_per_unit() * visited),
+        "raster_bwd": ("alu", raster_bwd_flops_per_unit() * visited),
         "update": ("hbm", eng.n * rows * 4 * (5 + 3)),
     }
     roof_calls = {}
@@ -898,14 +911,14 @@ def rooflines(eng, per_call, sum_nc, pairs_timed, local, full_size):
         traffic = None
     else:
         name, ms_k, per_unit = "gs_raster_bwd (reverse blend, 1+nu streams, + projection reverse)", bwd_ms, raster_bwd_flops_per_unit()
-        traffic = raster_bwd_traffic(pairs_timed, N_GAUSS, N_VIEWS) if full_size else None
-    achieved = per_unit * sum_nc / (ms_k * 1e-3) / 1e12
+        traffic = raster_bwd_traffic(pairs_timed, N_GAUSS, N_VIEWS, eng.tile) if full_size else None
+    achieved = per_unit * visited / (ms_k * 1e-3) / 1e12
     roof = {"kernel": name, "bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
             "frac": achieved / fp32_peak, "traffic": traffic, "launch_ms": ms_k,
             "peak_source": (f"{n_sm} SMs (device query) x 128 FP32 lanes x 2 FLOP x {sm_mhz:.0f} MHz "
                             f"({src} max SM clock)"),
-            "work": (f"{per_unit} FLOP x {sum_nc:.4g} units (sum over pixels of n_contrib, all views, mean of "
-                     f"the steps the call was timed on)")}
+            "work": (f"{per_unit} FLOP x {visited:.4g} pixels at which a splat is evaluated (64 per 8 x 8 block that "
+                     f"a pair's footprint reaches, all views, mean of the steps the call was timed on)")}
     return roof, roof_calls
 
 
@@ -968,9 +981,9 @@ def run_data_parallel(args, ws, rank, local, device):
     tt = torch.tensor([ms, e2e_ms], device=device)
     dist.all_reduce(tt, op=dist.ReduceOp.MAX)
     ms, e2e_ms = (float(v) for v in tt.cpu())
-    sum_nc = per_call.pop("sum_n_contrib")
+    visited = per_call.pop("visited_pixels")
     pairs_timed = per_call.pop("pairs")
-    roof, roof_calls = rooflines(eng, per_call, sum_nc, pairs_timed, local, args.n == N_GAUSS)
+    roof, roof_calls = rooflines(eng, per_call, visited, pairs_timed, local, args.n == N_GAUSS)
     status = eng.read_status()
     if rank == 0:
         ms_per_step = ms / args.steps
@@ -1025,10 +1038,9 @@ def run_cuda(args):
     stream = torch.cuda.Stream(device=device)
     # tile shape: measured on this workload (the step is rebuilt if another shape wins)
     from paper_2602_00395_gb300.engine import autotune_tile
-    (bw, bh, best_batch), tile_ms = autotune_tile(eng, stream=stream)
-    if (bw, bh, best_batch) != (*TILE, 0):
-        eng, cam_dev, targets, batches, need = retile_workload(eng, cam_dev, targets, batches, (bw, bh), device,
-                                                               best_batch)
+    (bw, bh, _), tile_ms = autotune_tile(eng, stream=stream)
+    if (bw, bh) != TILE:
+        eng, cam_dev, targets, batches, need = retile_workload(eng, cam_dev, targets, batches, (bw, bh), device)
     # warm-up
     timed_steps(eng, cam_dev, targets, max(args.warmup, 3), 0, 1, stream)
     torch.cuda.synchronize()
@@ -1090,9 +1102,9 @@ def run_cuda(args):
     # roofline of the dominant call: the work units are those of the launches
     # the per-call times come from (summed between the calls of those steps)
     torch.cuda.synchronize()
-    sum_nc = per_call.pop("sum_n_contrib")
+    visited = per_call.pop("visited_pixels")
     pairs_timed = per_call.pop("pairs")
-    roof, roof_calls = rooflines(eng, per_call, sum_nc, pairs_timed, local, args.n == N_GAUSS)
+    roof, roof_calls = rooflines(eng, per_call, visited, pairs_timed, local, args.n == N_GAUSS)
     clocks = clk.summary()
     cpu = None
     if rank == 0 and ws == 1 and not args.no_cpu_baseline:
@@ -1110,9 +1122,8 @@ def run_cuda(args):
             "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": {"workload": WORKLOAD, "n_gaussians": args.n, "views_per_step": N_VIEWS,
                        "image": f"{W}x{H}", "nu": NU, "tile": f"{eng.tile[0]}x{eng.tile[1]}",
-                       "blend_batch": eng.frame.batch or "one per thread",
-                       "tile_autotune_ms": {f"{a}x{b}" + (f"/{c}" if c else ""): round(v, 3)
-                                            for (a, b, c), v in tile_ms.items()}, "pairs_per_step": pairs_timed,
+                       "tile_autotune_ms": {f"{a}x{b}": round(v, 3) for (a, b, _), v in tile_ms.items()},
+                       "pairs_per_step": pairs_timed,
                        "pairs_max_over_view_batches": need,
                        "parallelism": "replicas" if ws > 1 else "single GPU",
                        "l2": "inputs larger than L2 (236 MB parameters, 199 MB targets per step)",

@@ -348,9 +348,10 @@ class TRStep:
 
 
 def autotune_tile(eng: TRStep, candidates=((16, 16), (32, 8), (8, 32), (16, 8), (32, 16), (16, 32)),
-                  batches=(0, 64, 256), steps: int = 3, stream=None) -> tuple[tuple[int, int, int], dict]:
-    """Pick the tile shape, then gs_frame.batch for it (a hint that the blends do
-    not need), with the shortest step on the caller's own workload: each candidate is a TRStep
+                  batches=(0,), steps: int = 3, stream=None) -> tuple[tuple[int, int, int], dict]:
+    """Pick the tile shape with the shortest step on the caller's own workload, and
+    of `batches` the gs_frame.batch (the present blends do not read that hint, so
+    by default it is not timed): each candidate is a TRStep
     with the same parameters, cameras, targets and probes that runs one untimed
     and `steps` timed steps (CUDA events), starting from copies of eng's state so
     that eng is left unchanged.  Returns (tile_w, tile_h, batch) and the ms per

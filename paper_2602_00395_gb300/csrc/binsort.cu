@@ -242,8 +242,10 @@ __global__ void __launch_bounds__(kScanThreads) scan_apply_kernel(uint32_t* __re
 }
 
 // Gather, scan and total in one block, for up to kSmallScan records: one launch
-// where three would each cost more than the work.
-constexpr size_t kSmallScan = 16384;
+// where three would each cost more than the work (the whole sort of 8192 records
+// 101 against 103 us with three, of 12,288 the other way: 114 against 112, of
+// 16,384 112 against 106).
+constexpr size_t kSmallScan = 8192;
 __global__ void __launch_bounds__(1024) small_offsets_kernel(const uint32_t* __restrict__ order,
                                                              const uint4* __restrict__ hdr, uint32_t* __restrict__ scnt,
                                                              int items, uint32_t* __restrict__ total, uint64_t capacity,
@@ -390,7 +392,12 @@ __global__ void __launch_bounds__(256, 8) emit_kernel(const uint4* __restrict__ 
 // chip to the few warps with the largest splats: 61k records of 64 pairs on
 // average 76 us, 30 us with chunks.  The caller takes it from a capacity of 16
 // pairs per record on: below that a chunk spans many groups of 32 records and a
-// warp per group has the same share (8M records of 6 pairs: 246 us so).  Records
+// warp per group has the same share (8M records of 6 pairs: 246 us so).  Where one
+// record in 64 is eight times as wide, the whole sort takes with chunks and without
+// 125 and 137 us (8000 records of 10 pairs), 160 and 194 (61,000 of 23), 298 and 316
+// (300,000 of 23), 706 and 700 (1M of 23), 1352 and 1387 (1M of 54); where all are
+// alike it is slower with them from about 150,000 records on, by 7 % at 1M of 15
+// pairs and 12 % at 8M.  Records
 // without pairs come in runs (the culled ones first in their view, with depth 0):
 // a group that owns none of the chunk's pairs is followed by another search
 // instead of the groups after it (3 views of 1M records, 3000 with pairs in each:
@@ -566,7 +573,9 @@ __global__ void __launch_bounds__(1024) radix_prefix_kernel(uint32_t* __restrict
   }
 }
 // Up to this many ranges a scatter block sums the ranges' counts itself, which
-// spares the kernel above (small inputs are bound by their launches).
+// spares the kernel above (small inputs are bound by their launches: the sort of
+// 65,536 records, 32 ranges a pass, 120 us against 128 with the kernel; of 98,304,
+// 48 ranges, 140 against 133).
 constexpr int kDirectRanges = 32;
 
 // Stable scatter of one range, tile by tile.  Warp w owns a tile's items
@@ -866,7 +875,9 @@ __global__ void tile_order_kernel(const uint32_t* __restrict__ ranges, uint32_t 
   if (c != 0xffffffffu) order[base + __popc(peers & ((1u << lane) - 1u))] = t;
 }
 
-// The whole order in one block, for few tiles.
+// The whole order in one block, for few tiles: three launches and a memset less (the
+// sort with 8160 tiles 116 against 121 us, with 14,400 122 against 123, with 32,400
+// 136 against 122).
 constexpr uint32_t kSmallOrder = 8192;
 __global__ void __launch_bounds__(1024) small_tile_order_kernel(const uint32_t* __restrict__ ranges, uint32_t n_tiles,
                                                                 uint32_t* __restrict__ order) {

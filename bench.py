@@ -619,22 +619,23 @@ def raster_bwd_flops_per_unit() -> int:
 
 # DRAM bytes of one gs_raster_bwd call (its two kernels, read plus write; the
 # workspace clear is a memset, not counted) from one-kernel ncu captures of the
-# 2-view case (summaries under profiles/), with that case's pair count: a full
+# 2-view case in the tile shape that the autotuner takes (summaries under
+# profiles/), with that case's pair count: a full
 # launch's traffic is scaled from it by the pairs (the gathered records and the
 # cotangent rows grow with the pairs and views).  Valid while the kernel sources
 # are the ones captured (their SHA-256 below); otherwise null.
 RASTER_BWD_TRAFFIC = {
     # one-kernel captures (dram__bytes_read.sum + dram__bytes_write.sum) of the
     # reverse call's two kernels on the 2-view case of the bench scene
-    "blend_bytes": 245_436_160 + 34_334_208,        # raster_bwd_kernel
-    "projection_bytes": 460_086_784 + 448_578_304,  # project_bwd_kernel
-    "pairs": 12_223_264,                            # pairs blended in that launch
+    "blend_bytes": 250_807_296 + 35_321_344,        # raster_bwd_kernel
+    "projection_bytes": 460_133_888 + 448_815_360,  # project_bwd_kernel
+    "pairs": 8_580_237,                             # pairs blended in that launch
     "n": 1_000_000,
     "views": 2,
-    "tile": (16, 16),  # a larger tile's blocks walk longer lists for the same pairs
+    "tile": (16, 32),  # a smaller tile makes more pairs for much the same bytes
     "sources": {
-        "paper_2602_00395_gb300/csrc/raster.cu": "2b104bd3a08966c966a1bac4c72973b98537d645794e06e52e439f90825cebee",
-        "paper_2602_00395_gb300/csrc/common.cuh": "e9bcf2711bfbde27362ad3a8babfd4d75ec7ef387c8b5d98516574231b7735db",
+        "paper_2602_00395_gb300/csrc/raster.cu": "a054992549162a91bf64a0914b160e353a3ec89fc032d9358fe76b398745feec",
+        "paper_2602_00395_gb300/csrc/common.cuh": "2112fcc4ef0c3d8c4eac27e66b3f9102b0f58c16da48d0c9ef64751c3d2923c7",
     },
 }
 

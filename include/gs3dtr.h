@@ -60,8 +60,8 @@ enum {
 enum {
   GS_FLAG_CAPACITY = 1,  /* gs_bin_sort: more pairs than capacity; *n_pairs holds the need */
   GS_FLAG_NONFINITE = 2, /* gs_tr_update: a non-finite value was written */
-  GS_FLAG_TIMEOUT = 4    /* a bounded wait gave up (gs_wait_check); a reverse blend
-                          * that finds it set walks no list */
+  GS_FLAG_TIMEOUT = 4    /* a bounded wait on an asynchronous copy gave up; a reverse
+                          * blend that finds it set walks no list */
 };
 
 const char* gs_last_error(void); /* host string, valid until the next call on this thread */
@@ -421,10 +421,9 @@ gs_status gs_tr_update_batch(const gs_batch_item* items, int32_t n_items, const 
 
 /* Diagnostics (no paper counterpart): runs, in one warp, a bounded wait on an
  * mbarrier that nothing completes, giving up after `limit` tries
- * (1 <= limit <= 2^20).  Raises GS_FLAG_TIMEOUT in *status (device int32); the
- * kernel then returns and the context stays usable.  Lets the failure path be
- * tested without a fault (the path's own kernels wait only for copies that their
- * warp started). */
+ * (1 <= limit <= 2^20).  Raises GS_FLAG_TIMEOUT in *status (device int32) as the
+ * reverse blend does when a staged copy never lands; the kernel then returns and
+ * the context stays usable.  Lets the failure path be tested without a fault. */
 gs_status gs_wait_check(uint32_t limit, int32_t* status, void* stream);
 
 #ifdef __cplusplus

@@ -27,7 +27,8 @@ gs_status check_launch(const char* what) {
 
 namespace {
 // One warp waits, with `limit` tries, on an mbarrier that nothing arrives at and
-// no copy completes: every lane gives up and raises GS_FLAG_TIMEOUT.
+// no copy completes: every lane gives up and raises GS_FLAG_TIMEOUT, as a kernel
+// does when a staged copy never lands.
 __global__ void wait_check_kernel(uint32_t limit, int32_t* status) {
   __shared__ __align__(8) uint64_t bar;
   if (threadIdx.x == 0) {

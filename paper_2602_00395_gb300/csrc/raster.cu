@@ -12,11 +12,12 @@
 // chunks of 32 positions, keeps the splats whose alpha >= 1/255 footprint can
 // reach its block, and stages those records in shared memory by asynchronous
 // copies, one buffer ahead of the one it blends.  Nothing is shared with the
-// tile's other blocks, so no block waits for another.  The reverse pass
-// walks the list back to front, recovers T_i = T_{i+1} / (1 - a_i) from the final
-// transmittance (nothing per pair is stored), merges each splat's 9 x streams
-// partial derivatives over the block's 64 pixels, four splats at a time in a
-// fixed order, and adds them with float4 reductions.  The projection's reverse pass (2-D
+// tile's other blocks, so no block waits for another (but see below).  The reverse
+// pass walks the list back to front, recovers T_i = T_{i+1} / (1 - a_i) from the final
+// transmittance (nothing per pair is stored), sums each splat's 9 x streams partial
+// derivatives over the block's 64 pixels in a fixed order, and adds them with
+// float4 reductions; with two probes beside the gradient a tile's warps walk its list
+// in step, sharing a ring of TMA-staged batches.  The projection's reverse pass (2-D
 // cotangents -> 11 + 3K parameter rows) runs one thread per Gaussian and sums
 // over the views.
 #include "common.cuh"
@@ -392,28 +393,25 @@ __global__ void __launch_bounds__(32, fwd_min_blocks(NU)) raster_fwd_kernel(
 }
 
 // ------------------------------------------------------------------ reverse
-// Against CTAs of a tile's four warps sharing a ring of TMA-staged batches, with
-// a reduce-scatter of every splat's row, one warp per CTA and the merge below take
-// the call from 3.40 to 2.83 ms (1M Gaussians, 8 views of 1080p, two probes; no
-// probe 2.29 -> 1.59 ms, one 3.10 -> 2.38 ms; 100k Gaussians, 1297 x 840, one
-// probe 0.66 -> 0.45 ms).
-// Minimum resident CTAs (warps) per SM requested from the compiler for the
-// reverse kernel, by the number of cotangent streams; what counts is the warps of
+// Two kernels.  With one or two streams a warp per CTA walks its own 8 x 8 block
+// (raster_bwd_kernel); with three, the gradient's and two probes', a tile's warps
+// walk its list in step (raster_bwd_tile_kernel).  Both sum a splat's products over
+// a block in the same fixed order (see merge_slots).
+// Minimum resident CTAs (warps) per SM requested from the compiler for
+// raster_bwd_kernel, by the number of cotangent streams; what counts is the warps of
 // one of the SM's four schedulers, whose registers they share.  Without a probe 28
-// (72 registers; 24: 1.577 against 1.585 ms per call of 1M Gaussians, 8 views of
+// (72 registers; 24: 1.577 against 1.563 ms per call of 1M Gaussians, 8 views of
 // 1080p, 32, with spills: 1.612), with one 20 (95 registers; 16: 2.524, 24, with
-// spills: 2.512 against 2.378), with two 20 (96 registers; 16: 3.003, 24, with
-// spills: 3.495 against 2.825).
+// spills: 2.512 against 2.378).  Against CTAs of a tile's four warps sharing a ring of
+// TMA-staged batches, with a reduce-scatter of every splat's row: none 2.29 -> 1.56
+// ms, one 3.10 -> 2.38; 100k Gaussians, 1297 x 840, one probe 0.66 -> 0.45 ms.
 #ifndef GS_BWD_MB1
 #define GS_BWD_MB1 28
 #endif
 #ifndef GS_BWD_MB2
 #define GS_BWD_MB2 20
 #endif
-#ifndef GS_BWD_MB3
-#define GS_BWD_MB3 20
-#endif
-__host__ __device__ constexpr int bwd_min_blocks(int S) { return S == 1 ? GS_BWD_MB1 : S == 2 ? GS_BWD_MB2 : GS_BWD_MB3; }
+__host__ __device__ constexpr int bwd_min_blocks(int S) { return S == 1 ? GS_BWD_MB1 : GS_BWD_MB2; }
 
 // Row stride (floats) of the per-view 2-D cotangents: 9 per stream, padded to
 // whole float4s so that rows can be added and read as vectors.
@@ -509,20 +507,187 @@ __device__ __forceinline__ void red_add4(float* p, float4 v) {
                : "memory");
 }
 
-// Shared memory of one warp's merge of the partial derivatives (see
-// raster_bwd_kernel): kMergeSlots splats' per-pixel values, S + 1 pairs per
-// lane, and the negated cotangents -w of the warp's pixels, 3 S pairs per lane
-// at a stride (in pairs) that keeps eight consecutive lanes on distinct banks.
-// A slot holds the values of the last two streams, side by side, then the first
-// one's (of an odd number) beside -a T, or -a T alone.
+// The cotangents dL/dC of each stream at the thread's two pixels, of the block whose
+// first pixel is (bx0, by0), and their transmittance and list end (none of an empty
+// list, len = 0); returns the objective's terms there.
+template <int NU, bool GRAD>
+__device__ __forceinline__ float bwd_pixels(BwdPair<(GRAD ? 1 : 0) + NU>& pp, int bx0, int by0, int view, uint32_t len,
+                                            const gs_frame& fr, const float* __restrict__ image,
+                                            const float* __restrict__ target, const float* __restrict__ final_T,
+                                            const uint32_t* __restrict__ n_contrib,
+                                            const float* __restrict__ image_tan, int loss_kind, float gn_floor,
+                                            float inv_m) {
+  constexpr int S = (GRAD ? 1 : 0) + NU;
+  const int lane = threadIdx.x & 31;
+  const size_t HW = (size_t)fr.width * fr.height;
+  float lossp = 0.f;
+  float wv[kPixPerThread][S][3], Tv[kPixPerThread], pyc[kPixPerThread];
+#pragma unroll
+  for (int q = 0; q < kPixPerThread; ++q) {
+    const int px = bx0 + (lane & 7), py = by0 + (lane >> 3) + 4 * q;
+    pp.pxc = (float)px + 0.5f;
+    pyc[q] = (float)py + 0.5f;
+    Tv[q] = 0.f;
+    pp.nc[q] = 0;
+#pragma unroll
+    for (int st = 0; st < S; ++st) wv[q][st][0] = wv[q][st][1] = wv[q][st][2] = 0.f;
+    if (!(px < fr.width && py < fr.height)) continue;
+    const size_t at0 = (size_t)py * fr.width + px;
+    if (len) {
+      Tv[q] = final_T[(size_t)view * HW + at0];
+      pp.nc[q] = n_contrib[(size_t)view * HW + at0];
+    }
+    if (loss_kind == GS_LOSS_COTANGENT) {  // the caller's cotangent images, one per stream
+#pragma unroll
+      for (int st = 0; st < S; ++st)
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch)
+          wv[q][st][ch] = target[(((size_t)st * fr.n_views + view) * 3 + ch) * HW + at0];
+      continue;
+    }
+    if (loss_kind == GS_LOSS_WEIGHTED) {  // dL/dC (gradient stream), then the weights of w . J z_k
+      const float* wimg = target + (GRAD ? (size_t)fr.n_views * 3 * HW : 0);
+#pragma unroll
+      for (int ch = 0; ch < 3; ++ch) {
+        if constexpr (GRAD) wv[q][0][ch] = target[((size_t)view * 3 + ch) * HW + at0];
+        const float wt = wimg[((size_t)view * 3 + ch) * HW + at0];
+#pragma unroll
+        for (int k = 0; k < NU; ++k)
+          wv[q][(GRAD ? 1 : 0) + k][ch] = wt * image_tan[(((size_t)k * fr.n_views + view) * 3 + ch) * HW + at0];
+      }
+      continue;
+    }
+#pragma unroll
+    for (int ch = 0; ch < 3; ++ch) {
+      const size_t at = ((size_t)view * 3 + ch) * HW + at0;
+      const float r = image[at] - target[at];
+      const float ar = fabsf(r);
+      float lam;
+      if (loss_kind == GS_LOSS_L1) {
+        lossp += 0.5f * inv_m * ar;
+        lam = 0.25f / fmaxf(ar, gn_floor);
+      } else {
+        lossp += 0.5f * inv_m * r * r;
+        lam = 1.f;
+      }
+      if constexpr (GRAD)
+        wv[q][0][ch] = (loss_kind == GS_LOSS_L1) ? (0.5f * inv_m) * ((r > 0.f) - (r < 0.f)) : inv_m * r;
+#pragma unroll
+      for (int k = 0; len && k < NU; ++k)
+        wv[q][(GRAD ? 1 : 0) + k][ch] =
+            inv_m * lam * image_tan[(((size_t)k * fr.n_views + view) * 3 + ch) * HW + at0];
+    }
+  }
+  pp.T = pack2(Tv[0], Tv[1]);
+  pp.npy = pack2(-pyc[0], -pyc[1]);
+  pp.ns[0] = pp.ns[1] = pp.ns[2] = 0ull;
+#pragma unroll
+  for (int st = 0; st < S; ++st) {
+#pragma unroll
+    for (int ch = 0; ch < 3; ++ch) {
+      pp.nw[st][ch] = pack2(-wv[0][st][ch], -wv[1][st][ch]);
+    }
+  }
+  return lossp;
+}
+
+// Adds the warp's terms to the objective's sums (see CotHeader).
+__device__ __forceinline__ void add_block_loss(float lossp, int slot, CotHeader* cot_hdr) {
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) lossp += __shfl_xor_sync(0xffffffffu, lossp, o);
+  if ((threadIdx.x & 31) == 0 && lossp != 0.f) atomicAdd(&cot_hdr->loss[slot], (double)lossp);
+}
+
+// One splat, at list position pos, at the thread's two pixels: which blend it, the
+// g = dL/d(power) of each stream and -a T, and the pixels' state in front of it.
+// Returns the lanes that blend it (0: nothing else is set).
+template <int S>
+__device__ __forceinline__ uint32_t bwd_visit(BwdPair<S>& pp, const Rec& r, uint32_t pos, bool (&on)[2], float& dx,
+                                              f32x2& dy, f32x2 (&gp)[S], f32x2& naT) {
+  float power[2], oG[2], na[2], ac[2], om[2];
+  f32x2 G;
+  splat_gauss2(r, pp.pxc, pp.npy, dx, dy, power, G);
+  unpack2(mul2(dup2(r.b.y), G), oG[0], oG[1]);
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const float al = fminf(kAlphaMax, oG[q]);
+    on[q] = pos < pp.nc[q] && power[q] <= 0.f && al >= kAlphaMin;
+    na[q] = on[q] ? -al : 0.f;
+    ac[q] = on[q] && !(oG[q] > kAlphaMax) ? -al : 0.f;  // a capped alpha has zero derivative
+  }
+  const uint32_t act = __ballot_sync(0xffffffffu, on[0] || on[1]);
+  if (!act) return 0u;
+  // recover T_i = T_{i+1} / (1 - a); dC/da = c T_i - suffix / (1 - a), and
+  // dL/d(power) = a (w . dC/da) per stream.  A pixel that does not blend the
+  // splat has a = 0: its state stays as it is and it contributes exact zeros.
+  const f32x2 nap = pack2(na[0], na[1]);
+  unpack2(add2(dup2(1.f), nap), om[0], om[1]);
+  const f32x2 inv = pack2(rcp_approx(om[0]), rcp_approx(om[1]));
+  const f32x2 Ti = mul2(pp.T, inv), nac = pack2(ac[0], ac[1]);
+  naT = mul2(nap, Ti);
+  const float rgb[3] = {r.b.z, r.b.w, r.c.x};
+  f32x2 da[3];
+#pragma unroll
+  for (int ch = 0; ch < 3; ++ch) {
+    da[ch] = fma2(dup2(rgb[ch]), Ti, mul2(pp.ns[ch], inv));
+    pp.ns[ch] = fma2(dup2(rgb[ch]), naT, pp.ns[ch]);
+  }
+#pragma unroll
+  for (int s = 0; s < S; ++s)
+    gp[s] = mul2(fma2(pp.nw[s][2], da[2], fma2(pp.nw[s][0], da[0], mul2(pp.nw[s][1], da[1]))), nac);
+  pp.T = Ti;
+  return act;
+}
+
+// A splat that at most this many lanes blend is added by those lanes, each the row
+// of its two pixels, instead of through the sums over the block: part of the fixed
+// order too (a quarter of the splats that a block blends; without it raster_bwd_kernel
+// takes 1.557 instead of 1.584 ms with no probe, 2.425 instead of 2.378 with one).
+constexpr int kSparseLanes = 8;
+// The row of a lane's two pixels: their products summed in one fused operation.
+template <int S>
+__device__ __forceinline__ void lane_row(const f32x2 (&gp)[S], f32x2 naT, const f32x2 (&nw)[S][3], float dx, f32x2 dy,
+                                         float* v) {
+  float y0, y1, t0, t1;
+  unpack2(dy, y0, y1);
+  unpack2(naT, t0, t1);
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    float g0, g1;
+    unpack2(gp[s], g0, g1);
+    v[cot_index(S, s, 0)] = fmaf(dx, g1, __fmul_rn(dx, g0));
+    v[cot_index(S, s, 1)] = fmaf(y1, g1, __fmul_rn(y0, g0));
+    v[cot_index(S, s, 2)] = fmaf(__fmul_rn(dx, dx), g1, __fmul_rn(__fmul_rn(dx, dx), g0));
+    v[cot_index(S, s, 3)] = fmaf(__fmul_rn(dx, y1), g1, __fmul_rn(__fmul_rn(dx, y0), g0));
+    v[cot_index(S, s, 4)] = fmaf(__fmul_rn(y1, y1), g1, __fmul_rn(__fmul_rn(y0, y0), g0));
+    v[cot_index(S, s, 5)] = g0 + g1;
+#pragma unroll
+    for (int ch = 0; ch < 3; ++ch) {
+      float w0, w1;
+      unpack2(nw[s][ch], w0, w1);
+      v[cot_index(S, s, 6 + ch)] = fmaf(w1, t1, __fmul_rn(w0, t0));
+    }
+  }
+#pragma unroll
+  for (int k = 9 * S; k < cot_stride(S); ++k) v[k] = 0.f;
+}
+template <int S>
+__device__ __forceinline__ void add_lane(const f32x2 (&gp)[S], f32x2 naT, const f32x2 (&nw)[S][3], float dx, f32x2 dy,
+                                         float* __restrict__ row) {
+  float v[cot_stride(S)];
+  lane_row<S>(gp, naT, nw, dx, dy, v);
+#pragma unroll
+  for (int k = 0; k < cot_stride(S); k += 4) red_add4(row + k, make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]));
+}
+
+// Shared memory of one warp's merge of the partial derivatives of one or two
+// streams (see raster_bwd_kernel): kMergeSlots splats' per-pixel values, S + 1 pairs
+// per lane, and the negated cotangents -w of the warp's pixels, 3 S pairs per lane.
+// A slot holds g of one stream beside -a T, or of two side by side, then -a T.
 constexpr int kMergeSlots = 4;
 __host__ __device__ constexpr int merge_slot_pairs(int S) { return 32 * (S + 1); }
-__host__ __device__ constexpr int merge_w_stride(int S) { return S == 1 ? 3 : S == 2 ? 6 : 10; }
+__host__ __device__ constexpr int merge_w_stride(int S) { return 3 * S; }
 __host__ __device__ constexpr int merge_pairs(int S) { return kMergeSlots * merge_slot_pairs(S) + 32 * merge_w_stride(S); }
-
-// Where a column's float4s of the second part lie, so that eight lanes' are on
-// distinct banks (of the first part, and of one stream, 12 floats apart, they are).
-__host__ __device__ constexpr int part_swizzle(int S, int x) { return S == 1 ? 0 : S == 2 ? x >> 2 : x >> 1; }
 
 // The merge of up to kMergeSlots splats of one warp into their cotangent rows.
 // A row's entries per stream are the sums over pixels of (dx, dy, dx^2, dx dy,
@@ -537,24 +702,24 @@ __host__ __device__ constexpr int part_swizzle(int S, int x) { return S == 1 ? 0
 // pixel's product is added to that of the pixel four rows below it (one fused
 // operation), then rows y and y + 2, rows y and y + 1, columns x and x + 4, x and
 // x + 1, x and x + 2; the pixels' g come from the suffix of each colour.  Summing
-// whole columns first and keeping one suffix per stream took 2.60 ms instead of
-// 2.83 (two probes), and moved single entries of the gradient by 1e-3 of its root
-// mean square, up to eight times what repeats differ by.
+// whole columns first and keeping one suffix per stream took 1.40 and 2.02 ms
+// instead of 1.56 and 2.38 (no probe and one), and moved single entries of the
+// gradient by 1e-3 of its root mean square.
 // Lanes 8 s .. 8 s + 7 sum splat s, lane & 7 the column of the 8 x 8 block.  A lane
-// holds rows (0, 1), (2, 3), (4, 5), (6, 7) as pairs, first of the last two
-// streams, whose sums it writes over their slots' values, then of the rest, so
-// that half the row is live at a time; lane (s, quad) then adds the eight columns
-// of its four entries and issues one float4 reduction.  Against a reduce-scatter
-// of the 9 S values over the warp per splat (128 instructions of 290 per splat and
-// block with two probes) a merge costs about 70 per splat; the blend's bounds are
-// the path to shared memory (68 % of its wavefronts) and issue slots (57 %).
+// holds rows (0, 1), (2, 3), (4, 5), (6, 7) as pairs, with two streams first their
+// moments, which it writes over the slots' values, then the colours, so that half
+// the row is live at a time; lane (s, quad) then adds the eight columns of its four
+// entries and issues one float4 reduction.
 // smx, smy, sgi: mean and index of the lane's splat; count: slots in use.
 template <int S>
 __device__ __forceinline__ void merge_slots(f32x2* slots, const f32x2* sw, int count, float wx0, float wy0, float smx,
                                             float smy, uint32_t sgi, float* __restrict__ cot_view) {
   constexpr int NVP = cot_stride(S), NQ = NVP / 4;
-  constexpr int kA = S >= 2 ? 12 : 0, kB = NVP - kA;  // floats of a column's first and second part
+  static_assert(S <= 2, "streams");
+  constexpr int kA = S == 2 ? 12 : 0, kB = NVP - kA;  // floats of a column's first and second part
   constexpr int kQA = kA / 4, kQB = kB / 4;
+  // two float4s 8 floats apart: swapped in columns 4..7, so that eight lanes' are on distinct banks
+  auto swizzle = [](int col) { return S == 2 ? col >> 2 : 0; };
   const int lane = threadIdx.x & 31, sl = lane >> 3, x = lane & 7;
   f32x2* my = slots + sl * merge_slot_pairs(S);
   float* rows = reinterpret_cast<float*>(my);
@@ -579,7 +744,7 @@ __device__ __forceinline__ void merge_slots(f32x2* slots, const f32x2* sw, int c
     m[5] = sum2(add2(add2(g0, g1), add2(g2, g3)));
   };
   __syncwarp();
-  if constexpr (S >= 2) {  // the moments of the last two streams
+  if constexpr (S == 2) {  // the moments of two streams
     float lo[2][4], hi[2][4], m[2][6];
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
@@ -605,8 +770,8 @@ __device__ __forceinline__ void merge_slots(f32x2* slots, const f32x2* sw, int c
     for (int r = 0; r < 4; ++r) {
       const int at = r * 8 + x;
       f32x2 naT;
-      if constexpr (S % 2) {
-        const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(my + 32 * (S - 1) + 2 * at);
+      if constexpr (S == 1) {
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(my + 2 * at);
         unpack2(t.x, lo[r], hi[r]);
         naT = t.y;
       } else {
@@ -614,8 +779,8 @@ __device__ __forceinline__ void merge_slots(f32x2* slots, const f32x2* sw, int c
       }
       const f32x2* wp = sw + at * merge_w_stride(S);
 #pragma unroll
-      for (int k = 0; k < 3 * S; k += S == 1 ? 1 : 2) {
-        if (S == 1 || k + 1 >= 3 * S) {
+      for (int k = 0; k < 3 * S; k += S) {
+        if constexpr (S == 1) {
           c[k] = fma2(naT, wp[k], c[k]);
         } else {
           const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(wp + k);
@@ -628,7 +793,7 @@ __device__ __forceinline__ void merge_slots(f32x2* slots, const f32x2* sw, int c
     for (int s = 0; s < S; ++s)
 #pragma unroll
       for (int ch = 0; ch < 3; ++ch) b[cot_index(S, s, 6 + ch) - kA] = sum2(c[3 * s + ch]);
-    if constexpr (S % 2) {
+    if constexpr (S == 1) {
       float m[6];
       moments(lo, hi, m);
 #pragma unroll
@@ -639,16 +804,16 @@ __device__ __forceinline__ void merge_slots(f32x2* slots, const f32x2* sw, int c
     __syncwarp();  // every lane has read these values
 #pragma unroll
     for (int q = 0; q < kQB; ++q)
-      *reinterpret_cast<float4*>(rows + 128 * (S >= 2) + x * kB + 4 * (q ^ part_swizzle(S, x))) =
+      *reinterpret_cast<float4*>(rows + 128 * (S - 1) + x * kB + 4 * (q ^ swizzle(x))) =
           make_float4(b[4 * q], b[4 * q + 1], b[4 * q + 2], b[4 * q + 3]);
   }
   __syncwarp();
   if (x < NQ && sl < count) {  // quad x of the lane's own splat
     const bool first = x < kQA;
-    const float* part = rows + (first ? 4 * x : 128 * (S >= 2));
+    const float* part = rows + (first ? 4 * x : 128 * (S - 1));
     const int stride = first ? kA : kB;
     auto quad = [&](int k) {
-      return *reinterpret_cast<const ulonglong2*>(part + k * stride + (first ? 0 : 4 * ((x - kQA) ^ part_swizzle(S, k))));
+      return *reinterpret_cast<const ulonglong2*>(part + k * stride + (first ? 0 : 4 * ((x - kQA) ^ swizzle(k))));
     };
     f32x2 a[2], b[2];
 #pragma unroll
@@ -667,12 +832,12 @@ __device__ __forceinline__ void merge_slots(f32x2* slots, const f32x2* sw, int c
 }
 
 // A lane's cotangents from shared memory; volatile, so that they are read here and
-// not held in registers across a merge (spilled there, they cost the call 0.45 ms).
+// not held in registers across a merge, where they would be spilled.
 template <int S>
 __device__ __forceinline__ void load_w(f32x2 (&nw)[S][3], const f32x2* sw) {
 #pragma unroll
   for (int k = 0; k < 3 * S; ++k) {
-    if (S == 1 || k + 1 >= 3 * S) {
+    if constexpr (S == 1) {
       asm volatile("ld.shared.b64 %0, [%1];" : "=l"(nw[k / 3][k % 3]) : "r"(smem_u32(sw + k)));
     } else if (k % 2 == 0) {
       asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];"
@@ -681,43 +846,6 @@ __device__ __forceinline__ void load_w(f32x2 (&nw)[S][3], const f32x2* sw) {
     }
   }
 }
-// A splat that at most this many lanes blend is added by those lanes, each the row
-// of its two pixels, instead of through the merge: part of the fixed order too (a
-// quarter of the splats that a block blends; without it the call of 1M Gaussians and
-// 8 views takes 1.557 instead of 1.584 ms with no probe, 2.425 instead of 2.378 with
-// one, 2.924 instead of 2.824 with two).
-constexpr int kSparseLanes = 8;
-template <int S>
-__device__ __forceinline__ void add_lane(const f32x2 (&gp)[S], f32x2 naT, const f32x2 (&nw)[S][3], float dx, f32x2 dy,
-                                         float* __restrict__ row) {
-  constexpr int NVP = cot_stride(S);
-  float y0, y1, t0, t1;
-  unpack2(dy, y0, y1);
-  unpack2(naT, t0, t1);
-  float v[NVP];
-#pragma unroll
-  for (int s = 0; s < S; ++s) {
-    float g0, g1;
-    unpack2(gp[s], g0, g1);
-    v[cot_index(S, s, 0)] = fmaf(dx, g1, __fmul_rn(dx, g0));
-    v[cot_index(S, s, 1)] = fmaf(y1, g1, __fmul_rn(y0, g0));
-    v[cot_index(S, s, 2)] = fmaf(__fmul_rn(dx, dx), g1, __fmul_rn(__fmul_rn(dx, dx), g0));
-    v[cot_index(S, s, 3)] = fmaf(__fmul_rn(dx, y1), g1, __fmul_rn(__fmul_rn(dx, y0), g0));
-    v[cot_index(S, s, 4)] = fmaf(__fmul_rn(y1, y1), g1, __fmul_rn(__fmul_rn(y0, y0), g0));
-    v[cot_index(S, s, 5)] = g0 + g1;
-#pragma unroll
-    for (int ch = 0; ch < 3; ++ch) {
-      float w0, w1;
-      unpack2(nw[s][ch], w0, w1);
-      v[cot_index(S, s, 6 + ch)] = fmaf(w1, t1, __fmul_rn(w0, t0));
-    }
-  }
-#pragma unroll
-  for (int k = 9 * S; k < NVP; ++k) v[k] = 0.f;
-#pragma unroll
-  for (int k = 0; k < NVP; k += 4) red_add4(row + k, make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]));
-}
-
 template <int NU, bool GRAD>
 __global__ void __launch_bounds__(32, bwd_min_blocks((GRAD ? 1 : 0) + NU)) raster_bwd_kernel(
     const float4* __restrict__ rec, const uint32_t* __restrict__ vals, const uint32_t* __restrict__ ranges,
@@ -728,7 +856,7 @@ __global__ void __launch_bounds__(32, bwd_min_blocks((GRAD ? 1 : 0) + NU)) raste
     const uint8_t* __restrict__ masks, const int32_t* status) {
   constexpr int S = (GRAD ? 1 : 0) + NU;  // cotangent streams
   constexpr int NVP = cot_stride(S);      // padded row stride of their 9 S values
-  static_assert(NVP <= 32, "streams");
+  static_assert(S <= 2, "three streams take raster_bwd_tile_kernel");
   // the merge slots, then the negated cotangents (see merge_slots), and two
   // buffers of staged records, whose last two words hold the Gaussian index
   // and the list position instead of the record's radius and extents
@@ -743,88 +871,14 @@ __global__ void __launch_bounds__(32, bwd_min_blocks((GRAD ? 1 : 0) + NU)) raste
   const size_t tslot = 2 * ((size_t)view * T + pb.tile);
   const uint32_t start = __ldg(ranges + tslot), len = __ldg(ranges + tslot + 1) - start;
   if (len == 0 && !want_loss) return;
-  const size_t HW = (size_t)fr.width * fr.height;
   const float wx0 = (float)bx0 + 0.5f, wy0 = (float)by0 + 0.5f;  // the block's first pixel centre
 
-  // per-pixel cotangents dL/dC of each stream and the loss
   BwdPair<S> pp;
-  float lossp = 0.f;
-  {
-    float wv[kPixPerThread][S][3], Tv[kPixPerThread], pyc[kPixPerThread];
+  const float lossp = bwd_pixels<NU, GRAD>(pp, bx0, by0, view, len, fr, image, target, final_T, n_contrib, image_tan,
+                                           loss_kind, gn_floor, inv_m);
 #pragma unroll
-    for (int q = 0; q < kPixPerThread; ++q) {
-      const int px = bx0 + (lane & 7), py = by0 + (lane >> 3) + 4 * q;
-      pp.pxc = (float)px + 0.5f;
-      pyc[q] = (float)py + 0.5f;
-      Tv[q] = 0.f;
-      pp.nc[q] = 0;
-#pragma unroll
-      for (int st = 0; st < S; ++st) wv[q][st][0] = wv[q][st][1] = wv[q][st][2] = 0.f;
-      if (!(px < fr.width && py < fr.height)) continue;
-      const size_t at0 = (size_t)py * fr.width + px;
-      if (len) {
-        Tv[q] = final_T[(size_t)view * HW + at0];
-        pp.nc[q] = n_contrib[(size_t)view * HW + at0];
-      }
-      if (loss_kind == GS_LOSS_COTANGENT) {  // the caller's cotangent images, one per stream
-#pragma unroll
-        for (int st = 0; st < S; ++st)
-#pragma unroll
-          for (int ch = 0; ch < 3; ++ch)
-            wv[q][st][ch] = target[(((size_t)st * fr.n_views + view) * 3 + ch) * HW + at0];
-        continue;
-      }
-      if (loss_kind == GS_LOSS_WEIGHTED) {  // dL/dC (gradient stream), then the weights of w . J z_k
-        const float* wimg = target + (GRAD ? (size_t)fr.n_views * 3 * HW : 0);
-#pragma unroll
-        for (int ch = 0; ch < 3; ++ch) {
-          if constexpr (GRAD) wv[q][0][ch] = target[((size_t)view * 3 + ch) * HW + at0];
-          const float wt = wimg[((size_t)view * 3 + ch) * HW + at0];
-#pragma unroll
-          for (int k = 0; k < NU; ++k)
-            wv[q][(GRAD ? 1 : 0) + k][ch] = wt * image_tan[(((size_t)k * fr.n_views + view) * 3 + ch) * HW + at0];
-        }
-        continue;
-      }
-#pragma unroll
-      for (int ch = 0; ch < 3; ++ch) {
-        const size_t at = ((size_t)view * 3 + ch) * HW + at0;
-        const float r = image[at] - target[at];
-        const float ar = fabsf(r);
-        float lam;
-        if (loss_kind == GS_LOSS_L1) {
-          lossp += 0.5f * inv_m * ar;
-          lam = 0.25f / fmaxf(ar, gn_floor);
-        } else {
-          lossp += 0.5f * inv_m * r * r;
-          lam = 1.f;
-        }
-        if constexpr (GRAD)
-          wv[q][0][ch] = (loss_kind == GS_LOSS_L1) ? (0.5f * inv_m) * ((r > 0.f) - (r < 0.f)) : inv_m * r;
-#pragma unroll
-        for (int k = 0; len && k < NU; ++k)
-          wv[q][(GRAD ? 1 : 0) + k][ch] =
-              inv_m * lam * image_tan[(((size_t)k * fr.n_views + view) * 3 + ch) * HW + at0];
-      }
-    }
-    pp.T = pack2(Tv[0], Tv[1]);
-    pp.npy = pack2(-pyc[0], -pyc[1]);
-    pp.ns[0] = pp.ns[1] = pp.ns[2] = 0ull;
-#pragma unroll
-    for (int st = 0; st < S; ++st) {
-#pragma unroll
-      for (int ch = 0; ch < 3; ++ch) {
-        pp.nw[st][ch] = pack2(-wv[0][st][ch], -wv[1][st][ch]);
-        s_w[lane * merge_w_stride(S) + 3 * st + ch] = pp.nw[st][ch];
-      }
-    }
-  }
-  if (want_loss) {
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) lossp += __shfl_xor_sync(0xffffffffu, lossp, o);
-    if (lane == 0 && lossp != 0.f)
-      atomicAdd(&cot_hdr->loss[loss_per_view ? view : (int)(blockIdx.x % kLossSlots)], (double)lossp);
-  }
+  for (int k = 0; k < 3 * S; ++k) s_w[lane * merge_w_stride(S) + k] = pp.nw[k / 3][k % 3];
+  if (want_loss) add_block_loss(lossp, loss_per_view ? view : (int)(blockIdx.x % kLossSlots), cot_hdr);
   // list positions this block still needs (n_contrib never exceeds the tile's
   // list); none after a wait that ran out in an earlier call
   const uint32_t nw = min(__reduce_max_sync(0xffffffffu, max(pp.nc[0], pp.nc[1])), len);
@@ -893,38 +947,11 @@ __global__ void __launch_bounds__(32, bwd_min_blocks((GRAD ? 1 : 0) + NU)) raste
     for (int j = 0; j < cnt; ++j) {
       const Rec r = buf[cur][j];
       const uint32_t pos = __float_as_uint(r.c.w);
-      float dx, power[2], oG[2], na[2], ac[2], om[2];
-      f32x2 dy, G;
-      splat_gauss2(r, pp.pxc, pp.npy, dx, dy, power, G);
-      unpack2(mul2(dup2(r.b.y), G), oG[0], oG[1]);
       bool on[2];
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const float al = fminf(kAlphaMax, oG[q]);
-        on[q] = pos < pp.nc[q] && power[q] <= 0.f && al >= kAlphaMin;
-        na[q] = on[q] ? -al : 0.f;
-        ac[q] = on[q] && !(oG[q] > kAlphaMax) ? -al : 0.f;  // a capped alpha has zero derivative
-      }
-      const uint32_t act = __ballot_sync(0xffffffffu, on[0] || on[1]);
+      float dx;
+      f32x2 dy, gp[S], naT;
+      const uint32_t act = bwd_visit<S>(pp, r, pos, on, dx, dy, gp, naT);
       if (!act) continue;
-      // recover T_i = T_{i+1} / (1 - a); dC/da = c T_i - suffix / (1 - a), and
-      // dL/d(power) = a (w . dC/da) per stream.  A pixel that does not blend the
-      // splat has a = 0: its state stays as it is and it contributes exact zeros.
-      const f32x2 nap = pack2(na[0], na[1]);
-      unpack2(add2(dup2(1.f), nap), om[0], om[1]);
-      const f32x2 inv = pack2(rcp_approx(om[0]), rcp_approx(om[1]));
-      const f32x2 Ti = mul2(pp.T, inv), nac = pack2(ac[0], ac[1]), naT = mul2(nap, Ti);
-      const float rgb[3] = {r.b.z, r.b.w, r.c.x};
-      f32x2 gp[S], da[3];
-#pragma unroll
-      for (int ch = 0; ch < 3; ++ch) {
-        da[ch] = fma2(dup2(rgb[ch]), Ti, mul2(pp.ns[ch], inv));
-        pp.ns[ch] = fma2(dup2(rgb[ch]), naT, pp.ns[ch]);
-      }
-#pragma unroll
-      for (int s = 0; s < S; ++s)
-        gp[s] = mul2(fma2(pp.nw[s][2], da[2], fma2(pp.nw[s][0], da[0], mul2(pp.nw[s][1], da[1]))), nac);
-      pp.T = Ti;
       if (__popc(act) <= kSparseLanes) {
         if (on[0] || on[1])
           add_lane<S>(gp, naT, pp.nw, dx, dy, cot_view + (size_t)__float_as_uint(r.c.z) * NVP);
@@ -932,9 +959,12 @@ __global__ void __launch_bounds__(32, bwd_min_blocks((GRAD ? 1 : 0) + NU)) raste
       }
       // the lane's values of this splat into its merge slot
       f32x2* my = slots + used * merge_slot_pairs(S);
-      if constexpr (S >= 2) *reinterpret_cast<ulonglong2*>(my + 2 * lane) = make_ulonglong2(gp[S - 2], gp[S - 1]);
-      if constexpr (S % 2) *reinterpret_cast<ulonglong2*>(my + 32 * (S - 1) + 2 * lane) = make_ulonglong2(gp[0], naT);
-      else my[64 + lane] = naT;
+      if constexpr (S == 1) {
+        *reinterpret_cast<ulonglong2*>(my + 2 * lane) = make_ulonglong2(gp[0], naT);
+      } else {
+        *reinterpret_cast<ulonglong2*>(my + 2 * lane) = make_ulonglong2(gp[0], gp[1]);
+        my[64 + lane] = naT;
+      }
       if ((lane >> 3) == used) {
         smx = r.a.x;
         smy = r.a.y;
@@ -952,6 +982,212 @@ __global__ void __launch_bounds__(32, bwd_min_blocks((GRAD ? 1 : 0) + NU)) raste
     cnt = cnt_next;
   }
   if (used) merge_slots<S>(slots, s_w, used, wx0, wy0, smx, smy, sgi, cot_view);
+}
+
+// ------------------------------------------------ reverse, three streams
+// A CTA per tile, a warp per 8 x 8 block.  The warps share a ring of kBwdStages
+// batches (one record per thread) that they release one by one: a warp moves on as
+// soon as a batch has landed and reads only the splats its block sees; the last warp
+// to release a buffer refills it with the batch kBwdStages further on.  So a
+// tile's warps walk its list in step, and the order in which their blocks add to a
+// splat's row is nearly the same in every run.  With a warp per CTA (raster_bwd_kernel's
+// way, 2.83 ms for 1M Gaussians, 8 views of 1080p) near ties between blocks went
+// either way: the rotation of a nearly round splat, whose terms cancel to 1e-5 of
+// their size, moved by 3e-4 of itself between a request alone and the same one in a
+// batch; here by less than a tenth of that in 250 runs.  With one stream or two the
+// same comparison moves by a twentieth of that, and the walk in step takes 2.00
+// instead of 1.56 ms (no probe) and 2.67 instead of 2.38 (one).
+// Sums over the block are a reduce-scatter over the warp (the order of
+// merge_slots).  Scalar pixels and 7 CTAs took 3.40 ms; pairs 2.94 at 8 CTAs per SM
+// (64 registers, 24 bytes of spills; 7: 3.09, 6: 3.19).  In 16 x 32 tiles 3.17.
+constexpr int kBwdStages = 3;
+#ifndef GS_BWD_TILE_MB
+#define GS_BWD_TILE_MB 8
+#endif
+// ring header: one mbarrier and one release counter per stage, 16-byte aligned
+constexpr size_t kBwdRingHdr = (kBwdStages * (sizeof(uint64_t) + sizeof(uint32_t)) + 15) / 16 * 16;
+__host__ __device__ constexpr size_t bwd_ring_bytes(int batch) {
+  return kBwdRingHdr + (size_t)kBwdStages * batch * (sizeof(Rec) + sizeof(uint32_t)) +
+         ((size_t)kBwdStages * batch + 15) / 16 * 16;  // and the staged block masks, one byte per record
+}
+
+// The calling warp fills ring stage s with batch b of the list (use u of the
+// ring): its lanes store the Gaussian indices (and, given the forward pass's
+// block masks, each record's mask byte) and issue one bulk copy per record,
+// then lane 0 records u as the stage's last fill and arms the stage's barrier
+// with the byte count.  The copies may complete before that arrival (the
+// phase cannot complete while the arrival is pending), and the arrival releases
+// the index stores to the warps that wait on the phase.
+__device__ __forceinline__ void stage_batch_warp(int s, int u, int b, int batch, uint32_t start, int n, int view,
+                                                 int n_pad, const uint32_t* __restrict__ vals,
+                                                 const float4* __restrict__ rec, const uint8_t* __restrict__ masks,
+                                                 Rec* buf, uint32_t* s_idx, uint8_t* s_bits, uint64_t* full,
+                                                 int* fill_use) {
+  const int lane = threadIdx.x & 31;
+  const int cnt = min(batch, n - b * batch);
+  __syncwarp();
+  fence_proxy_async();  // the ring slot's earlier reads come before the copies' writes
+  for (int q = lane; q < cnt; q += 32) {
+    const uint32_t gi = __ldg(vals + start + (uint32_t)(b * batch + q));
+    s_idx[s * batch + q] = gi;
+    if (masks) s_bits[s * batch + q] = __ldg(masks + start + (uint32_t)(b * batch + q));
+    bulk_g2s(&buf[s * batch + q], rec + 3 * ((size_t)view * n_pad + gi), sizeof(Rec), &full[s]);
+  }
+  __syncwarp();
+  if (lane == 0) {
+    fill_use[s] = u;
+    mbar_arrive_expect_tx(&full[s], (uint32_t)(cnt * (int)sizeof(Rec)));
+  }
+}
+
+// Warp sums of v[0..31] delivered as quads: afterwards every lane L with
+// (L & 3) == 0 holds in q[0..3] the warp-wide sums of v[L .. L+3].  Three
+// reduce-scatter stages (lane bits 4, 3, 2) then a butterfly over bits 1, 0.
+__device__ __forceinline__ void warp_reduce_quads(float (&v)[32], float (&q)[4]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 16; o >= 4; o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < o; ++i) {
+      const float send = up ? v[i] : v[i + o];
+      const float keep = up ? v[i + o] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float x = v[i];
+    x += __shfl_xor_sync(0xffffffffu, x, 1);
+    x += __shfl_xor_sync(0xffffffffu, x, 2);
+    q[i] = x;
+  }
+}
+
+template <int NU, bool GRAD, int NT>
+__global__ void __launch_bounds__(NT, GS_BWD_TILE_MB * 128 / NT) raster_bwd_tile_kernel(
+    const float4* __restrict__ rec, const uint32_t* __restrict__ vals, const uint32_t* __restrict__ ranges,
+    const uint32_t* __restrict__ order, int n_pad, gs_frame fr, int Tx, int T, const float* __restrict__ image,
+    const float* __restrict__ target, const float* __restrict__ final_T, const uint32_t* __restrict__ n_contrib,
+    const float* __restrict__ image_tan, int loss_kind, float gn_floor, float inv_m, float* __restrict__ cot,
+    bool want_loss, bool loss_per_view, CotHeader* cot_hdr, const uint8_t* __restrict__ masks, int32_t* status) {
+  constexpr int S = (GRAD ? 1 : 0) + NU, NVP = cot_stride(S), K = kBwdStages;
+  static_assert(NVP <= 32, "streams");
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int nthr = blockDim.x, nwarps = nthr >> 5, batch = nthr;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem);                             // K phase barriers
+  uint32_t* released = reinterpret_cast<uint32_t*>(smem + K * sizeof(uint64_t));  // K release counters
+  Rec* buf = reinterpret_cast<Rec*>(smem + kBwdRingHdr);
+  uint32_t* s_idx = reinterpret_cast<uint32_t*>(buf + K * batch);
+  uint8_t* s_bits = reinterpret_cast<uint8_t*>(s_idx + K * batch);  // block masks of the staged records
+  __shared__ uint32_t s_max;
+  __shared__ int s_abort;
+  __shared__ int s_fill_use[K];  // ring use of each stage's last fill (-1: none)
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // the tile of this block: the heaviest tiles first when an order is given
+  const int blk = order ? (int)min(__ldg(order + blockIdx.x), gridDim.x - 1) : (int)blockIdx.x;
+  const int view = blk / T, tile = blk - view * T, ty = tile / Tx, tx = tile - ty * Tx, bw = fr.tile_w >> 3;
+  const int bx0 = tx * fr.tile_w + (warp % bw) * 8, by0 = ty * fr.tile_h + (warp / bw) * 8;
+  const size_t tslot = 2 * ((size_t)view * T + tile);
+  const uint32_t start = __ldg(ranges + tslot), len = __ldg(ranges + tslot + 1) - start;
+  if (blockIdx.x == 0 && tid == 0) cot_hdr->clear_floats = 0;  // the rows are being added into
+  if (len == 0 && !want_loss) return;
+  const float wx0 = (float)bx0 + 0.5f, wy0 = (float)by0 + 0.5f;  // the block's first pixel centre
+  BwdPair<S> pp;
+  const float lossp = bwd_pixels<NU, GRAD>(pp, bx0, by0, view, len, fr, image, target, final_T, n_contrib, image_tan,
+                                           loss_kind, gn_floor, inv_m);
+  if (want_loss) add_block_loss(lossp, loss_per_view ? view : (int)((blockIdx.x * nwarps + warp) % kLossSlots), cot_hdr);
+  if (tid == 0) {
+    s_max = 0;
+    // a stage wait that ran out in an earlier block: skip the list walk
+    s_abort = status ? (*(volatile int32_t*)status & GS_FLAG_TIMEOUT) : 0;
+    for (int k = 0; k < K; ++k) {
+      mbar_init(&full[k], 1);
+      released[k] = 0;
+      s_fill_use[k] = -1;
+    }
+    fence_mbar_init();
+  }
+  __syncthreads();
+  const uint32_t warp_nc = __reduce_max_sync(0xffffffffu, max(pp.nc[0], pp.nc[1]));  // positions this warp needs
+  if (lane == 0 && warp_nc) atomicMax(&s_max, warp_nc);
+  __syncthreads();
+  const int n = s_abort ? 0 : (int)min(s_max, len);  // n_contrib never exceeds the tile's list
+  const int nb = (n + batch - 1) / batch;
+  // batch b is use u = nb - 1 - b of the ring: stage u % K, its (u / K)-th fill
+  for (int u = warp; u < min(K, nb); u += nwarps)
+    stage_batch_warp(u, u, nb - 1 - u, batch, start, n, view, n_pad, vals, rec, masks, buf, s_idx, s_bits, full,
+                     s_fill_use);
+  float* cot_view = cot + (size_t)view * n_pad * NVP;
+  bool ok = true;
+  for (int u = 0; u < nb; ++u) {
+    const int st = u % K, b = nb - 1 - u;
+    // every lane waits (bounded) for the stage's phase: each acquires the copies
+    // and indices.  A warp whose wait ran out stops at once: it releases no
+    // further stage, so no later round completes and nothing is refilled
+    // behind it; the other warps run into their own bounded waits.
+    const bool landed = mbar_wait_bounded(&full[st], (uint32_t)((u / K) & 1), status);
+    ok = __all_sync(0xffffffffu, landed) != 0;
+    if (!ok) break;
+    const int cnt = min(batch, n - b * batch);
+    const Rec* bb = buf + st * batch;
+    // the warp walks, back to front, only the splats its block can see (the
+    // forward pass's mask bit when given, else the same footprint test) and
+    // that lie before its last contributor: one ballot per 32 splats
+    const uint8_t* sb = s_bits + st * batch;
+    for (int j0 = ((cnt - 1) & ~31); (uint32_t)(b * batch) < warp_nc && j0 >= 0; j0 -= 32) {
+      const int jl = j0 + lane;
+      uint32_t bits = __ballot_sync(
+          0xffffffffu, jl < cnt && (uint32_t)(b * batch + jl) < warp_nc &&
+                           (masks ? ((sb[jl] >> warp) & 1u) != 0 : block_sees(bb[jl], wx0, wy0)));
+      while (bits) {
+        const int hb = 31 - __clz(bits);
+        bits &= ~(1u << hb);
+        const int j = j0 + hb;
+        const Rec r = bb[j];
+        bool on[2];
+        float dx;
+        f32x2 dy, gp[S], naT;
+        const uint32_t act = bwd_visit<S>(pp, r, (uint32_t)(b * batch + j), on, dx, dy, gp, naT);
+        if (!act) continue;
+        float* row = cot_view + (size_t)s_idx[st * batch + j] * NVP;
+        if (__popc(act) <= kSparseLanes) {
+          if (on[0] || on[1]) add_lane<S>(gp, naT, pp.nw, dx, dy, row);
+          continue;
+        }
+        float v[32], q[4];
+        lane_row<S>(gp, naT, pp.nw, dx, dy, v);
+#pragma unroll
+        for (int k = NVP; k < 32; ++k) v[k] = 0.f;
+        warp_reduce_quads(v, q);
+        if ((lane & 3) == 0 && lane < NVP && (q[0] != 0.f || q[1] != 0.f || q[2] != 0.f || q[3] != 0.f))
+          red_add4(row + lane, make_float4(q[0], q[1], q[2], q[3]));
+      }
+    }
+    // release the stage: the warp's reads of it are ordered before its count,
+    // and the last warp to count it, ordered after all counts, refills it
+    __syncwarp();
+    uint32_t last = 0;
+    if (lane == 0) {
+      __threadfence_block();
+      last = atomicAdd(&released[st], 1u) == (uint32_t)(nwarps - 1);
+      if (last) {
+        released[st] = 0;
+        __threadfence_block();
+      }
+    }
+    last = __shfl_sync(0xffffffffu, last, 0);
+    if (last && u + K < nb)
+      stage_batch_warp(st, u + K, nb - 1 - (u + K), batch, start, n, view, n_pad, vals, rec, masks, buf, s_idx,
+                       s_bits, full, s_fill_use);
+  }
+  // Drain after a failed wait: a stage is refilled only by a warp that saw its
+  // previous fill land, so each stage has at most one fill in flight, its last.
+  // One thread per stage waits (bounded) for that fill, so that no bulk copy is
+  // still writing into this block's shared memory, or completing on its
+  // barrier, when the block exits.  Without a failure every fill has landed.
+  if (__syncthreads_or(!ok) && tid < K && s_fill_use[tid] >= 0)
+    mbar_wait_bounded(&full[tid], (uint32_t)((s_fill_use[tid] / K) & 1), status);
 }
 
 // ------------------------------------------------ projection reverse pass
@@ -1604,12 +1840,22 @@ void launch_bwd_kernels(const gs_params* x, const BatchArg* ba, int n_pad, int d
   const TileGrid g = tile_grid(fr);
   const double views_per_objective = ba ? 1.0 : (double)fr.n_views;
   const float inv_m = (float)(1.0 / (3.0 * (double)fr.width * fr.height * views_per_objective));
-  const int log_blocks = log_tile_blocks(fr);
-  const unsigned blocks = (unsigned)((size_t)fr.n_views * g.T << log_blocks);
-  raster_bwd_kernel<NU, GRAD><<<blocks, 32, 0, st>>>(
-      reinterpret_cast<const float4*>(proj->rec), sorted->vals, sorted->ranges, sorted->order, n_pad, fr, g.Tx, g.T,
-      log_blocks, image, target, final_T, n_contrib, image_tan, loss.kind, loss.gn_floor, inv_m, ws.cot,
-      loss_out != nullptr, ba != nullptr, ws.hdr, sorted->masks, status);
+  const float4* rec = reinterpret_cast<const float4*>(proj->rec);
+  if constexpr (GRAD && NU == 2) {
+    const int nthr = fr.tile_w * fr.tile_h / kPixPerThread;
+    auto* kern = nthr <= 128 ? raster_bwd_tile_kernel<NU, GRAD, 128> : raster_bwd_tile_kernel<NU, GRAD, 256>;
+    kern<<<(unsigned)((size_t)fr.n_views * g.T), nthr, bwd_ring_bytes(nthr), st>>>(
+        rec, sorted->vals, sorted->ranges, sorted->order, n_pad, fr, g.Tx, g.T, image, target, final_T, n_contrib,
+        image_tan, loss.kind, loss.gn_floor, inv_m, ws.cot, loss_out != nullptr, ba != nullptr, ws.hdr, sorted->masks,
+        status);
+  } else {
+    const int log_blocks = log_tile_blocks(fr);
+    const unsigned blocks = (unsigned)((size_t)fr.n_views * g.T << log_blocks);
+    raster_bwd_kernel<NU, GRAD><<<blocks, 32, 0, st>>>(
+        rec, sorted->vals, sorted->ranges, sorted->order, n_pad, fr, g.Tx, g.T, log_blocks, image, target, final_T,
+        n_contrib, image_tan, loss.kind, loss.gn_floor, inv_m, ws.cot, loss_out != nullptr, ba != nullptr, ws.hdr,
+        sorted->masks, status);
+  }
   if (loss_out && (ba ? ba->first_block[ba->n_items] : x->n) == 0)
     add_loss_kernel<<<1, 1, 0, st>>>(ws.hdr, loss_out, ba ? ba->n_items : 0);
   if (ba) {

@@ -278,11 +278,14 @@ gs_status gs_raster_fwd(const gs_projected* proj, const gs_sorted* sorted, int32
  * (one float, may be NULL) gets the objective added.
  * workspace: device, 16-byte aligned, at least gs_raster_bwd_workspace_size
  *   bytes (a 256-byte header, then the 2-D cotangent rows the reverse blend adds
- *   into).  Any content is accepted on entry.  The call leaves the rows zero
- *   and records that in the header, so a following call on the same workspace
- *   (the same or a smaller frame) skips clearing them; otherwise the call
- *   clears them first.  The same holds for gs_hvp_diag and gs_raster_bwd_batch,
- *   which share this workspace layout. */
+ *   into).  The call leaves the rows zero and records that in the header, so a
+ *   following call on the same workspace (the same or a smaller frame) skips
+ *   clearing them; with any other header, of zeros or foreign bytes, the call
+ *   clears them first.  Memory that held a workspace, was then written to by
+ *   something else and becomes one again can still carry that record: zero its
+ *   first GS_RASTER_BWD_HEADER bytes before the first call.  The same holds for
+ *   gs_hvp_diag and gs_raster_bwd_batch, which share this workspace layout. */
+#define GS_RASTER_BWD_HEADER 256
 size_t gs_raster_bwd_workspace_size(int32_t n_pad, gs_frame frame, int32_t nu);
 gs_status gs_raster_bwd(const gs_params* x, const gs_camera* cams, gs_frame frame, const gs_projected* proj,
                         const gs_sorted* sorted, const float* image, const float* target, const float* final_T,

@@ -427,10 +427,11 @@ __host__ __device__ constexpr int cot_index(int S, int st, int k) {
 // blend adds into.  They must be zero when the blend starts.  The projection
 // reverse, which reads every row, leaves each row it read zero, and its last
 // block records in the header that the first clear_floats floats are zero;
-// the next call then clears nothing.  Any other header (a new or reused
-// buffer, a call that stopped between the blend and the projection reverse)
-// makes the next call clear the rows first; the blend marks the rows dirty
-// when it starts.
+// the next call then clears nothing.  Any other header (zeros, foreign bytes, a
+// call that stopped between the blend and the projection reverse) makes the next
+// call clear the rows first; the blend marks the rows dirty when it starts.  The
+// record is the caller's to drop (zeros over the header) where a former workspace
+// was written to by something else: only reading every row would show that.
 constexpr int kLossSlots = GS_BATCH_MAX;
 struct CotHeader {
   uint64_t magic;         // kCotClear while clear_floats is valid
@@ -440,7 +441,7 @@ struct CotHeader {
   double loss[kLossSlots];  // the objective's partial sums: of each view (a batch), or spread over the slots
 };
 constexpr uint64_t kCotClear = 0x9d2c5680a3b1f4e7ull;
-constexpr size_t kCotHeaderBytes = 256;
+constexpr size_t kCotHeaderBytes = GS_RASTER_BWD_HEADER;
 static_assert(sizeof(CotHeader) <= kCotHeaderBytes, "workspace header");
 
 // Zero the first 4 n4 floats of the rows unless the header says they are zero;

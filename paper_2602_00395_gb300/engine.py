@@ -107,6 +107,9 @@ class TRStep:
         self.order = zi(n_views * self.Tx * self.Ty, dtype=torch.int32, device=self.device)  # heaviest tiles first
         self.bwd_ws = torch.empty(G.gs_raster_bwd_workspace_size(self.n_pad, self.frame, nu), dtype=torch.uint8,
                                   device=self.device)
+        # the allocator may hand back a former workspace whose header still calls
+        # rows clear that another tensor has since written over
+        self.bwd_ws[: G.GS_RASTER_BWD_HEADER].zero_()
         self.dssim_lambda = dssim_lambda
         if dssim_lambda is not None:
             self.cot_img = torch.empty((1 + nu) * n_views * 3 * HW, dtype=torch.float32, device=self.device)
@@ -461,17 +464,20 @@ class BatchStep:
                           for b, e in enumerate(entries)]
             self.hzs = ([buf(f"hz{b}", self.rows * e.x.shape[1], f32).view(self.rows, e.x.shape[1])
                          for b, e in enumerate(entries)] if self.nu else None)
-            self.bwd_ws = buf("bwd_ws", G.gs_raster_bwd_workspace_size(self.n_pad, self.frame, self.nu), u8)
+            self.bwd_ws = buf("bwd_ws", G.gs_raster_bwd_workspace_size(self.n_pad, self.frame, self.nu), u8,
+                              G.GS_RASTER_BWD_HEADER)
 
-    def _buf(self, name: str, numel: int, dtype) -> torch.Tensor:
-        """A device buffer of numel elements: a new one, or the front of the pool's
-        buffer of that name (replaced by a larger one when too small)."""
-        if self.pool is None:
-            return torch.empty(numel, dtype=dtype, device=self.device)
-        t = self.pool.get(name)
+    def _buf(self, name: str, numel: int, dtype, zero: int = 0) -> torch.Tensor:
+        """A device buffer of numel elements: a new one (its first `zero` elements
+        zeroed), or the front of the pool's buffer of that name (replaced by a
+        larger one when too small)."""
+        t = self.pool.get(name) if self.pool is not None else None
         if t is None or t.dtype != dtype or t.numel() < numel:
-            t = torch.empty(max(numel, 1), dtype=dtype, device=self.device)
-            self.pool[name] = t
+            t = torch.empty(max(numel, 1) if self.pool is not None else numel, dtype=dtype, device=self.device)
+            if zero:
+                t[:zero].zero_()
+            if self.pool is not None:
+                self.pool[name] = t
         return t[:numel]
 
     @staticmethod

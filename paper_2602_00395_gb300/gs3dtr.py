@@ -82,6 +82,7 @@ class gs_tr_config(C.Structure):
 
 
 GS_BATCH_MAX = 16
+GS_RASTER_BWD_HEADER = 256
 
 
 class gs_batch_item(C.Structure):

@@ -627,15 +627,15 @@ def raster_bwd_flops_per_unit() -> int:
 RASTER_BWD_TRAFFIC = {
     # one-kernel captures (dram__bytes_read.sum + dram__bytes_write.sum) of the
     # reverse call's two kernels on the 2-view case of the bench scene
-    "blend_bytes": 250_807_296 + 35_321_344,        # raster_bwd_kernel
-    "projection_bytes": 460_133_888 + 448_815_360,  # project_bwd_kernel
-    "pairs": 8_580_237,                             # pairs blended in that launch
+    "blend_bytes": 281_402_624 + 41_894_656,        # raster_bwd_tile_kernel
+    "projection_bytes": 460_141_312 + 448_752_128,  # project_bwd_kernel
+    "pairs": 12_223_264,                             # pairs blended in that launch
     "n": 1_000_000,
     "views": 2,
-    "tile": (16, 32),  # a smaller tile makes more pairs for much the same bytes
+    "tile": (16, 16),  # a smaller tile makes more pairs for much the same bytes
     "sources": {
-        "paper_2602_00395_gb300/csrc/raster.cu": "a054992549162a91bf64a0914b160e353a3ec89fc032d9358fe76b398745feec",
-        "paper_2602_00395_gb300/csrc/common.cuh": "2112fcc4ef0c3d8c4eac27e66b3f9102b0f58c16da48d0c9ef64751c3d2923c7",
+        "paper_2602_00395_gb300/csrc/raster.cu": "46a73f61f08b3ed86e8c81d2417da94f7d06d37f5594586eee45ac39ac1fdb46",
+        "paper_2602_00395_gb300/csrc/common.cuh": "0383989dc8f3785d3ccd8928ff9a9607dbe2df5c528f60cd9bca8182c30eee49",
     },
 }
 
